@@ -381,7 +381,7 @@ struct Bars {
     uint64_t tfull[2];
     uint64_t tempty[2];
     uint64_t tfull2[2];
-    uint64_t mid_full;
+    uint64_t mid_full[2];  // by tile parity: a warp may finish tile j + 1 before another arrives for tile j
     uint64_t drain;
 };
 
@@ -458,7 +458,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_pass_kernel(const PassArgs a) 
             ptx::mbar_init(&bars.tempty[b], kEpiThreads);
             ptx::mbar_init(&bars.tfull2[b], 1);
         }
-        ptx::mbar_init(&bars.mid_full, kEpiThreads);
+        for (int b = 0; b < 2; ++b) ptx::mbar_init(&bars.mid_full[b], kEpiThreads);
         ptx::mbar_init(&bars.drain, 1);
         ptx::fence_mbar_init();
         s_abort = 0;
@@ -508,7 +508,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_pass_kernel(const PassArgs a) 
                     // inverse of tile j: its mid operand sits in tile j's own A stage
                     const int j = it - 1, b = j & 1, sj = j % S;
                     const long long tw = KX_CLK_NOW();
-                    ok = wait_bar(&bars.mid_full, (uint32_t)(j & 1), a, &s_abort);
+                    ok = wait_bar(&bars.mid_full[b], (uint32_t)((j >> 1) & 1), a, &s_abort);
                     KX_CLK_ADD(7, tw);
                     if (!ok) break;
                     ptx::tc_fence_after();
@@ -654,7 +654,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_pass_kernel(const PassArgs a) 
                 if (with_inv) {
                     ptx::fence_proxy_async_smem();
                     ptx::tc_fence_before();
-                    ptx::mbar_arrive(&bars.mid_full);
+                    ptx::mbar_arrive(&bars.mid_full[b]);
                     KX_CLK_ADD(10, tw);
                     tw = KX_CLK_NOW();
                     // inverse half of the previous tile (its MMA ran while this tile's forward half was processed)

@@ -169,6 +169,23 @@ def test_fused_and_unfused_middle_passes(kx, case, monkeypatch):
         assert abs(ex.item() - ex_ref) < TOL[1]["ex"] * abs(ex_ref)
 
 
+@pytest.mark.parametrize("n", [(48, 48, 64), (80, 16, 24)])
+def test_separate_passes_repeat_bit_identical(kx, n, monkeypatch):
+    """The separate middle passes with an odd number of 16-column chunks along x1:
+    the epilogue warps then have uneven work and run up to a tile apart, and the
+    inverse half of a tile has to wait for the slowest of them."""
+    sysd = system(n, (0.3,) * 3, (P, P, P), S, 16, 211)
+    psi = dev(workloads.make_orbitals(sysd).T)
+    plan = kx.Plan(n, sysd.h, sysd.bc, S, precision=1)
+    fused, _ = kx.kx_vx_apply(plan, psi)
+    monkeypatch.setenv("KX_SLAB", "0")
+    first, e0 = kx.kx_vx_apply(plan, psi)
+    for _ in range(12):
+        again, e1 = kx.kx_vx_apply(plan, psi)
+        assert torch.equal(first, again) and e0.item() == e1.item()
+    assert relmax(first.cpu().numpy(), fused.cpu().numpy()) < 2 * TOL[1]["vx"]
+
+
 def test_max_axis_128(kx):
     n, h, bc = (128, 8, 16), (0.2, 0.5, 0.5), (D, P, D)
     sysd = system(n, h, bc, S, 2, 29)
