@@ -46,9 +46,11 @@ constexpr int kProdThreads = 32 * kProdWarps;
 constexpr int kProdGroups = 2;                            // producer groups work on alternate tiles
 constexpr int kGroupThreads = kProdThreads / kProdGroups;  // 128: one thread per row for the K-major pass
 constexpr int kMmaWarp = kEpiWarps + kProdWarps;
-constexpr int kThreads = 32 * (kEpiWarps + kProdWarps + 1);
+constexpr int kMetaWarp = kMmaWarp + 1;
+constexpr int kThreads = 32 * (kEpiWarps + kProdWarps + 2);
+constexpr int kMetaRing = 8;  // >= the tiles a producer can be ahead of the epilogue (stages + 2 slots) + 1
 constexpr int kMaxStages = 4;
-constexpr size_t kSmemBudget = 222 * 1024;
+constexpr size_t kSmemBudget = 218 * 1024;  // dynamic; ~7 KB of static shared memory beside it
 
 // Optional per-role cycle counters (compile with -DKX_ROLE_CLOCKS): each CTA
 // writes kClk counters to PassArgs::clk[blockIdx.x * kClk + k].
@@ -141,52 +143,81 @@ __device__ __forceinline__ float item_in_max(const PassArgs &a, long long item) 
     return a.in_max[item];
 }
 
-// Per-tile source descriptors, computed once per tile by the producers: for
-// the MN-major passes one per group of 8 rows (row (m, k) of the group reads
-// p0 + k * kstride, 8 consecutive rows contiguous), for the K-major pass one per
-// row (chunk kc reads p0 + 8 kc).  p0 == nullptr marks rows past the end.
-struct SrcDesc {
-    const float *p0[128];
-    const float *p1[16];  // second orbital of the pair product (X3F pair mode)
-    float scale[128];
+// What the producers and the epilogue need to know about one tile, per group of
+// 8 rows (a group never straddles two items: every n is a multiple of 8).  Finding
+// it takes divisions and two or three dependent loads (item, pair, maxima),
+// about 1.5 k cycles, and both the producers and the epilogue spent them per tile (24-28%
+// of the epilogue's time at 96^3).  A warp of its own fetches it up to kMetaRing tiles
+// ahead: X3F 3.31 -> 2.95 ms, X3I 2.85 -> 2.63 ms per apply at 96^3 / 64 orbitals.
+// In the MN-major passes row (m, k) of group g reads p0[g] + k * kstride + m % 8, in
+// the K-major one row m reads the n1 values at p0[g] + (m % 8) n1.
+struct TileMeta {
+    const float *p0[16];   // nullptr: rows past the end
+    const float *p1[16];   // second orbital of the pair product (X3F pair mode)
+    long long obase[16];   // first output element of the group's first row
+    double w[16];          // X1: energy weight of the item
+    int item[16];
+    int local[16];         // first row of the group inside its item
+    float scale[16];       // power-of-two split scale of the source
+    int exp_[16];          // its exponent
+    float in_max[16];
 };
 
+// Lane g < 16 of the metadata warp: group g of a tile.
 template <int PASS>
-__device__ __forceinline__ void make_desc(const PassArgs &a, long long tile, SrcDesc &d, int ptid) {
+__device__ __forceinline__ void make_meta(const PassArgs &a, long long tile, TileMeta &d, int g) {
     const long long n12 = (long long)a.n1 * a.n2;
-    const int nd = (PASS == P_X1) ? 128 : 16;
-    if (ptid >= nd) return;
-    const long long R0 = tile * 128 + (PASS == P_X1 ? ptid : 8 * ptid);  // < 2^31: 32-bit division below
+    const long long R0 = tile * 128 + 8 * g;  // < 2^31: 32-bit division below
     if (R0 >= a.total_rows) {
-        d.p0[ptid] = nullptr;
-        if (PASS == P_X3F) d.p1[ptid] = nullptr;
-        d.scale[ptid] = 0.f;
+        d.p0[g] = nullptr;
+        if (PASS == P_X3F) d.p1[g] = nullptr;
+        d.obase[g] = 0;
+        d.w[g] = 0.0;
+        d.item[g] = 0;
+        d.local[g] = 0;
+        d.scale[g] = 0.f;
+        d.exp_[g] = 0;
+        d.in_max[g] = 0.f;
         return;
     }
     const unsigned rpp = (unsigned)a.rows_pp;
-    const long long item = (unsigned)R0 / rpp, local = (unsigned)R0 % rpp;
-    d.scale[ptid] = ldexpf(1.f, scale_exp(item_in_max<PASS>(a, item)));
+    const long long item = (unsigned)R0 / rpp, local = (unsigned)R0 - (unsigned)item * rpp;
+    const float mx = item_in_max<PASS>(a, item);
+    const int e = scale_exp(mx);
+    d.item[g] = (int)item;
+    d.local[g] = (int)local;
+    d.in_max[g] = mx;
+    d.exp_[g] = e;
+    d.scale[g] = ldexpf(1.f, e);
+    long long off;  // of the group's first row inside the item
     if (PASS == P_X1) {
-        d.p0[ptid] = a.in + item * a.N + local * a.n1;
-    } else if (PASS == P_X3F) {
-        if (a.rhs_mode) {
-            d.p0[ptid] = a.in + item * a.N + local;
-            d.p1[ptid] = nullptr;
-        } else {
+        off = local * a.n1;
+        double w = 0.0;
+        if (a.e_partial != nullptr && !a.rhs_mode) {
             const int2 ij = a.pairs[item];
-            d.p0[ptid] = a.psi32 + (long long)ij.x * a.N + local;
-            d.p1[ptid] = a.psi32 + (long long)ij.y * a.N + local;
+            w = (ij.x == ij.y) ? 1.0 : 2.0;
+            if (a.occ) w *= a.occ[ij.x] * a.occ[ij.y];
         }
+        d.w[g] = w;
     } else if (PASS == P_X2F || PASS == P_X2I) {
         const long long k3 = (unsigned)local / (unsigned)a.n1, x1 = (unsigned)local % (unsigned)a.n1;  // rows (k3, x1)
-        d.p0[ptid] = a.in + item * a.N + k3 * n12 + x1;
-    } else {  // P_X3I: rows = positions
-        d.p0[ptid] = a.in + item * a.N + local;
+        off = k3 * n12 + x1;
+    } else {  // rows = positions
+        off = local;
+    }
+    d.obase[g] = item * a.N + off;
+    if (PASS == P_X3F && !a.rhs_mode) {
+        const int2 ij = a.pairs[item];
+        d.p0[g] = a.psi32 + (long long)ij.x * a.N + off;
+        d.p1[g] = a.psi32 + (long long)ij.y * a.N + off;
+    } else {
+        d.p0[g] = a.in + item * a.N + off;
+        if (PASS == P_X3F) d.p1[g] = nullptr;
     }
 }
 
 template <int PASS, int U, bool TWO>
-__device__ __forceinline__ void produce_tile_u(const PassArgs &a, const SrcDesc &d, uint8_t *Ahi, uint8_t *Alo,
+__device__ __forceinline__ void produce_tile_u(const PassArgs &a, const TileMeta &d, uint8_t *Ahi, uint8_t *Alo,
                                                int ptid) {
     const int np = a.np;
     const int nkc = np >> 3;
@@ -207,9 +238,9 @@ __device__ __forceinline__ void produce_tile_u(const PassArgs &a, const SrcDesc 
                 if (PASS == P_X1) {
                     // lanes walk the 8-value chunks of one row, then the next row: contiguous reads
                     const int m = (int)(((unsigned)t * magic) >> 16), kc = t - m * nkc;
-                    p0 = d.p0[m];
+                    p0 = d.p0[m >> 3];
                     ok = p0 != nullptr && kc * 8 < a.nc;
-                    if (ok) p0 += kc * 8;
+                    if (ok) p0 += (m & 7) * a.n1 + kc * 8;
                 } else {
                     // lanes walk the 16 row groups at one k, then the next k: 16 x 32 contiguous bytes
                     const int g = t & 15, k = t >> 4;
@@ -243,7 +274,7 @@ __device__ __forceinline__ void produce_tile_u(const PassArgs &a, const SrcDesc 
             if (PASS == P_X1) {
                 const int m = (int)(((unsigned)t * magic) >> 16), kc = t - m * nkc;
                 off = (m >> 3) * (nkc * kCoreStride) + kc * kCoreStride + (m & 7) * 16;
-                sc = d.scale[m];
+                sc = d.scale[m >> 3];
             } else {
                 const int g = t & 15, k = t >> 4;
                 off = g * kCoreStride + (k >> 3) * (16 * kCoreStride) + (k & 7) * 16;
@@ -266,7 +297,7 @@ __device__ __forceinline__ void produce_tile_u(const PassArgs &a, const SrcDesc 
 // consecutive global addresses.  All loads of a batch of U tasks (a whole tile for n <= 96 when U = 12) are
 // issued before any is converted, so each thread keeps U*32 bytes in flight.
 template <int PASS>
-__device__ __forceinline__ void produce_tile(const PassArgs &a, const SrcDesc &d, uint8_t *Ahi, uint8_t *Alo,
+__device__ __forceinline__ void produce_tile(const PassArgs &a, const TileMeta &d, uint8_t *Ahi, uint8_t *Alo,
                                              int ptid) {
     if (PASS == P_X3F) {
         if (a.rhs_mode)
@@ -350,18 +381,6 @@ __device__ __forceinline__ bool wait_bar_warp(uint64_t *bar, uint32_t parity, co
     return __all_sync(0xffffffffu, ok);
 }
 
-// The threads of one producer group agree on `ok` and have finished their
-// previous tile (a named barrier of the group, then a vote through shared memory).
-__device__ __forceinline__ bool producers_agree(bool ok, int *flag, int gtid, int bar_id) {
-    if (gtid == 0) *flag = 1;
-    ptx::named_bar(bar_id, kGroupThreads);
-    if (!ok) *flag = 0;
-    ptx::named_bar(bar_id, kGroupThreads);
-    const bool r = *flag != 0;
-    ptx::named_bar(bar_id, kGroupThreads);
-    return r;
-}
-
 __device__ __forceinline__ void track_max(float *out_max, long long item, float m, bool valid) {
     if (out_max == nullptr) return;
     const long long item0 = __shfl_sync(0xffffffffu, item, 0);
@@ -383,6 +402,8 @@ struct Bars {
     uint64_t tfull2[2];
     uint64_t mid_full[2];  // by tile parity: a warp may finish tile j + 1 before another arrives for tile j
     uint64_t drain;
+    uint64_t meta_full[kMetaRing];
+    uint64_t meta_empty[kMetaRing];
 };
 
 // X1 epilogue, inverse half of tile j: wait for its inverse MMA, unscale and
@@ -435,8 +456,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_pass_kernel(const PassArgs a) 
     __shared__ uint32_t tmem_slot;
     __shared__ volatile int s_abort;
     __shared__ double s_red[kEpiWarps];
-    __shared__ SrcDesc sdesc[kProdGroups];
-    __shared__ int s_vote[kProdGroups];
+    __shared__ TileMeta smeta[kMetaRing];
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const bool with_inv = (PASS == P_X1) && !a.energy_only;
@@ -460,6 +480,10 @@ __global__ void __launch_bounds__(kThreads, 1) tc_pass_kernel(const PassArgs a) 
         }
         for (int b = 0; b < 2; ++b) ptx::mbar_init(&bars.mid_full[b], kEpiThreads);
         ptx::mbar_init(&bars.drain, 1);
+        for (int r = 0; r < kMetaRing; ++r) {
+            ptx::mbar_init(&bars.meta_full[r], 16);
+            ptx::mbar_init(&bars.meta_empty[r], kEpiWarps);
+        }
         ptx::fence_mbar_init();
         s_abort = 0;
     }
@@ -528,25 +552,35 @@ __global__ void __launch_bounds__(kThreads, 1) tc_pass_kernel(const PassArgs a) 
             }
         }
         __syncwarp();
+    } else if (warp == kMetaWarp) {
+        // ------------------------------------------------------------ tile metadata
+        if (lane < 16) {
+            for (int it = 0; it < n_my; ++it) {
+                const int r = it % kMetaRing;
+                if (it >= kMetaRing &&
+                    !wait_bar(&bars.meta_empty[r], (uint32_t)((it / kMetaRing - 1) & 1), a, &s_abort))
+                    break;
+                make_meta<PASS>(a, blockIdx.x + (long long)it * gridDim.x, smeta[r], lane);
+                ptx::mbar_arrive(&bars.meta_full[r]);
+            }
+        }
+        __syncwarp();
     } else if (warp >= kEpiWarps) {
         // ------------------------------------------------------------ producers
         const int ptid = tid - kEpiThreads;
         const int grp = ptid / kGroupThreads, gtid = ptid % kGroupThreads;
         const long long tp0 = KX_CLK_NOW();
         for (int it = grp; it < n_my; it += kProdGroups) {  // groups take alternate tiles
-            const int s = it % S;
+            const int s = it % S, r = it % kMetaRing;
             long long tw = KX_CLK_NOW();
-            bool ok = it < S || wait_bar(&bars.empty[s], (uint32_t)(((it / S) - 1) & 1), a, &s_abort);
+            if (it >= S && !wait_bar(&bars.empty[s], (uint32_t)(((it / S) - 1) & 1), a, &s_abort)) break;
             KX_CLK_ADD(1, tw);
             tw = KX_CLK_NOW();
-            ok = producers_agree(ok, &s_vote[grp], gtid, 2 + 2 * grp);
-            if (!ok) break;
-            make_desc<PASS>(a, blockIdx.x + (long long)it * gridDim.x, sdesc[grp], gtid);
-            ptx::named_bar(3 + 2 * grp, kGroupThreads);
+            if (!wait_bar(&bars.meta_full[r], (uint32_t)((it / kMetaRing) & 1), a, &s_abort)) break;
             KX_CLK_ADD(2, tw);
             tw = KX_CLK_NOW();
             uint8_t *Ahi = stage0 + s * stage_bytes;
-            produce_tile<PASS>(a, sdesc[grp], Ahi, Ahi + half_bytes, gtid);
+            produce_tile<PASS>(a, smeta[r], Ahi, Ahi + half_bytes, gtid);
             ptx::fence_proxy_async_smem();
             ptx::mbar_arrive(&bars.full[s]);
             KX_CLK_ADD(3, tw);
@@ -563,25 +597,19 @@ __global__ void __launch_bounds__(kThreads, 1) tc_pass_kernel(const PassArgs a) 
         float prev_unscale2 = 0.f;
         bool aborted = false;
         const long long te0 = KX_CLK_NOW();
-        const unsigned rpp = (unsigned)a.rows_pp;
-        // the per-item scale of a row is fetched one tile ahead (its loads are
-        // dependent L2 round trips that would otherwise follow the MMA wait)
-        auto row_in_max = [&](int j) {
-            const long long R = (blockIdx.x + (long long)j * gridDim.x) * 128 + m;
-            return (R < a.total_rows) ? item_in_max<PASS>(a, (unsigned)R / rpp) : 0.f;
-        };
-        float in_mx_next = n_my > 0 ? row_in_max(0) : 0.f;
         for (int it = 0; it < n_my; ++it) {
             const int b = it & 1;
             // row information and the per-item scale do not depend on the MMA:
-            // fetch them (and X1's first f chunk) before waiting for it
-            const long long tile = blockIdx.x + (long long)it * gridDim.x;
-            const long long R = tile * 128 + m;  // < 2^31
-            const bool valid = R < a.total_rows;
-            const long long item = valid ? (unsigned)R / rpp : 0;
-            const long long local = valid ? (unsigned)R % rpp : 0;
-            const float in_mx = in_mx_next;
-            if (it + 1 < n_my) in_mx_next = row_in_max(it + 1);
+            // take them (and fetch X1's first f chunk) before waiting for it
+            const int r = it % kMetaRing, g8 = m >> 3;
+            if (!wait_bar_warp(&bars.meta_full[r], (uint32_t)((it / kMetaRing) & 1), a, &s_abort)) break;
+            const bool valid = smeta[r].p0[g8] != nullptr;
+            const long long item = smeta[r].item[g8];
+            const long long local = smeta[r].local[g8] + (m & 7);
+            const long long obase = smeta[r].obase[g8] + (m & 7);  // X1: rows are n1 apart, see orow
+            const int e_in = smeta[r].exp_[g8];
+            const float in_mx = smeta[r].in_max[g8];
+            const double w_item = (PASS == P_X1) ? smeta[r].w[g8] : 0.0;
             float fpre[16];
             if (PASS == P_X1) {
 #pragma unroll
@@ -596,24 +624,22 @@ __global__ void __launch_bounds__(kThreads, 1) tc_pass_kernel(const PassArgs a) 
             }
             long long tw = KX_CLK_NOW();
             if (!wait_bar_warp(&bars.tfull[b], (uint32_t)((it >> 1) & 1), a, &s_abort)) break;
+            // the tile's producers are done with its metadata as well (their stage fed this MMA)
+            __syncwarp();
+            if (lane == 0) ptx::mbar_arrive(&bars.meta_empty[r]);
             KX_CLK_ADD(9, tw);
             tw = KX_CLK_NOW();
             ptx::tc_fence_after();
             const uint32_t ta = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(b * 2 * np);
             const uint32_t tb = ta + (uint32_t)np;
-            const float unscale = ldexpf(1.f, -(scale_exp(in_mx) + kVScaleExp));
+            const float unscale = ldexpf(1.f, -(e_in + kVScaleExp));
             float my_max = 0.f;
 
             if (PASS == P_X1) {
                 // forward half of tile it: energy, f scaling, mid operand into the tile's own A stage
                 const int e_mid = scale_exp(a.mid_bound * in_mx);
                 const float s_mid = ldexpf(1.f, e_mid);
-                double w = 0.0;
-                if (valid && a.e_partial != nullptr && !a.rhs_mode) {
-                    int2 ij = a.pairs[item];
-                    w = (ij.x == ij.y) ? 1.0 : 2.0;
-                    if (a.occ) w *= a.occ[ij.x] * a.occ[ij.y];
-                }
+                const double w = w_item;  // 0 for rows past the end and without the energy sum
                 uint8_t *midh = stage0 + (it % S) * stage_bytes;
                 float e_row = 0.f;
                 for (int c = hcol; c < nch; c += 2) {
@@ -675,16 +701,6 @@ __global__ void __launch_bounds__(kThreads, 1) tc_pass_kernel(const PassArgs a) 
                 // row base and column stride are computed once per tile
                 // output (row r, column c) at base(r) + c * ostride: [k3 or x3][position] or [k3][k2 or x2][x1]
                 const long long ostride = (PASS == P_X3F || PASS == P_X3I) ? n12 : (long long)a.n1;
-                long long obase = 0;
-                if (valid) {
-                    if (PASS == P_X3F || PASS == P_X3I) {
-                        obase = item * a.N + local;
-                    } else {
-                        const long long k3 = (unsigned)local / (unsigned)a.n1;
-                        const long long x1 = (unsigned)local % (unsigned)a.n1;
-                        obase = item * a.N + k3 * n12 + x1;
-                    }
-                }
                 for (int cb = 32 * hcol; cb < np; cb += 64) {
                     float v[32], vb[32];
                     const long long tl = KX_CLK_NOW();
