@@ -184,7 +184,8 @@ __global__ void __launch_bounds__(kEigThreads) eig1d_kernel(int n0, int n1, int 
     for (int k = tid; k < n; k += blockDim.x) lam[k] = lam_s[perm[k]];
 }
 
-// f(l1_k1 + l2_k2 + l3_k3) for every spectral point, float64 and float32.
+// f(l1_k1 + l2_k2 + l3_k3) for every spectral point, float64 (grid order) and float32
+// ([k3][k1 / 4][k2][k1 % 4]).
 __global__ void ftable_kernel(int n1, int n2, int n3, const double *l1, const double *l2, const double *l3,
                               int kind, double omega, double *f64, float *f32) {
     size_t N = (size_t)n1 * n2 * n3;
@@ -195,7 +196,8 @@ __global__ void ftable_kernel(int n1, int n2, int n3, const double *l1, const do
         int k3 = (int)(idx / ((size_t)n1 * n2));
         double f = kernel_f_value(kind, omega, l1[k1] + l2[k2] + l3[k3]);
         f64[idx] = f;
-        f32[idx] = (float)f;
+        // float32 in the tensor-core epilogues' order: rows k2 next to each other, four k1 each
+        f32[n1 % 4 ? idx : (((size_t)k3 * (n1 / 4) + k1 / 4) * n2 + k2) * 4 + k1 % 4] = (float)f;
     }
 }
 

@@ -107,10 +107,17 @@ struct PassArgs {
 };
 
 __device__ __forceinline__ int scale_exp(float mx) {
-    // e such that mx * 2^e < 2^14 (mx = m 2^k, m in [0.5, 1)  =>  e = 14 - k)
+    // e such that mx * 2^e < 2^14 (mx = m 2^k, m in [0.5, 1)  =>  e = 14 - k), from the
+    // exponent bits (frexpf only for subnormal maxima)
     int k = 0;
-    if (mx > 0.f && isfinite(mx)) frexpf(mx, &k);
+    if (mx > 0.f && isfinite(mx)) {
+        k = (__float_as_int(mx) >> 23) - 126;
+        if (k == -126) frexpf(mx, &k);
+    }
     return 14 - k;
+}
+__device__ __forceinline__ float pow2f(int e) {
+    return (unsigned)(e + 126) < 254u ? __int_as_float((e + 127) << 23) : ldexpf(1.f, e);
 }
 
 __device__ __forceinline__ void split8(const float *v, uint4 &hi, uint4 &lo) {
@@ -129,6 +136,23 @@ __device__ __forceinline__ void split8(const float *v, uint4 &hi, uint4 &lo) {
 __device__ __forceinline__ void ld8(const float *p, float *v) {
     float4 a = __ldg(reinterpret_cast<const float4 *>(p));
     float4 b = __ldg(reinterpret_cast<const float4 *>(p) + 1);
+    v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+    v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+}
+
+// One k-step leaves the second accumulator unwritten: the epilogues then add zeros
+// (one branch per chunk; a select and a bound test per element made the last stage
+// three times as long as the others at the same number of values).
+__device__ __forceinline__ void zero16(float *v) {
+#pragma unroll
+    for (int k = 0; k < 16; ++k) v[k] = 0.f;
+}
+
+// f(Lambda) of 8 columns of one row: the table holds [k3][k1 / 4][k2][k1 % 4], so that
+// the lanes of a warp (rows k2) read neighbouring 16-byte pieces; `ld4` = 4 n2.
+__device__ __forceinline__ void ld8f(const float *p, int ld4, float *v) {
+    const float4 a = __ldg(reinterpret_cast<const float4 *>(p));
+    const float4 b = __ldg(reinterpret_cast<const float4 *>(p + ld4));
     v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
     v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
 }
@@ -157,7 +181,7 @@ struct TileMeta {
     long long obase[16];   // first output element of the group's first row
     double w[16];          // X1: energy weight of the item
     int item[16];
-    int local[16];         // first row of the group inside its item
+    int foff[16];          // X1: offset of the group's first row in the f table
     float scale[16];       // power-of-two split scale of the source
     int exp_[16];          // its exponent
     float in_max[16];
@@ -174,7 +198,7 @@ __device__ __forceinline__ void make_meta(const PassArgs &a, long long tile, Til
         d.obase[g] = 0;
         d.w[g] = 0.0;
         d.item[g] = 0;
-        d.local[g] = 0;
+        d.foff[g] = 0;
         d.scale[g] = 0.f;
         d.exp_[g] = 0;
         d.in_max[g] = 0.f;
@@ -185,13 +209,14 @@ __device__ __forceinline__ void make_meta(const PassArgs &a, long long tile, Til
     const float mx = item_in_max<PASS>(a, item);
     const int e = scale_exp(mx);
     d.item[g] = (int)item;
-    d.local[g] = (int)local;
     d.in_max[g] = mx;
     d.exp_[g] = e;
-    d.scale[g] = ldexpf(1.f, e);
+    d.scale[g] = pow2f(e);
     long long off;  // of the group's first row inside the item
     if (PASS == P_X1) {
         off = local * a.n1;
+        const int k3 = (unsigned)local / (unsigned)a.n2, k2 = (unsigned)local % (unsigned)a.n2;  // rows (k3, k2)
+        d.foff[g] = (k3 * (a.n1 >> 2) * a.n2 + k2) * 4;
         double w = 0.0;
         if (a.e_partial != nullptr && !a.rhs_mode) {
             const int2 ij = a.pairs[item];
@@ -315,6 +340,26 @@ __device__ __forceinline__ void produce_tile(const PassArgs &a, const TileMeta &
 // the two small cross products are issued first into accumulator Da, and the
 // hi*hi chain is split over Da (even k-steps) and Db (odd k-steps); the
 // epilogue adds Da + Db with round-to-nearest.
+template <int NKS>
+__device__ __forceinline__ void issue_ksteps(uint32_t tmem_a, uint32_t tmem_b, uint32_t ah0, uint32_t al0, uint32_t a_up,
+                                             uint32_t bh0, uint32_t bl0, uint32_t b_up, uint32_t a_inc, uint32_t b_inc,
+                                             uint32_t idesc) {
+#pragma unroll
+    for (int ks = 0; ks < NKS; ++ks) {
+        const uint32_t da = ks * a_inc, db = ks * b_inc;
+        ptx::mma_f16_lo(tmem_a, ah0 + da, a_up, bl0 + db, b_up, idesc, ks > 0 ? 1u : 0u);
+        ptx::mma_f16_lo(tmem_a, al0 + da, a_up, bh0 + db, b_up, idesc, 1u);
+    }
+#pragma unroll
+    for (int ks = 0; ks < NKS; ++ks) {
+        const uint32_t da = ks * a_inc, db = ks * b_inc;
+        if (ks & 1)
+            ptx::mma_f16_lo(tmem_b, ah0 + da, a_up, bh0 + db, b_up, idesc, ks > 1 ? 1u : 0u);
+        else
+            ptx::mma_f16_lo(tmem_a, ah0 + da, a_up, bh0 + db, b_up, idesc, 1u);
+    }
+}
+
 __device__ __forceinline__ void issue_split_mma(uint32_t tmem_a, uint32_t tmem_b, uint32_t a_hi, uint32_t a_lo,
                                                 bool a_kmajor, uint32_t v_hi, uint32_t v_lo, bool inverse, int np) {
     const uint32_t idesc = ptx::idesc_f16(128, np, a_kmajor ? 0 : 1, inverse ? 0 : 1);
@@ -327,35 +372,35 @@ __device__ __forceinline__ void issue_split_mma(uint32_t tmem_a, uint32_t tmem_b
     const uint32_t b_lbo = inverse ? 128u : (uint32_t)(np * 16);
     const uint32_t b_sbo = inverse ? (uint32_t)(np * 16) : 128u;
     const uint32_t b_step = inverse ? 256u : (uint32_t)(np * 32);
-    const int nks = np >> 4;
     // descriptors built once; a k-step advances the start-address field (16-byte units)
-    const uint64_t ah0 = ptx::sdesc(a_hi, a_lbo, a_sbo), al0 = ptx::sdesc(a_lo, a_lbo, a_sbo);
-    const uint64_t bh0 = ptx::sdesc(v_hi, b_lbo, b_sbo), bl0 = ptx::sdesc(v_lo, b_lbo, b_sbo);
-    const uint64_t a_inc = a_step >> 4, b_inc = b_step >> 4;
-    {
-        uint64_t ah = ah0, al = al0, bh = bh0, bl = bl0;
-        ptx::mma_f16(tmem_a, ah, bl, idesc, 0u);
-        ptx::mma_f16(tmem_a, al, bh, idesc, 1u);
-        for (int ks = 1; ks < nks; ++ks) {
-            ah += a_inc;
-            al += a_inc;
-            bh += b_inc;
-            bl += b_inc;
-            ptx::mma_f16(tmem_a, ah, bl, idesc, 1u);
-            ptx::mma_f16(tmem_a, al, bh, idesc, 1u);
-        }
+    const uint64_t ah = ptx::sdesc(a_hi, a_lbo, a_sbo), al = ptx::sdesc(a_lo, a_lbo, a_sbo);
+    const uint64_t bh = ptx::sdesc(v_hi, b_lbo, b_sbo), bl = ptx::sdesc(v_lo, b_lbo, b_sbo);
+    const uint32_t a_up = (uint32_t)(ah >> 32), b_up = (uint32_t)(bh >> 32);
+    const uint32_t a_inc = a_step >> 4, b_inc = b_step >> 4;
+#define KX_ISSUE(n)                                                                                               \
+    case n:                                                                                                       \
+        issue_ksteps<n>(tmem_a, tmem_b, (uint32_t)ah, (uint32_t)al, a_up, (uint32_t)bh, (uint32_t)bl, b_up, a_inc, \
+                        b_inc, idesc);                                                                            \
+        break;
+    switch (np >> 4) {
+        KX_ISSUE(1)
+        KX_ISSUE(2)
+        KX_ISSUE(3)
+        KX_ISSUE(4)
+        KX_ISSUE(5)
+        KX_ISSUE(6)
+        KX_ISSUE(7)
+        KX_ISSUE(8)
+        default: break;
     }
-    {
-        uint64_t ah = ah0, bh = bh0;
-        for (int ks = 0; ks < nks; ++ks) {
-            if (ks & 1)
-                ptx::mma_f16(tmem_b, ah, bh, idesc, ks > 1 ? 1u : 0u);
-            else
-                ptx::mma_f16(tmem_a, ah, bh, idesc, 1u);
-            ah += a_inc;
-            bh += b_inc;
-        }
-    }
+#undef KX_ISSUE
+}
+
+// One arrival for a warp, after everything its lanes did before (their own proxy
+// fences included): 32 arrivals on one word would be served one by one.
+__device__ __forceinline__ void warp_arrive(uint64_t *bar) {
+    __syncwarp();
+    if ((threadIdx.x & 31) == 0) ptx::mbar_arrive(bar);
 }
 
 // Bounded wait shared by all roles: gives up when the limit elapses or another
@@ -409,25 +454,28 @@ struct Bars {
 // X1 epilogue, inverse half of tile j: wait for its inverse MMA, unscale and
 // store the row (float4 per 4 columns), track the maximum, release the slot.
 __device__ __forceinline__ bool x1_inverse_half(const PassArgs &a, Bars &bars, uint32_t tmem, int q, int hcol, int j,
-                                                int np, bool two_acc, bool valid, long long item, long long local,
-                                                float unscale2, volatile int *abort) {
+                                                int np, bool two_acc, const TileMeta &d, int m, volatile int *abort) {
     const int b = j & 1;
     if (!wait_bar_warp(&bars.tfull2[b], (uint32_t)((j >> 1) & 1), a, abort)) return false;
     ptx::tc_fence_after();
     const uint32_t ta = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(b * 2 * np);
     const uint32_t tb = ta + (uint32_t)np;
+    const int g8 = m >> 3;
+    const bool valid = d.p0[g8] != nullptr;
+    float *orow = a.out + d.obase[g8] + (m & 7) * a.n1;
+    const float unscale2 = pow2f(-(scale_exp(a.mid_bound * d.in_max[g8]) + kVScaleExp));
     float my_max = 0.f;
-    float *orow = a.out + item * a.N + local * a.n1;
     for (int c = hcol; c < (np >> 4); c += 2) {
         float v[16], vb[16];
         ptx::tmem_ld16x2(ta + 16 * c, tb + 16 * c, v, vb);
+        if (!two_acc) zero16(vb);
 #pragma unroll
         for (int h2 = 0; h2 < 2; ++h2) {  // store each 8-column half that lies inside the row
             if (!valid || 16 * c + 8 * h2 >= a.nc) continue;
             float wv[8];
 #pragma unroll
             for (int k = 0; k < 8; ++k) {
-                wv[k] = (two_acc ? v[8 * h2 + k] + vb[8 * h2 + k] : v[8 * h2 + k]) * unscale2;
+                wv[k] = (v[8 * h2 + k] + vb[8 * h2 + k]) * unscale2;
                 my_max = fmaxf(my_max, fabsf(wv[k]));
             }
             float4 *dst = reinterpret_cast<float4 *>(orow + 16 * c + 8 * h2);
@@ -435,9 +483,10 @@ __device__ __forceinline__ bool x1_inverse_half(const PassArgs &a, Bars &bars, u
             dst[1] = make_float4(wv[4], wv[5], wv[6], wv[7]);
         }
     }
-    track_max(a.out_max, item, my_max, valid);
+    track_max(a.out_max, d.item[g8], my_max, valid);
     ptx::tc_fence_before();
-    ptx::mbar_arrive(&bars.tempty[b]);
+    warp_arrive(&bars.tempty[b]);
+    warp_arrive(&bars.meta_empty[j % kMetaRing]);
     return true;
 }
 
@@ -470,15 +519,15 @@ __global__ void __launch_bounds__(kThreads, 1) tc_pass_kernel(const PassArgs a) 
     }
     if (tid == 0) {
         for (int s = 0; s < S; ++s) {
-            ptx::mbar_init(&bars.full[s], kGroupThreads);
+            ptx::mbar_init(&bars.full[s], kGroupThreads / 32);
             ptx::mbar_init(&bars.empty[s], 1);
         }
         for (int b = 0; b < 2; ++b) {
             ptx::mbar_init(&bars.tfull[b], 1);
-            ptx::mbar_init(&bars.tempty[b], kEpiThreads);
+            ptx::mbar_init(&bars.tempty[b], kEpiWarps);
             ptx::mbar_init(&bars.tfull2[b], 1);
         }
-        for (int b = 0; b < 2; ++b) ptx::mbar_init(&bars.mid_full[b], kEpiThreads);
+        for (int b = 0; b < 2; ++b) ptx::mbar_init(&bars.mid_full[b], kEpiWarps);
         ptx::mbar_init(&bars.drain, 1);
         for (int r = 0; r < kMetaRing; ++r) {
             ptx::mbar_init(&bars.meta_full[r], 16);
@@ -505,7 +554,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_pass_kernel(const PassArgs a) 
 
     if (warp == kMmaWarp) {
         // ------------------------------------------------------------ MMA issue
-        if (lane == 0) {
+        if (ptx::elect_one()) {
             const uint32_t sVhi = ptx::smem_u32(Vhi), sVlo = ptx::smem_u32(Vlo);
             const bool inv = (PASS == P_X2I || PASS == P_X3I);
             bool ok = true;
@@ -573,16 +622,16 @@ __global__ void __launch_bounds__(kThreads, 1) tc_pass_kernel(const PassArgs a) 
         for (int it = grp; it < n_my; it += kProdGroups) {  // groups take alternate tiles
             const int s = it % S, r = it % kMetaRing;
             long long tw = KX_CLK_NOW();
-            if (it >= S && !wait_bar(&bars.empty[s], (uint32_t)(((it / S) - 1) & 1), a, &s_abort)) break;
+            if (it >= S && !wait_bar_warp(&bars.empty[s], (uint32_t)(((it / S) - 1) & 1), a, &s_abort)) break;
             KX_CLK_ADD(1, tw);
             tw = KX_CLK_NOW();
-            if (!wait_bar(&bars.meta_full[r], (uint32_t)((it / kMetaRing) & 1), a, &s_abort)) break;
+            if (!wait_bar_warp(&bars.meta_full[r], (uint32_t)((it / kMetaRing) & 1), a, &s_abort)) break;
             KX_CLK_ADD(2, tw);
             tw = KX_CLK_NOW();
             uint8_t *Ahi = stage0 + s * stage_bytes;
             produce_tile<PASS>(a, smeta[r], Ahi, Ahi + half_bytes, gtid);
             ptx::fence_proxy_async_smem();
-            ptx::mbar_arrive(&bars.full[s]);
+            warp_arrive(&bars.full[s]);
             KX_CLK_ADD(3, tw);
         }
         KX_CLK_ADD(0, tp0);
@@ -592,9 +641,6 @@ __global__ void __launch_bounds__(kThreads, 1) tc_pass_kernel(const PassArgs a) 
         const int m = 32 * q + lane;  // TMEM lane == tile row of this thread
         const int nch = np >> 4;      // 16-column chunks
         double e_acc = 0.0;
-        bool prev_valid = false;  // X1: the tile whose inverse half is still pending
-        long long prev_item = 0, prev_local = 0;
-        float prev_unscale2 = 0.f;
         bool aborted = false;
         const long long te0 = KX_CLK_NOW();
         for (int it = 0; it < n_my; ++it) {
@@ -604,18 +650,19 @@ __global__ void __launch_bounds__(kThreads, 1) tc_pass_kernel(const PassArgs a) 
             const int r = it % kMetaRing, g8 = m >> 3;
             if (!wait_bar_warp(&bars.meta_full[r], (uint32_t)((it / kMetaRing) & 1), a, &s_abort)) break;
             const bool valid = smeta[r].p0[g8] != nullptr;
-            const long long item = smeta[r].item[g8];
-            const long long local = smeta[r].local[g8] + (m & 7);
-            const long long obase = smeta[r].obase[g8] + (m & 7);  // X1: rows are n1 apart, see orow
+            const int item = smeta[r].item[g8];
+            const long long obase = smeta[r].obase[g8] + (PASS == P_X1 ? (m & 7) * a.n1 : (m & 7));
             const int e_in = smeta[r].exp_[g8];
             const float in_mx = smeta[r].in_max[g8];
             const double w_item = (PASS == P_X1) ? smeta[r].w[g8] : 0.0;
+            const float *frow = (PASS == P_X1) ? a.f32 + smeta[r].foff[g8] + 4 * (m & 7) : nullptr;
+            const int ld4 = 4 * a.n2;
             float fpre[16];
             if (PASS == P_X1) {
 #pragma unroll
                 for (int h2 = 0; h2 < 2; ++h2) {
                     if (valid && 16 * hcol + 8 * h2 < a.nc) {
-                        ld8(a.f32 + local * a.n1 + 16 * hcol + 8 * h2, fpre + 8 * h2);
+                        ld8f(frow + (4 * hcol + 2 * h2) * ld4, ld4, fpre + 8 * h2);
                     } else {
 #pragma unroll
                         for (int k = 0; k < 8; ++k) fpre[8 * h2 + k] = 0.f;
@@ -625,20 +672,20 @@ __global__ void __launch_bounds__(kThreads, 1) tc_pass_kernel(const PassArgs a) 
             long long tw = KX_CLK_NOW();
             if (!wait_bar_warp(&bars.tfull[b], (uint32_t)((it >> 1) & 1), a, &s_abort)) break;
             // the tile's producers are done with its metadata as well (their stage fed this MMA)
-            __syncwarp();
-            if (lane == 0) ptx::mbar_arrive(&bars.meta_empty[r]);
+            // (X1 needs it once more, in the tile's inverse half)
+            if (!with_inv) warp_arrive(&bars.meta_empty[r]);
             KX_CLK_ADD(9, tw);
             tw = KX_CLK_NOW();
             ptx::tc_fence_after();
             const uint32_t ta = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(b * 2 * np);
             const uint32_t tb = ta + (uint32_t)np;
-            const float unscale = ldexpf(1.f, -(e_in + kVScaleExp));
+            const float unscale = pow2f(-(e_in + kVScaleExp));
             float my_max = 0.f;
 
             if (PASS == P_X1) {
                 // forward half of tile it: energy, f scaling, mid operand into the tile's own A stage
                 const int e_mid = scale_exp(a.mid_bound * in_mx);
-                const float s_mid = ldexpf(1.f, e_mid);
+                const float s_mid = pow2f(e_mid);
                 const double w = w_item;  // 0 for rows past the end and without the energy sum
                 uint8_t *midh = stage0 + (it % S) * stage_bytes;
                 float e_row = 0.f;
@@ -651,7 +698,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_pass_kernel(const PassArgs a) 
 #pragma unroll
                     for (int h2 = 0; h2 < 2; ++h2) {
                         if (valid && 16 * (c + 2) + 8 * h2 < a.nc) {
-                            ld8(a.f32 + local * a.n1 + 16 * (c + 2) + 8 * h2, fpre + 8 * h2);
+                            ld8f(frow + (4 * (c + 2) + 2 * h2) * ld4, ld4, fpre + 8 * h2);
                         } else {
 #pragma unroll
                             for (int k = 0; k < 8; ++k) fpre[8 * h2 + k] = 0.f;
@@ -659,9 +706,10 @@ __global__ void __launch_bounds__(kThreads, 1) tc_pass_kernel(const PassArgs a) 
                     }
                     float v[16], vb[16];
                     ptx::tmem_ld16x2(ta + 16 * c, tb + 16 * c, v, vb);
+                    if (!two_acc) zero16(vb);
 #pragma unroll
                     for (int k = 0; k < 16; ++k) {
-                        const float y = (two_acc ? v[k] + vb[k] : v[k]) * unscale;
+                        const float y = (v[k] + vb[k]) * unscale;
                         e_row = fmaf(fk[k] * y, y, e_row);
                         v[k] = fk[k] * y * s_mid;
                     }
@@ -680,20 +728,16 @@ __global__ void __launch_bounds__(kThreads, 1) tc_pass_kernel(const PassArgs a) 
                 if (with_inv) {
                     ptx::fence_proxy_async_smem();
                     ptx::tc_fence_before();
-                    ptx::mbar_arrive(&bars.mid_full[b]);
+                    warp_arrive(&bars.mid_full[b]);
                     KX_CLK_ADD(10, tw);
                     tw = KX_CLK_NOW();
                     // inverse half of the previous tile (its MMA ran while this tile's forward half was processed)
                     if (it >= 1) {
-                        if (!x1_inverse_half(a, bars, tmem, q, hcol, it - 1, np, two_acc, prev_valid, prev_item,
-                                             prev_local, prev_unscale2, &s_abort))
+                        if (!x1_inverse_half(a, bars, tmem, q, hcol, it - 1, np, two_acc,
+                                             smeta[(it - 1) % kMetaRing], m, &s_abort))
                             break;
                     }
                     KX_CLK_ADD(11, tw);
-                    prev_valid = valid;
-                    prev_item = item;
-                    prev_local = local;
-                    prev_unscale2 = ldexpf(1.f, -(e_mid + kVScaleExp));
                     continue;  // tile it's TMEM slot is released by its inverse half
                 }
             } else {
@@ -710,31 +754,42 @@ __global__ void __launch_bounds__(kThreads, 1) tc_pass_kernel(const PassArgs a) 
                         ptx::tmem_ld16x2(ta + cb, tb + cb, v, vb);
                     }
                     KX_CLK_ADD(11, tl);
+                    if (!two_acc) zero16(vb);  // np == 16
                     if (!valid) continue;
-                    const int w = min(32, a.nc - cb);
+                    // (nc is a multiple of 8: whole groups of 8 columns, no test per element)
+                    if (PASS == P_X3I && a.rhs_mode) {
+                        double *o = a.xout + obase + (long long)cb * ostride;
 #pragma unroll
-                    for (int k = 0; k < 32; ++k) {
-                        if (k >= w) break;
-                        const float y = (two_acc ? v[k] + vb[k] : v[k]) * unscale;
-                        const long long dst = obase + (long long)(cb + k) * ostride;
-                        if (PASS == P_X3I && a.rhs_mode) {
-                            a.xout[dst] = (double)y;
-                        } else {
-                            my_max = fmaxf(my_max, fabsf(y));
-                            a.out[dst] = y;
+                        for (int g = 0; g < 4; ++g) {
+                            if (cb + 8 * g >= a.nc) break;
+#pragma unroll
+                            for (int k = 8 * g; k < 8 * g + 8; ++k, o += ostride)
+                                *o = (double)((v[k] + vb[k]) * unscale);
+                        }
+                    } else {
+                        float *o = a.out + obase + (long long)cb * ostride;
+#pragma unroll
+                        for (int g = 0; g < 4; ++g) {
+                            if (cb + 8 * g >= a.nc) break;
+#pragma unroll
+                            for (int k = 8 * g; k < 8 * g + 8; ++k, o += ostride) {
+                                const float y = (v[k] + vb[k]) * unscale;
+                                my_max = fmaxf(my_max, fabsf(y));
+                                *o = y;
+                            }
                         }
                     }
                 }
                 track_max(a.out_max, item, my_max, valid);
             }
             ptx::tc_fence_before();
-            ptx::mbar_arrive(&bars.tempty[b]);
+            warp_arrive(&bars.tempty[b]);
             KX_CLK_ADD(10, tw);
         }
         KX_CLK_ADD(8, te0);
         if (PASS == P_X1 && with_inv && n_my >= 1 && !s_abort)
-            aborted = !x1_inverse_half(a, bars, tmem, q, hcol, n_my - 1, np, two_acc, prev_valid, prev_item, prev_local,
-                                       prev_unscale2, &s_abort);
+            aborted = !x1_inverse_half(a, bars, tmem, q, hcol, n_my - 1, np, two_acc, smeta[(n_my - 1) % kMetaRing], m,
+                                       &s_abort);
         (void)aborted;
         if (a.e_partial != nullptr) {
             double e = e_acc;
@@ -797,19 +852,22 @@ struct SlabArgs {
     const double *occ;
     int rhs_mode;
     int stage_in;           // the input plane is bulk-copied into shared memory before it is split
+    int share_v;            // V2 == V1 (same size, spacing and boundary): one shared copy
     int *status;
     long long timeout_cycles;
     long long *clk;         // role counters (only with KX_ROLE_CLOCKS)
 };
 
-constexpr int kSlabProdThreads = 96;
 constexpr int kSlabU = 8;            // producer loads in flight per thread
 // Warp roles: 16 epilogue warps (warp w reads TMEM lane quadrant w % 4, the
 // TMEM access rule; column half (w / 4) % 2; group w / 8), then 3 producer
-// warps, then the MMA warp.
+// warps, then the MMA warp.  A plane of at most 96 rows leaves one quadrant (32:
+// three) without rows: those epilogue warps work as producers instead (the split
+// of a plane runs beside the last epilogue stage and took as long as it: slab
+// time 8.54 -> 8.12 ms per apply at 96^3 / 64 orbitals).
 constexpr int kSlabEpiWarps = 16;
-constexpr int kSlabGroupThreads = 256;
-constexpr int kSlabMmaWarp = kSlabEpiWarps + kSlabProdThreads / 32;
+constexpr int kSlabProdWarps = 3;
+constexpr int kSlabMmaWarp = kSlabEpiWarps + kSlabProdWarps;
 constexpr int kSlabThreads = 32 * (kSlabMmaWarp + 1);
 
 struct SlabBars {
@@ -844,11 +902,10 @@ struct SlabUnit {
     double w;
 };
 
-__device__ __forceinline__ SlabUnit slab_unit(const SlabArgs &a, long long u) {
+__device__ __forceinline__ SlabUnit slab_unit(const SlabArgs &a, long long u, float b1, int2 ij) {
     SlabUnit r;
     r.item = (unsigned)u / (unsigned)a.n3;
-    r.k3 = (unsigned)u % (unsigned)a.n3;
-    const float b1 = __ldg(a.in_max + r.item);
+    r.k3 = (unsigned)u - (unsigned)r.item * (unsigned)a.n3;
     const float b2 = b1 * a.sq2, b3 = a.fmax * a.sq1 * b2, b4 = a.sq1 * b3;
     r.e1 = scale_exp(b1);
     r.e2 = scale_exp(b2);
@@ -856,7 +913,6 @@ __device__ __forceinline__ SlabUnit slab_unit(const SlabArgs &a, long long u) {
     r.e4 = scale_exp(b4);
     r.w = 0.0;
     if (a.e_partial != nullptr && !a.rhs_mode) {
-        const int2 ij = a.pairs[r.item];
         r.w = (ij.x == ij.y) ? 1.0 : 2.0;
         if (a.occ) r.w *= a.occ[ij.x] * a.occ[ij.y];
     }
@@ -869,16 +925,17 @@ __device__ __forceinline__ SlabUnit slab_unit(const SlabArgs &a, long long u) {
 __device__ __forceinline__ void slab_transpose_stage(uint32_t ta, uint32_t tb, int m, int h, int nrow, int nprow,
                                                      int ncol, bool two, float us, uint8_t *Ahi, uint8_t *Alo) {
     const int off_r = (m >> 3) * (16 * kCoreStride) + (m & 7) * 16;
+    if (m >= nrow) us = 0.f;  // padding rows hold zeros already: their operand rows were zero
     for (int c = 16 * h; c < ncol; c += 32) {
         float v[16], vb[16];
         ptx::tmem_ld16x2(ta + c, tb + c, v, vb);
+        if (!two) zero16(vb);
         if (m < nprow) {
 #pragma unroll
             for (int g8 = 0; g8 < 2; ++g8) {
                 float w[8];
 #pragma unroll
-                for (int k = 0; k < 8; ++k)
-                    w[k] = (m < nrow) ? (two ? v[8 * g8 + k] + vb[8 * g8 + k] : v[8 * g8 + k]) * us : 0.f;
+                for (int k = 0; k < 8; ++k) w[k] = (v[8 * g8 + k] + vb[8 * g8 + k]) * us;
                 store_split8(Ahi, Alo, ((c >> 3) + g8) * kCoreStride + off_r, w);
             }
         }
@@ -892,7 +949,7 @@ __global__ void __launch_bounds__(kSlabThreads, 1) tc_slab_kernel(const SlabArgs
     const size_t half_bytes = a_half_bytes(npm);
     uint8_t *V1hi = smem;
     uint8_t *V1lo = V1hi + np1 * np1 * 2;
-    uint8_t *V2hi = V1lo + np1 * np1 * 2;
+    uint8_t *V2hi = a.share_v ? V1hi : V1lo + np1 * np1 * 2;
     uint8_t *V2lo = V2hi + np2 * np2 * 2;
     uint8_t *buf0 = V2lo + np2 * np2 * 2;  // two A buffers (hi | lo), one per TMEM slot
     float *sin = reinterpret_cast<float *>(buf0 + 4 * half_bytes);  // input plane [x2][x1] (stage_in)
@@ -902,6 +959,11 @@ __global__ void __launch_bounds__(kSlabThreads, 1) tc_slab_kernel(const SlabArgs
     __shared__ double s_red[kSlabEpiWarps];
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int nq = (npm + 31) >> 5;              // TMEM lane quadrants with rows
+    const int n_help = 4 * (4 - nq);             // epilogue warps without rows
+    const int helper = (warp < kSlabEpiWarps && (warp & 3) >= nq) ? (warp & 3) - nq + (4 - nq) * (warp >> 2) : -1;
+    const int n_prod = 32 * (kSlabProdWarps + n_help);  // producer threads
+    const int group_threads = 64 * nq;           // epilogue threads of a group
 #ifdef KX_ROLE_CLOCKS
     long long clk_acc[kClk] = {0};
     const long long clk_t0 = clock64();
@@ -912,16 +974,17 @@ __global__ void __launch_bounds__(kSlabThreads, 1) tc_slab_kernel(const SlabArgs
     }
     if (tid == 0) {
         for (int b = 0; b < 2; ++b) {
-            ptx::mbar_init(&bars.full[b], kSlabProdThreads);
+            ptx::mbar_init(&bars.full[b], n_prod / 32);
             ptx::mbar_init(&bars.empty[b], 1);
             ptx::mbar_init(&bars.tfull[b], 1);
-            ptx::mbar_init(&bars.ready[b], kSlabGroupThreads);
+            ptx::mbar_init(&bars.ready[b], group_threads / 32);
         }
         ptx::mbar_init(&bars.in_full, 1);
         ptx::mbar_init(&bars.drain, 1);
         ptx::fence_mbar_init();
         s_abort = 0;
     }
+    if (tid < kSlabEpiWarps) s_red[tid] = 0.0;
     {
         const uint4 *s1 = reinterpret_cast<const uint4 *>(a.V1s);
         const uint4 *s2 = reinterpret_cast<const uint4 *>(a.V2s);
@@ -929,7 +992,8 @@ __global__ void __launch_bounds__(kSlabThreads, 1) tc_slab_kernel(const SlabArgs
         uint4 *d2 = reinterpret_cast<uint4 *>(V2hi);
         const int c1 = (4 * np1 * np1) / 16, c2 = (4 * np2 * np2) / 16;
         for (int i = tid; i < c1; i += blockDim.x) d1[i] = __ldg(s1 + i);
-        for (int i = tid; i < c2; i += blockDim.x) d2[i] = __ldg(s2 + i);
+        if (!a.share_v)
+            for (int i = tid; i < c2; i += blockDim.x) d2[i] = __ldg(s2 + i);
     }
     ptx::fence_proxy_async_smem();
     ptx::tc_fence_before();
@@ -944,7 +1008,7 @@ __global__ void __launch_bounds__(kSlabThreads, 1) tc_slab_kernel(const SlabArgs
         // Polls both slots and issues the next product of whichever is ready:
         // M1 of unit j needs its A1 (full) and the slot's previous unit through
         // stage E; M2..M4 need the group's previous stage (ready).
-        if (lane == 0) {
+        if (ptx::elect_one()) {
             const uint32_t sV1h = ptx::smem_u32(V1hi), sV1l = ptx::smem_u32(V1lo);
             const uint32_t sV2h = ptx::smem_u32(V2hi), sV2l = ptx::smem_u32(V2lo);
             int jn[2] = {0, 1}, sn[2] = {0, 0};
@@ -966,18 +1030,11 @@ __global__ void __launch_bounds__(kSlabThreads, 1) tc_slab_kernel(const SlabArgs
                     ptx::tc_fence_after();
                     const uint32_t sA = ptx::smem_u32(buf0 + g * 2 * half_bytes);
                     const uint32_t da = tmem + (uint32_t)(g * 2 * npm);
-                    if (st == 0)  // M1: A1 (MN-major) x V2 forward
-                        issue_split_mma(da, da + (uint32_t)npm, sA, sA + (uint32_t)half_bytes, false, sV2h, sV2l,
-                                        false, np2);
-                    else if (st == 1)  // M2: A2 (MN-major) x V1 forward
-                        issue_split_mma(da, da + (uint32_t)npm, sA, sA + (uint32_t)half_bytes, false, sV1h, sV1l,
-                                        false, np1);
-                    else if (st == 2)  // M3: A3 (K-major) x V1^T
-                        issue_split_mma(da, da + (uint32_t)npm, sA, sA + (uint32_t)half_bytes, true, sV1h, sV1l,
-                                        true, np1);
-                    else  // M4: A4 (MN-major) x V2^T
-                        issue_split_mma(da, da + (uint32_t)npm, sA, sA + (uint32_t)half_bytes, false, sV2h, sV2l,
-                                        true, np2);
+                    // M1: A1 (MN-major) x V2 forward; M2: A2 (MN-major) x V1 forward;
+                    // M3: A3 (K-major) x V1^T; M4: A4 (MN-major) x V2^T
+                    const bool ax2 = st == 0 || st == 3;
+                    issue_split_mma(da, da + (uint32_t)npm, sA, sA + (uint32_t)half_bytes, st == 2, ax2 ? sV2h : sV1h,
+                                    ax2 ? sV2l : sV1l, st >= 2, ax2 ? np2 : np1);
                     ptx::mma_commit(&bars.tfull[g]);
                     if (st == 3) ptx::mma_commit(&bars.empty[g]);
                     if (++sn[g] == 4) {
@@ -1006,9 +1063,9 @@ __global__ void __launch_bounds__(kSlabThreads, 1) tc_slab_kernel(const SlabArgs
             }
         }
         __syncwarp();
-    } else if (warp >= kSlabEpiWarps) {
+    } else if (warp >= kSlabEpiWarps || helper >= 0) {
         // ---------------------------------------------------------------- producers: A1 from global
-        const int ptid = tid - kSlabEpiWarps * 32;
+        const int ptid = helper >= 0 ? 32 * (kSlabProdWarps + helper) + lane : tid - kSlabEpiWarps * 32;
         const int ntask = 16 * np2;  // 16 row groups (x1) x np2 columns (x2)
         const int nlines = (int)((n12 * 4) >> 7);  // 128-byte lines of a slice (n1 % 8 == 0)
         const uint32_t plane_bytes = (uint32_t)(n12 * 4);
@@ -1027,6 +1084,10 @@ __global__ void __launch_bounds__(kSlabThreads, 1) tc_slab_kernel(const SlabArgs
             for (uint32_t o = 0; o < plane_bytes; o += 16384u)
                 ptx::bulk_load(dst + o, src + o, min(16384u, plane_bytes - o), &bars.in_full);
         };
+        auto plane_max = [&](int it) {
+            return __ldg(a.in_max + (unsigned)(blockIdx.x + (long long)it * gridDim.x) / (unsigned)a.n3);
+        };
+        float next_max = n_my > 0 ? plane_max(0) : 0.f;  // loaded one unit ahead
         int inflight = -1;  // unit whose plane copy thread 0 issued and has not yet waited for
         if (a.stage_in && ptid == 0 && n_my > 0) {
             issue_plane(0);
@@ -1037,7 +1098,7 @@ __global__ void __launch_bounds__(kSlabThreads, 1) tc_slab_kernel(const SlabArgs
             if (it + 2 < n_my) {
                 // pull the plane of unit it+2 into L2 while this unit waits for its buffer
                 const char *src = reinterpret_cast<const char *>(plane(it + 2));
-                for (int l = ptid; l < nlines; l += kSlabProdThreads) ptx::prefetch_l2(src + ((long long)l << 7));
+                for (int l = ptid; l < nlines; l += n_prod) ptx::prefetch_l2(src + ((long long)l << 7));
             }
             long long tw = KX_CLK_NOW();
             bool ok = it < 2 || slab_wait(&bars.empty[sl], (uint32_t)(((it >> 1) - 1) & 1), a, &s_abort);
@@ -1047,16 +1108,15 @@ __global__ void __launch_bounds__(kSlabThreads, 1) tc_slab_kernel(const SlabArgs
             if (ok && ptid == 0) inflight = -1;
             ok = ok && !s_abort;
             // with stage_in the producers meet at a named barrier below, so they leave together
-            if (a.stage_in) ok = ptx::named_bar_and(2, kSlabProdThreads, ok);
+            ok = a.stage_in ? ptx::named_bar_and(2, n_prod, ok) : (bool)__all_sync(0xffffffffu, ok);
             if (!ok) break;
-            const long long u = blockIdx.x + (long long)it * gridDim.x;
-            const long long item = (unsigned)u / (unsigned)a.n3;
-            const float sc = ldexpf(1.f, scale_exp(a.in_max[item]));
+            const float sc = pow2f(scale_exp(next_max));
+            if (it + 1 < n_my) next_max = plane_max(it + 1);
             uint8_t *Ahi = buf0 + sl * 2 * half_bytes;
             uint8_t *Alo = Ahi + half_bytes;
             if (a.stage_in) {
 #pragma unroll 4
-                for (int t = ptid; t < ntask; t += kSlabProdThreads) {
+                for (int t = ptid; t < ntask; t += n_prod) {
                     const int g = t & 15, k = t >> 4;
                     float v[8];
                     if (8 * g < a.n1 && k < a.n2) {
@@ -1071,20 +1131,20 @@ __global__ void __launch_bounds__(kSlabThreads, 1) tc_slab_kernel(const SlabArgs
                     store_split8(Ahi, Alo, g * kCoreStride + (k >> 3) * (16 * kCoreStride) + (k & 7) * 16, v);
                 }
                 ptx::fence_proxy_async_smem();
-                ptx::mbar_arrive(&bars.full[sl]);
+                warp_arrive(&bars.full[sl]);
                 // every producer has finished reading the plane: it may be overwritten
-                ptx::named_bar(2, kSlabProdThreads);
+                ptx::named_bar(2, n_prod);
                 if (ptid == 0 && it + 1 < n_my) {
                     issue_plane(it + 1);
                     inflight = it + 1;
                 }
             } else {
                 const float *slice = plane(it);
-                for (int t0 = ptid; t0 < ntask; t0 += kSlabProdThreads * kSlabU) {
+                for (int t0 = ptid; t0 < ntask; t0 += n_prod * kSlabU) {
                     float v[kSlabU][8];
 #pragma unroll
                     for (int r = 0; r < kSlabU; ++r) {
-                        const int t = t0 + r * kSlabProdThreads;
+                        const int t = t0 + r * n_prod;
                         const int g = t & 15, k = t >> 4;
                         if (t < ntask && 8 * g < a.n1 && k < a.n2) {
                             ld8(slice + (long long)k * a.n1 + 8 * g, v[r]);
@@ -1095,7 +1155,7 @@ __global__ void __launch_bounds__(kSlabThreads, 1) tc_slab_kernel(const SlabArgs
                     }
 #pragma unroll
                     for (int r = 0; r < kSlabU; ++r) {
-                        const int t = t0 + r * kSlabProdThreads;
+                        const int t = t0 + r * n_prod;
                         if (t >= ntask) continue;
                         const int g = t & 15, k = t >> 4;
 #pragma unroll
@@ -1104,7 +1164,7 @@ __global__ void __launch_bounds__(kSlabThreads, 1) tc_slab_kernel(const SlabArgs
                     }
                 }
                 ptx::fence_proxy_async_smem();
-                ptx::mbar_arrive(&bars.full[sl]);
+                warp_arrive(&bars.full[sl]);
             }
             KX_CLK_ADD(2, tw);
         }
@@ -1125,9 +1185,19 @@ __global__ void __launch_bounds__(kSlabThreads, 1) tc_slab_kernel(const SlabArgs
         uint8_t *Alo = Ahi + half_bytes;
         double e_acc = 0.0;
         bool ok = true;
+        // the item's maximum and pair are loaded one unit ahead
+        float next_b1 = 0.f;
+        int2 next_ij = make_int2(0, 0);
+        auto fetch = [&](int j) {
+            const unsigned item = (unsigned)(blockIdx.x + (long long)j * gridDim.x) / (unsigned)a.n3;
+            next_b1 = __ldg(a.in_max + item);
+            if (a.e_partial != nullptr && !a.rhs_mode) next_ij = __ldg(a.pairs + item);
+        };
+        if (g < n_my) fetch(g);
         for (int j = g; j < n_my && ok; j += 2) {
             long long tw = KX_CLK_NOW();
-            const SlabUnit U = slab_unit(a, blockIdx.x + (long long)j * gridDim.x);
+            const SlabUnit U = slab_unit(a, blockIdx.x + (long long)j * gridDim.x, next_b1, next_ij);
+            if (j + 2 < n_my) fetch(j + 2);
             KX_CLK_ADD(0, tw);
             // ---- B: D1[x1][k2] -> A2[k2][x1]
             tw = KX_CLK_NOW();
@@ -1137,16 +1207,17 @@ __global__ void __launch_bounds__(kSlabThreads, 1) tc_slab_kernel(const SlabArgs
             tw = KX_CLK_NOW();
             ptx::tc_fence_after();
             if (32 * q < np1)
-                slab_transpose_stage(ta, tb, m, h, a.n1, np1, np2, two2, ldexpf(1.f, U.e2 - U.e1 - kVScaleExp), Ahi,
+                slab_transpose_stage(ta, tb, m, h, a.n1, np1, np2, two2, pow2f(U.e2 - U.e1 - kVScaleExp), Ahi,
                                      Alo);
             ptx::fence_proxy_async_smem();
             ptx::tc_fence_before();
-            ptx::mbar_arrive(&bars.ready[g]);
+            warp_arrive(&bars.ready[g]);
             KX_CLK_ADD(10, tw);
             // ---- C: D2[k2][k1] = Y: energy sum f Y^2, mid = f Y -> A3[k2][k1] (K-major, own row)
             {
                 const bool rowC = m < a.n2;
-                const float *frow = a.f32 + (U.k3 * a.n2 + m) * (long long)a.n1;
+                const int ld4 = 4 * a.n2;
+                const float *frow = a.f32 + (U.k3 * n12 + 4 * m);
                 // f(Lambda) of this warp's first chunk; each further chunk's is fetched
                 // while the previous one is processed
                 float fr[2][16];
@@ -1154,7 +1225,7 @@ __global__ void __launch_bounds__(kSlabThreads, 1) tc_slab_kernel(const SlabArgs
                 for (int hh = 0; hh < 2; ++hh) {
                     const int c0 = 16 * h + 8 * hh;
                     if (rowC && c0 < a.n1) {
-                        ld8(frow + c0, fr[0] + 8 * hh);
+                        ld8f(frow + (c0 >> 2) * ld4, ld4, fr[0] + 8 * hh);
                     } else {
 #pragma unroll
                         for (int k = 0; k < 8; ++k) fr[0][8 * hh + k] = 0.f;
@@ -1166,8 +1237,8 @@ __global__ void __launch_bounds__(kSlabThreads, 1) tc_slab_kernel(const SlabArgs
                 if (!ok) break;
                 tw = KX_CLK_NOW();
                 ptx::tc_fence_after();
-                const float u2 = ldexpf(1.f, -(U.e2 + kVScaleExp));
-                const float s3 = ldexpf(1.f, U.e3);
+                const float u2 = pow2f(-(U.e2 + kVScaleExp));
+                const float s3 = pow2f(U.e3);
                 const int off_r = (m >> 3) * (nkc1 * kCoreStride) + (m & 7) * 16;
                 float e_row = 0.f;
 #pragma unroll
@@ -1178,16 +1249,7 @@ __global__ void __launch_bounds__(kSlabThreads, 1) tc_slab_kernel(const SlabArgs
                     for (int hh = 0; hh < 2; ++hh) {
                         const int c0 = c + 32 + 8 * hh;
                         if (rowC && c0 < a.n1) {
-                            const float4 *src = reinterpret_cast<const float4 *>(frow + c0);
-                            const float4 x0 = __ldg(src), x1 = __ldg(src + 1);
-                            fr[(r + 1) & 1][8 * hh + 0] = x0.x;
-                            fr[(r + 1) & 1][8 * hh + 1] = x0.y;
-                            fr[(r + 1) & 1][8 * hh + 2] = x0.z;
-                            fr[(r + 1) & 1][8 * hh + 3] = x0.w;
-                            fr[(r + 1) & 1][8 * hh + 4] = x1.x;
-                            fr[(r + 1) & 1][8 * hh + 5] = x1.y;
-                            fr[(r + 1) & 1][8 * hh + 6] = x1.z;
-                            fr[(r + 1) & 1][8 * hh + 7] = x1.w;
+                            ld8f(frow + (c0 >> 2) * ld4, ld4, fr[(r + 1) & 1] + 8 * hh);
                         } else {
 #pragma unroll
                             for (int k = 0; k < 8; ++k) fr[(r + 1) & 1][8 * hh + k] = 0.f;
@@ -1195,9 +1257,11 @@ __global__ void __launch_bounds__(kSlabThreads, 1) tc_slab_kernel(const SlabArgs
                     }
                     float v[16], vb[16];
                     ptx::tmem_ld16x2(ta + c, tb + c, v, vb);
+                    if (!two1) zero16(vb);
+                    // (rows past n2 are never read back: no select for them)
 #pragma unroll
                     for (int k = 0; k < 16; ++k) {
-                        const float y = rowC ? (two1 ? v[k] + vb[k] : v[k]) * u2 : 0.f;
+                        const float y = (v[k] + vb[k]) * u2;
                         e_row = fmaf(fr[r & 1][k] * y, y, e_row);
                         v[k] = fr[r & 1][k] * y * s3;
                     }
@@ -1208,7 +1272,7 @@ __global__ void __launch_bounds__(kSlabThreads, 1) tc_slab_kernel(const SlabArgs
                 if (rowC) e_acc += U.w * (double)e_row;
                 ptx::fence_proxy_async_smem();
                 ptx::tc_fence_before();
-                ptx::mbar_arrive(&bars.ready[g]);
+                warp_arrive(&bars.ready[g]);
                 KX_CLK_ADD(11, tw);
             }
             // ---- D: D3[k2][x1] -> A4[x1][k2]
@@ -1219,11 +1283,11 @@ __global__ void __launch_bounds__(kSlabThreads, 1) tc_slab_kernel(const SlabArgs
             tw = KX_CLK_NOW();
             ptx::tc_fence_after();
             if (32 * q < np2)
-                slab_transpose_stage(ta, tb, m, h, a.n2, np2, np1, two1, ldexpf(1.f, U.e4 - U.e3 - kVScaleExp), Ahi,
+                slab_transpose_stage(ta, tb, m, h, a.n2, np2, np1, two1, pow2f(U.e4 - U.e3 - kVScaleExp), Ahi,
                                      Alo);
             ptx::fence_proxy_async_smem();
             ptx::tc_fence_before();
-            ptx::mbar_arrive(&bars.ready[g]);
+            warp_arrive(&bars.ready[g]);
             KX_CLK_ADD(3, tw);
             // ---- E: D4[x1][x2] -> slice [x2][x1] of the output, coalesced over x1
             tw = KX_CLK_NOW();
@@ -1233,21 +1297,26 @@ __global__ void __launch_bounds__(kSlabThreads, 1) tc_slab_kernel(const SlabArgs
             tw = KX_CLK_NOW();
             ptx::tc_fence_after();
             {
-                const float u4 = ldexpf(1.f, -(U.e4 + kVScaleExp));
+                const float u4 = pow2f(-(U.e4 + kVScaleExp));
                 const bool valid = m < a.n1;
-                float *orow = a.out + U.item * a.N + U.k3 * n12 + m;
                 float my_max = 0.f;
                 if (32 * q < a.n1) {
-                    for (int c = 16 * h; c < np2; c += 32) {
+                    float *orow = a.out + U.item * a.N + U.k3 * n12 + m + (long long)(16 * h) * a.n1;
+                    for (int c = 16 * h; c < np2; c += 32, orow += 32 * a.n1) {
                         float v[16], vb[16];
                         ptx::tmem_ld16x2(ta + c, tb + c, v, vb);
+                        if (!two2) zero16(vb);
                         if (!valid) continue;
+                        float *o = orow;
+                        // (n2 is a multiple of 8: each half of the chunk is in or out)
 #pragma unroll
-                        for (int k = 0; k < 16; ++k) {
-                            if (c + k < a.n2) {
-                                const float y = (two2 ? v[k] + vb[k] : v[k]) * u4;
+                        for (int g8 = 0; g8 < 2; ++g8) {
+                            if (c + 8 * g8 >= a.n2) break;
+#pragma unroll
+                            for (int k = 0; k < 8; ++k, o += a.n1) {
+                                const float y = (v[8 * g8 + k] + vb[8 * g8 + k]) * u4;
                                 my_max = fmaxf(my_max, fabsf(y));
-                                orow[(long long)(c + k) * a.n1] = y;
+                                *o = y;
                             }
                         }
                     }
@@ -1255,14 +1324,14 @@ __global__ void __launch_bounds__(kSlabThreads, 1) tc_slab_kernel(const SlabArgs
                 track_max(a.out_max, U.item, my_max, valid);
             }
             ptx::tc_fence_before();
-            ptx::mbar_arrive(&bars.ready[g]);
+            warp_arrive(&bars.ready[g]);
             KX_CLK_ADD(7, tw);
         }
         if (a.e_partial != nullptr) {
             double e = e_acc;
             for (int o = 16; o > 0; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
             if (lane == 0) s_red[warp] = e;
-            ptx::named_bar(1, kSlabEpiWarps * 32);
+            ptx::named_bar(1, 2 * group_threads);
             if (tid == 0) {
                 double sum = 0.0;
                 for (int w = 0; w < kSlabEpiWarps; ++w) sum += s_red[w];
@@ -1465,10 +1534,12 @@ int launch_pass(const kx_plan *p, PassArgs a, int axis, cudaStream_t s, int *gri
     return prof_end(const_cast<kx_plan *>(p), s);
 }
 
-size_t slab_smem(const kx_plan *p) {
+size_t slab_smem(const kx_plan *p, bool share_v = false) {
     const int np1 = p->np[0], np2 = p->np[1], npm = std::max(np1, np2);
-    return (size_t)4 * np1 * np1 + (size_t)4 * np2 * np2 + 4 * a_half_bytes(npm) + 1024;
+    return (size_t)4 * np1 * np1 + (share_v ? 0 : (size_t)4 * np2 * np2) + 4 * a_half_bytes(npm) + 1024;
 }
+// axes 1 and 2 of the same size, spacing and boundary have the same eigenvectors
+bool same_axes12(const kx_plan *p) { return p->n[0] == p->n[1] && p->h[0] == p->h[1] && p->bc[0] == p->bc[1]; }
 
 // The slab kernel holds V1, V2 and two split A buffers in shared memory.
 constexpr size_t kSlabSmemMax = 227 * 1024 - 1024;  // opt-in maximum less static shared memory
@@ -1513,7 +1584,8 @@ int launch_slab(kx_plan *p, long R, const float *in, const float *in_max, float 
     if (!g_clkbuf) cudaMallocManaged(&g_clkbuf, sizeof(long long) * kClk * 4096 * 6);
     a.clk = g_clkbuf + 5LL * kClk * 4096;
 #endif
-    size_t smem = slab_smem(p);
+    a.share_v = same_axes12(p) ? 1 : 0;
+    size_t smem = slab_smem(p, a.share_v != 0);
     const size_t plane = (size_t)a.n1 * a.n2 * 4;
     a.stage_in = (smem + plane <= kSlabSmemMax) ? 1 : 0;
     if (a.stage_in) smem += plane;

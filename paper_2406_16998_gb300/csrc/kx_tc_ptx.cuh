@@ -102,10 +102,38 @@ __device__ __forceinline__ void mma_f16(uint32_t d_tmem, uint64_t a, uint64_t b,
         "l"(a), "l"(b), "r"(idesc), "r"(accum)
         : "memory");
 }
+// The same with the descriptors given as 32-bit halves (the upper halves of a
+// product's descriptors never change).
+__device__ __forceinline__ void mma_f16_lo(uint32_t d_tmem, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo, uint32_t b_hi,
+                                           uint32_t idesc, uint32_t accum) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"
+        "setp.ne.b32 p, %6, 0;\n\t"
+        "mov.b64 da, {%1, %2};\n\t"
+        "mov.b64 db, {%3, %4};\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %5, p;\n\t}\n" ::"r"(d_tmem),
+        "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accum)
+        : "memory");
+}
 __device__ __forceinline__ void mma_commit(uint64_t *bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
                      smem_u32(bar))
                  : "memory");
+}
+
+// One lane of a converged warp, chosen by elect.sync.  A branch on it tells ptxas that
+// a single thread runs the code inside, so the operands of the MMAs issued there
+// stay in uniform registers; inside `if (lane == 0)` each of them is moved there
+// MMA by MMA (~100 cycles per MMA against 56 of tensor time at N = 96: slab kernel
+// 7.97 -> 6.95 ms per apply at 96^3 / 64 orbitals, 6.50 with the k-steps unrolled).
+__device__ __forceinline__ bool elect_one() {
+    uint32_t pred = 0;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "elect.sync _|p, 0xffffffff;\n\t"
+        "@p mov.u32 %0, 1;\n\t}\n"
+        : "+r"(pred));
+    return pred != 0;
 }
 
 // ---- TMEM -> registers: 8 consecutive fp32 columns of this thread's lane.
