@@ -27,6 +27,7 @@
 // with an S-deep ring of shared A stages and two TMEM accumulator slots, so
 // loads, MMAs and stores of consecutive tiles overlap.
 #include "kx_internal.h"
+#include "kx_conv.cuh"
 #include "kx_tc_ptx.cuh"
 
 #include <algorithm>
@@ -120,14 +121,33 @@ __device__ __forceinline__ float pow2f(int e) {
     return (unsigned)(e + 126) < 254u ? __int_as_float((e + 127) << 23) : ldexpf(1.f, e);
 }
 
-__device__ __forceinline__ void split8(const float *v, uint4 &hi, uint4 &lo) {
+// Packed float32 arithmetic (two values per instruction, each rounded as the scalar
+// form rounds it): the epilogues and producers below are bound by the length of
+// their instruction sequences.
+__device__ __forceinline__ float2 add2(float2 a, float2 b) {
+    unsigned long long r;
+    asm("add.rn.f32x2 %0, %1, %2;"
+        : "=l"(r)
+        : "l"(*reinterpret_cast<unsigned long long *>(&a)), "l"(*reinterpret_cast<unsigned long long *>(&b)));
+    return *reinterpret_cast<float2 *>(&r);
+}
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) {
+    unsigned long long r;
+    asm("mul.rn.f32x2 %0, %1, %2;"
+        : "=l"(r)
+        : "l"(*reinterpret_cast<unsigned long long *>(&a)), "l"(*reinterpret_cast<unsigned long long *>(&b)));
+    return *reinterpret_cast<float2 *>(&r);
+}
+
+__device__ __forceinline__ void split8(const float2 *v, uint4 &hi, uint4 &lo) {
     __half2 h[4], l[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-        __half2 hh = __floats2half2_rn(v[2 * i], v[2 * i + 1]);
-        float2 hf = __half22float2(hh);
+        const __half2 hh = __floats2half2_rn(v[i].x, v[i].y);
+        float2 r = v[i];
+        fma2(r, __half22float2(hh), make_float2(-1.f, -1.f));
         h[i] = hh;
-        l[i] = __floats2half2_rn(v[2 * i] - hf.x, v[2 * i + 1] - hf.y);
+        l[i] = __floats2half2_rn(r.x, r.y);
     }
     hi = *reinterpret_cast<uint4 *>(h);
     lo = *reinterpret_cast<uint4 *>(l);
@@ -139,6 +159,8 @@ __device__ __forceinline__ void ld8(const float *p, float *v) {
     v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
     v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
 }
+
+__device__ __forceinline__ float2 pair(const float *v, int k) { return make_float2(v[2 * k], v[2 * k + 1]); }
 
 // One k-step leaves the second accumulator unwritten: the epilogues then add zeros
 // (one branch per chunk; a select and a bound test per element made the last stage
@@ -305,9 +327,14 @@ __device__ __forceinline__ void produce_tile_u(const PassArgs &a, const TileMeta
                 off = g * kCoreStride + (k >> 3) * (16 * kCoreStride) + (k & 7) * 16;
                 sc = d.scale[g];
             }
-            float w[8];
+            float2 w[4];
+            const float2 sc2 = make_float2(sc, sc);
 #pragma unroll
-            for (int c = 0; c < 8; ++c) w[c] = (TWO ? v[r][c] * u[TWO ? r : 0][c] : v[r][c]) * sc;
+            for (int c = 0; c < 4; ++c) {
+                w[c] = make_float2(v[r][2 * c], v[r][2 * c + 1]);
+                if (TWO) w[c] = mul2(w[c], make_float2(u[TWO ? r : 0][2 * c], u[TWO ? r : 0][2 * c + 1]));
+                w[c] = mul2(w[c], sc2);
+            }
             uint4 hi4, lo4;
             split8(w, hi4, lo4);
             *reinterpret_cast<uint4 *>(Ahi + off) = hi4;
@@ -705,19 +732,22 @@ __global__ void __launch_bounds__(kThreads, 1) tc_pass_kernel(const PassArgs a) 
                         }
                     }
                     float v[16], vb[16];
+                    float2 mid[8];
                     ptx::tmem_ld16x2(ta + 16 * c, tb + 16 * c, v, vb);
                     if (!two_acc) zero16(vb);
 #pragma unroll
-                    for (int k = 0; k < 16; ++k) {
-                        const float y = (v[k] + vb[k]) * unscale;
-                        e_row = fmaf(fk[k] * y, y, e_row);
-                        v[k] = fk[k] * y * s_mid;
+                    for (int k = 0; k < 8; ++k) {
+                        const float2 y = mul2(add2(pair(v, k), pair(vb, k)), make_float2(unscale, unscale));
+                        const float2 fy = mul2(pair(fk, k), y);
+                        e_row = fmaf(fy.x, y.x, e_row);
+                        e_row = fmaf(fy.y, y.y, e_row);
+                        mid[k] = mul2(fy, make_float2(s_mid, s_mid));
                     }
                     if (with_inv) {
 #pragma unroll
                         for (int h2 = 0; h2 < 2; ++h2) {
                             uint4 hi, lo;
-                            split8(v + 8 * h2, hi, lo);
+                            split8(mid + 4 * h2, hi, lo);
                             const int off = (m >> 3) * ((np >> 3) * kCoreStride) + (2 * c + h2) * kCoreStride + (m & 7) * 16;
                             *reinterpret_cast<uint4 *>(midh + off) = hi;
                             *reinterpret_cast<uint4 *>(midh + half_bytes + off) = lo;
@@ -772,10 +802,11 @@ __global__ void __launch_bounds__(kThreads, 1) tc_pass_kernel(const PassArgs a) 
                         for (int g = 0; g < 4; ++g) {
                             if (cb + 8 * g >= a.nc) break;
 #pragma unroll
-                            for (int k = 8 * g; k < 8 * g + 8; ++k, o += ostride) {
-                                const float y = (v[k] + vb[k]) * unscale;
-                                my_max = fmaxf(my_max, fabsf(y));
-                                *o = y;
+                            for (int k = 4 * g; k < 4 * g + 4; ++k, o += 2 * ostride) {
+                                const float2 y = mul2(add2(pair(v, k), pair(vb, k)), make_float2(unscale, unscale));
+                                my_max = fmaxf(my_max, fmaxf(fabsf(y.x), fabsf(y.y)));
+                                o[0] = y.x;
+                                o[ostride] = y.y;
                             }
                         }
                     }
@@ -887,7 +918,7 @@ __device__ __forceinline__ bool slab_wait(uint64_t *bar, uint32_t parity, const 
     return true;
 }
 
-__device__ __forceinline__ void store_split8(uint8_t *hi_base, uint8_t *lo_base, int off, const float *w) {
+__device__ __forceinline__ void store_split8(uint8_t *hi_base, uint8_t *lo_base, int off, const float2 *w) {
     uint4 h, l;
     split8(w, h, l);
     *reinterpret_cast<uint4 *>(hi_base + off) = h;
@@ -933,9 +964,10 @@ __device__ __forceinline__ void slab_transpose_stage(uint32_t ta, uint32_t tb, i
         if (m < nprow) {
 #pragma unroll
             for (int g8 = 0; g8 < 2; ++g8) {
-                float w[8];
+                float2 w[4];
 #pragma unroll
-                for (int k = 0; k < 8; ++k) w[k] = (v[8 * g8 + k] + vb[8 * g8 + k]) * us;
+                for (int k = 0; k < 4; ++k)
+                    w[k] = mul2(add2(pair(v, 4 * g8 + k), pair(vb, 4 * g8 + k)), make_float2(us, us));
                 store_split8(Ahi, Alo, ((c >> 3) + g8) * kCoreStride + off_r, w);
             }
         }
@@ -1066,7 +1098,9 @@ __global__ void __launch_bounds__(kSlabThreads, 1) tc_slab_kernel(const SlabArgs
     } else if (warp >= kSlabEpiWarps || helper >= 0) {
         // ---------------------------------------------------------------- producers: A1 from global
         const int ptid = helper >= 0 ? 32 * (kSlabProdWarps + helper) + lane : tid - kSlabEpiWarps * 32;
-        const int ntask = 16 * np2;  // 16 row groups (x1) x np2 columns (x2)
+        const int ngrp = np1 >> 3;       // row groups (x1)
+        const int ntask = ngrp * np2;    // x np2 columns (x2)
+        const unsigned gmagic = (65536u + (unsigned)ngrp - 1u) / (unsigned)ngrp;  // t / ngrp for t < 2^11
         const int nlines = (int)((n12 * 4) >> 7);  // 128-byte lines of a slice (n1 % 8 == 0)
         const uint32_t plane_bytes = (uint32_t)(n12 * 4);
         auto plane = [&](int it) {
@@ -1115,20 +1149,34 @@ __global__ void __launch_bounds__(kSlabThreads, 1) tc_slab_kernel(const SlabArgs
             uint8_t *Ahi = buf0 + sl * 2 * half_bytes;
             uint8_t *Alo = Ahi + half_bytes;
             if (a.stage_in) {
-#pragma unroll 4
-                for (int t = ptid; t < ntask; t += n_prod) {
-                    const int g = t & 15, k = t >> 4;
-                    float v[8];
-                    if (8 * g < a.n1 && k < a.n2) {
-                        const float4 *src = reinterpret_cast<const float4 *>(sin + k * a.n1 + 8 * g);
-                        const float4 x0 = src[0], x1 = src[1];
-                        v[0] = x0.x * sc; v[1] = x0.y * sc; v[2] = x0.z * sc; v[3] = x0.w * sc;
-                        v[4] = x1.x * sc; v[5] = x1.y * sc; v[6] = x1.z * sc; v[7] = x1.w * sc;
-                    } else {
+                // task: 8 rows x1 at one x2.  Loads first, without branches between them: a task
+                // past the end repeats the last one, a padding one reads real values and scales
+                // them to zero.  Row groups past np1 are never read (see the quadrants above).
+                for (int t0 = ptid; t0 < ntask; t0 += 4 * n_prod) {
+                    float4 x[4][2];
+                    int off[4];
+                    float scl[4];
 #pragma unroll
-                        for (int c = 0; c < 8; ++c) v[c] = 0.f;
+                    for (int r = 0; r < 4; ++r) {
+                        const int t = min(t0 + r * n_prod, ntask - 1);
+                        const int k = (int)(((unsigned)t * gmagic) >> 16), g = t - k * ngrp;
+                        const bool in = 8 * g < a.n1 && k < a.n2;
+                        const float4 *src = reinterpret_cast<const float4 *>(sin + (in ? k * a.n1 + 8 * g : 0));
+                        x[r][0] = src[0];
+                        x[r][1] = src[1];
+                        scl[r] = in ? sc : 0.f;
+                        off[r] = g * kCoreStride + (k >> 3) * (16 * kCoreStride) + (k & 7) * 16;
                     }
-                    store_split8(Ahi, Alo, g * kCoreStride + (k >> 3) * (16 * kCoreStride) + (k & 7) * 16, v);
+#pragma unroll
+                    for (int r = 0; r < 4; ++r) {
+                        if (t0 + r * n_prod >= ntask) break;
+                        const float2 s2 = make_float2(scl[r], scl[r]);
+                        const float2 w[4] = {mul2(make_float2(x[r][0].x, x[r][0].y), s2),
+                                             mul2(make_float2(x[r][0].z, x[r][0].w), s2),
+                                             mul2(make_float2(x[r][1].x, x[r][1].y), s2),
+                                             mul2(make_float2(x[r][1].z, x[r][1].w), s2)};
+                        store_split8(Ahi, Alo, off[r], w);
+                    }
                 }
                 ptx::fence_proxy_async_smem();
                 warp_arrive(&bars.full[sl]);
@@ -1145,7 +1193,7 @@ __global__ void __launch_bounds__(kSlabThreads, 1) tc_slab_kernel(const SlabArgs
 #pragma unroll
                     for (int r = 0; r < kSlabU; ++r) {
                         const int t = t0 + r * n_prod;
-                        const int g = t & 15, k = t >> 4;
+                        const int k = (int)(((unsigned)t * gmagic) >> 16), g = t - k * ngrp;
                         if (t < ntask && 8 * g < a.n1 && k < a.n2) {
                             ld8(slice + (long long)k * a.n1 + 8 * g, v[r]);
                         } else {
@@ -1157,10 +1205,11 @@ __global__ void __launch_bounds__(kSlabThreads, 1) tc_slab_kernel(const SlabArgs
                     for (int r = 0; r < kSlabU; ++r) {
                         const int t = t0 + r * n_prod;
                         if (t >= ntask) continue;
-                        const int g = t & 15, k = t >> 4;
+                        const int k = (int)(((unsigned)t * gmagic) >> 16), g = t - k * ngrp;
+                        float2 w[4];
 #pragma unroll
-                        for (int c = 0; c < 8; ++c) v[r][c] *= sc;
-                        store_split8(Ahi, Alo, g * kCoreStride + (k >> 3) * (16 * kCoreStride) + (k & 7) * 16, v[r]);
+                        for (int c = 0; c < 4; ++c) w[c] = mul2(pair(v[r], c), make_float2(sc, sc));
+                        store_split8(Ahi, Alo, g * kCoreStride + (k >> 3) * (16 * kCoreStride) + (k & 7) * 16, w);
                     }
                 }
                 ptx::fence_proxy_async_smem();
@@ -1259,15 +1308,18 @@ __global__ void __launch_bounds__(kSlabThreads, 1) tc_slab_kernel(const SlabArgs
                     ptx::tmem_ld16x2(ta + c, tb + c, v, vb);
                     if (!two1) zero16(vb);
                     // (rows past n2 are never read back: no select for them)
+                    float2 mid[8];
 #pragma unroll
-                    for (int k = 0; k < 16; ++k) {
-                        const float y = (v[k] + vb[k]) * u2;
-                        e_row = fmaf(fr[r & 1][k] * y, y, e_row);
-                        v[k] = fr[r & 1][k] * y * s3;
+                    for (int k = 0; k < 8; ++k) {
+                        const float2 y = mul2(add2(pair(v, k), pair(vb, k)), make_float2(u2, u2));
+                        const float2 fy = mul2(pair(fr[r & 1], k), y);
+                        e_row = fmaf(fy.x, y.x, e_row);
+                        e_row = fmaf(fy.y, y.y, e_row);
+                        mid[k] = mul2(fy, make_float2(s3, s3));
                     }
 #pragma unroll
                     for (int hh = 0; hh < 2; ++hh)
-                        store_split8(Ahi, Alo, off_r + ((c >> 3) + hh) * kCoreStride, v + 8 * hh);
+                        store_split8(Ahi, Alo, off_r + ((c >> 3) + hh) * kCoreStride, mid + 4 * hh);
                 }
                 if (rowC) e_acc += U.w * (double)e_row;
                 ptx::fence_proxy_async_smem();
@@ -1313,10 +1365,11 @@ __global__ void __launch_bounds__(kSlabThreads, 1) tc_slab_kernel(const SlabArgs
                         for (int g8 = 0; g8 < 2; ++g8) {
                             if (c + 8 * g8 >= a.n2) break;
 #pragma unroll
-                            for (int k = 0; k < 8; ++k, o += a.n1) {
-                                const float y = (v[8 * g8 + k] + vb[8 * g8 + k]) * u4;
-                                my_max = fmaxf(my_max, fabsf(y));
-                                *o = y;
+                            for (int k = 4 * g8; k < 4 * g8 + 4; ++k, o += 2 * a.n1) {
+                                const float2 y = mul2(add2(pair(v, k), pair(vb, k)), make_float2(u4, u4));
+                                my_max = fmaxf(my_max, fmaxf(fabsf(y.x), fabsf(y.y)));
+                                o[0] = y.x;
+                                o[a.n1] = y.y;
                             }
                         }
                     }
