@@ -232,9 +232,7 @@ static int reserve(kx_plan *p, int n_orb) {
     if ((rc = mp_reserve(p, n_orb))) return rc;
     if (p->precision == KX_FP64) {
         const long P = (long)n_orb * (n_orb + 1) / 2;
-        const size_t budget = (size_t)2 << 30;
-        long c = (long)std::max<size_t>(1, budget / (3 * p->N * sizeof(double)));
-        return ensure_workspace(p, fp64_workspace_bytes(p, std::min(c, P)));
+        return ensure_workspace(p, fp64_workspace_bytes(p, fp64_chunk(p, P)));
     }
     const long P = (long)n_orb * (n_orb + 1) / 2;
     const long chunk = std::min<long>(tc_default_chunk(p, n_orb), P);

@@ -119,6 +119,12 @@ struct kx_plan_s {
     float *d_fft_tw = nullptr;
     float *d_fft_f = nullptr;
 
+    // float64 path (fp64_setup): per axis the tables of the even and odd eigenvectors,
+    // the number of even ones, and f in the order even, odd along every axis
+    double *d_p64_tab[3] = {nullptr, nullptr, nullptr};
+    double *d_p64_f = nullptr;
+    int p64_he[3] = {0, 0, 0};
+
     int *d_status = nullptr;                          // bounded-wait status word
 
     kx::TuneParams tune;
@@ -183,6 +189,8 @@ int ensure_workspace(kx_plan *p, size_t bytes);
 int ensure_pairs(kx_plan *p, int n_orb, cudaStream_t s, long long begin = 0, long long end = -1);
 
 // ---- FP64 path (kx_fp64.cu)
+int fp64_setup(kx_plan *p);  // parity tables (synchronous; once per plan)
+long fp64_chunk(const kx_plan *p, long want);
 int fp64_apply_fL(kx_plan *p, int n_rhs, const double *b, double *x, cudaStream_t s);
 int fp64_vx(kx_plan *p, int n_orb, const double *psi, const double *occ, double *vx, double *ex,
             bool energy_only, cudaStream_t s, long pair_begin = 0, long pair_end = -1);

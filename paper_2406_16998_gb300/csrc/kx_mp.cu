@@ -986,6 +986,7 @@ int mp_set(kx_plan *p, int l_max) {
     e = cudaGetLastError();
     int rc = e == cudaSuccess ? KX_OK : cuda_error(e, "mp_fields_kernel launch");
     // h_k = f(L) g_k with the float64 solver (set-up, once per plan)
+    if (!rc) rc = fp64_setup(p);
     if (!rc) rc = fp64_apply_fL(p, K, Gk, p->d_mpH, nullptr);
     if (!rc) {
         to_f32_kernel<<<1024, 256>>>(p->d_mpR, p->d_mpR32, (long long)K * N);

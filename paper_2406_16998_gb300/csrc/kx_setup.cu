@@ -264,6 +264,8 @@ int plan_setup(kx_plan *p) {
     }
     if (p->precision == KX_FFT32)
         if (int rc = fft_setup(p)) return rc;
+    if (p->precision == KX_FP64)
+        if (int rc = fp64_setup(p)) return rc;
     double *d_fmax = nullptr;
     KX_CUDA_TRY(cudaMalloc(&d_fmax, sizeof(double)));
     fmax_kernel<<<1, 256>>>(p->d_f64, p->N, d_fmax);
@@ -280,7 +282,9 @@ void plan_free(kx_plan *p) {
         cudaFree(p->d_lam[a]);
         cudaFree(p->d_V[a]);
         cudaFree(p->d_Vs[a]);
+        cudaFree(p->d_p64_tab[a]);
     }
+    cudaFree(p->d_p64_f);
     cudaFree(p->d_f64);
     cudaFree(p->d_f32);
     cudaFree(p->d_fft_tw);

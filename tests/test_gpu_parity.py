@@ -115,6 +115,31 @@ def test_fp64_odd_sizes(kx):
     assert abs(ex.item() - ex_ref) < 1e-11 * abs(ex_ref)
 
 
+@pytest.mark.parametrize("n,bc", [((2, 3, 5), (P, P, D)), ((3, 2, 7), (D, P, P)), ((128, 2, 9), (P, D, D)),
+                                  ((5, 127, 4), (D, P, D)), ((6, 4, 128), (D, D, P)), ((33, 16, 31), (P, P, P)),
+                                  ((17, 66, 12), (D, D, D))])
+def test_fp64_parity_form(kx, n, bc):
+    """The float64 products by even and odd eigenvectors: even and odd sizes, the smallest
+    and largest axes, both boundaries on each axis (points that are their own mirror
+    image: the middle one, or 0 and n / 2), one and many right-hand sides (every tile width)."""
+    h = (0.4, 0.5, 0.45)
+    op = oracle.Plan(n, h, bc, S)
+    plan = kx.Plan(n, h, bc, S, precision=0)
+    for n_rhs in (1, 70):
+        b = workloads.random_field(op.N, n_rhs, 91)
+        ref = np.stack([oracle.apply_fL(op, b[:, r]) for r in range(n_rhs)], axis=1)
+        x = kx.kx_apply_fL(plan, dev(b.T)).cpu().numpy().T
+        assert relmax(x, ref) < 1e-11
+    psi = workloads.random_field(op.N, 3, 92)
+    occ = np.array([1.0, 0.7, 0.2])
+    vx_ref, ex_ref = oracle.vx_apply(op, psi, occ)
+    vx, ex = kx.kx_vx_apply(plan, dev(psi.T), dev(occ))
+    e_only = kx.kx_energy(plan, dev(psi.T), dev(occ))
+    assert relmax(vx.cpu().numpy().T, vx_ref) < 1e-11
+    assert abs(ex.item() - ex_ref) < 1e-11 * abs(ex_ref)
+    assert abs(e_only.item() - ex_ref) < 1e-11 * abs(ex_ref)
+
+
 def test_setup_eigendecomposition_and_ftable(kx):
     n, h, bc, kind = (24, 40, 16), (0.45, 0.4, 0.5), (D, P, D), S
     op = oracle.Plan(n, h, bc, kind)
