@@ -55,13 +55,27 @@ __global__ void gram_kernel(const double *__restrict__ psi, int na, const double
 }
 
 // M[e] = dV sum_k part[k][e] in a fixed order (deterministic); optional copies
-// of M and -M.
-__global__ void gram_reduce_kernel(const double *__restrict__ part, int n_slab, int n_e, double dV,
-                                   double *__restrict__ M, double *__restrict__ M_out, double *__restrict__ negM) {
-    int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= n_e) return;
+// of M and -M.  A CTA takes 32 entries, its 16 warps every 16th slab of them:
+// latency-bound on the slabs' loads (one thread per entry walking all 304 slabs of
+// a 64 x 64 product took 33.6 us).
+constexpr int kRedWarps = 16;
+__global__ void __launch_bounds__(32 * kRedWarps) gram_reduce_kernel(const double *__restrict__ part, int n_slab,
+                                                                     int n_e, double dV, double *__restrict__ M,
+                                                                     double *__restrict__ M_out,
+                                                                     double *__restrict__ negM) {
+    __shared__ double red[kRedWarps][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int e = blockIdx.x * 32 + lane;
     double s = 0.0;
-    for (int k = 0; k < n_slab; ++k) s += part[(long long)k * n_e + e];
+    if (e < n_e) {
+#pragma unroll 4
+        for (int k = warp; k < n_slab; k += kRedWarps) s += part[(long long)k * n_e + e];
+    }
+    red[warp][lane] = s;
+    __syncthreads();
+    if (warp != 0 || e >= n_e) return;
+    s = 0.0;
+    for (int w = 0; w < kRedWarps; ++w) s += red[w][lane];
     s *= dV;
     M[e] = s;
     if (M_out) M_out[e] = s;
@@ -69,47 +83,76 @@ __global__ void gram_reduce_kernel(const double *__restrict__ part, int n_slab, 
 }
 
 // In-place Cholesky of the symmetric positive definite A (lower triangle used):
-// A = L L^T; writes R = L^T (upper) to R.  One CTA; *bad = 1 if a pivot <= 0.
-__global__ void cholesky_kernel(double *__restrict__ A, int n, double *__restrict__ R, int *__restrict__ bad) {
-    __shared__ double piv;
+// A = L L^T; the diagonal of A receives the reciprocals of L's, *bad = 1 if a pivot
+// <= 0.  One CTA, the matrix in shared memory where it fits (n <= kCholSmemN).  A
+// serial chain of n pivots (square root, reciprocal, two barriers) over rank-1
+// updates of the lower triangle, a warp per row: 130 us at n = 64 with the
+// updates in global memory and a division per entry of the column.
+constexpr int kCholThreads = 512;
+constexpr int kCholSmemN = 160;  // 205 KB
+__global__ void __launch_bounds__(kCholThreads) cholesky_kernel(double *__restrict__ A, int n, int *__restrict__ bad) {
+    extern __shared__ double chol_sm[];
+    __shared__ double rpiv;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const bool in_smem = n <= kCholSmemN;
+    double *L = in_smem ? chol_sm : A;
+    const int ld = n;
+    if (in_smem)
+        for (int e = tid; e < n * n; e += kCholThreads) L[e] = A[e];
+    __syncthreads();
     for (int k = 0; k < n; ++k) {
-        if (threadIdx.x == 0) {
-            double d = A[k * n + k];
+        if (tid == 0) {
+            double d = L[k * ld + k];
             if (!(d > 0.0)) {
                 *bad = 1;
                 d = 1.0;
             }
-            piv = sqrt(d);
-            A[k * n + k] = piv;
+            rpiv = 1.0 / sqrt(d);
+            L[k * ld + k] = rpiv;
         }
         __syncthreads();
-        for (int i = k + 1 + threadIdx.x; i < n; i += blockDim.x) A[i * n + k] /= piv;
+        const double r = rpiv;
+        for (int i = k + 1 + tid; i < n; i += kCholThreads) L[i * ld + k] *= r;
         __syncthreads();
-        const int m = n - k - 1;
-        for (int e = threadIdx.x; e < m * m; e += blockDim.x) {
-            int i = k + 1 + e / m, j = k + 1 + e % m;
-            if (j <= i) A[i * n + j] -= A[i * n + k] * A[j * n + k];
+        for (int i = k + 1 + warp; i < n; i += kCholThreads / 32) {
+            const double lik = L[i * ld + k];
+            for (int j = k + 1 + lane; j <= i; j += 32) L[i * ld + j] = fma(-lik, L[j * ld + k], L[i * ld + j]);
         }
         __syncthreads();
     }
-    for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
-        int i = e / n, j = e % n;  // R[i][j] = L[j][i] for j >= i
-        R[e] = (j >= i) ? A[j * n + i] : 0.0;
-    }
+    if (in_smem)
+        for (int e = tid; e < n * n; e += kCholThreads) A[e] = L[e];
 }
 
-// Rinv = R^{-1} (upper triangular), one thread per column, back substitution.
-__global__ void triinv_kernel(const double *__restrict__ R, int n, double *__restrict__ Rinv) {
-    int j = blockIdx.x * blockDim.x + threadIdx.x;
+// Rinv = R^{-1} = L^{-T} (upper triangular) from cholesky_kernel's L, a warp per column:
+// solve R x = e_j from the last row up, lane l holding the running right-hand sides
+// of the rows l + 32 u, so that a step is one broadcast and n / 32 FMAs (143 us at
+// n = 64 with one thread per column).
+constexpr int kInvU = 8;  // n <= 256
+__global__ void __launch_bounds__(128) triinv_kernel(const double *__restrict__ L, int n, double *__restrict__ Rinv) {
+    const int lane = threadIdx.x & 31, j = blockIdx.x * 4 + (threadIdx.x >> 5);
     if (j >= n) return;
-    for (int i = n - 1; i >= 0; --i) {
-        double s = (i == j) ? 1.0 : 0.0;
-        if (i > j) {
-            Rinv[i * n + j] = 0.0;
-            continue;
+    double s[kInvU];
+#pragma unroll
+    for (int u = 0; u < kInvU; ++u) s[u] = (lane + 32 * u == j) ? 1.0 : 0.0;
+#pragma unroll
+    for (int ub = kInvU - 1; ub >= 0; --ub) {  // rows i = 32 ub + ib, descending
+        if (32 * ub > j) continue;
+        for (int ib = min(31, j - 32 * ub); ib >= 0; --ib) {
+            const int i = 32 * ub + ib;
+            const double x = __shfl_sync(0xffffffffu, s[ub], ib) * __ldg(L + i * n + i);
+            if (lane == ib) s[ub] = x;  // final
+#pragma unroll
+            for (int u = 0; u <= ub; ++u) {
+                const int k = lane + 32 * u;
+                if (k < i) s[u] = fma(-__ldg(L + i * n + k), x, s[u]);  // R[k][i] = L[i][k]
+            }
         }
-        for (int k = i + 1; k <= j; ++k) s -= R[i * n + k] * Rinv[k * n + j];
-        Rinv[i * n + j] = s / R[i * n + i];
+    }
+#pragma unroll
+    for (int u = 0; u < kInvU; ++u) {
+        const int k = lane + 32 * u;
+        if (k < n) Rinv[k * n + j] = k <= j ? s[u] : 0.0;
     }
 }
 
@@ -492,23 +535,25 @@ int launch_combination(kx_plan *p, const double *A, int na, const double *C, int
 int ace_run(kx_plan *p, int n_orb, const double *psi, const double *W, double *xi, double *M_out, cudaStream_t s) {
     const int n_slab = projection_split(p, n_orb, n_orb);
     const size_t nn = (size_t)n_orb * n_orb;
-    const size_t bytes = sizeof(double) * (nn * (size_t)n_slab + 4 * nn) + 256;
+    const size_t bytes = sizeof(double) * (nn * (size_t)n_slab + 3 * nn) + 256;
     int rc = ensure_workspace(p, bytes);
     if (rc) return rc;
     double *part = (double *)p->ws.ptr;
     double *M = part + nn * n_slab;
     double *A = M + nn;
-    double *R = A + nn;
-    double *Rinv = R + nn;
+    double *Rinv = A + nn;
     int *bad = reinterpret_cast<int *>(Rinv + nn);
     KX_CUDA_TRY(cudaMemsetAsync(bad, 0, sizeof(int), s));
     if ((rc = launch_projection(p, psi, n_orb, W, n_orb, nullptr, nullptr, part, n_slab, s))) return rc;
     if ((rc = prof_begin(p, PK_ACE, s))) return rc;
-    gram_reduce_kernel<<<(unsigned)((nn + 255) / 256), 256, 0, s>>>(part, n_slab, (int)nn, p->dV, M, M_out, A);
+    gram_reduce_kernel<<<(unsigned)((nn + 31) / 32), 32 * kRedWarps, 0, s>>>(part, n_slab, (int)nn, p->dV, M, M_out, A);
     KX_LAUNCH_CHECK("gram_reduce_kernel launch");
-    cholesky_kernel<<<1, 256, 0, s>>>(A, n_orb, R, bad);
+    const size_t chol_smem = n_orb <= kCholSmemN ? sizeof(double) * nn : 0;
+    KX_CUDA_TRY(cudaFuncSetAttribute(cholesky_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)(sizeof(double) * kCholSmemN * kCholSmemN)));
+    cholesky_kernel<<<1, kCholThreads, chol_smem, s>>>(A, n_orb, bad);
     KX_LAUNCH_CHECK("cholesky_kernel launch");
-    triinv_kernel<<<(n_orb + 127) / 128, 128, 0, s>>>(R, n_orb, Rinv);
+    triinv_kernel<<<(n_orb + 3) / 4, 128, 0, s>>>(A, n_orb, Rinv);
     KX_LAUNCH_CHECK("triinv_kernel launch");
     if ((rc = prof_end(p, s))) return rc;
     if ((rc = launch_combination(p, W, n_orb, Rinv, n_orb, 1.0, false, xi, s))) return rc;
@@ -530,7 +575,7 @@ int ace_apply_run(kx_plan *p, int n_xi, const double *xi, int n_vec, const doubl
     // P = dV xi^T phi, then out = -xi P
     if ((rc = launch_projection(p, xi, n_xi, phi, n_vec, nullptr, nullptr, part, n_split, s))) return rc;
     if ((rc = prof_begin(p, PK_ACE, s))) return rc;
-    gram_reduce_kernel<<<(unsigned)((ne + 255) / 256), 256, 0, s>>>(part, n_split, (int)ne, p->dV, P, nullptr,
+    gram_reduce_kernel<<<(unsigned)((ne + 31) / 32), 32 * kRedWarps, 0, s>>>(part, n_split, (int)ne, p->dV, P, nullptr,
                                                                     nullptr);
     KX_LAUNCH_CHECK("gram_reduce_kernel launch");
     if ((rc = prof_end(p, s))) return rc;
@@ -550,7 +595,7 @@ int grid_projection(kx_plan *p, const double *A, int na, const double *B, int nb
     double *part = (double *)p->ws.ptr;
     if ((rc = launch_projection(p, A, na, B, nb, w64, w32, part, n_split, s, kind))) return rc;
     if ((rc = prof_begin(p, kind, s))) return rc;
-    gram_reduce_kernel<<<(unsigned)((ne + 255) / 256), 256, 0, s>>>(part, n_split, (int)ne, scale, out, nullptr,
+    gram_reduce_kernel<<<(unsigned)((ne + 31) / 32), 32 * kRedWarps, 0, s>>>(part, n_split, (int)ne, scale, out, nullptr,
                                                                     nullptr);
     KX_LAUNCH_CHECK("gram_reduce_kernel launch");
     return prof_end(p, s);

@@ -1620,17 +1620,28 @@ __global__ void bloch_basis_kernel(BlochAxes ax, typename Cx<T>::t *Mf0, typenam
     const bool bloch = ax.bc[a] == KX_PERIODIC;
     const double th = ax.theta[a];
     const double inv_sqrt_n = 1.0 / sqrt((double)n);
+    // e^{i 2 pi t / n} (the angle m x reduced exactly to t) and e^{i theta x / n}: n values
+    // each, the float64 sine pairs of every entry took 28 us per pair of k-points
+    __shared__ double2 rt[kMaxN], ph[kMaxN];
+    if (bloch)
+        for (int t = threadIdx.x; t < 2 * n; t += blockDim.x) {
+            double sv, cv;
+            if (t < n) {
+                sincospi(2.0 * t / n, &sv, &cv);
+                rt[t] = make_double2(cv, sv);
+            } else {
+                sincos(th * (t - n) / n, &sv, &cv);
+                ph[t - n] = make_double2(cv, sv);
+            }
+        }
+    __syncthreads();
     for (int e = blockIdx.y * blockDim.x + threadIdx.x; e < n * n; e += gridDim.y * blockDim.x) {
         int x = e / n, m = e - x * n;
         double vr, vi;
         if (bloch) {
-            // e^{i 2 pi m x / n} with the angle reduced exactly, times e^{i theta x / n}
-            int t = (int)(((long long)m * x) % n);
-            double s1, c1, s2, c2;
-            sincospi(2.0 * t / n, &s1, &c1);
-            sincos(th * x / n, &s2, &c2);
-            vr = (c1 * c2 - s1 * s2) * inv_sqrt_n;
-            vi = (s1 * c2 + c1 * s2) * inv_sqrt_n;
+            const double2 r = rt[(m * x) % n], p = ph[x];
+            vr = (r.x * p.x - r.y * p.y) * inv_sqrt_n;
+            vi = (r.y * p.x + r.x * p.y) * inv_sqrt_n;
         } else {
             vr = ax.V[a][x * n + m];
             vi = 0.0;
@@ -1830,12 +1841,20 @@ __global__ void __launch_bounds__(kEThreads) bloch_energy_kernel(const double2 *
     }
 }
 
-__global__ void bloch_energy_final_kernel(const double *partial, int count, double half_dv, double *ex) {
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
-        double t = 0.0;
-        for (int i = 0; i < count; ++i) t += partial[i];
-        *ex = half_dv * t;
-    }
+// ex = half_dv sum partial: fixed strided sums and a fixed tree (75 us with one thread
+// for the 1,216 partials of four k-points).
+__global__ void __launch_bounds__(1024) bloch_energy_final_kernel(const double *partial, int count, double half_dv,
+                                                                  double *ex) {
+    __shared__ double red[32];
+    double t = 0.0;
+    for (int i = threadIdx.x; i < count; i += 1024) t += partial[i];
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = t;
+    __syncthreads();
+    if (threadIdx.x >= 32) return;
+    t = red[threadIdx.x];
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if (threadIdx.x == 0) *ex = half_dv * t;
 }
 
 inline size_t al256(size_t b) { return (b + 255) / 256 * 256; }
@@ -2481,7 +2500,7 @@ int bloch_all(kx_plan *p, int n_kpt, const double *theta, const double *wk, int 
                                                      wk[k], partial + (size_t)k * nb);
         KX_LAUNCH_CHECK("bloch_energy_kernel launch");
     }
-    bloch_energy_final_kernel<<<1, 32, 0, s>>>(partial, nb * n_kpt, 0.5 * p->dV, ex);
+    bloch_energy_final_kernel<<<1, 1024, 0, s>>>(partial, nb * n_kpt, 0.5 * p->dV, ex);
     KX_LAUNCH_CHECK("bloch_energy_final_kernel launch");
     return prof_end(p, s);
 }
@@ -2625,7 +2644,7 @@ int bloch_energy_only(kx_plan *p, int n_kpt, const double *theta, const double *
         }
     }
     if (int rc = prof_begin(p, PK_BLOCH_OTHER, s)) return rc;
-    bloch_energy_final_kernel<<<1, 32, 0, s>>>(partial, (int)(n_launch * slot), 1.0, ex);
+    bloch_energy_final_kernel<<<1, 1024, 0, s>>>(partial, (int)(n_launch * slot), 1.0, ex);
     KX_LAUNCH_CHECK("bloch_energy_final_kernel launch");
     return prof_end(p, s);
 }

@@ -1526,12 +1526,17 @@ __global__ void finalize_scalar_kernel(const float *__restrict__ acc, double *__
         vx[e] = -(double)acc[e];
 }
 
-__global__ void energy_add_kernel(const double *__restrict__ partial, int n, double factor, double *e_x) {
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
-        double s = 0.0;
-        for (int b = 0; b < n; ++b) s += partial[b];
-        *e_x += factor * s;
-    }
+// e_x += factor sum partial[0 .. n), n <= 1024: strided partial sums and a fixed tree
+// (one thread adding them took 10 us, a fifth of the smallest apply).
+__global__ void __launch_bounds__(128) energy_add_kernel(const double *__restrict__ partial, int n, double factor,
+                                                         double *e_x) {
+    __shared__ double red[4];
+    double s = 0.0;
+    for (int b = threadIdx.x; b < n; b += 128) s += partial[b];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+    __syncthreads();
+    if (threadIdx.x == 0) *e_x += factor * ((red[0] + red[1]) + (red[2] + red[3]));
 }
 
 // Failure-path self-test: wait on an mbarrier phase that nothing completes; the
@@ -1702,7 +1707,7 @@ int run_passes(kx_plan *p, PassArgs a, long R, float *T0, float *T1, float *mx, 
             return rc;
         if (ex) {
             if ((rc = prof_begin(p, PK_FINAL, s))) return rc;
-            energy_add_kernel<<<1, 32, 0, s>>>(partial, grid, -0.5 * p->dV, ex);
+            energy_add_kernel<<<1, 128, 0, s>>>(partial, grid, -0.5 * p->dV, ex);
             KX_LAUNCH_CHECK("energy_add_kernel launch");
             if ((rc = prof_end(p, s))) return rc;
         }
@@ -1738,7 +1743,7 @@ int run_passes(kx_plan *p, PassArgs a, long R, float *T0, float *T1, float *mx, 
     if ((rc = launch_pass<P_X1>(p, a, 0, s, &grid))) return rc;
     if (ex) {
         if ((rc = prof_begin(p, PK_FINAL, s))) return rc;
-        energy_add_kernel<<<1, 32, 0, s>>>(partial, grid, -0.5 * p->dV, ex);
+        energy_add_kernel<<<1, 128, 0, s>>>(partial, grid, -0.5 * p->dV, ex);
         KX_LAUNCH_CHECK("energy_add_kernel launch");
         if ((rc = prof_end(p, s))) return rc;
     }
