@@ -122,10 +122,8 @@ int ensure_pairs(kx_plan *p, int n_orb, cudaStream_t s, long long begin, long lo
             Group g{};
             g.first_item = (int)(pairs.size() / 2);
             g.n_items = 0;
-            g.n_slots = (IB == JB) ? bi : bi + bj;
-            for (int t = 0; t < bi; ++t) g.orb[t] = I0 + t;
-            if (IB != JB)
-                for (int t = 0; t < bj; ++t) g.orb[bi + t] = J0 + t;
+            g.blk_i = IB;
+            g.blk_j = IB == JB ? -1 : JB;
             for (int si = 0; si < bi; ++si) {
                 for (int sj = (IB == JB ? si : 0); sj < (IB == JB ? bi : bj); ++sj, ++k) {
                     if (k < begin || k >= end) continue;
@@ -145,12 +143,15 @@ int ensure_pairs(kx_plan *p, int n_orb, cudaStream_t s, long long begin, long lo
         }
     }
     first.push_back((int)(pairs.size() / 2));
-    std::vector<int> last(n_orb, -1), maxorb(groups.size(), 0);
+    std::vector<int> last(n_orb, -1), span(2 * (size_t)n_orb, -1), maxorb(groups.size(), 0);
     for (size_t gi = 0; gi < groups.size(); ++gi)
-        for (int t = 0; t < groups[gi].n_slots; ++t) {
-            last[groups[gi].orb[t]] = (int)gi;
-            maxorb[gi] = std::max(maxorb[gi], groups[gi].orb[t]);
-        }
+        for (int blk : {groups[gi].blk_i, groups[gi].blk_j})
+            for (int o = blk * kOrbBlock; blk >= 0 && o < std::min(n_orb, (blk + 1) * kOrbBlock); ++o) {
+                last[o] = (int)gi;
+                if (span[2 * o] < 0) span[2 * o] = (int)gi;
+                span[2 * o + 1] = (int)gi;
+                maxorb[gi] = std::max(maxorb[gi], o);
+            }
     const size_t P = pairs.size() / 2;
     if (P > p->pairs_cap) {
         cudaFree(p->d_pairs);
@@ -178,6 +179,15 @@ int ensure_pairs(kx_plan *p, int n_orb, cudaStream_t s, long long begin, long lo
         if (e != cudaSuccess) return cuda_error(e, "pair mask cudaMalloc");
         p->pair_mask_cap = mask.size();
     }
+    if ((size_t)n_orb > p->orb_span_cap) {
+        cudaFree(p->d_orb_span);
+        p->d_orb_span = nullptr;
+        p->orb_span_cap = 0;
+        cudaError_t e = cudaMalloc(&p->d_orb_span, sizeof(int) * 2 * n_orb);
+        if (e != cudaSuccess) return cuda_error(e, "orbital span cudaMalloc");
+        p->orb_span_cap = (size_t)n_orb;
+    }
+    KX_CUDA_TRY(cudaMemcpy(p->d_orb_span, span.data(), sizeof(int) * span.size(), cudaMemcpyHostToDevice));
     KX_CUDA_TRY(cudaMemcpy(p->d_pair_mask, mask.data(), mask.size(), cudaMemcpyHostToDevice));
     if (P) {
         KX_CUDA_TRY(cudaMemcpy(p->d_pairs, pairs.data(), sizeof(int) * 2 * P, cudaMemcpyHostToDevice));

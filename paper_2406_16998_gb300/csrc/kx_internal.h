@@ -34,11 +34,10 @@ constexpr int kGroupSlots = 2 * kOrbBlock;
 
 // One accumulation group: the pairs of one orbital block pair (I, J), I <= J
 // (a contiguous run of items), touching at most kGroupSlots orbitals.
-struct Group {
+struct alignas(16) Group {
     int first_item;
     int n_items;
-    int n_slots;
-    int orb[kGroupSlots];
+    int blk_i, blk_j;  // orbital blocks I < J, or J = -1 for a diagonal pair (I, I)
 };
 constexpr int kTile = 128;       // tcgen05 M (rows of pencils per tile)
 constexpr float kVScale = 16384.f;  // V operand scale 2^14 (|V| <= 1)
@@ -142,6 +141,8 @@ struct kx_plan_s {
     int *d_pairs = nullptr;       // int2 per item (i, j), i <= j
     int *d_item_slot = nullptr;   // int2 per item: slots of i and j inside its group
     int *d_groups = nullptr;      // kx::Group per group
+    int *d_orb_span = nullptr;    // int2 per orbital: its first and last group (-1: none)
+    size_t orb_span_cap = 0;
     size_t pairs_cap = 0, groups_cap = 0;
     std::vector<int> h_group_first;  // first item of each group (+ sentinel)
     std::vector<int> h_orb_last;     // per orbital: index of the last group that touches it (-1: none)

@@ -295,6 +295,7 @@ void plan_free(kx_plan *p) {
     cudaFree(p->d_pairs);
     cudaFree(p->d_item_slot);
     cudaFree(p->d_groups);
+    cudaFree(p->d_orb_span);
     cudaFree(p->d_pair_mask);
     p->d_pair_mask = nullptr;
     mp_free(p);

@@ -1409,95 +1409,234 @@ __global__ void __launch_bounds__(kSlabThreads, 1) tc_slab_kernel(const SlabArgs
     }
 }
 
-// Accumulation of one chunk, group by group: one thread per four grid points
-// visits the group's items in order, adding g_j psi_j phi_ij to orbital i and
-// g_i psi_i phi_ij to orbital j in shared-memory partial sums (one per orbital
-// slot of the group, <= kGroupSlots), then adds the partial sums into the fp32
-// accumulators.  All of a group's global loads (phi of every item, psi and the
-// old accumulator of every slot) are issued before the first is used.  Every
-// accumulator element is owned by one thread per launch and chunks run in a
-// fixed order, so the result is deterministic.
+// Accumulation of one chunk, group by group: one thread per W grid points visits a
+// group's items in order, adding g_j psi_j phi_ij to orbital i and g_i psi_i phi_ij to
+// orbital j in partial sums (one per orbital of the group's two blocks), then adds
+// those to the orbitals' running sums.  Every sum is owned by one thread per launch
+// and groups and chunks run in a fixed order, so the result is deterministic.
+//
+// Bound by memory traffic.  Consecutive groups share one of their two orbital
+// blocks (the pair list walks rows or columns of block pairs), so a thread keeps two
+// blocks, orbitals and running sums, in its own column of shared memory and exchanges
+// only the block that changes: per pair 4N bytes of phi and 3N of orbitals and sums
+// (with both blocks exchanged 6N).  An orbital's sum starts from zero at its first
+// group and leaves negated, as Vx psi, after its last (no fill before, no pass after).
+// The state lives in the thread, so groups need no barrier; the 16 phi loads of a
+// group and those of a new block are issued together.  96^3, 64 orbitals: 2.15 ms
+// an apply (7N bytes a pair: 13 GB, 6.0 TB/s) against 3.20 ms with both blocks
+// exchanged per group and 0.29 ms for the fills and the negating pass.  W = 4 where
+// rows are whole 16-byte pieces, else 1.
 constexpr int kAccThreads = 128;
 constexpr int kGroupItems = kOrbBlock * kOrbBlock;
 
-__global__ void __launch_bounds__(kAccThreads) acc_kernel(const float *__restrict__ phi, const Group *__restrict__ groups,
-                                                         int g0, int g1, int item0, const int2 *__restrict__ item_slot,
-                                                         const float *__restrict__ psi32, const double *__restrict__ occ,
-                                                         float *__restrict__ acc, long long N) {
-    __shared__ float4 ps[kGroupSlots][kAccThreads];
-    __shared__ float4 as[kGroupSlots][kAccThreads];
-    __shared__ Group G;
-    __shared__ float gs[kGroupSlots];
-    __shared__ int2 sl_s[kGroupItems];
-    const int tid = threadIdx.x;
-    const long long N4 = N >> 2;
-    const long long x4 = (long long)blockIdx.x * kAccThreads + tid;
-    const bool valid = x4 < N4;
-    const float4 *phi4 = reinterpret_cast<const float4 *>(phi);
-    const float4 *psi4 = reinterpret_cast<const float4 *>(psi32);
-    float4 *acc4 = reinterpret_cast<float4 *>(acc);
-    const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int g = g0; g < g1; ++g) {
+template <int W> struct alignas(4 * W) Pts {
+    float v[W];
+};
+template <int W> __device__ __forceinline__ Pts<W> ld_pts(const float *p) {
+    return *reinterpret_cast<const Pts<W> *>(p);
+}
+
+struct AccArgs {
+    const float *phi;
+    const Group *groups;
+    int g0, g1, item0, n_orb;
+    const int2 *item_slot;
+    const int2 *orb_span;   // first and last group of each orbital
+    const float *psi32;
+    const double *occ;
+    float *acc;
+    double *vx;
+    int vx_vec;             // vx rows are 16-byte aligned
+    int acc_init;           // the sums start from acc (multipole correction), not from zero
+    long long N;
+    const double *e_partial;  // energy partials of the chunk, added by the first CTA (nullable)
+    int e_count;
+    double e_factor;
+    double *ex;
+};
+
+template <int W>
+__global__ void __launch_bounds__(kAccThreads, 3) acc_kernel(const AccArgs a) {
+    using P = Pts<W>;
+    extern __shared__ __align__(16) unsigned char acc_sm[];
+    P(*ps)[kAccThreads] = reinterpret_cast<P(*)[kAccThreads]>(acc_sm);  // orbitals of the two blocks
+    P(*av)[kAccThreads] = ps + kGroupSlots;                             // their running sums
+    P(*as)[kAccThreads] = av + kGroupSlots;                             // a partial group's sums
+    const int tid = threadIdx.x, lane = tid & 31;
+    const long long x = (blockIdx.x * (long long)kAccThreads + tid) * W;
+    const bool valid = x < a.N;
+    if (blockIdx.x == 0 && a.e_count > 0) {
+        __shared__ double red[kAccThreads / 32];
+        double s = 0.0;
+        for (int b = tid; b < a.e_count; b += kAccThreads) s += a.e_partial[b];
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (lane == 0) red[tid >> 5] = s;
         __syncthreads();
-        if (tid == 0) G = groups[g];
-        __syncthreads();
-        const int ns = G.n_slots, ni = G.n_items, fi = G.first_item;
-        if (tid < ns) gs[tid] = occ ? (float)occ[G.orb[tid]] : 1.f;
-        if (tid < ni) sl_s[tid] = item_slot[fi + tid];
-        float4 f[kGroupItems], o[kGroupSlots];
+        if (tid == 0) *a.ex += a.e_factor * ((red[0] + red[1]) + (red[2] + red[3]));
+    }
+    int cur[2] = {-1, -1};  // blocks held in the halves [0, 4) and [4, 8)
+    float gl = 1.f;         // occupation of slot `lane`
+    // running sums of half h back to memory before group g: Vx psi if the orbital is done
+    auto evict = [&](int h, int g) {
+        if (cur[h] < 0) return;
 #pragma unroll
-        for (int k = 0; k < kGroupItems; ++k)
-            f[k] = (valid && k < ni) ? __ldg(phi4 + (long long)(fi + k - item0) * N4 + x4) : z;
+        for (int s = 0; s < kOrbBlock; ++s) {
+            const int o = cur[h] * kOrbBlock + s;
+            if (o >= a.n_orb) break;
+            const P v = av[4 * h + s][tid];
+            if (!valid) continue;
+            if (__ldg(a.orb_span + o).y < g) {
+                double *d = a.vx + (long long)o * a.N + x;
+                if (W == 4 && a.vx_vec) {
+                    reinterpret_cast<double2 *>(d)[0] = make_double2(-(double)v.v[0], -(double)v.v[W > 1 ? 1 : 0]);
+                    reinterpret_cast<double2 *>(d)[1] =
+                        make_double2(-(double)v.v[W > 2 ? 2 : 0], -(double)v.v[W > 3 ? 3 : 0]);
+                } else {
 #pragma unroll
-        for (int s = 0; s < kGroupSlots; ++s) {
-            if (s < ns) {
-                const long long off = (long long)G.orb[s] * N4 + x4;
-                ps[s][tid] = valid ? __ldg(psi4 + off) : z;
-                o[s] = valid ? acc4[off] : z;
-                as[s][tid] = z;
+                    for (int c = 0; c < W; ++c) d[c] = -(double)v.v[c];
+                }
+            } else {
+                *reinterpret_cast<P *>(a.acc + (long long)o * a.N + x) = v;
             }
         }
-        __syncthreads();
+    };
+    auto load = [&](int h, int blk, int g) {
+        cur[h] = blk;
+        P p[kOrbBlock], q[kOrbBlock];
+#pragma unroll
+        for (int s = 0; s < kOrbBlock; ++s) {
+            const int o = blk * kOrbBlock + s;
+#pragma unroll
+            for (int c = 0; c < W; ++c) p[s].v[c] = q[s].v[c] = 0.f;
+            if (o < a.n_orb && valid) {
+                p[s] = ld_pts<W>(a.psi32 + (long long)o * a.N + x);
+                if (a.acc_init || __ldg(a.orb_span + o).x != g) q[s] = ld_pts<W>(a.acc + (long long)o * a.N + x);
+            }
+        }
+#pragma unroll
+        for (int s = 0; s < kOrbBlock; ++s) {
+            ps[4 * h + s][tid] = p[s];
+            av[4 * h + s][tid] = q[s];
+        }
+        const int o = blk * kOrbBlock + (lane & 3);
+        if ((lane >> 2) == h) gl = (a.occ && o < a.n_orb) ? (float)a.occ[o] : 1.f;
+    };
+    int4 next = __ldg(reinterpret_cast<const int4 *>(a.groups + a.g0));
+    for (int g = a.g0; g < a.g1; ++g) {
+        const int fi = next.x, ni = next.y, bi = next.z, bj = next.w;
+        if (g + 1 < a.g1) next = __ldg(reinterpret_cast<const int4 *>(a.groups + g + 1));
+        P f[kGroupItems];
 #pragma unroll
         for (int k = 0; k < kGroupItems; ++k) {
-            if (k >= ni) break;
-            const int2 sl = sl_s[k];
-            const float4 pj = ps[sl.y][tid];
-            const float gj = gs[sl.y];
-            float4 ai = as[sl.x][tid];
-            ai.x = fmaf(gj * pj.x, f[k].x, ai.x);
-            ai.y = fmaf(gj * pj.y, f[k].y, ai.y);
-            ai.z = fmaf(gj * pj.z, f[k].z, ai.z);
-            ai.w = fmaf(gj * pj.w, f[k].w, ai.w);
-            as[sl.x][tid] = ai;
-            if (sl.x != sl.y) {
-                const float4 pi = ps[sl.x][tid];
-                const float gi = gs[sl.x];
-                float4 aj = as[sl.y][tid];
-                aj.x = fmaf(gi * pi.x, f[k].x, aj.x);
-                aj.y = fmaf(gi * pi.y, f[k].y, aj.y);
-                aj.z = fmaf(gi * pi.z, f[k].z, aj.z);
-                aj.w = fmaf(gi * pi.w, f[k].w, aj.w);
-                as[sl.y][tid] = aj;
+            if (k < ni && valid) {
+                f[k] = ld_pts<W>(a.phi + (long long)(fi + k - a.item0) * a.N + x);
+            } else {
+#pragma unroll
+                for (int c = 0; c < W; ++c) f[k].v[c] = 0.f;
             }
         }
-        if (valid) {
+        // halves of I and J: where they already are, if anywhere
+        int hi;
+        if (bj < 0)
+            hi = cur[1] == bi ? 1 : 0;
+        else
+            hi = (cur[1] == bi || cur[0] == bj) && !(cur[0] == bi || cur[1] == bj) ? 1 : 0;
+        const int hj = 1 - hi;
+        if (cur[hi] != bi) {
+            evict(hi, g);
+            load(hi, bi, g);
+        }
+        if (bj >= 0 && cur[hj] != bj) {
+            evict(hj, g);
+            load(hj, bj, g);
+        }
+        if (bj >= 0 && ni == kGroupItems) {
+            // a whole block pair: the partial sums stay in registers
+            P si[kOrbBlock], sj[kOrbBlock], pj[kOrbBlock];
+#pragma unroll
+            for (int s = 0; s < kOrbBlock; ++s) {
+                const float gj = __shfl_sync(0xffffffffu, gl, 4 * hj + s);
+                pj[s] = ps[4 * hj + s][tid];
+#pragma unroll
+                for (int c = 0; c < W; ++c) {
+                    si[s].v[c] = sj[s].v[c] = 0.f;
+                    pj[s].v[c] = gj * pj[s].v[c];
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < kOrbBlock; ++i) {
+                const float gi = __shfl_sync(0xffffffffu, gl, 4 * hi + i);
+                P pi = ps[4 * hi + i][tid];
+#pragma unroll
+                for (int c = 0; c < W; ++c) pi.v[c] = gi * pi.v[c];
+#pragma unroll
+                for (int j = 0; j < kOrbBlock; ++j) {
+#pragma unroll
+                    for (int c = 0; c < W; ++c) {
+                        si[i].v[c] = fmaf(pj[j].v[c], f[4 * i + j].v[c], si[i].v[c]);
+                        sj[j].v[c] = fmaf(pi.v[c], f[4 * i + j].v[c], sj[j].v[c]);
+                    }
+                }
+            }
+#pragma unroll
+            for (int s = 0; s < kOrbBlock; ++s) {
+                P u = av[4 * hi + s][tid], v = av[4 * hj + s][tid];
+#pragma unroll
+                for (int c = 0; c < W; ++c) {
+                    u.v[c] += si[s].v[c];
+                    v.v[c] += sj[s].v[c];
+                }
+                av[4 * hi + s][tid] = u;
+                av[4 * hj + s][tid] = v;
+            }
+        } else {
+            // diagonal, ragged or cut block pairs: slots from the item table
+            const int mi = 4 * hi, mj = bj >= 0 ? 4 * hj - kOrbBlock : 4 * hi;  // slots of J count on from 4
+            P z;
+#pragma unroll
+            for (int c = 0; c < W; ++c) z.v[c] = 0.f;
+#pragma unroll
+            for (int s = 0; s < kGroupSlots; ++s) as[s][tid] = z;
+#pragma unroll
+            for (int k = 0; k < kGroupItems; ++k) {
+                if (k >= ni) break;
+                const int2 sl = __ldg(a.item_slot + fi + k);
+                const int ii = mi + sl.x, jj = mj + sl.y;
+                const float gj = __shfl_sync(0xffffffffu, gl, jj), gi = __shfl_sync(0xffffffffu, gl, ii);
+                const P pj = ps[jj][tid];
+                P u = as[ii][tid];
+#pragma unroll
+                for (int c = 0; c < W; ++c) u.v[c] = fmaf(gj * pj.v[c], f[k].v[c], u.v[c]);
+                as[ii][tid] = u;
+                if (ii != jj) {
+                    const P pi = ps[ii][tid];
+                    P v = as[jj][tid];
+#pragma unroll
+                    for (int c = 0; c < W; ++c) v.v[c] = fmaf(gi * pi.v[c], f[k].v[c], v.v[c]);
+                    as[jj][tid] = v;
+                }
+            }
 #pragma unroll
             for (int s = 0; s < kGroupSlots; ++s) {
-                if (s < ns) {
-                    const float4 d = as[s][tid];
-                    acc4[(long long)G.orb[s] * N4 + x4] =
-                        make_float4(o[s].x + d.x, o[s].y + d.y, o[s].z + d.z, o[s].w + d.w);
-                }
+                P u = av[s][tid];
+                const P d = as[s][tid];
+#pragma unroll
+                for (int c = 0; c < W; ++c) u.v[c] += d.v[c];
+                av[s][tid] = u;
             }
         }
     }
+    evict(0, a.g1);
+    evict(1, a.g1);
 }
+template <int W> constexpr size_t acc_smem() { return 3 * kGroupSlots * kAccThreads * sizeof(Pts<W>); }
 
 // psi (fp64) -> psi32 and per-vector max |value|.
+// *zero (nullable, the energy of the call) starts from 0.
 __global__ void prep_kernel(const double *__restrict__ src, float *__restrict__ dst, float *__restrict__ vmax,
-                            int n_vec, long long N) {
+                            int n_vec, long long N, double *__restrict__ zero) {
     const int v = blockIdx.y;
+    if (zero && blockIdx.x == 0 && v == 0 && threadIdx.x == 0) *zero = 0.0;
     float m = 0.f;
     for (long long x = blockIdx.x * (long long)blockDim.x + threadIdx.x; x < N; x += (long long)gridDim.x * blockDim.x) {
         const float f = (float)src[(long long)v * N + x];
@@ -1686,11 +1825,23 @@ float fmax_sqrt(const kx_plan *p) {
     return (float)(p->fmax * std::sqrt((double)p->n[0]) * 1.0001);
 }
 
+// ex += the energy of `grid` partials, now or, with e_count, later by acc_kernel.
+int add_energy(kx_plan *p, const double *partial, int grid, double *ex, int *e_count, cudaStream_t s) {
+    if (e_count) {
+        *e_count = grid;
+        return KX_OK;
+    }
+    if (int rc = prof_begin(p, PK_FINAL, s)) return rc;
+    energy_add_kernel<<<1, 128, 0, s>>>(partial, grid, -0.5 * p->dV, ex);
+    KX_LAUNCH_CHECK("energy_add_kernel launch");
+    return prof_end(p, s);
+}
+
 // The five passes over R items: X3F writes T0, X2F T0->T1, X1 T1->T0, X2I
 // T0->T1, X3I T1->T0 (or xout in vector mode).  mx holds four rows of per-item
 // maxima, mx_stride apart.
 int run_passes(kx_plan *p, PassArgs a, long R, float *T0, float *T1, float *mx, long mx_stride, double *ex,
-               double *partial, bool energy_only, double *xout, cudaStream_t s) {
+               double *partial, bool energy_only, double *xout, cudaStream_t s, int *e_count = nullptr) {
     int rc;
     float *mx1 = mx, *mx2 = mx + mx_stride, *mx3 = mx + 2 * mx_stride, *mx4 = mx + 3 * mx_stride;
     a.rows_pp = (long long)p->n[0] * p->n[1];
@@ -1705,12 +1856,7 @@ int run_passes(kx_plan *p, PassArgs a, long R, float *T0, float *T1, float *mx, 
         if ((rc = launch_slab(p, R, T0, mx1, T1, mx4, ex ? partial : nullptr, a.pairs, a.occ, a.rhs_mode, s,
                               &grid)))
             return rc;
-        if (ex) {
-            if ((rc = prof_begin(p, PK_FINAL, s))) return rc;
-            energy_add_kernel<<<1, 128, 0, s>>>(partial, grid, -0.5 * p->dV, ex);
-            KX_LAUNCH_CHECK("energy_add_kernel launch");
-            if ((rc = prof_end(p, s))) return rc;
-        }
+        if (ex && (rc = add_energy(p, partial, grid, ex, e_count, s))) return rc;
         a.e_partial = nullptr;
         a.energy_only = 0;
         a.rows_pp = (long long)p->n[0] * p->n[1];
@@ -1741,12 +1887,7 @@ int run_passes(kx_plan *p, PassArgs a, long R, float *T0, float *T1, float *mx, 
     a.energy_only = energy_only ? 1 : 0;
     int grid = 0;
     if ((rc = launch_pass<P_X1>(p, a, 0, s, &grid))) return rc;
-    if (ex) {
-        if ((rc = prof_begin(p, PK_FINAL, s))) return rc;
-        energy_add_kernel<<<1, 128, 0, s>>>(partial, grid, -0.5 * p->dV, ex);
-        KX_LAUNCH_CHECK("energy_add_kernel launch");
-        if ((rc = prof_end(p, s))) return rc;
-    }
+    if (ex && (rc = add_energy(p, partial, grid, ex, energy_only ? nullptr : e_count, s))) return rc;
     a.e_partial = nullptr;
     a.energy_only = 0;
     if (energy_only) return KX_OK;
@@ -1791,7 +1932,7 @@ size_t tc_workspace_bytes(const kx_plan *p, int n_vec, long chunk) {
            4096;
 }
 
-// Vx psi rows [o0, o1) = -acc, then the plan's final-rows hook (if set).
+// Vx psi rows [o0, o1) = -acc (rows no group touches, with a multipole correction).
 int finalize_rows(kx_plan *p, const float *acc, double *vx, int o0, int o1, cudaStream_t s) {
     if (o1 <= o0) return KX_OK;
     const long long n = (long long)(o1 - o0) * (long long)p->N;
@@ -1804,9 +1945,7 @@ int finalize_rows(kx_plan *p, const float *acc, double *vx, int o0, int o1, cuda
         finalize_scalar_kernel<<<(unsigned)std::min<long long>((n + 255) / 256, 8LL * p->num_sms), 256, 0, s>>>(
             acc + off, vx + off, n);
     KX_LAUNCH_CHECK("finalize_kernel launch");
-    if (int rc = prof_end(p, s)) return rc;
-    if (p->final_hook.fn) p->final_hook.fn(p->final_hook.ctx, o0, o1, s);
-    return KX_OK;
+    return prof_end(p, s);
 }
 
 int tc_vx(kx_plan *p, int n_orb, const double *psi, const double *occ, double *vx, double *ex, bool energy_only,
@@ -1824,13 +1963,15 @@ int tc_vx(kx_plan *p, int n_orb, const double *psi, const double *occ, double *v
     TcLayout L = carve(p, n_orb, chunk, !energy_only);
     const long long N = (long long)p->N;
 
-    KX_CUDA_TRY(cudaMemsetAsync(L.orb_max, 0, sizeof(float) * n_orb, s));
+    // maxima of the orbitals and of the first chunk's items (neighbours in the workspace)
+    KX_CUDA_TRY(cudaMemsetAsync(L.orb_max, 0, (size_t)((char *)(L.mx + 4 * chunk) - (char *)L.orb_max), s));
     // fp64 -> fp32 copies and maxima of orbitals [o0, o1)
     auto prep_range = [&](int o0, int o1) -> int {
         if (o1 <= o0) return KX_OK;
         dim3 g((unsigned)std::min<long long>((N + 255) / 256, 64), (unsigned)(o1 - o0));
         if (int r = prof_begin(p, PK_PREP, s)) return r;
-        prep_kernel<<<g, 256, 0, s>>>(psi + (size_t)o0 * N, L.psi32 + (size_t)o0 * N, L.orb_max + o0, o1 - o0, N);
+        prep_kernel<<<g, 256, 0, s>>>(psi + (size_t)o0 * N, L.psi32 + (size_t)o0 * N, L.orb_max + o0, o1 - o0, N,
+                                      o0 == 0 ? ex : nullptr);
         KX_LAUNCH_CHECK("prep_kernel launch");
         return prof_end(p, s);
     };
@@ -1859,16 +2000,29 @@ int tc_vx(kx_plan *p, int n_orb, const double *psi, const double *occ, double *v
         return k;
     };
     const std::vector<int> &maxorb = p->h_group_maxorb;
-    if (ex) KX_CUDA_TRY(cudaMemsetAsync(ex, 0, sizeof(double), s));
-    if (!energy_only) {
-        // with multipole boundary values the accumulator starts from the boundary
-        // correction (tensor-core form), otherwise from zero
-        if (mp_tc_eligible(p, n_orb, psi)) {
-            if ((rc = mp_correct_into_acc(p, n_orb, psi, occ, L.acc, ex, s))) return rc;
-        } else {
-            KX_CUDA_TRY(cudaMemsetAsync(L.acc, 0, sizeof(float) * (size_t)n_orb * N, s));
+    // with multipole boundary values the accumulator starts from the boundary
+    // correction (tensor-core form), otherwise from zero
+    const bool acc_init = !energy_only && mp_tc_eligible(p, n_orb, psi);
+    if (acc_init && (rc = mp_correct_into_acc(p, n_orb, psi, occ, L.acc, ex, s))) return rc;
+    if (pieces && n_groups == 0 && ex) KX_CUDA_TRY(cudaMemsetAsync(ex, 0, sizeof(double), s));
+    // rows [o0, o1) are final once the work queued so far has run: those no group
+    // touches are filled here, the others were written by acc_kernel
+    auto finish_rows = [&](int o0, int o1) -> int {
+        for (int o = o0; o < o1;) {
+            int e = o;
+            while (e < o1 && p->h_orb_last[e] < 0) ++e;
+            if (e > o) {
+                if (acc_init) {
+                    if (int r = finalize_rows(p, L.acc, vx, o, e, s)) return r;
+                } else {
+                    KX_CUDA_TRY(cudaMemsetAsync(vx + (size_t)o * N, 0, sizeof(double) * (size_t)(e - o) * N, s));
+                }
+            }
+            o = e + 1;
         }
-    }
+        if (o1 > o0 && p->final_hook.fn) p->final_hook.fn(p->final_hook.ctx, o0, o1, s);
+        return KX_OK;
+    };
     const int2 *pairs = reinterpret_cast<const int2 *>(p->d_pairs);
     const float mid_bound = fmax_sqrt(p);
 
@@ -1909,7 +2063,8 @@ int tc_vx(kx_plan *p, int n_orb, const double *psi, const double *occ, double *v
         }
         const long c0 = first[g0];
         const long R = first[g1] - c0;
-        KX_CUDA_TRY(cudaMemsetAsync(L.mx, 0, sizeof(float) * 4 * chunk, s));
+        if (g0 > 0) KX_CUDA_TRY(cudaMemsetAsync(L.mx, 0, sizeof(float) * 4 * chunk, s));
+        int e_count = 0;
         PassArgs a{};
         a.pairs = pairs + c0;
         a.psi32 = L.psi32;
@@ -1921,28 +2076,51 @@ int tc_vx(kx_plan *p, int n_orb, const double *psi, const double *occ, double *v
             rc = fft_passes(p, R, pairs + c0, L.psi32, 0, occ, reinterpret_cast<float2 *>(L.T1), L.T0, nullptr, ex,
                             L.partial, energy_only, s);
         else
-            rc = run_passes(p, a, R, L.T0, L.T1, L.mx, chunk, ex, L.partial, energy_only, nullptr, s);
+            rc = run_passes(p, a, R, L.T0, L.T1, L.mx, chunk, ex, L.partial, energy_only, nullptr, s, &e_count);
         if (rc) return rc;
         if (!energy_only) {
-            const unsigned blocks = (unsigned)((N / 4 + kAccThreads - 1) / kAccThreads);
+            AccArgs ac{};
+            ac.phi = L.T0;
+            ac.groups = reinterpret_cast<const Group *>(p->d_groups);
+            ac.g0 = g0;
+            ac.g1 = g1;
+            ac.item0 = (int)c0;
+            ac.n_orb = n_orb;
+            ac.item_slot = reinterpret_cast<const int2 *>(p->d_item_slot);
+            ac.orb_span = reinterpret_cast<const int2 *>(p->d_orb_span);
+            ac.psi32 = L.psi32;
+            ac.occ = occ;
+            ac.acc = L.acc;
+            ac.vx = vx;
+            ac.vx_vec = (reinterpret_cast<uintptr_t>(vx) & 15) == 0;
+            ac.acc_init = acc_init ? 1 : 0;
+            ac.N = N;
+            ac.e_partial = L.partial;
+            ac.e_count = ex ? e_count : 0;
+            ac.e_factor = -0.5 * p->dV;
+            ac.ex = ex;
             if ((rc = prof_begin(p, PK_ACC, s))) return rc;
-            acc_kernel<<<blocks, kAccThreads, 0, s>>>(L.T0, reinterpret_cast<const Group *>(p->d_groups), g0, g1,
-                                                     (int)c0, reinterpret_cast<const int2 *>(p->d_item_slot),
-                                                     L.psi32, occ, L.acc, N);
+            if (N % 4 == 0) {  // rows of whole 16-byte pieces
+                KX_CUDA_TRY(cudaFuncSetAttribute(acc_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                 (int)acc_smem<4>()));
+                acc_kernel<4><<<(unsigned)((N / 4 + kAccThreads - 1) / kAccThreads), kAccThreads, acc_smem<4>(), s>>>(ac);
+            } else {
+                acc_kernel<1><<<(unsigned)((N + kAccThreads - 1) / kAccThreads), kAccThreads, acc_smem<1>(), s>>>(ac);
+            }
             KX_LAUNCH_CHECK("acc_kernel launch");
             if ((rc = prof_end(p, s))) return rc;
         }
         if (!energy_only) {
-            // rows whose last group is done are final: negate them into vx now
+            // rows whose last group is done are final
             int o_done = o_fin;
             while (o_done < n_orb && p->h_orb_last[o_done] < g1) ++o_done;
-            if ((rc = finalize_rows(p, L.acc, vx, o_fin, o_done, s))) return rc;
+            if ((rc = finish_rows(o_fin, o_done))) return rc;
             o_fin = o_done;
         }
         g0 = g1;
     }
     if (pieces && (rc = need(n_orb))) return rc;  // every piece is on the device when the call's work ends
-    if (!energy_only) return finalize_rows(p, L.acc, vx, o_fin, n_orb, s);
+    if (!energy_only) return finish_rows(o_fin, n_orb);
     return KX_OK;
 }
 
@@ -1965,7 +2143,7 @@ int tc_apply_fL(kx_plan *p, int n_rhs, const double *b, double *x, cudaStream_t 
         KX_CUDA_TRY(cudaMemsetAsync(L.mx, 0, sizeof(float) * 4 * chunk, s));
         dim3 g((unsigned)std::min<long long>((N + 255) / 256, 64), (unsigned)R);
         if ((rc = prof_begin(p, PK_PREP, s))) return rc;
-        prep_kernel<<<g, 256, 0, s>>>(b + c0 * N, L.psi32, L.orb_max, (int)R, N);
+        prep_kernel<<<g, 256, 0, s>>>(b + c0 * N, L.psi32, L.orb_max, (int)R, N, nullptr);
         KX_LAUNCH_CHECK("prep_kernel launch");
         if ((rc = prof_end(p, s))) return rc;
         PassArgs a{};
@@ -2053,7 +2231,7 @@ int tc_apply_fL_noalloc(kx_plan *p, int n_rhs, const double *b, double *x, cudaS
     float *mx = src_max + kNoAllocMaxVec;  // four per-item maxima rows of kNoAllocMaxVec
     KX_CUDA_TRY(cudaMemsetAsync(src_max, 0, 5 * kNoAllocMaxVec * sizeof(float), s));
     dim3 g((unsigned)std::min<long long>((N + 255) / 256, 64), (unsigned)n_rhs);
-    prep_kernel<<<g, 256, 0, s>>>(b, b32, src_max, n_rhs, N);
+    prep_kernel<<<g, 256, 0, s>>>(b, b32, src_max, n_rhs, N, nullptr);
     KX_LAUNCH_CHECK("prep_kernel launch");
     PassArgs a{};
     a.rhs_mode = 1;

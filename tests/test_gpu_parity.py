@@ -8,6 +8,8 @@ Tolerances (stated once, used everywhere below):
              product carries ~2^-22 relative error, six chained products plus fp32
              accumulation stay well inside these bounds).
 """
+import os
+
 import numpy as np
 import pytest
 
@@ -478,6 +480,35 @@ def test_fft_vx_and_energy_match_oracle(kx):
     assert relmax(vx.cpu().numpy().T, vx_ref) < TOL[1]["vx"]
     assert abs(ex.item() - ex_ref) < TOL[1]["ex"] * abs(ex_ref)
     assert abs(e_only - ex_ref) < TOL[1]["ex"] * abs(ex_ref)
+
+
+@pytest.mark.parametrize("n_orb", [1, 3, 4, 5, 8, 13])
+@pytest.mark.parametrize("n", [(9, 10, 15), (12, 10, 9)])
+def test_fft_vx_ragged_blocks_and_points(kx, n, n_orb):
+    """The accumulation with whole, diagonal and ragged orbital blocks on grids whose
+    point count is not and is a multiple of four (scalar and 16-byte accumulation),
+    the whole list, in chunks that split the block rows, and a range of it."""
+    h, bc = (0.45, 0.5, 0.4), (P, P, P)
+    sysd = system(n, h, bc, S, n_orb, 97)
+    psi = workloads.random_field(n[0] * n[1] * n[2], n_orb, 98)
+    occ = np.random.default_rng(3).uniform(0.2, 1.0, n_orb)
+    op = oracle.Plan(n, h, bc, S)
+    vx_ref, ex_ref = oracle.vx_apply(op, psi, occ)
+    plan = kx.Plan(n, h, bc, S, precision=kx.KX_FFT32)
+    vx, ex = kx.kx_vx_apply(plan, dev(psi.T), dev(occ))
+    assert relmax(vx.cpu().numpy().T, vx_ref) < TOL[1]["vx"]
+    assert abs(ex.item() - ex_ref) < TOL[1]["ex"] * abs(ex_ref)
+    n_p = n_orb * (n_orb + 1) // 2
+    os.environ["KX_CHUNK_PAIRS"] = "20"
+    try:
+        vx20, _ = kx.kx_vx_apply(plan, dev(psi.T), dev(occ))
+    finally:
+        del os.environ["KX_CHUNK_PAIRS"]
+    assert torch.equal(vx, vx20)
+    parts = [kx.kx_vx_apply_pairs(plan, dev(psi.T), b, e, dev(occ))
+             for b, e in ((0, n_p // 3), (n_p // 3, n_p // 3), (n_p // 3, n_p))]
+    assert relmax(sum(v for v, _ in parts).cpu().numpy().T, vx_ref) < TOL[1]["vx"]
+    assert abs(sum(e.item() for _, e in parts) - ex_ref) < TOL[1]["ex"] * abs(ex_ref)
 
 
 def test_fft_rejects_unsupported_grids(kx):
