@@ -22,8 +22,10 @@
 // Each pass kernel is persistent (one CTA per SM) and warp-specialised:
 //   warps 0-7   epilogue (TMEM lane quadrant = warp % 4, one tile row per
 //               thread; warps 0-3 and 4-7 take alternate column blocks)
-//   warps 8-15  producers: global fp32 -> scale -> fp16 hi/lo -> shared stage
-//   warp 16     TMEM allocation and MMA issue (one thread)
+//   warps 8-17  producers: global fp32 -> scale -> fp16 hi/lo -> shared stage (20 warps
+//               are what 96 registers a thread allow)
+//   warp 18     TMEM allocation and MMA issue (one thread)
+//   warp 19     tile metadata, ahead of both
 // with an S-deep ring of shared A stages and two TMEM accumulator slots, so
 // loads, MMAs and stores of consecutive tiles overlap.
 #include "kx_internal.h"
@@ -41,11 +43,11 @@ namespace {
 enum PassKind { P_X3F = 0, P_X2F = 1, P_X1 = 2, P_X2I = 3, P_X3I = 4 };
 
 constexpr int kEpiWarps = 8;   // two per TMEM lane quadrant, alternate 16/32-column blocks
-constexpr int kProdWarps = 8;
+constexpr int kProdWarps = 10;
 constexpr int kEpiThreads = 32 * kEpiWarps;
 constexpr int kProdThreads = 32 * kProdWarps;
 constexpr int kProdGroups = 2;                            // producer groups work on alternate tiles
-constexpr int kGroupThreads = kProdThreads / kProdGroups;  // 128: one thread per row for the K-major pass
+constexpr int kGroupThreads = kProdThreads / kProdGroups;
 constexpr int kMmaWarp = kEpiWarps + kProdWarps;
 constexpr int kMetaWarp = kMmaWarp + 1;
 constexpr int kThreads = 32 * (kEpiWarps + kProdWarps + 2);
@@ -270,7 +272,7 @@ __device__ __forceinline__ void produce_tile_u(const PassArgs &a, const TileMeta
     const int nkc = np >> 3;
     const int ntask = 16 * np;  // 128 rows x np columns / 8
     const unsigned magic = (65536u + (unsigned)nkc - 1u) / (unsigned)nkc;  // t / nkc == (t * magic) >> 16 for t < 2^11
-    const long long kstride = (PASS == P_X3F || PASS == P_X3I) ? (long long)a.n1 * a.n2 : (long long)a.n1;
+    const int kstride = (PASS == P_X3F || PASS == P_X3I) ? a.n1 * a.n2 : a.n1;
     for (int t0 = ptid; t0 < ntask; t0 += kGroupThreads * U) {
         float v[U][8];
         float u[TWO ? U : 1][8];
@@ -346,9 +348,11 @@ __device__ __forceinline__ void produce_tile_u(const PassArgs &a, const TileMeta
 // Producer side: stage one 128-row tile of the A operand (scaled, split).
 // Task t covers 8 consecutive values: MN-major row group g = t%16 at k = t/16;
 // K-major row m = t/nkc, chunk kc = t%nkc.  Consecutive lanes therefore read
-// consecutive global addresses.  All loads of a batch of U tasks (a whole tile for n <= 96 when U = 12) are
-// issued before any is converted, so each thread keeps U*32 bytes in flight.
-template <int PASS>
+// consecutive global addresses.  All loads of a batch of U tasks are issued before
+// any is converted, so each thread keeps U*32 bytes in flight (twice that for the
+// pair product's two orbitals, in batches of 4); U is what splits a thread's tasks
+// into even batches (pass_batch).
+template <int PASS, int U>
 __device__ __forceinline__ void produce_tile(const PassArgs &a, const TileMeta &d, uint8_t *Ahi, uint8_t *Alo,
                                              int ptid) {
     if (PASS == P_X3F) {
@@ -357,7 +361,7 @@ __device__ __forceinline__ void produce_tile(const PassArgs &a, const TileMeta &
         else
             produce_tile_u<PASS, 4, true>(a, d, Ahi, Alo, ptid);
     } else {
-        produce_tile_u<PASS, 8, false>(a, d, Ahi, Alo, ptid);
+        produce_tile_u<PASS, U, false>(a, d, Ahi, Alo, ptid);
     }
 }
 
@@ -517,7 +521,7 @@ __device__ __forceinline__ bool x1_inverse_half(const PassArgs &a, Bars &bars, u
     return true;
 }
 
-template <int PASS>
+template <int PASS, int U>
 __global__ void __launch_bounds__(kThreads, 1) tc_pass_kernel(const PassArgs a) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -656,7 +660,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_pass_kernel(const PassArgs a) 
             KX_CLK_ADD(2, tw);
             tw = KX_CLK_NOW();
             uint8_t *Ahi = stage0 + s * stage_bytes;
-            produce_tile<PASS>(a, smeta[r], Ahi, Ahi + half_bytes, gtid);
+            produce_tile<PASS, U>(a, smeta[r], Ahi, Ahi + half_bytes, gtid);
             ptx::fence_proxy_async_smem();
             warp_arrive(&bars.full[s]);
             KX_CLK_ADD(3, tw);
@@ -1703,6 +1707,23 @@ size_t pass_smem(int np, int stages, bool with_mid) {
     return (size_t)4 * np * np + (size_t)(stages + (with_mid ? 1 : 0)) * stage_bytes_of(np) + kStagingBytes + 1024;
 }
 
+// Producer batch of a pass kernel: a thread has ceil(16 np / kGroupThreads) tasks a
+// tile; at np = 96 its 10 tasks take 2.60 ms as 5 + 5 and 2.70 as 8 + 2 (X3I per apply
+// at 96^3 / 64 orbitals), at np = 80 its 8 are one batch.
+int pass_batch(int np) {
+    const int tasks = (16 * np + kGroupThreads - 1) / kGroupThreads;
+    if (tasks == 9 || tasks == 10) return 5;
+    return tasks == 8 || tasks <= 6 ? 8 : 7;
+}
+
+template <int PASS, int U>
+int launch_pass_u(const PassArgs &a, int grid, size_t smem, cudaStream_t s) {
+    KX_CUDA_TRY(cudaFuncSetAttribute(tc_pass_kernel<PASS, U>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    tc_pass_kernel<PASS, U><<<grid, kThreads, smem, s>>>(a);
+    KX_LAUNCH_CHECK("tc_pass_kernel launch");
+    return KX_OK;
+}
+
 template <int PASS>
 int launch_pass(const kx_plan *p, PassArgs a, int axis, cudaStream_t s, int *grid_out) {
     a.nc = p->n[axis];
@@ -1721,13 +1742,16 @@ int launch_pass(const kx_plan *p, PassArgs a, int axis, cudaStream_t s, int *gri
     a.stages = pass_stages(a.np, false);  // X1's mid operand reuses its tile's A stage
     if (p->tune.pass_stages > 0) a.stages = std::min(a.stages, p->tune.pass_stages);
     const size_t smem = pass_smem(a.np, a.stages, false);
-    KX_CUDA_TRY(cudaFuncSetAttribute(tc_pass_kernel<PASS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     const long long n_tiles = (a.total_rows + 127) / 128;
     const int grid = (int)std::max(1LL, std::min<long long>(n_tiles, (long long)p->num_sms));
     if (grid_out) *grid_out = grid;
     if (int rc = prof_begin(const_cast<kx_plan *>(p), PK_X3F + PASS, s)) return rc;
-    tc_pass_kernel<PASS><<<grid, kThreads, smem, s>>>(a);
-    KX_LAUNCH_CHECK("tc_pass_kernel launch");
+    const int u = PASS == P_X3F ? 8 : pass_batch(a.np);  // X3F has its own batches
+    int rc;
+    if (PASS == P_X3F || u == 8) rc = launch_pass_u<PASS, 8>(a, grid, smem, s);
+    else if (u == 7) rc = launch_pass_u<PASS, PASS == P_X3F ? 8 : 7>(a, grid, smem, s);
+    else rc = launch_pass_u<PASS, PASS == P_X3F ? 8 : 5>(a, grid, smem, s);
+    if (rc) return rc;
     return prof_end(const_cast<kx_plan *>(p), s);
 }
 
