@@ -392,9 +392,10 @@ __device__ __forceinline__ void issue_ksteps(uint32_t tmem_a, uint32_t tmem_b, u
 }
 
 __device__ __forceinline__ void issue_split_mma(uint32_t tmem_a, uint32_t tmem_b, uint32_t a_hi, uint32_t a_lo,
-                                                bool a_kmajor, uint32_t v_hi, uint32_t v_lo, bool inverse, int np) {
+                                                bool a_kmajor, uint32_t v_hi, uint32_t v_lo, bool inverse, int np,
+                                                int row_groups = 16) {
     const uint32_t idesc = ptx::idesc_f16(128, np, a_kmajor ? 0 : 1, inverse ? 0 : 1);
-    const uint32_t a_lbo = a_kmajor ? (uint32_t)kCoreStride : (uint32_t)(16 * kCoreStride);
+    const uint32_t a_lbo = a_kmajor ? (uint32_t)kCoreStride : (uint32_t)(row_groups * kCoreStride);
     const uint32_t a_sbo = a_kmajor ? (uint32_t)((np >> 3) * kCoreStride) : (uint32_t)kCoreStride;
     const uint32_t a_step = 2 * a_lbo;  // one k-step = two core matrices along K
     // V stored as 8x8 core matrices, row block of 8 x-rows = np*16 bytes.
@@ -865,16 +866,25 @@ __global__ void __launch_bounds__(kThreads, 1) tc_pass_kernel(const PassArgs a) 
 //   D   D3 -> A4[x1][k2] (MN-major, written by the thread owning row k2)
 //   M4  A4 x V2^T                                    -> D4[x1][x2]
 //   E   D4 -> global slice [x2][x1] (coalesced), per-item maximum
-// Two units are in flight: unit j uses TMEM slot, A buffer and epilogue
-// warpgroup j & 1, so the two groups run their stage chains independently and
+// E_x alone (ENERGY) stops after C.
+// Two units are in flight: unit j uses TMEM slot and epilogue group j & 1 and A
+// buffer j mod nbuf, so the two groups run their stage chains independently and
 // the single MMA thread serves whichever group is ready.  Split scales are
 // powers of two from bounds: each orthogonal mode product grows max|.| by at
 // most sqrt(n), the scaling by at most fmax.
+//
+// What bounds it is each group's chain: four products of 18 MMAs (1.0-1.3 k cycles
+// each at 96^2, on one tensor pipe for both groups) and the four stages between them
+// (1.5-2.9 k cycles), ~18 k cycles a unit.  A third A buffer takes the split of the
+// next plane (3.3 k cycles) out of the chain, where it stood beside stage E:
+// 6.24 -> 5.34 ms per apply at 96^3 / 64 orbitals, 10.4 -> 8.65 at 80^3 / 96.  Small
+// planes share a unit (slab_planes): 0.29 -> 0.17 ms at 56x40x48 / 24 orbitals.
 // ---------------------------------------------------------------------------
 struct SlabArgs {
     int n1, n2, n3, np1, np2;
     long long N;
-    long long total_units;  // items * n3
+    long long total_units;  // items * n3 / pp
+    int pp;                 // planes per unit: 1, or 2 (4) where a plane fits 64 (32) rows
     const float *in;
     float *out;
     const __half *V1s, *V2s;
@@ -888,12 +898,13 @@ struct SlabArgs {
     int rhs_mode;
     int stage_in;           // the input plane is bulk-copied into shared memory before it is split
     int share_v;            // V2 == V1 (same size, spacing and boundary): one shared copy
+    int nbuf;               // A buffers (2 or 3)
     int *status;
     long long timeout_cycles;
     long long *clk;         // role counters (only with KX_ROLE_CLOCKS)
 };
 
-constexpr int kSlabU = 8;            // producer loads in flight per thread
+constexpr int kSlabU = 6;            // producer loads in flight per thread
 // Warp roles: 16 epilogue warps (warp w reads TMEM lane quadrant w % 4, the
 // TMEM access rule; column half (w / 4) % 2; group w / 8), then 3 producer
 // warps, then the MMA warp.  A plane of at most 96 rows leaves one quadrant (32:
@@ -904,9 +915,34 @@ constexpr int kSlabEpiWarps = 16;
 constexpr int kSlabProdWarps = 3;
 constexpr int kSlabMmaWarp = kSlabEpiWarps + kSlabProdWarps;
 constexpr int kSlabThreads = 32 * (kSlabMmaWarp + 1);
+constexpr int kSlabMaxBuf = 3;
+// Units whose constants are kept: a slot is refilled eight units on, when two later
+// units of the same group have been through their stages.
+constexpr int kSlabRing = 8;
+
+// Planes of a unit: small ones share the 128 rows of a product (consecutive k3 of one
+// item; n3 is a multiple of 8), plane p on the rows from 128 p / pp on.  Everything but
+// the row offsets is per row, so stages and products serve all of them at once.
+__host__ __device__ constexpr int slab_planes(int npm) { return npm <= 32 ? 4 : npm <= 64 ? 2 : 1; }
+// An A buffer holds only the row groups (8 rows) of the quadrants in use, a product's
+// remaining rows up to 128 read what lies behind (their results are never read):
+// hi + lo 41.5 KB at 96^2 instead of 55.3.
+__host__ __device__ constexpr int slab_quadrants(int npm) { return slab_planes(npm) > 1 ? 4 : (npm + 31) / 32; }
+__host__ __device__ constexpr size_t slab_half_bytes(int npm) {
+    return (size_t)(npm / 8) * 4 * slab_quadrants(npm) * kCoreStride;
+}
 
 struct SlabBars {
-    uint64_t full[2], empty[2], tfull[2], ready[2], in_full, drain;
+    uint64_t full[kSlabMaxBuf], empty[kSlabMaxBuf], tfull[2], ready[2], in_full, drain;
+};
+
+// Constants of one unit: unscale and rescale factors of its stages, output and f
+// offsets, the item and its energy weight.
+struct SlabUnit {
+    float us2, u2, s3, us4, u4;
+    int item, foff;
+    double w;
+    long long out0;
 };
 
 __device__ __forceinline__ bool slab_wait(uint64_t *bar, uint32_t parity, const SlabArgs &a, volatile int *abort) {
@@ -929,37 +965,14 @@ __device__ __forceinline__ void store_split8(uint8_t *hi_base, uint8_t *lo_base,
     *reinterpret_cast<uint4 *>(lo_base + off) = l;
 }
 
-// Per-unit constants of the epilogue: item, slice, the four split exponents and
-// the pair's energy weight.
-struct SlabUnit {
-    long long item, k3;
-    int e1, e2, e3, e4;
-    double w;
-};
-
-__device__ __forceinline__ SlabUnit slab_unit(const SlabArgs &a, long long u, float b1, int2 ij) {
-    SlabUnit r;
-    r.item = (unsigned)u / (unsigned)a.n3;
-    r.k3 = (unsigned)u - (unsigned)r.item * (unsigned)a.n3;
-    const float b2 = b1 * a.sq2, b3 = a.fmax * a.sq1 * b2, b4 = a.sq1 * b3;
-    r.e1 = scale_exp(b1);
-    r.e2 = scale_exp(b2);
-    r.e3 = scale_exp(b3);
-    r.e4 = scale_exp(b4);
-    r.w = 0.0;
-    if (a.e_partial != nullptr && !a.rhs_mode) {
-        r.w = (ij.x == ij.y) ? 1.0 : 2.0;
-        if (a.occ) r.w *= a.occ[ij.x] * a.occ[ij.y];
-    }
-    return r;
-}
-
-// Epilogue stage B or D for one warp: D row m (a TMEM lane) becomes K column m
-// of the next MN-major operand; 8 consecutive D columns (M values) per 16-byte
-// store.  Rows m >= nrow (padding) give zeros; rows m >= nprow are not written.
-__device__ __forceinline__ void slab_transpose_stage(uint32_t ta, uint32_t tb, int m, int h, int nrow, int nprow,
-                                                     int ncol, bool two, float us, uint8_t *Ahi, uint8_t *Alo) {
-    const int off_r = (m >> 3) * (16 * kCoreStride) + (m & 7) * 16;
+// Epilogue stage B or D for one warp: D row m of a plane (a TMEM lane) becomes K
+// column m of the next MN-major operand; 8 consecutive D columns (M values, from
+// the plane's first row group gp on) per 16-byte store.  Rows m >= nrow (padding)
+// give zeros; rows m >= nprow are not written.
+__device__ __forceinline__ void slab_transpose_stage(uint32_t ta, uint32_t tb, int m, int gp, int h, int nrow,
+                                                     int nprow, int ncol, bool two, float us, int kcore, uint8_t *Ahi,
+                                                     uint8_t *Alo) {
+    const int off_r = (m >> 3) * kcore + (m & 7) * 16 + gp * kCoreStride;
     if (m >= nrow) us = 0.f;  // padding rows hold zeros already: their operand rows were zero
     for (int c = 16 * h; c < ncol; c += 32) {
         float v[16], vb[16];
@@ -978,40 +991,44 @@ __device__ __forceinline__ void slab_transpose_stage(uint32_t ta, uint32_t tb, i
     }
 }
 
+template <bool ENERGY, bool MULTI>
 __global__ void __launch_bounds__(kSlabThreads, 1) tc_slab_kernel(const SlabArgs a) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const int np1 = a.np1, np2 = a.np2, npm = max(np1, np2);
-    const size_t half_bytes = a_half_bytes(npm);
-    uint8_t *V1hi = smem;
+    const int nbuf = a.nbuf;
+    const int nq = slab_quadrants(npm);          // TMEM lane quadrants with rows
+    const int rg = 4 * nq, kcore = rg * kCoreStride;
+    const int pp = MULTI ? a.pp : 1;                      // planes per unit
+    const int row_sh = !MULTI ? 7 : pp == 2 ? 6 : 5;      // log2 of the 128 / pp rows of each
+    const size_t half_bytes = slab_half_bytes(npm);
+    uint8_t *buf0 = smem;  // A buffers (hi | lo)
+    uint8_t *V1hi = buf0 + nbuf * 2 * half_bytes;
     uint8_t *V1lo = V1hi + np1 * np1 * 2;
     uint8_t *V2hi = a.share_v ? V1hi : V1lo + np1 * np1 * 2;
     uint8_t *V2lo = V2hi + np2 * np2 * 2;
-    uint8_t *buf0 = V2lo + np2 * np2 * 2;  // two A buffers (hi | lo), one per TMEM slot
-    float *sin = reinterpret_cast<float *>(buf0 + 4 * half_bytes);  // input plane [x2][x1] (stage_in)
+    float *sin = reinterpret_cast<float *>(V2lo + np2 * np2 * 2);  // input plane [x2][x1] (stage_in)
     __shared__ SlabBars bars;
+    __shared__ SlabUnit units[kSlabRing];
     __shared__ uint32_t tmem_slot;
     __shared__ volatile int s_abort;
     __shared__ double s_red[kSlabEpiWarps];
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int nq = (npm + 31) >> 5;              // TMEM lane quadrants with rows
     const int n_help = 4 * (4 - nq);             // epilogue warps without rows
     const int helper = (warp < kSlabEpiWarps && (warp & 3) >= nq) ? (warp & 3) - nq + (4 - nq) * (warp >> 2) : -1;
     const int n_prod = 32 * (kSlabProdWarps + n_help);  // producer threads
     const int group_threads = 64 * nq;           // epilogue threads of a group
-#ifdef KX_ROLE_CLOCKS
-    long long clk_acc[kClk] = {0};
-    const long long clk_t0 = clock64();
-#endif
     if (warp == kSlabMmaWarp) {
         ptx::tmem_alloc(&tmem_slot, 512);
         ptx::tmem_relinquish();
     }
     if (tid == 0) {
-        for (int b = 0; b < 2; ++b) {
+        for (int b = 0; b < kSlabMaxBuf; ++b) {
             ptx::mbar_init(&bars.full[b], n_prod / 32);
             ptx::mbar_init(&bars.empty[b], 1);
+        }
+        for (int b = 0; b < 2; ++b) {
             ptx::mbar_init(&bars.tfull[b], 1);
             ptx::mbar_init(&bars.ready[b], group_threads / 32);
         }
@@ -1038,17 +1055,20 @@ __global__ void __launch_bounds__(kSlabThreads, 1) tc_slab_kernel(const SlabArgs
     const uint32_t tmem = tmem_slot;
     const int n_my = (int)((a.total_units - blockIdx.x + gridDim.x - 1) / gridDim.x);
     const long long n12 = (long long)a.n1 * a.n2;
+    constexpr int kLast = ENERGY ? 1 : 3;  // last product of a unit
 
     if (warp == kSlabMmaWarp) {
         // ---------------------------------------------------------------- MMA issue
         // Polls both slots and issues the next product of whichever is ready:
         // M1 of unit j needs its A1 (full) and the slot's previous unit through
-        // stage E; M2..M4 need the group's previous stage (ready).
+        // its last stage; M2..M4 need the group's previous stage (ready).
         if (ptx::elect_one()) {
             const uint32_t sV1h = ptx::smem_u32(V1hi), sV1l = ptx::smem_u32(V1lo);
             const uint32_t sV2h = ptx::smem_u32(V2hi), sV2l = ptx::smem_u32(V2lo);
             int jn[2] = {0, 1}, sn[2] = {0, 0};
+            int buf[2] = {0, 1}, par[2] = {0, 0};  // of unit jn[g]: A buffer and its use's parity
             bool ok = true;
+            int idle = 0;
             long long last = clock64();
             while (ok && (jn[0] < n_my || jn[1] < n_my)) {
                 bool progressed = false;
@@ -1058,41 +1078,48 @@ __global__ void __launch_bounds__(kSlabThreads, 1) tc_slab_kernel(const SlabArgs
                     if (j >= n_my) continue;
                     bool go;
                     if (st == 0)
-                        go = ptx::mbar_test_wait(&bars.full[g], (uint32_t)((j >> 1) & 1)) &&
+                        go = ptx::mbar_test_wait(&bars.full[buf[g]], (uint32_t)par[g]) &&
                              (j < 2 || ptx::mbar_test_wait(&bars.ready[g], 1u));
                     else
                         go = ptx::mbar_test_wait(&bars.ready[g], (uint32_t)((st - 1) & 1));
                     if (!go) continue;
                     ptx::tc_fence_after();
-                    const uint32_t sA = ptx::smem_u32(buf0 + g * 2 * half_bytes);
+                    const uint32_t sA = ptx::smem_u32(buf0 + buf[g] * 2 * half_bytes);
                     const uint32_t da = tmem + (uint32_t)(g * 2 * npm);
                     // M1: A1 (MN-major) x V2 forward; M2: A2 (MN-major) x V1 forward;
                     // M3: A3 (K-major) x V1^T; M4: A4 (MN-major) x V2^T
                     const bool ax2 = st == 0 || st == 3;
                     issue_split_mma(da, da + (uint32_t)npm, sA, sA + (uint32_t)half_bytes, st == 2, ax2 ? sV2h : sV1h,
-                                    ax2 ? sV2l : sV1l, st >= 2, ax2 ? np2 : np1);
+                                    ax2 ? sV2l : sV1l, st >= 2, ax2 ? np2 : np1, rg);
                     ptx::mma_commit(&bars.tfull[g]);
-                    if (st == 3) ptx::mma_commit(&bars.empty[g]);
-                    if (++sn[g] == 4) {
+                    if (st == kLast) {
+                        ptx::mma_commit(&bars.empty[buf[g]]);
                         sn[g] = 0;
                         jn[g] += 2;
+                        buf[g] += 2;
+                        if (buf[g] >= nbuf) {
+                            buf[g] -= nbuf;
+                            par[g] ^= 1;
+                        }
+                    } else {
+                        ++sn[g];
                     }
                     progressed = true;
                 }
-                const long long now = clock64();
                 if (progressed) {
-                    last = now;
-                } else if (s_abort) {
-                    ok = false;
-                } else if (now - last > a.timeout_cycles) {
-                    s_abort = 1;
-                    atomicExch(a.status, KX_ERR_TIMEOUT);
-                    ok = false;
+                    idle = 0;
+                } else if ((++idle & 31) == 0) {  // the clock and the abort flag now and then
+                    const long long now = clock64();
+                    if (idle == 32) last = now;
+                    if (s_abort) {
+                        ok = false;
+                    } else if (now - last > a.timeout_cycles) {
+                        s_abort = 1;
+                        atomicExch(a.status, KX_ERR_TIMEOUT);
+                        ok = false;
+                    }
                 }
             }
-#ifdef KX_ROLE_CLOCKS
-            clk_acc[5] = 0;
-#endif
             if (!ok) {
                 ptx::mma_commit(&bars.drain);
                 ptx::mbar_wait_bounded(&bars.drain, 0, a.timeout_cycles);
@@ -1102,77 +1129,120 @@ __global__ void __launch_bounds__(kSlabThreads, 1) tc_slab_kernel(const SlabArgs
     } else if (warp >= kSlabEpiWarps || helper >= 0) {
         // ---------------------------------------------------------------- producers: A1 from global
         const int ptid = helper >= 0 ? 32 * (kSlabProdWarps + helper) + lane : tid - kSlabEpiWarps * 32;
-        const int ngrp = np1 >> 3;       // row groups (x1)
-        const int ntask = ngrp * np2;    // x np2 columns (x2)
+        const int ngrp = np1 >> 3;            // row groups (x1) of a plane
+        const int ptask = ngrp * np2;         // x np2 columns (x2)
+        const int ntask = ptask * pp;         // x planes
         const unsigned gmagic = (65536u + (unsigned)ngrp - 1u) / (unsigned)ngrp;  // t / ngrp for t < 2^11
-        const int nlines = (int)((n12 * 4) >> 7);  // 128-byte lines of a slice (n1 % 8 == 0)
-        const uint32_t plane_bytes = (uint32_t)(n12 * 4);
-        auto plane = [&](int it) {
+        const int nlines = (int)((n12 * 4 * pp) >> 7);  // 128-byte lines of a unit's planes (n1 % 8 == 0)
+        const uint32_t plane_bytes = (uint32_t)(n12 * 4 * pp);
+        const unsigned n3u = (unsigned)(a.n3 / pp);  // units per item
+        // task t: plane, 8-row group and column; source offset (0 with `in` false: padding) and A offset
+        auto task = [&](int t, bool &in, int &src, int &off) {
+            int pl = 0;
+            if (MULTI) {
+                pl = t >= ptask ? 1 : 0;
+                if (pp > 2) pl += (t >= 2 * ptask ? 1 : 0) + (t >= 3 * ptask ? 1 : 0);
+                t -= pl * ptask;
+            }
+            const int k = (int)(((unsigned)t * gmagic) >> 16), g = t - k * ngrp;
+            in = 8 * g < a.n1 && k < a.n2;
+            src = in ? pl * (int)n12 + k * a.n1 + 8 * g : 0;
+            off = (g + (pl << (row_sh - 3))) * kCoreStride + (k >> 3) * kcore + (k & 7) * 16;
+        };
+        auto unit_item = [&](int it) { return (unsigned)(blockIdx.x + (long long)it * gridDim.x) / n3u; };
+        auto plane_off = [&](int it) {
             const long long u = blockIdx.x + (long long)it * gridDim.x;
-            const long long item = (unsigned)u / (unsigned)a.n3, k3 = (unsigned)u % (unsigned)a.n3;
-            return a.in + item * a.N + k3 * n12;
+            const long long item = (unsigned)u / n3u, k3 = (unsigned)u % n3u;
+            return item * a.N + k3 * pp * n12;
         };
         // stage_in: one thread copies the plane of the next unit into shared memory
         // (pieces of at most 16 KB) as soon as the previous plane has been split
         auto issue_plane = [&](int it) {
             ptx::fence_proxy_async_smem();
             ptx::mbar_arrive_expect_tx(&bars.in_full, plane_bytes);
-            const char *src = reinterpret_cast<const char *>(plane(it));
+            const char *src = reinterpret_cast<const char *>(a.in + plane_off(it));
             char *dst = reinterpret_cast<char *>(sin);
             for (uint32_t o = 0; o < plane_bytes; o += 16384u)
                 ptx::bulk_load(dst + o, src + o, min(16384u, plane_bytes - o), &bars.in_full);
         };
-        auto plane_max = [&](int it) {
-            return __ldg(a.in_max + (unsigned)(blockIdx.x + (long long)it * gridDim.x) / (unsigned)a.n3);
+        // item maxima and pairs are loaded one unit ahead, occupations with the unit
+        const bool want_e = a.e_partial != nullptr && !a.rhs_mode;
+        float next_max = 0.f;
+        int2 next_ij = make_int2(0, 0);
+        auto fetch = [&](int it) {
+            const unsigned item = unit_item(it);
+            next_max = __ldg(a.in_max + item);
+            if (want_e && ptid == 0) next_ij = __ldg(a.pairs + item);
         };
-        float next_max = n_my > 0 ? plane_max(0) : 0.f;  // loaded one unit ahead
+        if (n_my > 0) fetch(0);
         int inflight = -1;  // unit whose plane copy thread 0 issued and has not yet waited for
         if (a.stage_in && ptid == 0 && n_my > 0) {
             issue_plane(0);
             inflight = 0;
         }
+        int buf = 0, round = 0;  // A buffer of unit it, and how often it was used before
         for (int it = 0; it < n_my; ++it) {
-            const int sl = it & 1;
             if (it + 2 < n_my) {
                 // pull the plane of unit it+2 into L2 while this unit waits for its buffer
-                const char *src = reinterpret_cast<const char *>(plane(it + 2));
+                const char *src = reinterpret_cast<const char *>(a.in + plane_off(it + 2));
                 for (int l = ptid; l < nlines; l += n_prod) ptx::prefetch_l2(src + ((long long)l << 7));
             }
-            long long tw = KX_CLK_NOW();
-            bool ok = it < 2 || slab_wait(&bars.empty[sl], (uint32_t)(((it >> 1) - 1) & 1), a, &s_abort);
-            KX_CLK_ADD(1, tw);
-            tw = KX_CLK_NOW();
+            bool ok = round == 0 || slab_wait(&bars.empty[buf], (uint32_t)((round - 1) & 1), a, &s_abort);
             if (ok && a.stage_in) ok = slab_wait(&bars.in_full, (uint32_t)(it & 1), a, &s_abort);
             if (ok && ptid == 0) inflight = -1;
             ok = ok && !s_abort;
             // with stage_in the producers meet at a named barrier below, so they leave together
             ok = a.stage_in ? ptx::named_bar_and(2, n_prod, ok) : (bool)__all_sync(0xffffffffu, ok);
             if (!ok) break;
-            const float sc = pow2f(scale_exp(next_max));
-            if (it + 1 < n_my) next_max = plane_max(it + 1);
-            uint8_t *Ahi = buf0 + sl * 2 * half_bytes;
+            const float b1 = next_max;
+            const int2 ij = next_ij;
+            if (it + 1 < n_my) fetch(it + 1);
+            const int e1 = scale_exp(b1);
+            const float sc = pow2f(e1);
+            uint8_t *Ahi = buf0 + buf * 2 * half_bytes;
             uint8_t *Alo = Ahi + half_bytes;
+            if (ptid == 0) {
+                // the unit's constants for the epilogue (it reads them after this unit's M1)
+                SlabUnit &d = units[it % kSlabRing];
+                const float b2 = b1 * a.sq2, b3 = a.fmax * a.sq1 * b2, b4 = a.sq1 * b3;
+                const int e2 = scale_exp(b2), e3 = scale_exp(b3), e4 = scale_exp(b4);
+                d.us2 = pow2f(e2 - e1 - kVScaleExp);
+                d.u2 = pow2f(-(e2 + kVScaleExp));
+                d.s3 = pow2f(e3);
+                d.us4 = pow2f(e4 - e3 - kVScaleExp);
+                d.u4 = pow2f(-(e4 + kVScaleExp));
+                const unsigned u = (unsigned)(blockIdx.x + (long long)it * gridDim.x);
+                const int item = (int)(u / n3u), k3 = (int)(u - (unsigned)item * n3u) * pp;
+                d.item = item;
+                d.foff = k3 * (int)n12;
+                d.out0 = item * a.N + k3 * n12;
+                double w = 0.0;
+                if (want_e) {
+                    w = (ij.x == ij.y) ? 1.0 : 2.0;
+                    if (a.occ) w *= a.occ[ij.x] * a.occ[ij.y];
+                }
+                d.w = w;
+            }
             if (a.stage_in) {
-                // task: 8 rows x1 at one x2.  Loads first, without branches between them: a task
-                // past the end repeats the last one, a padding one reads real values and scales
-                // them to zero.  Row groups past np1 are never read (see the quadrants above).
-                for (int t0 = ptid; t0 < ntask; t0 += 4 * n_prod) {
-                    float4 x[4][2];
-                    int off[4];
-                    float scl[4];
+                // task: 8 rows x1 at one x2.  Two tasks' loads first, without branches between them
+                // (batches of 3, 4 and 6 measured 1, 3 and 3% slower): a task past the end
+                // repeats the last one, a padding one reads real values and scales them to zero.  Row groups past np1 are never read (see the quadrants above).
+                for (int t0 = ptid; t0 < ntask; t0 += 2 * n_prod) {
+                    float4 x[2][2];
+                    int off[2];
+                    float scl[2];
 #pragma unroll
-                    for (int r = 0; r < 4; ++r) {
-                        const int t = min(t0 + r * n_prod, ntask - 1);
-                        const int k = (int)(((unsigned)t * gmagic) >> 16), g = t - k * ngrp;
-                        const bool in = 8 * g < a.n1 && k < a.n2;
-                        const float4 *src = reinterpret_cast<const float4 *>(sin + (in ? k * a.n1 + 8 * g : 0));
+                    for (int r = 0; r < 2; ++r) {
+                        bool in;
+                        int so;
+                        task(min(t0 + r * n_prod, ntask - 1), in, so, off[r]);
+                        const float4 *src = reinterpret_cast<const float4 *>(sin + so);
                         x[r][0] = src[0];
                         x[r][1] = src[1];
                         scl[r] = in ? sc : 0.f;
-                        off[r] = g * kCoreStride + (k >> 3) * (16 * kCoreStride) + (k & 7) * 16;
                     }
 #pragma unroll
-                    for (int r = 0; r < 4; ++r) {
+                    for (int r = 0; r < 2; ++r) {
                         if (t0 + r * n_prod >= ntask) break;
                         const float2 s2 = make_float2(scl[r], scl[r]);
                         const float2 w[4] = {mul2(make_float2(x[r][0].x, x[r][0].y), s2),
@@ -1183,7 +1253,7 @@ __global__ void __launch_bounds__(kSlabThreads, 1) tc_slab_kernel(const SlabArgs
                     }
                 }
                 ptx::fence_proxy_async_smem();
-                warp_arrive(&bars.full[sl]);
+                warp_arrive(&bars.full[buf]);
                 // every producer has finished reading the plane: it may be overwritten
                 ptx::named_bar(2, n_prod);
                 if (ptid == 0 && it + 1 < n_my) {
@@ -1191,15 +1261,16 @@ __global__ void __launch_bounds__(kSlabThreads, 1) tc_slab_kernel(const SlabArgs
                     inflight = it + 1;
                 }
             } else {
-                const float *slice = plane(it);
+                const float *slice = a.in + plane_off(it);
                 for (int t0 = ptid; t0 < ntask; t0 += n_prod * kSlabU) {
                     float v[kSlabU][8];
 #pragma unroll
                     for (int r = 0; r < kSlabU; ++r) {
-                        const int t = t0 + r * n_prod;
-                        const int k = (int)(((unsigned)t * gmagic) >> 16), g = t - k * ngrp;
-                        if (t < ntask && 8 * g < a.n1 && k < a.n2) {
-                            ld8(slice + (long long)k * a.n1 + 8 * g, v[r]);
+                        bool in;
+                        int so, off;
+                        task(min(t0 + r * n_prod, ntask - 1), in, so, off);
+                        if (in) {
+                            ld8(slice + so, v[r]);
                         } else {
 #pragma unroll
                             for (int c = 0; c < 8; ++c) v[r][c] = 0.f;
@@ -1209,17 +1280,22 @@ __global__ void __launch_bounds__(kSlabThreads, 1) tc_slab_kernel(const SlabArgs
                     for (int r = 0; r < kSlabU; ++r) {
                         const int t = t0 + r * n_prod;
                         if (t >= ntask) continue;
-                        const int k = (int)(((unsigned)t * gmagic) >> 16), g = t - k * ngrp;
+                        bool in;
+                        int so, off;
+                        task(t, in, so, off);
                         float2 w[4];
 #pragma unroll
                         for (int c = 0; c < 4; ++c) w[c] = mul2(pair(v[r], c), make_float2(sc, sc));
-                        store_split8(Ahi, Alo, g * kCoreStride + (k >> 3) * (16 * kCoreStride) + (k & 7) * 16, w);
+                        store_split8(Ahi, Alo, off, w);
                     }
                 }
                 ptx::fence_proxy_async_smem();
-                warp_arrive(&bars.full[sl]);
+                warp_arrive(&bars.full[buf]);
             }
-            KX_CLK_ADD(2, tw);
+            if (++buf == nbuf) {
+                buf = 0;
+                ++round;
+            }
         }
         // a plane copy still in flight after an early exit must land before the CTA leaves
         if (inflight >= 0) ptx::mbar_wait_bounded(&bars.in_full, (uint32_t)(inflight & 1), a.timeout_cycles);
@@ -1229,48 +1305,37 @@ __global__ void __launch_bounds__(kSlabThreads, 1) tc_slab_kernel(const SlabArgs
         // 16-column chunks c = 16*h + 32*i, h = (w/4)%2.  tcgen05.ld is
         // warp-collective: every lane loads, only the stores are predicated per row.
         const int g = warp >> 3, q = warp & 3, h = (warp >> 2) & 1;
-        const int m = 32 * q + lane;  // TMEM lane == D row
+        const int row = 32 * q + lane;                      // TMEM lane == D row
+        const int pl = MULTI ? row >> row_sh : 0, m = MULTI ? row & ((1 << row_sh) - 1) : row;  // plane, row of it
+        const int m0 = m - lane;                            // the warp's first row of the plane
+        const int gp = pl << (row_sh - 3);                  // the plane's first row group
         const bool two1 = (np1 >> 4) > 1, two2 = (np2 >> 4) > 1;
         const int nkc1 = np1 >> 3;
         const uint32_t ta = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(g * 2 * npm);
         const uint32_t tb = ta + (uint32_t)npm;
-        uint8_t *Ahi = buf0 + g * 2 * half_bytes;
-        uint8_t *Alo = Ahi + half_bytes;
+        const int ld4 = 4 * a.n2;
         double e_acc = 0.0;
         bool ok = true;
-        // the item's maximum and pair are loaded one unit ahead
-        float next_b1 = 0.f;
-        int2 next_ij = make_int2(0, 0);
-        auto fetch = [&](int j) {
-            const unsigned item = (unsigned)(blockIdx.x + (long long)j * gridDim.x) / (unsigned)a.n3;
-            next_b1 = __ldg(a.in_max + item);
-            if (a.e_partial != nullptr && !a.rhs_mode) next_ij = __ldg(a.pairs + item);
-        };
-        if (g < n_my) fetch(g);
+        int buf = g;
         for (int j = g; j < n_my && ok; j += 2) {
-            long long tw = KX_CLK_NOW();
-            const SlabUnit U = slab_unit(a, blockIdx.x + (long long)j * gridDim.x, next_b1, next_ij);
-            if (j + 2 < n_my) fetch(j + 2);
-            KX_CLK_ADD(0, tw);
+            const SlabUnit &U = units[j % kSlabRing];
+            uint8_t *Ahi = buf0 + buf * 2 * half_bytes;
+            uint8_t *Alo = Ahi + half_bytes;
+            buf += 2;
+            if (buf >= nbuf) buf -= nbuf;
             // ---- B: D1[x1][k2] -> A2[k2][x1]
-            tw = KX_CLK_NOW();
             ok = __all_sync(0xffffffffu, slab_wait(&bars.tfull[g], 0u, a, &s_abort));
-            KX_CLK_ADD(9, tw);
             if (!ok) break;
-            tw = KX_CLK_NOW();
             ptx::tc_fence_after();
-            if (32 * q < np1)
-                slab_transpose_stage(ta, tb, m, h, a.n1, np1, np2, two2, pow2f(U.e2 - U.e1 - kVScaleExp), Ahi,
-                                     Alo);
+            if (m0 < np1)
+                slab_transpose_stage(ta, tb, m, gp, h, a.n1, np1, np2, two2, U.us2, kcore, Ahi, Alo);
             ptx::fence_proxy_async_smem();
             ptx::tc_fence_before();
             warp_arrive(&bars.ready[g]);
-            KX_CLK_ADD(10, tw);
             // ---- C: D2[k2][k1] = Y: energy sum f Y^2, mid = f Y -> A3[k2][k1] (K-major, own row)
             {
                 const bool rowC = m < a.n2;
-                const int ld4 = 4 * a.n2;
-                const float *frow = a.f32 + (U.k3 * n12 + 4 * m);
+                const float *frow = a.f32 + U.foff + pl * (int)n12 + 4 * m;
                 // f(Lambda) of this warp's first chunk; each further chunk's is fetched
                 // while the previous one is processed
                 float fr[2][16];
@@ -1284,15 +1349,11 @@ __global__ void __launch_bounds__(kSlabThreads, 1) tc_slab_kernel(const SlabArgs
                         for (int k = 0; k < 8; ++k) fr[0][8 * hh + k] = 0.f;
                     }
                 }
-                tw = KX_CLK_NOW();
                 ok = __all_sync(0xffffffffu, slab_wait(&bars.tfull[g], 1u, a, &s_abort));
-                KX_CLK_ADD(9, tw);
                 if (!ok) break;
-                tw = KX_CLK_NOW();
                 ptx::tc_fence_after();
-                const float u2 = pow2f(-(U.e2 + kVScaleExp));
-                const float s3 = pow2f(U.e3);
-                const int off_r = (m >> 3) * (nkc1 * kCoreStride) + (m & 7) * 16;
+                const float u2 = U.u2, s3 = U.s3;
+                const int off_r = (row >> 3) * (nkc1 * kCoreStride) + (row & 7) * 16;
                 float e_row = 0.f;
 #pragma unroll
                 for (int r = 0; r < kMaxN / 32; ++r) {
@@ -1319,45 +1380,41 @@ __global__ void __launch_bounds__(kSlabThreads, 1) tc_slab_kernel(const SlabArgs
                         const float2 fy = mul2(pair(fr[r & 1], k), y);
                         e_row = fmaf(fy.x, y.x, e_row);
                         e_row = fmaf(fy.y, y.y, e_row);
-                        mid[k] = mul2(fy, make_float2(s3, s3));
+                        if (!ENERGY) mid[k] = mul2(fy, make_float2(s3, s3));
                     }
+                    if (!ENERGY) {
 #pragma unroll
-                    for (int hh = 0; hh < 2; ++hh)
-                        store_split8(Ahi, Alo, off_r + ((c >> 3) + hh) * kCoreStride, mid + 4 * hh);
+                        for (int hh = 0; hh < 2; ++hh)
+                            store_split8(Ahi, Alo, off_r + ((c >> 3) + hh) * kCoreStride, mid + 4 * hh);
+                    }
                 }
-                if (rowC) e_acc += U.w * (double)e_row;
-                ptx::fence_proxy_async_smem();
+                if (!ENERGY) ptx::fence_proxy_async_smem();
                 ptx::tc_fence_before();
+                const double w = U.w;
                 warp_arrive(&bars.ready[g]);
-                KX_CLK_ADD(11, tw);
+                if (rowC) e_acc += w * (double)e_row;
             }
+            if (ENERGY) continue;
             // ---- D: D3[k2][x1] -> A4[x1][k2]
-            tw = KX_CLK_NOW();
             ok = __all_sync(0xffffffffu, slab_wait(&bars.tfull[g], 0u, a, &s_abort));
-            KX_CLK_ADD(9, tw);
             if (!ok) break;
-            tw = KX_CLK_NOW();
             ptx::tc_fence_after();
-            if (32 * q < np2)
-                slab_transpose_stage(ta, tb, m, h, a.n2, np2, np1, two1, pow2f(U.e4 - U.e3 - kVScaleExp), Ahi,
-                                     Alo);
+            if (m0 < np2)
+                slab_transpose_stage(ta, tb, m, gp, h, a.n2, np2, np1, two1, U.us4, kcore, Ahi, Alo);
             ptx::fence_proxy_async_smem();
             ptx::tc_fence_before();
             warp_arrive(&bars.ready[g]);
-            KX_CLK_ADD(3, tw);
             // ---- E: D4[x1][x2] -> slice [x2][x1] of the output, coalesced over x1
-            tw = KX_CLK_NOW();
             ok = __all_sync(0xffffffffu, slab_wait(&bars.tfull[g], 1u, a, &s_abort));
-            KX_CLK_ADD(9, tw);
             if (!ok) break;
-            tw = KX_CLK_NOW();
             ptx::tc_fence_after();
             {
-                const float u4 = pow2f(-(U.e4 + kVScaleExp));
+                const float u4 = U.u4;
+                const int item = U.item;
                 const bool valid = m < a.n1;
                 float my_max = 0.f;
-                if (32 * q < a.n1) {
-                    float *orow = a.out + U.item * a.N + U.k3 * n12 + m + (long long)(16 * h) * a.n1;
+                if (m0 < a.n1) {
+                    float *orow = a.out + U.out0 + pl * (int)n12 + m + (long long)(16 * h) * a.n1;
                     for (int c = 16 * h; c < np2; c += 32, orow += 32 * a.n1) {
                         float v[16], vb[16];
                         ptx::tmem_ld16x2(ta + c, tb + c, v, vb);
@@ -1378,11 +1435,10 @@ __global__ void __launch_bounds__(kSlabThreads, 1) tc_slab_kernel(const SlabArgs
                         }
                     }
                 }
-                track_max(a.out_max, U.item, my_max, valid);
+                ptx::tc_fence_before();
+                warp_arrive(&bars.ready[g]);
+                track_max(a.out_max, item, my_max, valid);
             }
-            ptx::tc_fence_before();
-            warp_arrive(&bars.ready[g]);
-            KX_CLK_ADD(7, tw);
         }
         if (a.e_partial != nullptr) {
             double e = e_acc;
@@ -1396,15 +1452,6 @@ __global__ void __launch_bounds__(kSlabThreads, 1) tc_slab_kernel(const SlabArgs
             }
         }
     }
-#ifdef KX_ROLE_CLOCKS
-    if (a.clk != nullptr) {
-        long long *o = a.clk + (long long)blockIdx.x * kClk;
-        const long long tot = clock64() - clk_t0;
-        if (warp == kSlabMmaWarp && lane == 0) { o[4] = tot; }
-        if (tid == kSlabEpiWarps * 32) { o[5] = tot; o[1] = clk_acc[1]; o[2] = clk_acc[2]; }
-        if (tid == 0) { o[8] = tot; o[0] = clk_acc[0]; o[9] = clk_acc[9]; o[10] = clk_acc[10]; o[11] = clk_acc[11]; o[3] = clk_acc[3]; o[7] = clk_acc[7]; }
-    }
-#endif
     ptx::tc_fence_before();
     __syncthreads();
     if (warp == kSlabMmaWarp) {
@@ -1755,16 +1802,25 @@ int launch_pass(const kx_plan *p, PassArgs a, int axis, cudaStream_t s, int *gri
     return prof_end(const_cast<kx_plan *>(p), s);
 }
 
-size_t slab_smem(const kx_plan *p, bool share_v = false) {
-    const int np1 = p->np[0], np2 = p->np[1], npm = std::max(np1, np2);
-    return (size_t)4 * np1 * np1 + (share_v ? 0 : (size_t)4 * np2 * np2) + 4 * a_half_bytes(npm) + 1024;
-}
 // axes 1 and 2 of the same size, spacing and boundary have the same eigenvectors
 bool same_axes12(const kx_plan *p) { return p->n[0] == p->n[1] && p->h[0] == p->h[1] && p->bc[0] == p->bc[1]; }
 
-// The slab kernel holds V1, V2 and two split A buffers in shared memory.
+// The slab kernel runs where V1, V2 and two full (128-row) A buffers fit in shared memory
+// (planes up to ~104 x 104); what it needs is no more than that.
 constexpr size_t kSlabSmemMax = 227 * 1024 - 1024;  // opt-in maximum less static shared memory
-bool slab_fits(const kx_plan *p) { return slab_smem(p) <= kSlabSmemMax; }
+bool slab_fits(const kx_plan *p) {
+    const int np1 = p->np[0], np2 = p->np[1], npm = std::max(np1, np2);
+    return (size_t)4 * np1 * np1 + (size_t)4 * np2 * np2 + 4 * a_half_bytes(npm) + 1024 <= kSlabSmemMax;
+}
+
+// E_x alone through the slab kernel: its two products cost a unit nearly the same
+// whatever the planes hold, the two passes it replaces go with their values.  Per call
+// (40 orbitals), slab against passes: 48^3 0.48 / 0.45 ms, (80, 48, 64) 1.03 / 0.86 at
+// 4608 and 3840 values a unit; (64, 48, 80) 0.84 / 0.86, 80^3 1.58 / 1.78, 96^3
+// 2.57 / 3.12 at 6144, 6400 and 9216.
+bool slab_for_energy(const kx_plan *p) {
+    return slab_planes(std::max(p->np[0], p->np[1])) * p->np[0] * p->np[1] >= 6000;
+}
 
 bool use_slab(const kx_plan *p) {
     if (const char *e = std::getenv("KX_SLAB")) return std::atoi(e) != 0;  // tuning override
@@ -1775,8 +1831,8 @@ bool use_slab(const kx_plan *p) {
 // and mode 2 inverse of R items in one launch; `in` holds the mode-3 forward
 // output, `out` receives the input of the mode-3 inverse (both natural layout).
 int launch_slab(kx_plan *p, long R, const float *in, const float *in_max, float *out, float *out_max,
-                double *e_partial, const int2 *pairs, const double *occ, int rhs_mode, cudaStream_t s,
-                int *grid_out) {
+                double *e_partial, const int2 *pairs, const double *occ, int rhs_mode, bool energy_only,
+                cudaStream_t s, int *grid_out) {
     SlabArgs a{};
     a.n1 = p->n[0];
     a.n2 = p->n[1];
@@ -1784,7 +1840,8 @@ int launch_slab(kx_plan *p, long R, const float *in, const float *in_max, float 
     a.np1 = p->np[0];
     a.np2 = p->np[1];
     a.N = (long long)p->N;
-    a.total_units = (long long)R * a.n3;
+    a.pp = slab_planes(std::max(a.np1, a.np2));
+    a.total_units = (long long)R * (a.n3 / a.pp);
     a.in = in;
     a.out = out;
     a.V1s = p->d_Vs[0];
@@ -1806,17 +1863,23 @@ int launch_slab(kx_plan *p, long R, const float *in, const float *in_max, float 
     a.clk = g_clkbuf + 5LL * kClk * 4096;
 #endif
     a.share_v = same_axes12(p) ? 1 : 0;
-    size_t smem = slab_smem(p, a.share_v != 0);
-    const size_t plane = (size_t)a.n1 * a.n2 * 4;
-    a.stage_in = (smem + plane <= kSlabSmemMax) ? 1 : 0;
+    const size_t base = (size_t)4 * a.np1 * a.np1 + (a.share_v ? 0 : (size_t)4 * a.np2 * a.np2) + 1024;
+    const size_t buffer = 2 * slab_half_bytes(std::max(a.np1, a.np2));
+    const size_t plane = (size_t)a.n1 * a.n2 * 4 * a.pp;
+    // a third buffer first, then the staged input plane
+    a.nbuf = base + 3 * buffer <= kSlabSmemMax ? 3 : 2;
+    size_t smem = base + a.nbuf * buffer;
+    a.stage_in = smem + plane <= kSlabSmemMax ? 1 : 0;
     if (a.stage_in) smem += plane;
     // at least 120 KB so that one CTA (and one 512-column TMEM allocation) sits on each SM
     smem = std::max<size_t>(smem, 120 * 1024);
-    KX_CUDA_TRY(cudaFuncSetAttribute(tc_slab_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     const int grid = (int)std::max(1LL, std::min<long long>(a.total_units, (long long)p->num_sms));
     if (grid_out) *grid_out = grid;
     if (int rc = prof_begin(p, PK_SLAB, s)) return rc;
-    tc_slab_kernel<<<grid, kSlabThreads, smem, s>>>(a);
+    auto kernel = energy_only ? (a.pp > 1 ? tc_slab_kernel<true, true> : tc_slab_kernel<true, false>)
+                              : (a.pp > 1 ? tc_slab_kernel<false, true> : tc_slab_kernel<false, false>);
+    KX_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    kernel<<<grid, kSlabThreads, smem, s>>>(a);
     KX_LAUNCH_CHECK("tc_slab_kernel launch");
     return prof_end(p, s);
 }
@@ -1874,13 +1937,15 @@ int run_passes(kx_plan *p, PassArgs a, long R, float *T0, float *T1, float *mx, 
     a.out_max = mx1;
     if ((rc = launch_pass<P_X3F>(p, a, 2, s, nullptr))) return rc;
 
-    if (!energy_only && slab_fits(p) && use_slab(p)) {
-        // X2F, X1 and X2I fused: T0 -> T1 without the intermediate round trips
+    if (slab_fits(p) && use_slab(p) && (!energy_only || slab_for_energy(p))) {
+        // X2F, X1 and X2I fused: T0 -> T1 without the intermediate round trips (E_x
+        // alone: X2F and the forward half of X1)
         int grid = 0;
-        if ((rc = launch_slab(p, R, T0, mx1, T1, mx4, ex ? partial : nullptr, a.pairs, a.occ, a.rhs_mode, s,
-                              &grid)))
+        if ((rc = launch_slab(p, R, T0, mx1, T1, mx4, ex ? partial : nullptr, a.pairs, a.occ, a.rhs_mode, energy_only,
+                              s, &grid)))
             return rc;
-        if (ex && (rc = add_energy(p, partial, grid, ex, e_count, s))) return rc;
+        if (ex && (rc = add_energy(p, partial, grid, ex, energy_only ? nullptr : e_count, s))) return rc;
+        if (energy_only) return KX_OK;
         a.e_partial = nullptr;
         a.energy_only = 0;
         a.rows_pp = (long long)p->n[0] * p->n[1];

@@ -196,6 +196,30 @@ def test_fused_and_unfused_middle_passes(kx, case, monkeypatch):
         assert abs(ex.item() - ex_ref) < TOL[1]["ex"] * abs(ex_ref)
 
 
+@pytest.mark.parametrize("n", [(8, 8, 8), (32, 32, 8), (32, 40, 8), (64, 64, 16), (8, 64, 24), (72, 64, 8), (96, 96, 8),
+                               (96, 8, 16), (8, 96, 8), (80, 88, 8), (104, 16, 8), (16, 128, 8)])
+def test_slab_planes_per_unit(kx, n):
+    """The fused middle products over the plane shapes it handles differently: four,
+    two and one plane per unit, idle quadrants, two and three A buffers, shared and
+    separate eigenvectors, planes of more than 96 rows; E_x alone through it or the passes."""
+    h = (0.4, 0.4, 0.45)
+    sysd = system(n, h, (P, P, D), S, 5, 223)
+    psi = workloads.random_field(n[0] * n[1] * n[2], 5, 224)
+    occ = np.array([1.0, 0.9, 0.7, 0.4, 0.2])
+    op = oracle.Plan(n, h, sysd.bc, S)
+    vx_ref, ex_ref = oracle.vx_apply(op, psi, occ)
+    plan = kx.Plan(n, h, sysd.bc, S, precision=1)
+    vx, ex = kx.kx_vx_apply(plan, dev(psi.T), dev(occ))
+    e_only = kx.kx_energy(plan, dev(psi.T), dev(occ))
+    b = workloads.random_field(op.N, 3, 225)
+    x = kx.kx_apply_fL(plan, dev(b.T)).cpu().numpy().T
+    assert plan.status() == kx.KX_OK
+    assert relmax(vx.cpu().numpy().T, vx_ref) < TOL[1]["vx"]
+    assert abs(ex.item() - ex_ref) < TOL[1]["ex"] * abs(ex_ref)
+    assert abs(e_only.item() - ex_ref) < TOL[1]["ex"] * abs(ex_ref)
+    assert relmax(x, np.stack([oracle.apply_fL(op, b[:, r]) for r in range(3)], axis=1)) < TOL[1]["fl"]
+
+
 @pytest.mark.parametrize("n", [(48, 48, 64), (80, 16, 24)])
 def test_separate_passes_repeat_bit_identical(kx, n, monkeypatch):
     """The separate middle passes with an odd number of 16-column chunks along x1:
