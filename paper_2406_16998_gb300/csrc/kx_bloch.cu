@@ -2108,6 +2108,12 @@ inline bool bp0_axis(const kx_plan *p) {
     return bp_axes(p) && tc_axis(p, 0) && p->n[0] == 64 && (p->N / 64) % 128 == 0;
 }
 
+// Axes 1 and 2 two products per kernel (kx_bloch_fused.cu): planes of 64 x 64 points, two
+// of which are a tile of 128 rows (969 -> 485 us for the four products of 256 pairs at
+// 64^3).  A plane of 32-point axes would fill half the tile's columns and leave the
+// kernel's time per value as it is, so those sizes keep the single products.
+inline bool bp_fused(const kx_plan *p) { return bp_axes(p) && tc_axis(p, 0) && p->n[0] == 64 && p->n[1] == 64; }
+
 template <bool FORM>
 int launch_bp0(kx_plan *p, long long R, const float2 *in, float2 *out, const __half *Bs, const float2 *P,
                const float2 *F, const float *in_max, const float *pmax, const float *fmax, long long r0, int n_orb,
@@ -2365,17 +2371,31 @@ int bloch_sweep(kx_plan *p, int n_kpt, const double *theta, const double *wk, in
             const long long r1 = std::min(pairs, r0 + L.chunk);
             const long long R = r1 - r0;
             int rc;
+            T2 *X = B;  // the solved chunk
             if constexpr (sizeof(T) == 4) {
                 auto Bf = [&](int a) { return reinterpret_cast<const __half *>(ws + L.Bf[a]); };
                 auto Bi = [&](int a) { return reinterpret_cast<const __half *>(ws + L.Bi[a]); };
-                if (bp0_axis(p))
+                if (bp_fused(p)) {
+                    // axes 1 and 2 two products at a time, on planes; axis 3 between them
+                    float *mx0 = reinterpret_cast<float *>(ws + L.mx0), *mx1 = reinterpret_cast<float *>(ws + L.mx1);
+                    if ((rc = bloch_fused_forward(p, R, Pq, F, B, Bf(0), Bf(1), reinterpret_cast<const float *>(ws + L.Pmax),
+                                                  reinterpret_cast<const float *>(ws + L.Fmax), r0, n_orb, mx0, s)))
+                        return rc;
+                    if ((rc = launch_bp<1>(p, 2, R, B, A, Bf(2), f, mx0, nullptr, nullptr, 0, n_orb, mx1, s))) return rc;
+                    if ((rc = launch_bp<0>(p, 2, R, A, B, Bi(2), nullptr, mx1, nullptr, nullptr, 0, n_orb, mx0, s)))
+                        return rc;
+                    rc = bloch_fused_inverse(p, R, B, A, Bi(1), Bi(0), mx0, s);
+                    X = A;
+                } else if (bp0_axis(p))
                     rc = launch_bp0<true>(p, R, nullptr, A, Bf(0), Pq, F, nullptr, reinterpret_cast<const float *>(ws + L.Pmax),
                                           reinterpret_cast<const float *>(ws + L.Fmax), r0, n_orb, s);
                 else
                     rc = tc_axis(p, 0) ? launch_tc<true, 0>(p, 0, R, nullptr, A, Bf(0), nullptr, Pq, F, n_orb, r0, s)
                                        : launch_form<T>(p, R, A, Mf[0], Pq, F, n_orb, r0, s);
                 if (rc) return rc;
-                if (bp_axes(p)) {
+                if (bp_fused(p)) {
+                    // done above
+                } else if (bp_axes(p)) {
                     // axes 2 and 3 with per-item scales: the bound from the orbital
                     // maxima, then the maxima each product records
                     float *mx0 = reinterpret_cast<float *>(ws + L.mx0), *mx1 = reinterpret_cast<float *>(ws + L.mx1);
@@ -2405,7 +2425,9 @@ int bloch_sweep(kx_plan *p, int n_kpt, const double *theta, const double *wk, in
                              : launch_pipe<T, 0>(p, 1, R, B, A, Mi[1], nullptr, s);
                     if (rc) return rc;
                 }
-                if (bp0_axis(p))
+                if (bp_fused(p))
+                    rc = KX_OK;
+                else if (bp0_axis(p))
                     rc = launch_bp0<false>(p, R, A, B, Bi(0), nullptr, nullptr,
                                            reinterpret_cast<const float *>(ws + L.mx1), nullptr, nullptr, 0, n_orb, s);
                 else
@@ -2429,11 +2451,11 @@ int bloch_sweep(kx_plan *p, int n_kpt, const double *theta, const double *wk, in
             const int ab = (int)std::min<long long>((nv * N / per + 255) / 256, 8LL * p->num_sms);
             if constexpr (sizeof(T) == 4) {
                 if (pairs2)
-                    bloch_accum2_kernel<false><<<ab, 256, 0, s>>>(B, r0, r1, n_orb, Pq, occ_q, wk[q],
+                    bloch_accum2_kernel<false><<<ab, 256, 0, s>>>(X, r0, r1, n_orb, Pq, occ_q, wk[q],
                                                                   reinterpret_cast<double2 *>(out_k), N);
             }
             if (!pairs2)
-                bloch_accum_kernel<T><<<ab, 256, 0, s>>>(B, r0, r1, n_orb, Pq, occ_q, wk[q],
+                bloch_accum_kernel<T><<<ab, 256, 0, s>>>(X, r0, r1, n_orb, Pq, occ_q, wk[q],
                                                          reinterpret_cast<double2 *>(out_k), N);
             KX_LAUNCH_CHECK("bloch_accum_kernel launch");
             if (reverse) {
@@ -2441,10 +2463,10 @@ int bloch_sweep(kx_plan *p, int n_kpt, const double *theta, const double *wk, in
                 double2 *out_q = reinterpret_cast<double2 *>(out_all) + (size_t)q * n_orb * N;
                 if constexpr (sizeof(T) == 4) {
                     if (pairs2)
-                        bloch_accum2_kernel<true><<<rb, 256, 0, s>>>(B, r0, r1, n_orb, F, occ_k, wk[k], out_q, N);
+                        bloch_accum2_kernel<true><<<rb, 256, 0, s>>>(X, r0, r1, n_orb, F, occ_k, wk[k], out_q, N);
                 }
                 if (!pairs2)
-                    bloch_accum_rev_kernel<T><<<rb, 256, 0, s>>>(B, r0, r1, n_orb, F, occ_k, wk[k], out_q, N);
+                    bloch_accum_rev_kernel<T><<<rb, 256, 0, s>>>(X, r0, r1, n_orb, F, occ_k, wk[k], out_q, N);
                 KX_LAUNCH_CHECK("bloch_accum_rev_kernel launch");
             }
             if ((rc = prof_end(p, s))) return rc;
@@ -2609,7 +2631,11 @@ int bloch_energy_only(kx_plan *p, int n_kpt, const double *theta, const double *
                 int rc;
                 if constexpr (sizeof(T) == 4) {
                     auto Bf = [&](int a) { return reinterpret_cast<const __half *>(ws + L.Bf[a]); };
-                    if (bp0_axis(p))
+                    if (bp_fused(p))
+                        rc = bloch_fused_forward(p, R, Pq, F, B, Bf(0), Bf(1), reinterpret_cast<const float *>(ws + L.Pmax),
+                                                 reinterpret_cast<const float *>(ws + L.Fmax), r0, n_orb,
+                                                 reinterpret_cast<float *>(ws + L.mx0), s);
+                    else if (bp0_axis(p))
                         rc = launch_bp0<true>(p, R, nullptr, A, Bf(0), Pq, F, nullptr, reinterpret_cast<const float *>(ws + L.Pmax),
                                               reinterpret_cast<const float *>(ws + L.Fmax), r0, n_orb, s);
                     else
@@ -2620,7 +2646,8 @@ int bloch_energy_only(kx_plan *p, int n_kpt, const double *theta, const double *
                         float *mx0 = reinterpret_cast<float *>(ws + L.mx0);
                         const float *pm = reinterpret_cast<const float *>(ws + L.Pmax);
                         const float *fm = reinterpret_cast<const float *>(ws + L.Fmax);
-                        if ((rc = launch_bp<0>(p, 1, R, A, B, Bf(1), nullptr, nullptr, pm, fm, r0, n_orb, mx0, s)))
+                        if (!bp_fused(p) &&
+                            (rc = launch_bp<0>(p, 1, R, A, B, Bf(1), nullptr, nullptr, pm, fm, r0, n_orb, mx0, s)))
                             return rc;
                         if ((rc = launch_bp<2>(p, 2, R, B, nullptr, Bf(2), f, mx0, nullptr, nullptr, 0, n_orb, nullptr,
                                                s, ea)))

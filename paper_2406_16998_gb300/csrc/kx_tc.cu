@@ -109,60 +109,12 @@ struct PassArgs {
     long long *clk;        // role counters (only with KX_ROLE_CLOCKS)
 };
 
-__device__ __forceinline__ int scale_exp(float mx) {
-    // e such that mx * 2^e < 2^14 (mx = m 2^k, m in [0.5, 1)  =>  e = 14 - k), from the
-    // exponent bits (frexpf only for subnormal maxima)
-    int k = 0;
-    if (mx > 0.f && isfinite(mx)) {
-        k = (__float_as_int(mx) >> 23) - 126;
-        if (k == -126) frexpf(mx, &k);
-    }
-    return 14 - k;
-}
-__device__ __forceinline__ float pow2f(int e) {
-    return (unsigned)(e + 126) < 254u ? __int_as_float((e + 127) << 23) : ldexpf(1.f, e);
-}
-
-// Packed float32 arithmetic (two values per instruction, each rounded as the scalar
-// form rounds it): the epilogues and producers below are bound by the length of
-// their instruction sequences.
-__device__ __forceinline__ float2 add2(float2 a, float2 b) {
-    unsigned long long r;
-    asm("add.rn.f32x2 %0, %1, %2;"
-        : "=l"(r)
-        : "l"(*reinterpret_cast<unsigned long long *>(&a)), "l"(*reinterpret_cast<unsigned long long *>(&b)));
-    return *reinterpret_cast<float2 *>(&r);
-}
-__device__ __forceinline__ float2 mul2(float2 a, float2 b) {
-    unsigned long long r;
-    asm("mul.rn.f32x2 %0, %1, %2;"
-        : "=l"(r)
-        : "l"(*reinterpret_cast<unsigned long long *>(&a)), "l"(*reinterpret_cast<unsigned long long *>(&b)));
-    return *reinterpret_cast<float2 *>(&r);
-}
-
-__device__ __forceinline__ void split8(const float2 *v, uint4 &hi, uint4 &lo) {
-    __half2 h[4], l[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const __half2 hh = __floats2half2_rn(v[i].x, v[i].y);
-        float2 r = v[i];
-        fma2(r, __half22float2(hh), make_float2(-1.f, -1.f));
-        h[i] = hh;
-        l[i] = __floats2half2_rn(r.x, r.y);
-    }
-    hi = *reinterpret_cast<uint4 *>(h);
-    lo = *reinterpret_cast<uint4 *>(l);
-}
-
 __device__ __forceinline__ void ld8(const float *p, float *v) {
     float4 a = __ldg(reinterpret_cast<const float4 *>(p));
     float4 b = __ldg(reinterpret_cast<const float4 *>(p) + 1);
     v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
     v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
 }
-
-__device__ __forceinline__ float2 pair(const float *v, int k) { return make_float2(v[2 * k], v[2 * k + 1]); }
 
 // One k-step leaves the second accumulator unwritten: the epilogues then add zeros
 // (one branch per chunk; a select and a bound test per element made the last stage

@@ -86,6 +86,13 @@ __device__ __forceinline__ uint64_t sdesc(uint32_t saddr, uint32_t lbo, uint32_t
     d |= (uint64_t)1 << 46;
     return d;
 }
+// The same for the 128-byte swizzle (layout type 2; atoms of 8 rows x 128 bytes, 1024-byte
+// aligned, the 16-byte chunks of a row XORed with the row).  K along the rows: sbo
+// between 8-row groups along M/N (lbo unused).  M/N along the rows: lbo between 64-value
+// halves, sbo between 8-row groups along K.
+__device__ __forceinline__ uint64_t sdesc_sw128(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
+    return sdesc(saddr, lbo, sbo) | (uint64_t)2 << 61;
+}
 // Instruction descriptor of kind::f16: fp16 A and B, fp32 D, dense, M x N,
 // A/B major-ness (0 = K-major, 1 = MN-major).
 __host__ __device__ constexpr uint32_t idesc_f16(int M, int N, int a_mn, int b_mn) {
@@ -317,6 +324,13 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 template <int n>
 __device__ __forceinline__ void cp_async_wait() {
     asm volatile("cp.async.wait_group %0;" ::"n"(n) : "memory");
+}
+
+// 32 bytes (aligned) in one store: a whole sector.
+__device__ __forceinline__ void st_global_32(void *p, const float *v) {
+    asm volatile("st.global.v8.f32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(p), "f"(v[0]), "f"(v[1]), "f"(v[2]),
+                 "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7])
+                 : "memory");
 }
 
 __device__ __forceinline__ void prefetch_l2(const void *p) {

@@ -1084,6 +1084,48 @@ def test_kpoint_pass_kernels_and_tile_kernels(kx, case, monkeypatch):
     assert relmax(out[("5", "1")], out[(None, "1")]) < TOL_K[prec][0]
 
 
+@pytest.mark.parametrize("n3,bc,n_orb,counts,chunk", [
+    (64, (P, P, D), 3, (2, 1, 1), None),  # 9 pairs: more tiles than SMs, fewer than two rounds of them
+    (64, (P, D, P), 2, (2, 1, 1), "3"),  # chunks that split a vector's bands
+    (32, (P, P, P), 3, (1, 2, 1), None),  # the shorter third axis
+    (32, (D, P, P), 1, (1, 1, 2), None),  # fewer tiles than SMs
+])
+def test_kpoint_fused_products(kx, n3, bc, n_orb, counts, chunk, monkeypatch):
+    """Planes of 64 x 64 points run two products per kernel; KX_BLOCH_PASS=0 takes the
+    single products.  Both match the oracle, for Vx, E_x alone and vectors at one k-point."""
+    prec = 1
+    sysd = system((64, 64, n3), (0.3, 0.35, 0.4), bc, U if D in bc else S, n_orb, 380 + n3)
+    theta, wk = workloads.kpoint_grid(sysd, counts)
+    psi = workloads.make_bloch_orbitals(sysd, theta)
+    occ = np.random.default_rng(n3).uniform(0.3, 1.0, (len(wk), n_orb))
+    base = oracle.Plan(sysd.n, sysd.h, sysd.bc, sysd.kernel)
+    vx_ref, ex_ref = oracle.vx_kpoints(base, theta, wk, psi, occ)
+    plan = kx.Plan(sysd.n, sysd.h, sysd.bc, sysd.kernel, precision=prec)
+    if chunk:
+        monkeypatch.setenv("KX_CHUNK_PAIRS", chunk)
+    dpsi, docc = to_dev_orbitals(psi), dev(occ)
+    out = {}
+    for bp in ("1", "0"):
+        monkeypatch.setenv("KX_BLOCH_PASS", bp)
+        plan.profile(True)
+        vx, ex = kx.kx_vx_kpoints(plan, theta, wk, dpsi, docc)
+        torch.cuda.synchronize()
+        assert plan.status() == kx.KX_OK
+        chunks = -(-n_orb * n_orb // int(chunk)) if chunk else 1
+        n_k = len(wk)
+        assert plan.profile_read()["bloch"][1] == (4 if bp == "1" else 6) * chunks * n_k * (n_k + 1) // 2
+        e_only = kx.kx_energy_kpoints(plan, theta, wk, dpsi, docc).item()
+        one = kx.kx_vx_apply_kpoint(plan, theta, wk, dpsi, 1, dpsi[1].contiguous(), docc)
+        torch.cuda.synchronize()
+        vx = vx.cpu().numpy().transpose(0, 2, 1)
+        assert relmax(vx, vx_ref) < TOL_K[prec][0], bp
+        assert relmax(one.cpu().numpy().T, vx_ref[1]) < TOL_K[prec][0], bp
+        assert abs(ex.item() - ex_ref) < TOL_K[prec][1] * abs(ex_ref), bp
+        assert abs(e_only - ex_ref) < TOL_K[prec][1] * abs(ex_ref), bp
+        out[bp] = vx
+    assert relmax(out["1"], out["0"]) < TOL_K[prec][0]
+
+
 @pytest.mark.parametrize("prec", [0, 1])
 def test_kpoint_apply_to_vectors_in_chunks(kx, prec, monkeypatch):
     """Vx at one k-point on arbitrary complex vectors, with chunks of 4 pairs that
