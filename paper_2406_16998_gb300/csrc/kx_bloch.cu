@@ -1653,18 +1653,34 @@ __global__ void bloch_basis_kernel(BlochAxes ax, typename Cx<T>::t *Mf0, typenam
         v.y = -v.y;
         Mf[x * n + m] = v;
     }
-    if (blockIdx.y != 0) return;
+    // eigenvalues: a block takes every gridDim.y-th of them, a thread one of their cosines
+    // (one thread per eigenvalue in a single block was the whole kernel's time, 20 us)
     const int mo = ax.order / 2;
     const double ih2 = 1.0 / (ax.h[a] * ax.h[a]);
-    for (int m = threadIdx.x; m < n; m += blockDim.x) {
-        if (bloch) {
-            double kap = (2.0 * M_PI * m + th) / n;
-            double s = fd_weight(mo, 0);
-            for (int p = 1; p <= mo; ++p) s += 2.0 * fd_weight(mo, p) * cos(p * kap);
-            lam[m] = s * ih2;
-        } else {
+    const int nm = (n - (int)blockIdx.y + (int)gridDim.y - 1) / (int)gridDim.y;
+    if (!bloch) {
+        for (int i = threadIdx.x; i < nm; i += blockDim.x) {
+            const int m = blockIdx.y + i * gridDim.y;
             lam[m] = ax.lam[a][m];
         }
+        return;
+    }
+    __syncthreads();  // rt and ph are free
+    double *wt = &rt[0].x, *cs = &ph[0].x;  // weights w_0, 2 w_p; cosines
+    for (int i = threadIdx.x; i < nm * mo + mo + 1; i += blockDim.x) {
+        if (i < nm * mo) {
+            const int m = blockIdx.y + (i / mo) * gridDim.y, p = i % mo + 1;
+            cs[i] = cos(p * ((2.0 * M_PI * m + th) / n));
+        } else {
+            const int p = i - nm * mo;
+            wt[p] = p == 0 ? fd_weight(mo, 0) : 2.0 * fd_weight(mo, p);
+        }
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < nm; i += blockDim.x) {
+        double s = wt[0];
+        for (int p = 1; p <= mo; ++p) s += wt[p] * cs[i * mo + p - 1];
+        lam[blockIdx.y + i * gridDim.y] = s * ih2;
     }
 }
 
@@ -1813,6 +1829,147 @@ __global__ void __launch_bounds__(256, 3) bloch_accum2_kernel(const float2 *__re
         o[0] = o0;
         o[1] = o1;
     }
+}
+
+// Both sums of a float32 chunk in one pass over it, for up to MB bands and an even N: out_v
+// as bloch_accum_kernel and, when REV, out_m as bloch_accum_rev_kernel, same terms in the
+// same order per point.  The kernels above are bound by the loads in flight, read a
+// vector from L2 per item besides the chunk, and convert a weight per term on the float64
+// pipe.  Here a block has 128 points; a vector's items come through a ring of kAccStages
+// bulk copies (1 KB per item), the points' bands psi_m and the reversed sums stay in
+// registers.  256 pairs at 64^3 (537 MB): forward alone 135 -> 124 us, both 265 ->
+// 150 us (floors 104 and 128 us with the sums read and written).  Two stages: blocks per SM
+// count for more than depth (four: 187 and 141 us).
+constexpr int kAccPoints = 128, kAccStages = 2;
+
+struct AccBoth {
+    const float2 *X, *P, *F;
+    long long r0, r1, N;
+    int n_orb;
+    const double *occ_q, *occ_k;
+    double wq, wk;
+    double2 *out_k, *out_q;
+    int *status;
+};
+
+// a b - c d and a b + c d, rounded as the compiler rounds them in the kernels above
+__device__ __forceinline__ float acc_sub(float a, float b, float c, float d) { return fmaf(a, b, -__fmul_rn(c, d)); }
+__device__ __forceinline__ float acc_add(float a, float b, float c, float d) { return fmaf(c, d, __fmul_rn(a, b)); }
+
+template <int MB, bool REV>
+__global__ void __launch_bounds__(kAccPoints) bloch_accum_both_kernel(const AccBoth a) {
+    extern __shared__ __align__(16) unsigned char bloch_smem[];
+    float2 *ring = reinterpret_cast<float2 *>(bloch_smem);  // kAccStages x MB x kAccPoints
+    __shared__ uint64_t full[kAccStages];
+    __shared__ float s_cq[MB];
+    const int tid = threadIdx.x, n_orb = a.n_orb;
+    const long long N = a.N, x0 = (long long)blockIdx.x * kAccPoints, x = x0 + tid;
+    const bool in = x < N;
+    const int v_lo = (int)(a.r0 / n_orb), v_hi = (int)((a.r1 - 1) / n_orb);
+    if (tid == 0) {
+        for (int i = 0; i < kAccStages; ++i) ptx::mbar_init(&full[i], 1);
+        ptx::fence_mbar_init();
+    }
+    if (tid < n_orb) s_cq[tid] = (float)(a.wq * (a.occ_q ? a.occ_q[tid] : 1.0));
+    __syncthreads();
+    // the chunk holds bands [m0, m1) of vector v
+    auto lo = [&](int v) { return (int)max(0LL, a.r0 - (long long)v * n_orb); };
+    auto hi = [&](int v) { return (int)min((long long)n_orb, a.r1 - (long long)v * n_orb); };
+    auto fill = [&](int v) {
+        const int st = (v - v_lo) % kAccStages, m0 = lo(v), m1 = hi(v);
+        const uint32_t bytes = (uint32_t)min((long long)kAccPoints, N - x0) * 8;  // a multiple of 16
+        ptx::mbar_arrive_expect_tx(&full[st], bytes * (uint32_t)(m1 - m0));
+        for (int m = m0; m < m1; ++m)
+            ptx::bulk_load(ring + (st * MB + m) * kAccPoints, a.X + ((long long)v * n_orb + m - a.r0) * N + x0, bytes,
+                           &full[st]);
+    };
+    if (tid == 0)
+        for (int v = v_lo; v <= v_hi && v < v_lo + kAccStages; ++v) fill(v);
+    float2 p[MB], rev[REV ? MB : 1];
+#pragma unroll
+    for (int m = 0; m < MB; ++m) p[m] = m < n_orb && in ? a.P[m * N + x] : make_float2(0.f, 0.f);
+    if (REV)
+#pragma unroll
+        for (int m = 0; m < MB; ++m) rev[m] = make_float2(0.f, 0.f);
+    // a vector's own loads a step ahead
+    double2 o_next = make_double2(0.0, 0.0);
+    float2 f_next = make_float2(0.f, 0.f);
+    double w_next = 1.0;
+    auto next = [&](int v) {
+        if (in) o_next = a.out_k[v * N + x];
+        if (REV) {
+            if (in) f_next = a.F[v * N + x];
+            if (a.occ_k) w_next = a.occ_k[v];
+        }
+    };
+    next(v_lo);
+    if (REV && in && (tid & 7) == 0)  // the reversed outputs into L2 (a 128-byte line per 8 points)
+        for (int m = 0; m < n_orb; ++m) ptx::prefetch_l2(a.out_q + m * N + x);
+    for (int v = v_lo; v <= v_hi; ++v) {
+        const int i = v - v_lo, m0 = lo(v), m1 = hi(v);
+        double2 o = o_next;
+        const float2 f = f_next;
+        const float ck = REV ? (float)(a.wk * w_next) : 0.f;
+        if (v < v_hi) next(v + 1);
+        const bool ok = ptx::mbar_wait_bounded(&full[i % kAccStages], (uint32_t)((i / kAccStages) & 1), 2000000000LL);
+        if (ok) {
+            const float2 *xs = ring + (i % kAccStages) * MB * kAccPoints + tid;
+            float sr = 0.f, si = 0.f;
+#pragma unroll
+            for (int m = 0; m < MB; ++m) {
+                if (m < m0 || m >= m1) continue;
+                const float2 xx = xs[m * kAccPoints], y = p[m];
+                sr = fmaf(s_cq[m], acc_sub(y.x, xx.x, y.y, xx.y), sr);  // P X
+                si = fmaf(s_cq[m], acc_add(y.x, xx.y, y.y, xx.x), si);
+                if (REV) {  // F conj(X)
+                    float2 &t = rev[REV ? m : 0];
+                    t.x = fmaf(ck, acc_add(f.y, xx.y, f.x, xx.x), t.x);
+                    t.y = fmaf(ck, acc_sub(f.y, xx.x, f.x, xx.y), t.y);
+                }
+            }
+            o.x -= f32_to_f64(sr);
+            o.y -= f32_to_f64(si);
+            if (in) a.out_k[v * N + x] = o;
+        } else {
+            atomicExch(a.status, KX_ERR_TIMEOUT);
+        }
+        if (__syncthreads_or(!ok)) break;  // every thread is done with this stage, or a wait gave up
+        if (tid == 0 && v + kAccStages <= v_hi) fill(v + kAccStages);
+    }
+    if constexpr (REV) {
+#pragma unroll
+        for (int g = 0; g < MB; g += 4) {
+            double2 o[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (g + u < n_orb && in) o[u] = a.out_q[(g + u) * N + x];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                if (g + u >= n_orb || !in) continue;
+                o[u].x -= f32_to_f64(rev[g + u].x);
+                o[u].y -= f32_to_f64(rev[g + u].y);
+                a.out_q[(g + u) * N + x] = o[u];
+            }
+        }
+    }
+}
+
+template <int MB>
+int launch_accum_both(const AccBoth &a, cudaStream_t s) {
+    const int smem = kAccStages * MB * kAccPoints * (int)sizeof(float2);
+    static bool attr = false;  // once per instantiation
+    if (!attr) {
+        KX_CUDA_TRY(cudaFuncSetAttribute(bloch_accum_both_kernel<MB, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         smem));
+        KX_CUDA_TRY(cudaFuncSetAttribute(bloch_accum_both_kernel<MB, false>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+        attr = true;
+    }
+    const unsigned blocks = (unsigned)((a.N + kAccPoints - 1) / kAccPoints);
+    if (a.out_q) bloch_accum_both_kernel<MB, true><<<blocks, kAccPoints, smem, s>>>(a);
+    else bloch_accum_both_kernel<MB, false><<<blocks, kAccPoints, smem, s>>>(a);
+    KX_LAUNCH_CHECK("bloch_accum_both_kernel launch");
+    return KX_OK;
 }
 
 // partial[k * nb + b] = w_k sum_n g_kn sum_x Re(conj(psi_kn[x]) vx_kn[x]) over a
@@ -2444,30 +2601,46 @@ int bloch_sweep(kx_plan *p, int n_kpt, const double *theta, const double *wk, in
                 if ((rc = launch_pipe<T, 0>(p, 0, R, A, B, Mi[0], nullptr, s))) return rc;
             }
             if ((rc = prof_begin(p, PK_BLOCH_OTHER, s))) return rc;
-            const long long nv = (r1 - 1) / n_orb - r0 / n_orb + 1;
-            // float32 sums with an even N: two points per thread (16-byte loads)
-            const bool pairs2 = sizeof(T) == 4 && N % 2 == 0;
-            const long long per = pairs2 ? 2 : 1;
-            const int ab = (int)std::min<long long>((nv * N / per + 255) / 256, 8LL * p->num_sms);
+            // float32 sums of up to 24 bands, even N (16-byte copies): both in one pass; more bands would
+            // not fit the registers
+            double2 *out_q = reverse ? reinterpret_cast<double2 *>(out_all) + (size_t)q * n_orb * N : nullptr;
+            const bool both = sizeof(T) == 4 && n_orb <= 24 && N % 2 == 0;
             if constexpr (sizeof(T) == 4) {
-                if (pairs2)
-                    bloch_accum2_kernel<false><<<ab, 256, 0, s>>>(X, r0, r1, n_orb, Pq, occ_q, wk[q],
-                                                                  reinterpret_cast<double2 *>(out_k), N);
+                if (both) {
+                    const AccBoth acc = {X,     Pq, F, r0, r1, N, n_orb, occ_q, occ_k, wk[q], wk[k], reinterpret_cast<double2 *>(out_k),
+                                         out_q, p->d_status};
+                    rc = n_orb <= 4    ? launch_accum_both<4>(acc, s)
+                         : n_orb <= 8  ? launch_accum_both<8>(acc, s)
+                         : n_orb <= 16 ? launch_accum_both<16>(acc, s)
+                                       : launch_accum_both<24>(acc, s);
+                    if (rc) return rc;
+                }
             }
-            if (!pairs2)
-                bloch_accum_kernel<T><<<ab, 256, 0, s>>>(X, r0, r1, n_orb, Pq, occ_q, wk[q],
-                                                         reinterpret_cast<double2 *>(out_k), N);
-            KX_LAUNCH_CHECK("bloch_accum_kernel launch");
-            if (reverse) {
-                const int rb = (int)std::min<long long>((n_orb * N / per + 255) / 256, 8LL * p->num_sms);
-                double2 *out_q = reinterpret_cast<double2 *>(out_all) + (size_t)q * n_orb * N;
+            if (!both) {
+                const long long nv = (r1 - 1) / n_orb - r0 / n_orb + 1;
+                // float32 sums with an even N: two points per thread (16-byte loads)
+                const bool pairs2 = sizeof(T) == 4 && N % 2 == 0;
+                const long long per = pairs2 ? 2 : 1;
+                const int ab = (int)std::min<long long>((nv * N / per + 255) / 256, 8LL * p->num_sms);
                 if constexpr (sizeof(T) == 4) {
                     if (pairs2)
-                        bloch_accum2_kernel<true><<<rb, 256, 0, s>>>(X, r0, r1, n_orb, F, occ_k, wk[k], out_q, N);
+                        bloch_accum2_kernel<false><<<ab, 256, 0, s>>>(X, r0, r1, n_orb, Pq, occ_q, wk[q],
+                                                                      reinterpret_cast<double2 *>(out_k), N);
                 }
                 if (!pairs2)
-                    bloch_accum_rev_kernel<T><<<rb, 256, 0, s>>>(X, r0, r1, n_orb, F, occ_k, wk[k], out_q, N);
-                KX_LAUNCH_CHECK("bloch_accum_rev_kernel launch");
+                    bloch_accum_kernel<T><<<ab, 256, 0, s>>>(X, r0, r1, n_orb, Pq, occ_q, wk[q],
+                                                             reinterpret_cast<double2 *>(out_k), N);
+                KX_LAUNCH_CHECK("bloch_accum_kernel launch");
+                if (reverse) {
+                    const int rb = (int)std::min<long long>((n_orb * N / per + 255) / 256, 8LL * p->num_sms);
+                    if constexpr (sizeof(T) == 4) {
+                        if (pairs2)
+                            bloch_accum2_kernel<true><<<rb, 256, 0, s>>>(X, r0, r1, n_orb, F, occ_k, wk[k], out_q, N);
+                    }
+                    if (!pairs2)
+                        bloch_accum_rev_kernel<T><<<rb, 256, 0, s>>>(X, r0, r1, n_orb, F, occ_k, wk[k], out_q, N);
+                    KX_LAUNCH_CHECK("bloch_accum_rev_kernel launch");
+                }
             }
             if ((rc = prof_end(p, s))) return rc;
         }

@@ -1126,6 +1126,30 @@ def test_kpoint_fused_products(kx, n3, bc, n_orb, counts, chunk, monkeypatch):
     assert relmax(out["1"], out["0"]) < TOL_K[prec][0]
 
 
+@pytest.mark.parametrize("n,n_orb,chunk,prec", [
+    ((16, 8, 8), 1, None, 1), ((16, 8, 8), 4, "3", 1), ((8, 8, 16), 5, "7", 1),  # bands per thread of 4 and 8
+    ((8, 16, 8), 9, "20", 1), ((16, 8, 8), 16, None, 1), ((16, 16, 8), 17, "50", 1),  # of 16 and 24
+    ((16, 8, 16), 24, None, 1), ((16, 8, 16), 25, None, 1),  # the largest, and beyond it the two-pass sums
+    ((12, 10, 9), 6, "11", 2),  # points not a multiple of a block's
+])
+def test_kpoint_sums_of_both_directions(kx, n, n_orb, chunk, prec, monkeypatch):
+    """The sums over a chunk read forward and reversed in one pass, over the band counts a
+    thread holds, with chunks that split a vector's bands."""
+    sysd = system(n, (0.4, 0.45, 0.5), (P, P, P), S, n_orb, 390 + n_orb)
+    theta, wk = workloads.kpoint_grid(sysd, (2, 1, 1))
+    psi = workloads.make_bloch_orbitals(sysd, theta)
+    occ = np.random.default_rng(n_orb).uniform(0.3, 1.0, (len(wk), n_orb))
+    vx_ref, ex_ref = oracle.vx_kpoints(oracle.Plan(sysd.n, sysd.h, sysd.bc, sysd.kernel), theta, wk, psi, occ)
+    plan = kx.Plan(sysd.n, sysd.h, sysd.bc, sysd.kernel, precision=prec)
+    if chunk:
+        monkeypatch.setenv("KX_CHUNK_PAIRS", chunk)
+    vx, ex = kx.kx_vx_kpoints(plan, theta, wk, to_dev_orbitals(psi), dev(occ))
+    torch.cuda.synchronize()
+    assert plan.status() == kx.KX_OK
+    assert relmax(vx.cpu().numpy().transpose(0, 2, 1), vx_ref) < TOL_K[1][0]
+    assert abs(ex.item() - ex_ref) < TOL_K[1][1] * abs(ex_ref)
+
+
 @pytest.mark.parametrize("prec", [0, 1])
 def test_kpoint_apply_to_vectors_in_chunks(kx, prec, monkeypatch):
     """Vx at one k-point on arbitrary complex vectors, with chunks of 4 pairs that
