@@ -50,20 +50,25 @@ template <typename T2> __device__ __forceinline__ T2 cmul_conj(T2 a, T2 b) {  //
     return r;
 }
 
-// res[j][u] = sum_k Ms[k][w + 8u] Ts[k][l + 32j] for the warp w and lane l of
-// the calling thread (operand padded to NCP = 8U columns).  float32: two packed
+// A warp's U operand columns lie next to each other, an even number of places apart from
+// the next warp's, so that a broadcast load takes two of them.
+__host__ __device__ constexpr int padded_outputs(int U) { return (U + 1) / 2 * 2; }
+
+// res[j][u] = sum_k Ms[k][w UP + u] Ts[k][l + 32j] for the warp w and lane l of
+// the calling thread (operand padded to NCP = 8 UP columns).  float32: two packed
 // accumulators per output, (sum a_re v, sum a_im v), combined at the end.
 template <typename T, int PQ, int U>
 __device__ __forceinline__ void tile_products(const typename Cx<T>::t *Ts, const typename Cx<T>::t *Ms, int ld,
                                               int n, int lane, int warp, typename Cx<T>::t (&res)[PQ][U]) {
-    constexpr int NCP = 8 * U;
+    constexpr int UP = padded_outputs(U), NCP = 8 * UP;
     if constexpr (sizeof(T) == 4) {
         float2 accA[PQ][U], accB[PQ][U];
 #pragma unroll
         for (int j = 0; j < PQ; ++j)
 #pragma unroll
             for (int u = 0; u < U; ++u) accA[j][u] = accB[j][u] = make_float2(0.f, 0.f);
-        const float2 *mcol = Ms + warp;
+        // a warp's operand columns are neighbours: two of them per (broadcast) load
+        const float2 *mcol = Ms + warp * UP;
         const float2 *tcol = Ts + lane;
 #pragma unroll 2
         for (int k = 0; k < n; ++k) {
@@ -75,13 +80,16 @@ __device__ __forceinline__ void tile_products(const typename Cx<T>::t *Ts, const
                 ai[j] = make_float2(a.y, a.y);
             }
 #pragma unroll
-            for (int u = 0; u < U; ++u) {
-                const float2 v = mcol[k * NCP + 8 * u];
+            for (int u = 0; u < U; u += 2) {
+                const float4 v2 = *reinterpret_cast<const float4 *>(mcol + k * NCP + u);
+                const float2 v[2] = {make_float2(v2.x, v2.y), make_float2(v2.z, v2.w)};
 #pragma unroll
-                for (int j = 0; j < PQ; ++j) {
-                    fma2(accA[j][u], ar[j], v);
-                    fma2(accB[j][u], ai[j], v);
-                }
+                for (int e = 0; e < 2 && u + e < U; ++e)
+#pragma unroll
+                    for (int j = 0; j < PQ; ++j) {
+                        fma2(accA[j][u + e], ar[j], v[e]);
+                        fma2(accB[j][u + e], ai[j], v[e]);
+                    }
             }
         }
 #pragma unroll
@@ -100,7 +108,7 @@ __device__ __forceinline__ void tile_products(const typename Cx<T>::t *Ts, const
                 const double2 a = Ts[k * ld + lane + 32 * j];
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
-                    const double2 v = Ms[k * NCP + warp + 8 * u];
+                    const double2 v = Ms[k * NCP + warp * UP + u];
                     res[j][u].x = fma(a.x, v.x, fma(-a.y, v.y, res[j][u].x));
                     res[j][u].y = fma(a.x, v.y, fma(a.y, v.x, res[j][u].y));
                 }
@@ -110,16 +118,17 @@ __device__ __forceinline__ void tile_products(const typename Cx<T>::t *Ts, const
 }
 
 // Stage the output columns [c0, c0 + ncy) of the operand (n x n, M[k][c]) with
-// zero padding up to NCP = 8U columns.
+// zero padding up to NCP = 8 UP columns.
 template <typename T, int U>
 __device__ __forceinline__ void stage_operand(typename Cx<T>::t *Ms, const typename Cx<T>::t *__restrict__ M, int n,
                                               int c0, int ncy, int lane, int warp) {
-    constexpr int NCP = 8 * U;
+    constexpr int UP = padded_outputs(U), NCP = 8 * UP;
     for (int k = warp; k < n; k += kBWarps)
-        for (int cl = lane; cl < NCP; cl += 32) {
+        for (int i = lane; i < NCP; i += 32) {
             typename Cx<T>::t z;
             z.x = z.y = (T)0;
-            Ms[k * NCP + cl] = cl < ncy ? M[(size_t)k * n + c0 + cl] : z;
+            const int u = i % UP, cl = i / UP * U + u;
+            Ms[k * NCP + i] = u < U && cl < ncy ? M[(size_t)k * n + c0 + cl] : z;
         }
 }
 
@@ -127,8 +136,7 @@ __device__ __forceinline__ void stage_operand(typename Cx<T>::t *Ms, const typen
 // items, out[r][x2, x3][c] = sum_k M[k][c] rho_r[x2, x3][k], where item r is the
 // pair (v, m) = divmod(r0 + r, n_orb) and rho_r = conj(P_m) F_v is formed while
 // the tile is loaded.  Pencils q (N / n per item), QB = 32 PQ of them per CTA;
-// warp w owns the output columns c0 + w + 8u (u < U, operand zero-padded to
-// 8U columns), lane l the pencils l + 32j (j < PQ).  Chunk-relative indices
+// warp w owns the output columns c0 + w U + u (u < U, operand zero-padded), lane l the pencils l + 32j (j < PQ).  Chunk-relative indices
 // stay below 2^31 and pair indices below 2^24 (checked at launch and entry).
 template <typename T, int U>
 __global__ void __launch_bounds__(kBThreads) bloch_form_kernel(
@@ -138,7 +146,7 @@ __global__ void __launch_bounds__(kBThreads) bloch_form_kernel(
     using T2 = typename Cx<T>::t;
     constexpr int PQ = pencils_per_thread<T>();
     constexpr int QB = 32 * PQ;
-    constexpr int NCP = 8 * U;
+    constexpr int NCP = 8 * padded_outputs(U);
     extern __shared__ __align__(16) unsigned char bloch_smem[];
     T2 *Ms = reinterpret_cast<T2 *>(bloch_smem);  // n x NCP
     T2 *Ts = Ms + (size_t)n * NCP;                // n x (QB + 1): Ts[k * ld + ql]
@@ -173,7 +181,7 @@ __global__ void __launch_bounds__(kBThreads) bloch_form_kernel(
         if (ql >= nq) continue;
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            const int cl = warp + 8 * u;
+            const int cl = warp * U + u;
             if (cl < ncy) Ts[cl * ld + ql] = res[j][u];
         }
     }
@@ -208,7 +216,7 @@ __global__ void __launch_bounds__(kBThreads) bloch_mode_pipe_kernel(
     using T2 = typename Cx<T>::t;
     constexpr int PQ = pencils_per_thread<T>();
     constexpr int QB = 32 * PQ;
-    constexpr int NCP = 8 * U;
+    constexpr int NCP = 8 * padded_outputs(U);
     extern __shared__ __align__(16) unsigned char bloch_smem[];
     T2 *Ms = reinterpret_cast<T2 *>(bloch_smem);  // n x NCP
     const int ld = QB + 1;
@@ -282,7 +290,7 @@ __global__ void __launch_bounds__(kBThreads) bloch_mode_pipe_kernel(
             T ej = 0;
 #pragma unroll
             for (int u = 0; u < U; ++u) {
-                const int cl = warp + 8 * u;
+                const int cl = warp * U + u;
                 if (cl < ncy) {
                     T2 v = res[j][u];
                     if constexpr (EPI == 1) {
@@ -2022,14 +2030,14 @@ inline size_t al256(size_t b) { return (b + 255) / 256 * 256; }
 template <typename T> int outputs_for(int nc) {
     const int need = (nc + kBWarps - 1) / kBWarps;
     if (sizeof(T) == 8) return need <= 2 ? 2 : (need <= 4 ? 4 : 8);
-    return need <= 2 ? 2 : need <= 4 ? 4 : need <= 6 ? 6 : need <= 8 ? 8 : need <= 12 ? 12 : 16;
+    return need <= 2 ? 2 : need <= 8 ? need : need <= 10 ? 10 : need <= 12 ? 12 : 16;
 }
 
 template <typename T>
 void choose_split(int n, int *nc, int *n_split, int *U, size_t *smem) {
     using T2 = typename Cx<T>::t;
     const int max_cols = kBWarps * (sizeof(T) == 4 ? 16 : 8);
-    auto bytes = [n](int u) { return sizeof(T2) * ((size_t)n * 8 * u + (size_t)n * (tile_pencils<T>() + 1)); };
+    auto bytes = [n](int u) { return sizeof(T2) * ((size_t)n * 8 * padded_outputs(u) + (size_t)n * (tile_pencils<T>() + 1)); };
     int c = std::min(n, max_cols);
     while (bytes(outputs_for<T>(c)) > kBSmemTarget && c > kBWarps) c = (c + 1) / 2;
     *nc = c;
@@ -2076,7 +2084,11 @@ int launch_form(kx_plan *p, long long R, typename Cx<T>::t *out, const typename 
     else if (U == 4) rc = KX_BLOCH_FORM(4);
     else if (U == 8) rc = KX_BLOCH_FORM(8);
     else if constexpr (sizeof(T) == 4) {
-        if (U == 6) rc = KX_BLOCH_FORM(6);
+        if (U == 3) rc = KX_BLOCH_FORM(3);
+        else if (U == 5) rc = KX_BLOCH_FORM(5);
+        else if (U == 6) rc = KX_BLOCH_FORM(6);
+        else if (U == 7) rc = KX_BLOCH_FORM(7);
+        else if (U == 10) rc = KX_BLOCH_FORM(10);
         else if (U == 12) rc = KX_BLOCH_FORM(12);
         else rc = KX_BLOCH_FORM(16);
     } else {
@@ -2093,7 +2105,7 @@ template <typename T>
 void choose_split_pipe(int n, int *nc, int *n_split, int *U, size_t *smem) {
     using T2 = typename Cx<T>::t;
     const int max_cols = kBWarps * (sizeof(T) == 4 ? 16 : 8);
-    auto bytes = [n](int u) { return sizeof(T2) * ((size_t)n * 8 * u + 2 * (size_t)n * (tile_pencils<T>() + 1)); };
+    auto bytes = [n](int u) { return sizeof(T2) * ((size_t)n * 8 * padded_outputs(u) + 2 * (size_t)n * (tile_pencils<T>() + 1)); };
     int c = std::min(n, max_cols);
     while (bytes(outputs_for<T>(c)) > kBSmemPipeMax && c > kBWarps) c = (c + 1) / 2;
     *nc = c;
@@ -2147,7 +2159,11 @@ int launch_pipe(kx_plan *p, int axis, long long R, const typename Cx<T>::t *in, 
     else if (U == 4) rc = KX_BLOCH_PIPE(4);
     else if (U == 8) rc = KX_BLOCH_PIPE(8);
     else if constexpr (sizeof(T) == 4) {
-        if (U == 6) rc = KX_BLOCH_PIPE(6);
+        if (U == 3) rc = KX_BLOCH_PIPE(3);
+        else if (U == 5) rc = KX_BLOCH_PIPE(5);
+        else if (U == 6) rc = KX_BLOCH_PIPE(6);
+        else if (U == 7) rc = KX_BLOCH_PIPE(7);
+        else if (U == 10) rc = KX_BLOCH_PIPE(10);
         else if (U == 12) rc = KX_BLOCH_PIPE(12);
         else rc = KX_BLOCH_PIPE(16);
     } else {
