@@ -271,61 +271,49 @@ __global__ void __launch_bounds__(kBThreads) bloch_mode_pipe_kernel(
         const int nq = min(QB, n_cols - q0);
         T2 res[PQ][U];
         tile_products<T, PQ, U>(cur, Ms, ld, n, lane, warp, res);
-        __syncthreads();
+        __syncthreads();  // cur is free (and the buffer the next iteration copies into was, before)
 #pragma unroll
         for (int j = 0; j < PQ; ++j) {
             const int ql = lane + 32 * j;
             if (ql >= nq) continue;
-            int i_in = 0;
+            const int q = q0 + ql, o = q / inner, i_in = q - o * inner;
             double wj = 0.0;
-            if constexpr (EPI != 0) {
-                const int item = (q0 + ql) / inner;
-                i_in = (q0 + ql) - item * inner;
-                if constexpr (EPI == 2) {
-                    const long long rr = ea.r0 + item;
-                    const long long vv = rr / ea.n_orb, mm = rr - vv * ea.n_orb;
-                    wj = ea.cb * (ea.occ_q ? ea.occ_q[mm] : 1.0) * (ea.occ_k ? ea.occ_k[vv] : 1.0);
-                }
+            if constexpr (EPI == 2) {
+                const long long rr = ea.r0 + o;
+                const long long vv = rr / ea.n_orb, mm = rr - vv * ea.n_orb;
+                wj = ea.cb * (ea.occ_q ? ea.occ_q[mm] : 1.0) * (ea.occ_k ? ea.occ_k[vv] : 1.0);
             }
             T ej = 0;
+            // strided pencils: neighbours in neighbouring lanes, stored as they are
+            T2 *dst = out + (size_t)o * n * inner + i_in;
 #pragma unroll
             for (int u = 0; u < U; ++u) {
                 const int cl = warp * U + u;
                 if (cl < ncy) {
                     T2 v = res[j][u];
-                    if constexpr (EPI == 1) {
+                    if constexpr (EPI != 0) {
                         const T fv = f[(size_t)(c0 + cl) * inner + i_in];
-                        v.x *= fv;
-                        v.y *= fv;
+                        if constexpr (EPI == 1) {
+                            v.x *= fv;
+                            v.y *= fv;
+                        } else {
+                            ej = fma(fv, v.x * v.x + v.y * v.y, ej);
+                        }
                     }
-                    if constexpr (EPI == 2) {
-                        const T fv = f[(size_t)(c0 + cl) * inner + i_in];
-                        ej = fma(fv, v.x * v.x + v.y * v.y, ej);
-                    } else {
-                        cur[cl * ld + ql] = v;
+                    if constexpr (EPI != 2) {
+                        if (inner == 1) cur[cl * ld + ql] = v;
+                        else dst[(size_t)(c0 + cl) * inner] = v;
                     }
                 }
             }
             if constexpr (EPI == 2) e_acc += wj * (double)ej;
         }
+        if (EPI == 2 || inner != 1) continue;
+        // contiguous pencils through shared memory
         __syncthreads();
-        if constexpr (EPI == 2) continue;  // no output
-        if (inner == 1) {
-            for (int ql = warp; ql < nq; ql += kBWarps) {
-                T2 *dst = out + (size_t)(q0 + ql) * n + c0;
-                for (int cl = lane; cl < ncy; cl += 32) dst[cl] = cur[cl * ld + ql];
-            }
-        } else {
-#pragma unroll
-            for (int j = 0; j < PQ; ++j) {
-                const int ql = lane + 32 * j;
-                if (ql < nq) {
-                    const int q = q0 + ql;
-                    const int o = q / inner;
-                    T2 *dst = out + (size_t)o * n * inner + (q - o * inner);
-                    for (int cl = warp; cl < ncy; cl += kBWarps) dst[(size_t)(c0 + cl) * inner] = cur[cl * ld + ql];
-                }
-            }
+        for (int ql = warp; ql < nq; ql += kBWarps) {
+            T2 *dst = out + (size_t)(q0 + ql) * n + c0;
+            for (int cl = lane; cl < ncy; cl += 32) dst[cl] = cur[cl * ld + ql];
         }
         __syncthreads();
     }
