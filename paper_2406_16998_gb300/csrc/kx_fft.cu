@@ -16,15 +16,27 @@
 // stages are spread over the CTA's threads (lines x butterflies); lines of 80
 // points instead take a four-step transform (16 x 5) held in registers.
 #include "kx_internal.h"
+#include "kx_conv.cuh"
 
 #include <cmath>
+#include <type_traits>
 #include <vector>
 
 namespace kx {
 namespace {
 
-constexpr int kFftLine = 32;  // lines per CTA in pass B (40 KB of shared memory at n3 = 80: 5 CTAs per SM)
+// What bounds the passes is instruction issue and the barriers between their phases, not
+// memory (588 pairs at 80^3, passes A, B, C: 1588, 1042, 1202 us; floors 89, 178 and
+// 177 us): hence lines fixed per thread in pass B (885 us, 768 with five CTAs per SM),
+// neighbouring values loaded and stored together, packed sums, and planes in place
+// (A 1480 -> 1261 us, with the paired loads 862; C 1034 -> 824 us).
+constexpr int kFftLine = 32;  // lines per CTA in pass B (five CTAs per SM)
+constexpr int kFftLineThreads = 256;  // a warp's lanes are the lines
 constexpr int kFftPlaneThreads = 512;  // passes A and C: two planes (2 x 104 KB at 80^2) and 32 warps per SM
+
+// planes transformed in place: one buffer (52 KB at 80^2), four CTAs per SM whose barriers
+// fall apart
+constexpr int kFftInPlaceThreads = 256;
 
 struct FftAxis {
     int n, nr;
@@ -48,6 +60,12 @@ __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
 __device__ __forceinline__ unsigned fast_div(unsigned x, unsigned m) { return m ? __umulhi(x, m) : x; }
 __device__ __forceinline__ unsigned div_magic(unsigned d) { return d > 1 ? 0xFFFFFFFFu / d + 1u : 0u; }
 
+// Complex sums in one packed instruction (the transforms are bound by instruction issue).
+__device__ __forceinline__ float2 csub(float2 a, float2 b) {
+    fma2(a, b, make_float2(-1.f, -1.f));
+    return a;
+}
+
 // u = DFT_R(v) with W the twiddle table of the line (exp(-2 pi i t / n)),
 // nR = n / R; sg = -1 conjugates (inverse).  Radix 2 and 4 by additions and
 // multiplications by +-i, radix 3 and 5 from the table.
@@ -55,17 +73,15 @@ template <int R>
 __device__ __forceinline__ void dft_small(float2 *v, const float2 *W, int nR, float sg) {
     if (R == 2) {
         const float2 a = v[0], b = v[1];
-        v[0] = make_float2(a.x + b.x, a.y + b.y);
-        v[1] = make_float2(a.x - b.x, a.y - b.y);
+        v[0] = add2(a, b);
+        v[1] = csub(a, b);
     } else if (R == 4) {
         // (-i sg) (x, y) = (sg y, -sg x)
-        const float2 a = make_float2(v[0].x + v[2].x, v[0].y + v[2].y);
-        const float2 b = make_float2(v[0].x - v[2].x, v[0].y - v[2].y);
-        const float2 c = make_float2(v[1].x + v[3].x, v[1].y + v[3].y);
-        const float2 t = make_float2(v[1].x - v[3].x, v[1].y - v[3].y);
+        const float2 a = add2(v[0], v[2]), b = csub(v[0], v[2]);
+        const float2 c = add2(v[1], v[3]), t = csub(v[1], v[3]);
         const float2 d = make_float2(sg * t.y, -sg * t.x);
-        v[0] = make_float2(a.x + c.x, a.y + c.y);
-        v[2] = make_float2(a.x - c.x, a.y - c.y);
+        v[0] = add2(a, c);
+        v[2] = csub(a, c);
         v[1] = make_float2(b.x + d.x, b.y + d.y);
         v[3] = make_float2(b.x - d.x, b.y - d.y);
     } else {
@@ -89,18 +105,22 @@ __device__ __forceinline__ void dft_small(float2 *v, const float2 *W, int nR, fl
 
 // One Stockham stage of radix R over nl lines at once, spread over the CTA:
 // line l's element k sits at a[l * lstride + k * st] (scratch b, same
-// layout).  lines_fast picks the task order: consecutive threads take
+// layout; nl, lstride and st at compile time where NL, LS and ST are not 0).  lines_fast picks the task order: consecutive threads take
 // consecutive lines (element stride st > 1: neighbouring lines are adjacent)
 // or consecutive butterflies of one line (st == 1).
-template <int R>
+template <int R, int NL, int LS, int ST>
 __device__ __forceinline__ void fft_stage(const float2 *a, float2 *b, int n, int Ns, int nl, int lstride, int st,
-                                          bool lines_fast, const float2 *W, float sg) {
+                                          const float2 *W, float sg) {
+    constexpr bool lines_fast = ST != 1;
+    if (NL) nl = NL;
+    if (LS) lstride = LS;
+    if (ST) st = ST;
     const int nR = n / R, tstep = n / (Ns * R);
     const unsigned m_fast = div_magic(lines_fast ? nl : nR), m_ns = div_magic(Ns);
     for (int task = threadIdx.x; task < nl * nR; task += blockDim.x) {
         int l, j;
         if (lines_fast) {
-            j = (int)fast_div(task, m_fast);
+            j = NL ? task / max(NL, 1) : (int)fast_div(task, m_fast);
             l = task - j * nl;
         } else {
             l = (int)fast_div(task, m_fast);
@@ -137,13 +157,11 @@ __device__ __forceinline__ void fft_stage(const float2 *a, float2 *b, int n, int
 // W5 and W16 are the constants cos, sin of 2 pi k / 5 and 2 pi k / 16; W80
 // comes from the line's twiddle table.  sg = -1 conjugates (inverse).
 __device__ __forceinline__ void dft4_reg(float2 &v0, float2 &v1, float2 &v2, float2 &v3, float sg) {
-    const float2 a = make_float2(v0.x + v2.x, v0.y + v2.y);
-    const float2 b = make_float2(v0.x - v2.x, v0.y - v2.y);
-    const float2 c = make_float2(v1.x + v3.x, v1.y + v3.y);
-    const float2 t = make_float2(v1.x - v3.x, v1.y - v3.y);
+    const float2 a = add2(v0, v2), b = csub(v0, v2);
+    const float2 c = add2(v1, v3), t = csub(v1, v3);
     const float2 d = make_float2(sg * t.y, -sg * t.x);  // -i sg t
-    v0 = make_float2(a.x + c.x, a.y + c.y);
-    v2 = make_float2(a.x - c.x, a.y - c.y);
+    v0 = add2(a, c);
+    v2 = csub(a, c);
     v1 = make_float2(b.x + d.x, b.y + d.y);
     v3 = make_float2(b.x - d.x, b.y - d.y);
 }
@@ -151,17 +169,15 @@ __device__ __forceinline__ void dft4_reg(float2 &v0, float2 &v1, float2 &v2, flo
 __device__ __forceinline__ void dft5_reg(float2 *x, float sg) {
     constexpr float c1 = 0.30901699437494742f, c2 = -0.80901699437494742f;  // cos 2pi/5, cos 4pi/5
     constexpr float s1 = 0.95105651629515357f, s2 = 0.58778525229247313f;   // sin 2pi/5, sin 4pi/5
-    const float2 t1 = make_float2(x[1].x + x[4].x, x[1].y + x[4].y);
-    const float2 t2 = make_float2(x[2].x + x[3].x, x[2].y + x[3].y);
-    const float2 t3 = make_float2(x[1].x - x[4].x, x[1].y - x[4].y);
-    const float2 t4 = make_float2(x[2].x - x[3].x, x[2].y - x[3].y);
+    const float2 t1 = add2(x[1], x[4]), t2 = add2(x[2], x[3]);
+    const float2 t3 = csub(x[1], x[4]), t4 = csub(x[2], x[3]);
     const float2 a1 = make_float2(x[0].x + c1 * t1.x + c2 * t2.x, x[0].y + c1 * t1.y + c2 * t2.y);
     const float2 a2 = make_float2(x[0].x + c2 * t1.x + c1 * t2.x, x[0].y + c2 * t1.y + c1 * t2.y);
     const float2 b1 = make_float2(s1 * t3.x + s2 * t4.x, s1 * t3.y + s2 * t4.y);
     const float2 b2 = make_float2(s2 * t3.x - s1 * t4.x, s2 * t3.y - s1 * t4.y);
     const float2 m1 = make_float2(sg * b1.y, -sg * b1.x);  // -i sg b1
     const float2 m2 = make_float2(sg * b2.y, -sg * b2.x);
-    x[0] = make_float2(x[0].x + t1.x + t2.x, x[0].y + t1.y + t2.y);
+    x[0] = add2(add2(x[0], t1), t2);
     x[1] = make_float2(a1.x + m1.x, a1.y + m1.y);
     x[4] = make_float2(a1.x - m1.x, a1.y - m1.y);
     x[2] = make_float2(a2.x + m2.x, a2.y + m2.y);
@@ -204,62 +220,75 @@ __device__ __forceinline__ void dft16_reg(float2 *x, float sg) {
     for (int k = 0; k < 16; ++k) x[k] = y[k];
 }
 
-// 80-point transforms of nl lines (layout as in fft_stage), a -> b -> a; returns a.
-__device__ float2 *fft80_lines(float2 *a, float2 *b, int nl, int lstride, int st, const float2 *W, bool inv) {
+// 80-point transforms of nl lines (layout as in fft_stage), in place: phase 1 writes the
+// places it read, phase 2 (at most one task per thread) keeps its values in registers
+// over a barrier.  Every thread of the CTA must call it; it ends with a barrier.
+template <int NL, int LS, int ST>
+__device__ __forceinline__ void fft80_lines(float2 *a, int nl, int lstride, int st, const float2 *W, bool inv) {
+    if (NL) nl = NL;
+    if (LS) lstride = LS;
+    if (ST) st = ST;
     const float sg = inv ? -1.f : 1.f;
     const unsigned m_nl = div_magic(nl);
     for (int task = threadIdx.x; task < nl * 16; task += blockDim.x) {  // phase 1: (line, p)
-        const int p = (int)fast_div(task, m_nl), l = task - p * nl;
-        const float2 *al = a + l * lstride;
+        const int p = NL ? task / max(NL, 1) : (int)fast_div(task, m_nl), l = task - p * nl;
+        float2 *al = a + l * lstride + p * st;
         float2 x[5];
 #pragma unroll
-        for (int q = 0; q < 5; ++q) x[q] = al[(p + 16 * q) * st];
+        for (int q = 0; q < 5; ++q) x[q] = al[16 * q * st];
         dft5_reg(x, sg);
-        float2 *bl = b + l * lstride;
-        bl[p * st] = x[0];
+        al[0] = x[0];
 #pragma unroll
         for (int k5 = 1; k5 < 5; ++k5) {
             float2 w = W[p * k5];
             w.y *= sg;
-            bl[(16 * k5 + p) * st] = cmul(x[k5], w);
+            al[16 * k5 * st] = cmul(x[k5], w);
         }
     }
     __syncthreads();
-    for (int task = threadIdx.x; task < nl * 5; task += blockDim.x) {  // phase 2: (line, k5)
-        const int k5 = (int)fast_div(task, m_nl), l = task - k5 * nl;
-        const float2 *bl = b + l * lstride + 16 * k5 * st;
+    {  // phase 2: (line, k5)
+        const int task = threadIdx.x;
+        const int k5 = NL ? task / max(NL, 1) : (int)fast_div(task, m_nl), l = task - k5 * nl;
         float2 x[16];
+        if (task < nl * 5) {
+            const float2 *bl = a + l * lstride + 16 * k5 * st;
 #pragma unroll
-        for (int p = 0; p < 16; ++p) x[p] = bl[p * st];
-        dft16_reg(x, sg);
-        float2 *al = a + l * lstride;
+            for (int p = 0; p < 16; ++p) x[p] = bl[p * st];
+            dft16_reg(x, sg);
+        }
+        __syncthreads();
+        if (task < nl * 5) {
+            float2 *al = a + l * lstride + k5 * st;
 #pragma unroll
-        for (int k16 = 0; k16 < 16; ++k16) al[(k5 + 5 * k16) * st] = x[k16];
+            for (int k16 = 0; k16 < 16; ++k16) al[5 * k16 * st] = x[k16];
+        }
     }
     __syncthreads();
-    return a;
 }
 
 // Stockham FFT of nl lines (see fft_stage for the layout) by the whole CTA;
 // the inverse uses conjugate twiddles and is unnormalised.  Returns the buffer
 // that holds the result (a or b, by the number of stages).  Every thread of
 // the CTA must call it; it ends with a barrier.
-__device__ float2 *fft_lines(float2 *a, float2 *b, const FftAxis &ax, int nl, int lstride, int st, const float2 *W,
-                             bool inv) {
-    if (ax.n == 80) return fft80_lines(a, b, nl, lstride, st, W, inv);
+template <int NL, int LS, int ST>
+__device__ __forceinline__ float2 *fft_lines(float2 *a, float2 *b, const FftAxis &ax, int nl, int lstride, int st,
+                                             const float2 *W, bool inv) {
+    if (ax.n == 80) {
+        fft80_lines<NL, LS, ST>(a, nl, lstride, st, W, inv);
+        return a;
+    }
     const float sg = inv ? -1.f : 1.f;
-    const bool lines_fast = st != 1;
     int Ns = 1;
     for (int s = 0; s < ax.nr; ++s) {
         const int R = ax.radix[s];
         if (R == 4)
-            fft_stage<4>(a, b, ax.n, Ns, nl, lstride, st, lines_fast, W, sg);
+            fft_stage<4, NL, LS, ST>(a, b, ax.n, Ns, nl, lstride, st, W, sg);
         else if (R == 2)
-            fft_stage<2>(a, b, ax.n, Ns, nl, lstride, st, lines_fast, W, sg);
+            fft_stage<2, NL, LS, ST>(a, b, ax.n, Ns, nl, lstride, st, W, sg);
         else if (R == 3)
-            fft_stage<3>(a, b, ax.n, Ns, nl, lstride, st, lines_fast, W, sg);
+            fft_stage<3, NL, LS, ST>(a, b, ax.n, Ns, nl, lstride, st, W, sg);
         else
-            fft_stage<5>(a, b, ax.n, Ns, nl, lstride, st, lines_fast, W, sg);
+            fft_stage<5, NL, LS, ST>(a, b, ax.n, Ns, nl, lstride, st, W, sg);
         __syncthreads();
         float2 *t = a;
         a = b;
@@ -273,14 +302,23 @@ __device__ __forceinline__ void load_twiddles(const float2 *__restrict__ tw, flo
     for (int i = threadIdx.x; i < 3 * 128; i += blockDim.x) Ws[i] = tw[i];
 }
 
+template <int V> struct FftVec;
+template <> struct FftVec<1> { using t = float; };
+template <> struct FftVec<2> { using t = float2; };
+
 // Pass A: x3 plane blockIdx.x of item blockIdx.y; source psi_i psi_j (pairs) or src32.
-__global__ void __launch_bounds__(kFftPlaneThreads) fft_plane_fwd_kernel(const FftGeom G, const int2 *__restrict__ pairs,
+// IN_PLACE: one buffer (packed row j in row 2j), for planes both of whose axes take the
+// four-step transform.
+template <bool IN_PLACE>
+__global__ void __launch_bounds__(IN_PLACE ? kFftInPlaceThreads : kFftPlaneThreads, IN_PLACE ? 4 : 2)
+    fft_plane_fwd_kernel(const FftGeom G, const int2 *__restrict__ pairs,
                                                             const float *__restrict__ src32, int rhs,
                                                             float2 *__restrict__ C) {
     extern __shared__ float2 fsm[];
     __shared__ float2 Ws[3 * 128];
     const int ld = G.n1 + 1;  // padded rows
-    float2 *A = fsm, *B = fsm + (size_t)G.n2 * ld;
+    float2 *A = fsm, *B = IN_PLACE ? fsm : fsm + (size_t)G.n2 * ld;
+    const int lj = IN_PLACE ? 2 * ld : ld;  // between packed rows
     const int x3 = blockIdx.x;
     const long long item = blockIdx.y;
     const float *p0, *p1 = nullptr;
@@ -292,38 +330,56 @@ __global__ void __launch_bounds__(kFftPlaneThreads) fft_plane_fwd_kernel(const F
         p1 = src32 + (long long)ij.y * G.N + x3 * G.n12;
     }
     load_twiddles(G.tw, Ws);
-    const unsigned m_n1 = div_magic(G.n1);  // plane index e < 2^14: multiply-high division by n1
-    // four loads in flight per thread before their values are stored
-    for (int e0 = threadIdx.x; e0 < G.n12; e0 += 4 * blockDim.x) {
-        float v[4];
+    const int n2p = (G.n2 + 1) / 2;
+    // rows 2j and 2j + 1 as the real and imaginary parts of packed row j (an odd last row
+    // pairs with zeros), two neighbouring values at a time where n1 is even; the loads of
+    // two steps in flight per thread
+    auto fill = [&](auto vec) {
+        constexpr int V = decltype(vec)::value;
+        using T = typename FftVec<V>::t;
+        const int nv = G.n1 / V;
+        const unsigned m_nv = div_magic(nv);
+        for (int e0 = threadIdx.x; e0 < n2p * nv; e0 += 2 * blockDim.x) {
+            T q[2][4];
+            int at[2];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int e = e0 + u * blockDim.x;
-            v[u] = e < G.n12 ? (p1 ? __ldg(p0 + e) * __ldg(p1 + e) : __ldg(p0 + e)) : 0.f;
-        }
+            for (int u = 0; u < 2; ++u) {
+                const int e = e0 + u * blockDim.x;
+                const int j = (int)fast_div(e, m_nv), x1 = (e - j * nv) * V;
+                const int o = 2 * j * G.n1 + x1;
+                at[u] = e < n2p * nv ? j * lj + x1 : -1;
+                if (at[u] < 0) continue;
+                const bool two = 2 * j + 1 < G.n2;
+                q[u][0] = __ldg(reinterpret_cast<const T *>(p0 + o));
+                q[u][1] = two ? __ldg(reinterpret_cast<const T *>(p0 + o + G.n1)) : T{};
+                if (p1) {
+                    q[u][2] = __ldg(reinterpret_cast<const T *>(p1 + o));
+                    q[u][3] = two ? __ldg(reinterpret_cast<const T *>(p1 + o + G.n1)) : T{};
+                }
+            }
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int e = e0 + u * blockDim.x;
-            if (e >= G.n12) break;
-            const int x2 = (int)fast_div(e, m_n1), x1 = e - x2 * G.n1;
-            // rows 2j and 2j + 1 as the real and imaginary parts of packed row j
-            float *z = reinterpret_cast<float *>(A + (x2 >> 1) * ld + x1);
-            z[x2 & 1] = v[u];
-            if (x2 == G.n2 - 1 && (x2 & 1) == 0) z[1] = 0.f;  // an odd last row pairs with zeros
+            for (int u = 0; u < 2; ++u) {
+                if (at[u] < 0) continue;
+                const float *v = reinterpret_cast<const float *>(q[u]);
+#pragma unroll
+                for (int c = 0; c < V; ++c)
+                    A[at[u] + c] = p1 ? make_float2(v[c] * v[2 * V + c], v[V + c] * v[3 * V + c]) : make_float2(v[c], v[V + c]);
+            }
         }
-    }
+    };
+    if (G.n1 % 2 == 0) fill(std::integral_constant<int, 2>());
+    else fill(std::integral_constant<int, 1>());
     __syncthreads();
     // rows along x1: one complex transform per two real rows, Z = DFT(a + i b),
     // then A(k) = (Z(k) + conj Z(-k)) / 2 and B(k) = (Z(k) - conj Z(-k)) / 2i for
     // the kept columns k1 < h1 into the other buffer's rows 2j and 2j + 1
-    const int n2p = (G.n2 + 1) / 2;
-    float2 *Z = fft_lines(A, B, G.ax[0], n2p, ld, 1, Ws, false);
-    float2 *R1 = (Z == A) ? B : A;
+    float2 *Z = fft_lines<0, 0, 1>(A, B, G.ax[0], n2p, lj, 1, Ws, false);
+    float2 *R1 = IN_PLACE ? A : (Z == A) ? B : A;  // in place: only the thread itself reads what it overwrites
     {
         const unsigned m_h1 = div_magic(G.h1);
         for (int e = threadIdx.x; e < n2p * G.h1; e += blockDim.x) {
             const int j = (int)fast_div(e, m_h1), k = e - j * G.h1;
-            const float2 z = Z[j * ld + k], zc = Z[j * ld + (k == 0 ? 0 : G.n1 - k)];
+            const float2 z = Z[j * lj + k], zc = Z[j * lj + (k == 0 ? 0 : G.n1 - k)];
             R1[2 * j * ld + k] = make_float2(0.5f * (z.x + zc.x), 0.5f * (z.y - zc.y));
             if (2 * j + 1 < G.n2) R1[(2 * j + 1) * ld + k] = make_float2(0.5f * (z.y + zc.y), -0.5f * (z.x - zc.x));
         }
@@ -331,7 +387,7 @@ __global__ void __launch_bounds__(kFftPlaneThreads) fft_plane_fwd_kernel(const F
     __syncthreads();
     // columns along x2 for k1 < h1 only: the source is real, so its spectrum is
     // Hermitian and the columns k1 > n1 / 2 are conjugates of kept ones
-    const float2 *R2 = fft_lines(R1, Z, G.ax[1], G.h1, 1, ld, Ws + 128, false);
+    const float2 *R2 = fft_lines<0, 1, 0>(R1, Z, G.ax[1], G.h1, 1, ld, Ws + 128, false);
     float2 *dst = C + item * G.N + x3 * G.nh;  // [k2][k1 < h1]
     const unsigned m_h1 = div_magic(G.h1);
     for (int e = threadIdx.x; e < G.nh; e += blockDim.x) {
@@ -342,62 +398,64 @@ __global__ void __launch_bounds__(kFftPlaneThreads) fft_plane_fwd_kernel(const F
 
 // Pass B: kFftLine lines along x3 (plane positions blockIdx.x * kFftLine + l) of
 // item blockIdx.y: transform, f scaling, energy sum, inverse transform.
-__global__ void __launch_bounds__(256) fft_axis3_kernel(const FftGeom G, float2 *__restrict__ C,
+__global__ void __launch_bounds__(kFftLineThreads, 5) fft_axis3_kernel(const FftGeom G, float2 *__restrict__ C,
                                                         const float *__restrict__ ftab,
                                                         const int2 *__restrict__ pairs,
                                                         const double *__restrict__ occ, int rhs, int energy_only,
                                                         double *__restrict__ e_part) {
     extern __shared__ float2 fsm[];
     __shared__ float2 Ws[3 * 128];
-    __shared__ double red[8];
+    __shared__ double red[kFftLineThreads / 32];
     float2 *A = fsm, *B = fsm + (size_t)G.n3 * kFftLine;
     const int tid = threadIdx.x;
     const long long item = blockIdx.y;
     const long long p0 = (long long)blockIdx.x * kFftLine;
     float2 *col = C + item * G.N + p0;
     load_twiddles(G.tw, Ws);
-    for (int e0 = tid; e0 < G.n3 * kFftLine; e0 += 4 * blockDim.x) {  // e = x3 * kFftLine + l, four in flight
+    // a thread has one line (its lane) and every 8th point of it, so that what depends on
+    // the line is worked out once
+    static_assert(kFftLine == 32, "lanes are lines");
+    constexpr int NW = kFftLineThreads / 32;
+    const int l = tid & 31, wp = tid >> 5;
+    const bool in = p0 + l < G.nh;
+    for (int x0 = wp; x0 < G.n3; x0 += 4 * NW) {  // four loads in flight
         float2 v[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-            const int e = e0 + u * blockDim.x;
-            const int x3 = e / kFftLine, l = e % kFftLine;
-            v[u] = (e < G.n3 * kFftLine && p0 + l < G.nh) ? col[x3 * G.nh + l] : make_float2(0.f, 0.f);
+            const int x3 = x0 + u * NW;
+            v[u] = x3 < G.n3 && in ? col[x3 * G.nh + l] : make_float2(0.f, 0.f);
         }
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int e = e0 + u * blockDim.x;
-            if (e < G.n3 * kFftLine) A[e] = v[u];
-        }
+        for (int u = 0; u < 4; ++u)
+            if (x0 + u * NW < G.n3) A[(x0 + u * NW) * kFftLine + l] = v[u];
     }
     __syncthreads();
-    float2 *Rr = fft_lines(A, B, G.ax[2], kFftLine, 1, kFftLine, Ws + 256, false);
+    float2 *Rr = fft_lines<kFftLine, 1, kFftLine>(A, B, G.ax[2], kFftLine, 1, kFftLine, Ws + 256, false);
     float2 *Or = (Rr == A) ? B : A;
     // energy by Parseval over the half spectrum: the columns 0 < k1 < n1 / 2 stand
     // for themselves and their conjugates (weight 2), k1 = 0 and k1 = n1 / 2 once
-    float ef = 0.f;  // at most n3 * kFftLine / blockDim = 16 terms per thread
-    const unsigned m_h1 = div_magic(G.h1);
-    for (int k = tid; k < G.n3 * kFftLine; k += blockDim.x) {
-        const int k3 = k / kFftLine, l = k % kFftLine;
+    float ef = 0.f;  // at most 16 terms per thread
+    float wk = 0.f;
+    const float *fp = ftab;
+    if (in) {
         const int p = (int)p0 + l;  // < nh < 2^14
-        float f = 0.f, wk = 0.f;
-        if (p < G.nh) {
-            const int k2 = (int)fast_div(p, m_h1), k1 = p - k2 * G.h1;
-            f = __ldg(ftab + k3 * G.n12 + (long long)k2 * G.n1 + k1);
-            wk = (k1 == 0 || 2 * k1 == G.n1) ? 1.f : 2.f;
-        }
-        const float2 y = Rr[k];
+        const int k2 = (int)fast_div(p, div_magic(G.h1)), k1 = p - k2 * G.h1;
+        fp += k2 * G.n1 + k1;
+        wk = (k1 == 0 || 2 * k1 == G.n1) ? 1.f : 2.f;
+    }
+#pragma unroll 5
+    for (int k3 = wp; k3 < G.n3; k3 += NW) {
+        const float f = in ? __ldg(fp + k3 * G.n12) : 0.f;
+        const float2 y = Rr[k3 * kFftLine + l];
         ef = fmaf(f * wk, y.x * y.x + y.y * y.y, ef);
-        Rr[k] = make_float2(y.x * f, y.y * f);
+        Rr[k3 * kFftLine + l] = make_float2(y.x * f, y.y * f);
     }
     double e = (double)ef;
     __syncthreads();
     if (!energy_only) {
-        const float2 *R2 = fft_lines(Rr, Or, G.ax[2], kFftLine, 1, kFftLine, Ws + 256, true);
-        for (int k = tid; k < G.n3 * kFftLine; k += blockDim.x) {
-            const int x3 = k / kFftLine, l = k % kFftLine;
-            if (p0 + l < G.nh) col[x3 * G.nh + l] = R2[k];
-        }
+        const float2 *R2 = fft_lines<kFftLine, 1, kFftLine>(Rr, Or, G.ax[2], kFftLine, 1, kFftLine, Ws + 256, true);
+        if (in)
+            for (int x3 = wp; x3 < G.n3; x3 += NW) col[x3 * G.nh + l] = R2[x3 * kFftLine + l];
     }
     if (e_part != nullptr) {
         double w = 0.0;
@@ -412,7 +470,7 @@ __global__ void __launch_bounds__(256) fft_axis3_kernel(const FftGeom G, float2 
         __syncthreads();
         if (tid == 0) {
             double sum = 0.0;
-            for (int k = 0; k < (int)(blockDim.x >> 5); ++k) sum += red[k];
+            for (int k = 0; k < NW; ++k) sum += red[k];
             e_part[item * gridDim.x + blockIdx.x] = sum;
         }
     }
@@ -420,12 +478,15 @@ __global__ void __launch_bounds__(256) fft_axis3_kernel(const FftGeom G, float2 
 
 // Pass C: inverse 2D transform of x3 plane blockIdx.x of item blockIdx.y; real part / N
 // into out32 (fp32) or out64 (fp64, right-hand-side mode).
-__global__ void __launch_bounds__(kFftPlaneThreads) fft_plane_inv_kernel(const FftGeom G, const float2 *__restrict__ C,
+template <bool IN_PLACE>
+__global__ void __launch_bounds__(IN_PLACE ? kFftInPlaceThreads : kFftPlaneThreads, IN_PLACE ? 4 : 2)
+    fft_plane_inv_kernel(const FftGeom G, const float2 *__restrict__ C,
                                                             float *__restrict__ out32, double *__restrict__ out64) {
     extern __shared__ float2 fsm[];
     __shared__ float2 Ws[3 * 128];
     const int ld = G.n1 + 1;
-    float2 *A = fsm, *B = fsm + (size_t)G.n2 * ld;
+    float2 *A = fsm, *B = IN_PLACE ? fsm : fsm + (size_t)G.n2 * ld;
+    const int lj = IN_PLACE ? 2 * ld : ld;  // between packed rows
     const int x3 = blockIdx.x;
     const long long item = blockIdx.y;
     const float2 *src = C + item * G.N + x3 * G.nh;  // [k2][k1 < h1]
@@ -448,38 +509,51 @@ __global__ void __launch_bounds__(kFftPlaneThreads) fft_plane_inv_kernel(const F
         }
     }
     __syncthreads();
-    float2 *R1 = fft_lines(A, B, G.ax[1], G.h1, 1, ld, Ws + 128, true);  // kept columns: along x2
-    float2 *Zp = (R1 == A) ? B : A;
+    float2 *R1 = fft_lines<0, 1, 0>(A, B, G.ax[1], G.h1, 1, ld, Ws + 128, true);  // kept columns: along x2
+    float2 *Zp = IN_PLACE ? A : (R1 == A) ? B : A;  // in place: columns past h1 are free
     // two rows per complex inverse along x1: packed row j holds Z(k) = A(k) + i B(k)
     // for every k1, A and B the spectra of rows 2j and 2j + 1, whose columns
     // k1 > n1 / 2 are the conjugates of kept ones (the inverse along x3 and x2 of a
     // Hermitian spectrum leaves every row Hermitian in k1); the inverse of Z is
     // then row 2j in its real part and row 2j + 1 in its imaginary part
     const int n2p = (G.n2 + 1) / 2;
-    for (int e = threadIdx.x; e < n2p * G.n1; e += blockDim.x) {
-        const int j = (int)fast_div(e, m_n1), k = e - j * G.n1;
-        const bool kept = k < G.h1;
-        const int ks = kept ? k : G.n1 - k;
-        float2 a = R1[2 * j * ld + ks];
-        float2 b = (2 * j + 1 < G.n2) ? R1[(2 * j + 1) * ld + ks] : make_float2(0.f, 0.f);
-        if (!kept) {
-            a.y = -a.y;
-            b.y = -b.y;
-        }
-        Zp[j * ld + k] = make_float2(a.x - b.y, a.y + b.x);
+    for (int e = threadIdx.x; e < n2p * G.h1; e += blockDim.x) {  // column k and its mirror n1 - k
+        const int j = (int)fast_div(e, m_h1), k = e - j * G.h1;
+        const float2 a = R1[2 * j * ld + k];
+        const float2 b = (2 * j + 1 < G.n2) ? R1[(2 * j + 1) * ld + k] : make_float2(0.f, 0.f);
+        Zp[j * lj + k] = make_float2(a.x - b.y, a.y + b.x);
+        const int km = G.n1 - k;
+        if (km >= G.h1 && km < G.n1) Zp[j * lj + km] = make_float2(a.x + b.y, b.x - a.y);
     }
     __syncthreads();
-    const float2 *R2 = fft_lines(Zp, R1, G.ax[0], n2p, ld, 1, Ws, true);  // packed rows: along x1
+    const float2 *R2 = fft_lines<0, 0, 1>(Zp, R1, G.ax[0], n2p, lj, 1, Ws, true);  // packed rows: along x1
     const float inv_n = 1.f / (float)G.N;
     const long long base = item * G.N + x3 * G.n12;
-    for (int e = threadIdx.x; e < G.n12; e += blockDim.x) {
-        const int x2 = (int)fast_div(e, m_n1);
-        const float2 z = R2[(x2 >> 1) * ld + e - x2 * G.n1];
-        const float v = ((x2 & 1) ? z.y : z.x) * inv_n;
-        if (out64)
-            out64[base + e] = (double)v;
-        else
-            out32[base + e] = v;
+    if (G.n1 % 2 == 0 && out32) {  // two neighbouring values per store
+        const int nv = G.n1 / 2;
+        const unsigned m_nv = div_magic(nv);
+        for (int e = threadIdx.x; e < n2p * nv; e += blockDim.x) {
+            const int j = (int)fast_div(e, m_nv), x1 = 2 * (e - j * nv);
+            const float2 z0 = R2[j * lj + x1], z1 = R2[j * lj + x1 + 1];
+            float *o = out32 + base + 2 * j * G.n1 + x1;
+            *reinterpret_cast<float2 *>(o) = make_float2(z0.x * inv_n, z1.x * inv_n);
+            if (2 * j + 1 < G.n2) *reinterpret_cast<float2 *>(o + G.n1) = make_float2(z0.y * inv_n, z1.y * inv_n);
+        }
+        return;
+    }
+    for (int e = threadIdx.x; e < n2p * G.n1; e += blockDim.x) {
+        const int j = (int)fast_div(e, m_n1), x1 = e - j * G.n1;
+        const float2 z = R2[j * lj + x1];
+        const long long o = base + 2 * j * G.n1 + x1;
+        const float v0 = z.x * inv_n, v1 = z.y * inv_n;
+        const bool two = 2 * j + 1 < G.n2;
+        if (out64) {
+            out64[o] = (double)v0;
+            if (two) out64[o + G.n1] = (double)v1;
+        } else {
+            out32[o] = v0;
+            if (two) out32[o + G.n1] = v1;
+        }
     }
 }
 
@@ -529,8 +603,12 @@ FftGeom geom(const kx_plan *p) {
     return G;
 }
 
-size_t plane_smem(const kx_plan *p) { return sizeof(float2) * 2 * (size_t)p->n[1] * (p->n[0] + 1); }
-size_t line_smem(const kx_plan *p) { return sizeof(float2) * 2 * (size_t)p->n[2] * kFftLine; }
+// both plane axes by the four-step transform, whose second phase has a task per thread at most
+bool plane_in_place(const kx_plan *p) { return p->n[0] == 80 && p->n[1] == 80; }
+size_t plane_smem(const kx_plan *p) {
+    return sizeof(float2) * (plane_in_place(p) ? 1 : 2) * (size_t)p->n[1] * (p->n[0] + 1);
+}
+size_t line_smem(const kx_plan *p) { return sizeof(float2) * (p->n[2] == 80 ? 1 : 2) * (size_t)p->n[2] * kFftLine; }
 
 }  // namespace
 
@@ -599,17 +677,21 @@ int fft_passes(kx_plan *p, long R, const int2 *pairs, const float *src32, int rh
                float *out32, double *out64, double *ex, double *partial, bool energy_only, cudaStream_t s) {
     const FftGeom G = geom(p);
     const size_t ps = plane_smem(p), ls = line_smem(p);
-    KX_CUDA_TRY(cudaFuncSetAttribute(fft_plane_fwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ps));
-    KX_CUDA_TRY(cudaFuncSetAttribute(fft_plane_inv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ps));
+    const bool ip = plane_in_place(p);
+    auto fwd = ip ? fft_plane_fwd_kernel<true> : fft_plane_fwd_kernel<false>;
+    auto inv = ip ? fft_plane_inv_kernel<true> : fft_plane_inv_kernel<false>;
+    const int pt = ip ? kFftInPlaceThreads : kFftPlaneThreads;
+    KX_CUDA_TRY(cudaFuncSetAttribute(fwd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ps));
+    KX_CUDA_TRY(cudaFuncSetAttribute(inv, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ps));
     KX_CUDA_TRY(cudaFuncSetAttribute(fft_axis3_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ls));
     int rc;
     const dim3 gp((unsigned)p->n[2], (unsigned)R);
     if ((rc = prof_begin(p, PK_FFT, s))) return rc;
-    fft_plane_fwd_kernel<<<gp, kFftPlaneThreads, ps, s>>>(G, pairs, src32, rhs, C);
+    fwd<<<gp, pt, ps, s>>>(G, pairs, src32, rhs, C);
     KX_LAUNCH_CHECK("fft_plane_fwd_kernel launch");
     const unsigned groups = (unsigned)((G.nh + kFftLine - 1) / kFftLine);  // pass B: half-spectrum positions
     double *e_part = (ex != nullptr && !rhs) ? partial : nullptr;
-    fft_axis3_kernel<<<dim3(groups, (unsigned)R), 256, ls, s>>>(G, C, p->d_fft_f, pairs, occ, rhs,
+    fft_axis3_kernel<<<dim3(groups, (unsigned)R), kFftLineThreads, ls, s>>>(G, C, p->d_fft_f, pairs, occ, rhs,
                                                                     energy_only ? 1 : 0, e_part);
     KX_LAUNCH_CHECK("fft_axis3_kernel launch");
     if (e_part) {
@@ -617,7 +699,7 @@ int fft_passes(kx_plan *p, long R, const int2 *pairs, const float *src32, int rh
         KX_LAUNCH_CHECK("fft_energy_reduce_kernel launch");
     }
     if (!energy_only) {
-        fft_plane_inv_kernel<<<gp, kFftPlaneThreads, ps, s>>>(G, C, out32, out64);
+        inv<<<gp, pt, ps, s>>>(G, C, out32, out64);
         KX_LAUNCH_CHECK("fft_plane_inv_kernel launch");
     }
     return prof_end(p, s);

@@ -506,6 +506,24 @@ def test_fft_vx_and_energy_match_oracle(kx):
     assert abs(e_only - ex_ref) < TOL[1]["ex"] * abs(ex_ref)
 
 
+@pytest.mark.parametrize("n", [
+    (80, 80, 4), (80, 9, 5), (10, 80, 6), (9, 80, 4), (6, 5, 80),  # four-step lines: both plane axes, one, the third
+    (8, 15, 36), (15, 8, 12),  # value pairs along an even axis 1, single values along an odd one
+])
+def test_fft_line_and_plane_forms(kx, n):
+    h, bc = (0.45, 0.5, 0.4), (P, P, P)
+    op = oracle.Plan(n, h, bc, S)
+    psi = workloads.random_field(op.N, 3, 87)
+    plan = kx.Plan(n, h, bc, S, precision=kx.KX_FFT32)
+    ref = np.stack([oracle.apply_fL(op, psi[:, r]) for r in range(3)], axis=1)
+    x = kx.kx_apply_fL(plan, dev(psi.T)).cpu().numpy().T
+    assert relmax(x, ref) < TOL[1]["fl"]
+    vx_ref, ex_ref = oracle.vx_apply(op, psi, None)
+    vx, ex = kx.kx_vx_apply(plan, dev(psi.T))
+    assert relmax(vx.cpu().numpy().T, vx_ref) < TOL[1]["vx"]
+    assert abs(ex.item() - ex_ref) < TOL[1]["ex"] * abs(ex_ref)
+
+
 @pytest.mark.parametrize("n_orb", [1, 3, 4, 5, 8, 13])
 @pytest.mark.parametrize("n", [(9, 10, 15), (12, 10, 9)])
 def test_fft_vx_ragged_blocks_and_points(kx, n, n_orb):
