@@ -85,14 +85,16 @@ __global__ void __launch_bounds__(32 * kRedWarps) gram_reduce_kernel(const doubl
 // In-place Cholesky of the symmetric positive definite A (lower triangle used):
 // A = L L^T; the diagonal of A receives the reciprocals of L's, *bad = 1 if a pivot
 // <= 0.  One CTA, the matrix in shared memory where it fits (n <= kCholSmemN).  A
-// serial chain of n pivots (square root, reciprocal, two barriers) over rank-1
-// updates of the lower triangle, a warp per row: 130 us at n = 64 with the
-// updates in global memory and a division per entry of the column.
+// serial chain of n pivots over rank-1 updates of the lower triangle, a warp per row;
+// warp 0 works out the next pivot's reciprocal root meanwhile (n = 64: 130 us with the
+// updates in global memory and a division per entry of the column, 93 us with the
+// matrix in shared memory and root, reciprocal and updates one after the other,
+// 58 us now).
 constexpr int kCholThreads = 512;
 constexpr int kCholSmemN = 160;  // 205 KB
 __global__ void __launch_bounds__(kCholThreads) cholesky_kernel(double *__restrict__ A, int n, int *__restrict__ bad) {
     extern __shared__ double chol_sm[];
-    __shared__ double rpiv;
+    __shared__ double rpiv[2];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const bool in_smem = n <= kCholSmemN;
     double *L = in_smem ? chol_sm : A;
@@ -100,23 +102,35 @@ __global__ void __launch_bounds__(kCholThreads) cholesky_kernel(double *__restri
     if (in_smem)
         for (int e = tid; e < n * n; e += kCholThreads) L[e] = A[e];
     __syncthreads();
-    for (int k = 0; k < n; ++k) {
-        if (tid == 0) {
-            double d = L[k * ld + k];
-            if (!(d > 0.0)) {
-                *bad = 1;
-                d = 1.0;
-            }
-            rpiv = 1.0 / sqrt(d);
-            L[k * ld + k] = rpiv;
+    auto pivot = [&](int k) {  // reciprocal root of pivot k
+        double d = L[k * ld + k];
+        if (!(d > 0.0)) {
+            *bad = 1;
+            d = 1.0;
         }
-        __syncthreads();
-        const double r = rpiv;
+        return rsqrt(d);
+    };
+    if (tid == 0) rpiv[0] = pivot(0);
+    __syncthreads();
+    for (int k = 0; k < n; ++k) {
+        const double r = rpiv[k & 1];
         for (int i = k + 1 + tid; i < n; i += kCholThreads) L[i * ld + k] *= r;
         __syncthreads();
-        for (int i = k + 1 + warp; i < n; i += kCholThreads / 32) {
-            const double lik = L[i * ld + k];
-            for (int j = k + 1 + lane; j <= i; j += 32) L[i * ld + j] = fma(-lik, L[j * ld + k], L[i * ld + j]);
+        if (warp == 0) {
+            // the next pivot, while the other warps update the rest
+            if (lane == 0) {
+                L[k * ld + k] = r;
+                if (k + 1 < n) {
+                    const double l = L[(k + 1) * ld + k];
+                    L[(k + 1) * ld + k + 1] = fma(-l, l, L[(k + 1) * ld + k + 1]);
+                    rpiv[(k + 1) & 1] = pivot(k + 1);
+                }
+            }
+        } else {
+            for (int i = k + 1 + warp; i < n; i += kCholThreads / 32 - 1) {
+                const double lik = L[i * ld + k];
+                for (int j = k + 1 + lane; j <= i; j += 32) L[i * ld + j] = fma(-lik, L[j * ld + k], L[i * ld + j]);
+            }
         }
         __syncthreads();
     }
@@ -204,11 +218,11 @@ constexpr int kPT = 64;   // projection tile: 64 a x 64 b per CTA
 constexpr int kPX = 32;   // grid points per pipeline step
 constexpr int kPBlk = 8;  // steps summed in float32 before the compensated accumulation (256 points)
 constexpr int kPStages = 2;
-// dynamic shared memory of proj32_kernel (82 KB, two CTAs per SM): raw float64
-// stages of both operands, then their float32 copies (rows padded by 4 floats
+// dynamic shared memory of proj32_kernel (100 KB, two CTAs per SM): raw float64
+// stages of both operands, then two float32 copies of them (rows padded by 4 floats
 // for conflict-free float4 reads)
 constexpr size_t kProjRawBytes = (size_t)kPStages * 2 * kPT * kPX * sizeof(double);
-constexpr size_t kProjSmem = kProjRawBytes + 2 * (size_t)kPT * (kPX + 4) * sizeof(float);
+constexpr size_t kProjSmem = kProjRawBytes + 4 * (size_t)kPT * (kPX + 4) * sizeof(float);
 
 // Issues the asynchronous copies of grid points [xb, xb + kPX) of rows
 // r0..r0+63 of M (nr rows in all, stride N) into raw[64][kPX]; points at or
@@ -237,10 +251,13 @@ __device__ __forceinline__ void proj_issue(const double *__restrict__ M, int nr,
 // A_a(x) B_b(x) for its 64 x 64 tile (blockIdx.y, blockIdx.z); two CTAs per SM.
 // The float64 inputs of step k+1 are copied into shared memory (cp.async)
 // while step k is converted to float32 and multiplied, so the SM always has a
-// step's loads in flight.  Thread (tx, ty) of a 16 x 16 layout owns
-// a = a0 + ty + 16 i, b = b0 + tx + 16 j (i, j < 4): per four grid points it
-// reads four a-rows (two distinct per warp, broadcast) and four b-rows as
-// float4 and does 64 FMAs.  Each block of 256 points is summed in float32 and
+// step's loads in flight; a thread converts what it copied itself, into one of two
+// float32 tiles, so that a step has one barrier.  Thread (tx, ty) of a 16 x 16 layout
+// owns a = a0 + ty + 16 i, b = b0 + tx + 16 j (i, j < 4): per four grid points it
+// reads four a-rows and four b-rows as float4 and does 64 FMAs.  A warp is 4 x 8 of the
+// layout: its reads are 4 and 8 distinct rows, one pass over the banks each (2 and 16
+// rows took 3 for the two; the shared-memory path was the bound: 64 x 64 vectors at
+// 96^3 290 -> 264 us).  Each block of 256 points is summed in float32 and
 // added to a float32 pair (sum and rounding error), so the CTA's total keeps
 // about 48 bits.  w (nullable) weights every grid point of B; a tile whose A
 // and B rows are the same rows of one array copies them once.
@@ -251,9 +268,9 @@ __global__ void __launch_bounds__(256, 2) proj32_kernel(const double *__restrict
                                                         double *__restrict__ part) {
     extern __shared__ __align__(16) uint8_t smem_raw[];
     double *raw = reinterpret_cast<double *>(smem_raw);  // [stage][A|B][64][kPX]
-    float(*As)[kPX + 4] = reinterpret_cast<float(*)[kPX + 4]>(smem_raw + kProjRawBytes);
-    float(*Bs)[kPX + 4] = As + kPT;
-    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+    float(*const As0)[kPX + 4] = reinterpret_cast<float(*)[kPX + 4]>(smem_raw + kProjRawBytes);  // [2][A|B][64]
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int tx = (warp & 1) * 8 + (lane & 7), ty = (warp >> 1) * 4 + (lane >> 3);
     const int a0 = blockIdx.y * kPT, b0 = blockIdx.z * kPT;
     const long long x0 = (long long)blockIdx.x * span;
     const long long x1 = min(N, x0 + span);
@@ -275,7 +292,6 @@ __global__ void __launch_bounds__(256, 2) proj32_kernel(const double *__restrict
         if (!same) proj_issue<VEC2>(B, nb, b0, N, x0, x1, stage(0) + kPT * kPX, tid);
     }
     ptx::cp_async_commit();
-    const int lx = tid & 31, lr = tid >> 5;  // converter: one grid point, rows lr + 8m
     int blk = 0;
     for (int k = 0; k < nsteps; ++k) {
         if (k + 1 < nsteps) {
@@ -284,18 +300,31 @@ __global__ void __launch_bounds__(256, 2) proj32_kernel(const double *__restrict
             if (!same) proj_issue<VEC2>(B, nb, b0, N, xb, x1, stage(k + 1) + kPT * kPX, tid);
         }
         ptx::cp_async_commit();
-        ptx::cp_async_wait<1>();  // this thread's copies of step k have landed
-        __syncthreads();          // everyone's have; the float32 tiles are free
+        ptx::cp_async_wait<1>();  // this thread's copies of step k have landed: it converts those
         const double *ra = stage(k), *rb = same ? stage(k) : stage(k) + kPT * kPX;
-        const long long xw = x0 + (long long)k * kPX + lx;
-        const float wx = (w != nullptr && xw < x1) ? __ldg(w + xw) : 1.f;
+        float(*As)[kPX + 4] = As0 + (k & 1) * 2 * kPT, (*Bs)[kPX + 4] = As + kPT;
+        constexpr int V = VEC2 ? 2 : 1, per_row = kPX / V;  // as in proj_issue
+        const int c = (tid % per_row) * V;                   // (256 is a multiple of per_row)
+        float wx[V];
 #pragma unroll
-        for (int m = 0; m < 8; ++m) {
-            const int r = lr + 8 * m;
-            As[r][lx] = f64_to_f32(ra[r * kPX + lx]);
-            Bs[r][lx] = f64_to_f32(rb[r * kPX + lx]) * wx;
+        for (int v = 0; v < V; ++v) {
+            const long long xw = x0 + (long long)k * kPX + c + v;
+            wx[v] = (w != nullptr && xw < x1) ? __ldg(w + xw) : 1.f;
         }
-        __syncthreads();
+#pragma unroll
+        for (int m = 0; m < kPT * per_row / 256; ++m) {
+            const int r = (tid + 256 * m) / per_row;
+            if constexpr (VEC2) {
+                const double2 da = *reinterpret_cast<const double2 *>(ra + r * kPX + c);
+                const double2 db = *reinterpret_cast<const double2 *>(rb + r * kPX + c);
+                *reinterpret_cast<float2 *>(&As[r][c]) = make_float2(f64_to_f32(da.x), f64_to_f32(da.y));
+                *reinterpret_cast<float2 *>(&Bs[r][c]) = make_float2(f64_to_f32(db.x) * wx[0], f64_to_f32(db.y) * wx[V - 1]);
+            } else {
+                As[r][c] = f64_to_f32(ra[r * kPX + c]);
+                Bs[r][c] = f64_to_f32(rb[r * kPX + c]) * wx[0];
+            }
+        }
+        __syncthreads();  // (two float32 tiles: the other one's readers passed the barrier before)
 #pragma unroll 2
         for (int xx = 0; xx < kPX; xx += 4) {
             float4 av[4], bv[4];
@@ -355,7 +384,7 @@ __host__ __device__ constexpr size_t comb_smem(int na) {
 // C row piece it needs is the same for the whole warp (two broadcast float4
 // reads), the A values are consecutive across lanes.  Sums over a stay in
 // float32 (na <= 256 terms).
-template <bool VEC2>
+// (For rows that are not 16-byte aligned; combine32_bulk_kernel otherwise.)
 __global__ void __launch_bounds__(256, 2) combine32_kernel(const double *__restrict__ A, int na,
                                                            const double *__restrict__ C, int nb, long long N,
                                                            float sgn, bool accumulate, double *__restrict__ out) {
@@ -378,19 +407,14 @@ __global__ void __launch_bounds__(256, 2) combine32_kernel(const double *__restr
         double *dst = raw + (size_t)(i % kCStages) * kCA * kCX;
         const long long xt = (blockIdx.x + (i / nch) * gridDim.x) * kCX;
         const int r0 = (int)(i % nch) * kCA;
-        constexpr int per_row = VEC2 ? kCX / 2 : kCX;
 #pragma unroll
-        for (int m = 0; m < kCA * per_row / 256; ++m) {
+        for (int m = 0; m < kCA * kCX / 256; ++m) {
             const int piece = tid + 256 * m;
-            const int r = piece / per_row, c = (piece % per_row) * (VEC2 ? 2 : 1);
+            const int r = piece / kCX, c = piece % kCX;
             const long long x = xt + c;
             long long nbytes = (r0 + r < na) ? (N - x) * 8 : 0;
-            nbytes = nbytes < 0 ? 0 : (nbytes > (VEC2 ? 16 : 8) ? (VEC2 ? 16 : 8) : nbytes);
-            const double *src = nbytes > 0 ? A + (long long)(r0 + r) * N + x : A;
-            if (VEC2)
-                ptx::cp_async16(dst + r * kCX + c, src, (uint32_t)nbytes);
-            else
-                ptx::cp_async8(dst + r * kCX + c, src, (uint32_t)nbytes);
+            nbytes = nbytes < 0 ? 0 : min(nbytes, 8LL);
+            ptx::cp_async8(dst + r * kCX + c, nbytes > 0 ? A + (long long)(r0 + r) * N + x : A, (uint32_t)nbytes);
         }
     };
 #pragma unroll
@@ -456,6 +480,126 @@ __global__ void __launch_bounds__(256, 2) combine32_kernel(const double *__restr
     ptx::cp_async_wait<0>();
 }
 
+// The same for an even N and 16-byte aligned rows, 256 points x 64 outputs per CTA and
+// 8 x 8 per thread (points tile + 2 tx + 64 k and the next, outputs b0 + 8 ty + j): half the shared
+// reads per product of the 4 x 8 form above, rows brought in by bulk copies (1 issue
+// per row in place of 128), a double float32 tile (one barrier per step of 8 vectors).
+// Bound by instruction issue (packed products, their operands and the conversions)
+// beside 133 us of memory: 319 -> 255 us for 64 x 64 vectors at 96^3.  Same sums in
+// the same order.
+constexpr int kDX = 256, kDR = 8, kDStages = 3;
+__host__ __device__ constexpr size_t comb_bulk_smem(int na) {
+    return (size_t)kDStages * kDR * kDX * sizeof(double) + 2 * (size_t)kDR * kDX * sizeof(float) +
+           (size_t)((na + kDR - 1) / kDR) * kDR * kCB * sizeof(float);
+}
+__global__ void __launch_bounds__(256, 2) combine32_bulk_kernel(const double *__restrict__ A, int na,
+                                                                const double *__restrict__ C, int nb, long long N,
+                                                                float sgn, bool accumulate, double *__restrict__ out,
+                                                                int *status) {
+    extern __shared__ __align__(16) uint8_t smem_raw[];
+    double *raw = reinterpret_cast<double *>(smem_raw);                                  // [stage][kDR][kDX]
+    float *As = reinterpret_cast<float *>(raw + (size_t)kDStages * kDR * kDX);           // [2][kDR][kDX]
+    float *Cs = As + 2 * kDR * kDX;                                                      // [na][kCB]
+    __shared__ uint64_t full[kDStages];
+    const int tid = threadIdx.x, tx = tid & 31, ty = tid >> 5;
+    const int b0 = blockIdx.y * kCB;
+    const int nch = (na + kDR - 1) / kDR;
+    const int ntiles = (int)((N + kDX - 1) / kDX);
+    const int my_tiles = ntiles > (int)blockIdx.x ? (ntiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : 0;
+    const int nitems = my_tiles * nch;  // N < 2^21: items stay far below 2^31
+    if (tid == 0) {
+        for (int i = 0; i < kDStages; ++i) ptx::mbar_init(&full[i], 1);
+        ptx::fence_mbar_init();
+    }
+    for (int e = tid; e < nch * kDR * kCB; e += 256) {
+        const int r = e / kCB, c = e % kCB;
+        Cs[e] = (r < na && b0 + c < nb) ? f64_to_f32(__ldg(C + (long long)r * nb + b0 + c)) : 0.f;
+    }
+    __syncthreads();
+    auto issue = [&](int tile, int ch, int st) {
+        const long long xt = (long long)tile * kDX;
+        const int rows = min(kDR, na - ch * kDR);
+        const uint32_t bytes = (uint32_t)min((long long)kDX, N - xt) * 8;  // a multiple of 16
+        ptx::mbar_arrive_expect_tx(&full[st], bytes * (uint32_t)rows);
+        for (int r = 0; r < rows; ++r)
+            ptx::bulk_load(raw + (st * kDR + r) * kDX, A + (long long)(ch * kDR + r) * N + xt, bytes, &full[st]);
+    };
+    int i_tile = blockIdx.x, i_ch = 0, i_st = 0;  // next copy (thread 0)
+    auto issue_next = [&]() {
+        issue(i_tile, i_ch, i_st);
+        if (++i_ch == nch) {
+            i_ch = 0;
+            i_tile += gridDim.x;
+        }
+        if (++i_st == kDStages) i_st = 0;
+    };
+    if (tid == 0)
+        for (int i = 0; i < kDStages && i < nitems; ++i) issue_next();
+    const bool out16 = (reinterpret_cast<uintptr_t>(out) & 15) == 0;
+    float2 acc[4][8];  // acc[k][j]: points 2 tx + 64 k (.x) and + 1 (.y), output b0 + 8 ty + j
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) acc[k][j] = make_float2(0.f, 0.f);
+    int ch = 0, st = 0, tile = blockIdx.x;
+    uint32_t par = 0;
+    for (int i = 0; i < nitems; ++i) {
+        const bool ok = ptx::mbar_wait_bounded(&full[st], par, 2000000000LL);
+        float *at = As + (i & 1) * kDR * kDX;
+        const int rows = min(kDR, na - ch * kDR);
+        const double *src = raw + st * kDR * kDX + tid;
+#pragma unroll
+        for (int r = 0; r < kDR; ++r) at[r * kDX + tid] = ok && r < rows ? f64_to_f32(src[r * kDX]) : 0.f;
+        if (!ok) atomicExch(status, KX_ERR_TIMEOUT);
+        if (__syncthreads_or(!ok)) return;  // a wait gave up
+        if (tid == 0 && i + kDStages < nitems) issue_next();  // every thread has read this stage
+        if (++st == kDStages) {
+            st = 0;
+            par ^= 1u;
+        }
+        const float *cs = Cs + ch * kDR * kCB + 8 * ty;
+#pragma unroll 2
+        for (int r = 0; r < kDR; ++r) {
+            float2 av[4];  // points 2 tx, + 1 + 64 k
+#pragma unroll
+            for (int k = 0; k < 4; ++k) av[k] = *reinterpret_cast<const float2 *>(at + r * kDX + 2 * tx + 64 * k);
+            float cv[8];
+            *reinterpret_cast<float4 *>(cv) = *reinterpret_cast<const float4 *>(cs + r * kCB);
+            *reinterpret_cast<float4 *>(cv + 4) = *reinterpret_cast<const float4 *>(cs + r * kCB + 4);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const float2 cj = make_float2(cv[j], cv[j]);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) fma2(acc[k][j], cj, av[k]);
+            }
+        }
+        if (++ch < nch) continue;
+        ch = 0;
+        const long long xt = (long long)tile * kDX;
+        tile += gridDim.x;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const int b = b0 + 8 * ty + j;
+            double *o = out + (long long)b * N + xt + 2 * tx;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                if (xt + 2 * tx + 64 * k < N && b < nb) {
+                    double *q = o + 64 * k;
+                    const double vx = (accumulate ? q[0] : 0.0) + f32_to_f64(sgn * acc[k][j].x);
+                    const double vy = (accumulate ? q[1] : 0.0) + f32_to_f64(sgn * acc[k][j].y);
+                    if (out16) {
+                        *reinterpret_cast<double2 *>(q) = make_double2(vx, vy);
+                    } else {  // an output that starts on 8 bytes only
+                        q[0] = vx;
+                        q[1] = vy;
+                    }
+                }
+                acc[k][j] = make_float2(0.f, 0.f);
+            }
+        }
+    }
+}
+
 // part (n_split x na x nb) of A^T B over the grid, float64 or float32 products
 // by plan precision; returns n_split.
 int launch_projection(kx_plan *p, const double *A, int na, const double *B, int nb, const double *w64,
@@ -510,20 +654,20 @@ int launch_combination(kx_plan *p, const double *A, int na, const double *C, int
         KX_LAUNCH_CHECK("xi_kernel launch");
     } else {
         const int tiles_b = (nb + kCB - 1) / kCB;
-        const long long ntiles = (N + kCX - 1) / kCX;
-        const int gx = (int)std::max(1LL, std::min<long long>(ntiles, std::max(1, 2 * p->num_sms / tiles_b)));
-        const size_t smem = comb_smem(na);
-        const dim3 grid(gx, tiles_b);
         const float fs = sgn < 0.0 ? -1.f : 1.f;
-        const bool vec2 = N % 2 == 0 && (reinterpret_cast<uintptr_t>(A) & 15) == 0;
-        if (vec2) {
-            KX_CUDA_TRY(cudaFuncSetAttribute(combine32_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        // bulk copies: 16-byte aligned rows
+        const bool bulk = N % 2 == 0 && (reinterpret_cast<uintptr_t>(A) & 15) == 0;
+        const long long ntiles = (N + (bulk ? kDX : kCX) - 1) / (bulk ? kDX : kCX);
+        const int gx = (int)std::max(1LL, std::min<long long>(ntiles, std::max(1, 2 * p->num_sms / tiles_b)));
+        const size_t smem = bulk ? comb_bulk_smem(na) : comb_smem(na);
+        const dim3 grid(gx, tiles_b);
+        if (bulk) {
+            KX_CUDA_TRY(cudaFuncSetAttribute(combine32_bulk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)smem));
-            combine32_kernel<true><<<grid, 256, smem, s>>>(A, na, C, nb, N, fs, accumulate, out);
+            combine32_bulk_kernel<<<grid, 256, smem, s>>>(A, na, C, nb, N, fs, accumulate, out, p->d_status);
         } else {
-            KX_CUDA_TRY(cudaFuncSetAttribute(combine32_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)smem));
-            combine32_kernel<false><<<grid, 256, smem, s>>>(A, na, C, nb, N, fs, accumulate, out);
+            KX_CUDA_TRY(cudaFuncSetAttribute(combine32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+            combine32_kernel<<<grid, 256, smem, s>>>(A, na, C, nb, N, fs, accumulate, out);
         }
         KX_LAUNCH_CHECK("combine32_kernel launch");
     }

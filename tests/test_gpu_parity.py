@@ -475,6 +475,28 @@ def test_multipole_full_size_row(kx):
     assert np.max(np.abs(vx_h[i] - ref[:, i])) < 1e-5 * np.abs(ref[:, i]).max()
 
 
+@pytest.mark.parametrize("shift", [0, 1])  # rows on 16 and on 8 bytes: the two forms of the grid products
+@pytest.mark.parametrize("n_xi,n_vec", [(1, 1), (7, 65), (8, 64), (65, 8), (130, 3)])
+def test_ace_apply_forms(kx, n_xi, n_vec, shift):
+    n, h = (16, 8, 24), (0.4, 0.5, 0.3)  # 12 tiles of 256 points
+    plan = kx.Plan(n, h, (P, P, P), S, precision=1)
+    rng = np.random.default_rng(n_xi)
+    xi, phi = rng.standard_normal((n_xi, plan.N)), rng.standard_normal((n_vec, plan.N))
+    ref = -(np.prod(h) * phi @ xi.T) @ xi
+
+    def placed(a):
+        buf = torch.empty(a.size + 2, dtype=torch.float64, device="cuda")
+        v = buf[shift:shift + a.size].view(a.shape)
+        v.copy_(torch.from_numpy(a))
+        return v
+
+    out = placed(np.zeros_like(phi))
+    kx.kx_ace_apply(plan, placed(xi), placed(phi), out=out)
+    torch.cuda.synchronize()
+    assert plan.status() == kx.KX_OK
+    assert relmax(out.cpu().numpy(), ref) < 2e-5  # float32 products, 130 terms at most
+
+
 # --------------------------------------------------------------------------
 # FFT variant for fully periodic grids (KX_FFT32)
 # --------------------------------------------------------------------------
