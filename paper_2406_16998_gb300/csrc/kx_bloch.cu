@@ -2269,10 +2269,10 @@ inline bool bp0_axis(const kx_plan *p) {
     return bp_axes(p) && tc_axis(p, 0) && p->n[0] == 64 && (p->N / 64) % 128 == 0;
 }
 
-// Axes 1 and 2 two products per kernel (kx_bloch_fused.cu): planes of 64 x 64 points, two
-// of which are a tile of 128 rows (969 -> 485 us for the four products of 256 pairs at
-// 64^3).  A plane of 32-point axes would fill half the tile's columns and leave the
-// kernel's time per value as it is, so those sizes keep the single products.
+// Two products per kernel (kx_bloch_fused.cu): planes of 64 x 64 points, two of which are
+// a tile of 128 rows (1428 -> 873 us for the six products of 256 pairs at 64^3).  A
+// plane of 32-point axes would fill half the tile's columns and leave the kernel's time
+// per value as it is, so those sizes keep the single products.
 inline bool bp_fused(const kx_plan *p) { return bp_axes(p) && tc_axis(p, 0) && p->n[0] == 64 && p->n[1] == 64; }
 
 template <bool FORM>
@@ -2328,7 +2328,7 @@ inline int vector_maxima(kx_plan *p, const float2 *x, long long N, int n_vec, fl
 // the orbitals and vectors and their maxima (float32 plans), chunk buffers A and
 // B and two per-item maximum arrays.
 struct BlochLayout {
-    size_t Mf[3], Mi[3], lam[3], Bf[3], Bi[3], f, P, F, Pmax, Fmax, mx0, mx1, A, B, partial, total;
+    size_t Mf[3], Mi[3], lam[3], Bf[3], Bi[3], f, P, F, Pmax, Fmax, mx0, mx1, mid, A, B, partial, total;
     long long chunk;
 };
 
@@ -2376,6 +2376,8 @@ BlochLayout bloch_layout(const kx_plan *p, int n_orb, int n_vec, int n_kpt, size
     off += f32 ? al256(sizeof(float) * chunk) : 0;
     L.mx1 = off;
     off += f32 ? al256(sizeof(float) * chunk) : 0;
+    L.mid = off;  // tiles' maxima between fused products, 32 per item, two sets
+    off += f32 && bp_fused(p) ? al256(sizeof(int) * 64 * chunk) : 0;
     L.A = off;
     off += al256(sizeof(T2) * N * chunk);
     L.B = off;
@@ -2532,21 +2534,19 @@ int bloch_sweep(kx_plan *p, int n_kpt, const double *theta, const double *wk, in
             const long long r1 = std::min(pairs, r0 + L.chunk);
             const long long R = r1 - r0;
             int rc;
-            T2 *X = B;  // the solved chunk
             if constexpr (sizeof(T) == 4) {
                 auto Bf = [&](int a) { return reinterpret_cast<const __half *>(ws + L.Bf[a]); };
                 auto Bi = [&](int a) { return reinterpret_cast<const __half *>(ws + L.Bi[a]); };
                 if (bp_fused(p)) {
-                    // axes 1 and 2 two products at a time, on planes; axis 3 between them
+                    // two products at a time; the items' and tiles' maxima zeroed together
                     float *mx0 = reinterpret_cast<float *>(ws + L.mx0), *mx1 = reinterpret_cast<float *>(ws + L.mx1);
+                    int *mid = reinterpret_cast<int *>(ws + L.mid);
+                    KX_CUDA_TRY(cudaMemsetAsync(mx0, 0, L.A - L.mx0, s));
                     if ((rc = bloch_fused_forward(p, R, Pq, F, B, Bf(0), Bf(1), reinterpret_cast<const float *>(ws + L.Pmax),
                                                   reinterpret_cast<const float *>(ws + L.Fmax), r0, n_orb, mx0, s)))
                         return rc;
-                    if ((rc = launch_bp<1>(p, 2, R, B, A, Bf(2), f, mx0, nullptr, nullptr, 0, n_orb, mx1, s))) return rc;
-                    if ((rc = launch_bp<0>(p, 2, R, A, B, Bi(2), nullptr, mx1, nullptr, nullptr, 0, n_orb, mx0, s)))
-                        return rc;
-                    rc = bloch_fused_inverse(p, R, B, A, Bi(1), Bi(0), mx0, s);
-                    X = A;
+                    if ((rc = bloch_fused_middle(p, R, B, A, Bf(2), Bi(2), f, mx0, mid, mx1, s))) return rc;
+                    rc = bloch_fused_inverse(p, R, A, B, Bi(1), Bi(0), mx1, mid + 32 * R, s);
                 } else if (bp0_axis(p))
                     rc = launch_bp0<true>(p, R, nullptr, A, Bf(0), Pq, F, nullptr, reinterpret_cast<const float *>(ws + L.Pmax),
                                           reinterpret_cast<const float *>(ws + L.Fmax), r0, n_orb, s);
@@ -2611,7 +2611,7 @@ int bloch_sweep(kx_plan *p, int n_kpt, const double *theta, const double *wk, in
             const bool both = sizeof(T) == 4 && n_orb <= 24 && N % 2 == 0;
             if constexpr (sizeof(T) == 4) {
                 if (both) {
-                    const AccBoth acc = {X,     Pq, F, r0, r1, N, n_orb, occ_q, occ_k, wk[q], wk[k], reinterpret_cast<double2 *>(out_k),
+                    const AccBoth acc = {B,     Pq, F, r0, r1, N, n_orb, occ_q, occ_k, wk[q], wk[k], reinterpret_cast<double2 *>(out_k),
                                          out_q, p->d_status};
                     rc = n_orb <= 4    ? launch_accum_both<4>(acc, s)
                          : n_orb <= 8  ? launch_accum_both<8>(acc, s)
@@ -2628,21 +2628,21 @@ int bloch_sweep(kx_plan *p, int n_kpt, const double *theta, const double *wk, in
                 const int ab = (int)std::min<long long>((nv * N / per + 255) / 256, 8LL * p->num_sms);
                 if constexpr (sizeof(T) == 4) {
                     if (pairs2)
-                        bloch_accum2_kernel<false><<<ab, 256, 0, s>>>(X, r0, r1, n_orb, Pq, occ_q, wk[q],
+                        bloch_accum2_kernel<false><<<ab, 256, 0, s>>>(B, r0, r1, n_orb, Pq, occ_q, wk[q],
                                                                       reinterpret_cast<double2 *>(out_k), N);
                 }
                 if (!pairs2)
-                    bloch_accum_kernel<T><<<ab, 256, 0, s>>>(X, r0, r1, n_orb, Pq, occ_q, wk[q],
+                    bloch_accum_kernel<T><<<ab, 256, 0, s>>>(B, r0, r1, n_orb, Pq, occ_q, wk[q],
                                                              reinterpret_cast<double2 *>(out_k), N);
                 KX_LAUNCH_CHECK("bloch_accum_kernel launch");
                 if (reverse) {
                     const int rb = (int)std::min<long long>((n_orb * N / per + 255) / 256, 8LL * p->num_sms);
                     if constexpr (sizeof(T) == 4) {
                         if (pairs2)
-                            bloch_accum2_kernel<true><<<rb, 256, 0, s>>>(X, r0, r1, n_orb, F, occ_k, wk[k], out_q, N);
+                            bloch_accum2_kernel<true><<<rb, 256, 0, s>>>(B, r0, r1, n_orb, F, occ_k, wk[k], out_q, N);
                     }
                     if (!pairs2)
-                        bloch_accum_rev_kernel<T><<<rb, 256, 0, s>>>(X, r0, r1, n_orb, F, occ_k, wk[k], out_q, N);
+                        bloch_accum_rev_kernel<T><<<rb, 256, 0, s>>>(B, r0, r1, n_orb, F, occ_k, wk[k], out_q, N);
                     KX_LAUNCH_CHECK("bloch_accum_rev_kernel launch");
                 }
             }
@@ -2808,11 +2808,12 @@ int bloch_energy_only(kx_plan *p, int n_kpt, const double *theta, const double *
                 int rc;
                 if constexpr (sizeof(T) == 4) {
                     auto Bf = [&](int a) { return reinterpret_cast<const __half *>(ws + L.Bf[a]); };
-                    if (bp_fused(p))
+                    if (bp_fused(p)) {
+                        KX_CUDA_TRY(cudaMemsetAsync(ws + L.mx0, 0, sizeof(float) * R, s));
                         rc = bloch_fused_forward(p, R, Pq, F, B, Bf(0), Bf(1), reinterpret_cast<const float *>(ws + L.Pmax),
                                                  reinterpret_cast<const float *>(ws + L.Fmax), r0, n_orb,
                                                  reinterpret_cast<float *>(ws + L.mx0), s);
-                    else if (bp0_axis(p))
+                    } else if (bp0_axis(p))
                         rc = launch_bp0<true>(p, R, nullptr, A, Bf(0), Pq, F, nullptr, reinterpret_cast<const float *>(ws + L.Pmax),
                                               reinterpret_cast<const float *>(ws + L.Fmax), r0, n_orb, s);
                     else

@@ -238,8 +238,10 @@ int bloch_energy(kx_plan *p, int n_kpt, const double *theta, const double *wk, i
 int bloch_fused_forward(kx_plan *p, long long R, const float2 *P, const float2 *F, float2 *out, const __half *B1,
                         const __half *B2, const float *pmax, const float *fmax, long long r0, int n_orb,
                         float *out_max, cudaStream_t s);
+int bloch_fused_middle(kx_plan *p, long long R, const float2 *in, float2 *out, const __half *Bf, const __half *Bi,
+                       const float *f, const float *in_max, int *mid, float *out_max, cudaStream_t s);
 int bloch_fused_inverse(kx_plan *p, long long R, const float2 *in, float2 *out, const __half *B2, const __half *B1,
-                        const float *in_max, cudaStream_t s);
+                        const float *in_max, int *mid, cudaStream_t s);
 
 // ---- multipole boundary values (kx_mp.cu)
 int mp_set(kx_plan *p, int l_max);

@@ -1153,7 +1153,7 @@ def test_kpoint_fused_products(kx, n3, bc, n_orb, counts, chunk, monkeypatch):
         assert plan.status() == kx.KX_OK
         chunks = -(-n_orb * n_orb // int(chunk)) if chunk else 1
         n_k = len(wk)
-        assert plan.profile_read()["bloch"][1] == (4 if bp == "1" else 6) * chunks * n_k * (n_k + 1) // 2
+        assert plan.profile_read()["bloch"][1] == (3 if bp == "1" else 6) * chunks * n_k * (n_k + 1) // 2
         e_only = kx.kx_energy_kpoints(plan, theta, wk, dpsi, docc).item()
         one = kx.kx_vx_apply_kpoint(plan, theta, wk, dpsi, 1, dpsi[1].contiguous(), docc)
         torch.cuda.synchronize()
