@@ -11,6 +11,7 @@
 // axes keep the plan's real eigenvectors.  The forward transform contracts with
 // conj(Vk), the inverse with Vk.  The six complex mode products run on the
 // tensor cores (split fp16 products, float32 plans, axes of 32 or 64 points:
+// two products per kernel, kx_bloch_fused.cu, on planes of 64 x 64 points; else
 // the pass kernels with per-item scales, bloch_pass_kernel and
 // bloch_pass0_kernel, when every axis qualifies, else bloch_tc_ws_kernel with
 // per-tile scales) or on the CUDA cores (float64 for KX_FP64 plans, float32 with

@@ -16,8 +16,8 @@
 //        back with V1^T                                       [A K-major]
 //   X2I  contract k2 with V2^T                                [A MN-major]
 //   X3I  contract k3 with V3^T, write phi (pair mode) or f(L)b (vector mode)
-// then acc_kernel adds g_j psi_j phi_ij and g_i psi_i phi_ij into the fp32
-// accumulators, one thread per four grid points, group by group.
+// then acc_kernel adds g_j psi_j phi_ij and g_i psi_i phi_ij, group by group, one thread
+// per four grid points with a block of orbitals and their sums resident.
 //
 // Each pass kernel is persistent (one CTA per SM) and warp-specialised:
 //   warps 0-7   epilogue (TMEM lane quadrant = warp % 4, one tile row per
@@ -55,8 +55,8 @@ constexpr int kMetaRing = 8;  // >= the tiles a producer can be ahead of the epi
 constexpr int kMaxStages = 4;
 constexpr size_t kSmemBudget = 218 * 1024;  // dynamic; ~7 KB of static shared memory beside it
 
-// Optional per-role cycle counters (compile with -DKX_ROLE_CLOCKS): each CTA
-// writes kClk counters to PassArgs::clk[blockIdx.x * kClk + k].
+// Optional per-role cycle counters of the pass kernels (compile with -DKX_ROLE_CLOCKS): each
+// CTA writes kClk counters to PassArgs::clk[blockIdx.x * kClk + k].
 constexpr int kClk = 12;
 #ifdef KX_ROLE_CLOCKS
 long long *g_clkbuf = nullptr;
@@ -853,7 +853,6 @@ struct SlabArgs {
     int nbuf;               // A buffers (2 or 3)
     int *status;
     long long timeout_cycles;
-    long long *clk;         // role counters (only with KX_ROLE_CLOCKS)
 };
 
 constexpr int kSlabU = 6;            // producer loads in flight per thread
@@ -1735,7 +1734,7 @@ int launch_pass(const kx_plan *p, PassArgs a, int axis, cudaStream_t s, int *gri
     a.status = p->d_status;
     a.timeout_cycles = 4000000000LL;  // ~2 s at the SM clock
 #ifdef KX_ROLE_CLOCKS
-    if (!g_clkbuf) cudaMallocManaged(&g_clkbuf, sizeof(long long) * kClk * 4096 * 6);
+    if (!g_clkbuf) cudaMallocManaged(&g_clkbuf, sizeof(long long) * kClk * 4096 * 5);
     a.clk = g_clkbuf + (long long)PASS * kClk * 4096;
 #endif
     a.stages = pass_stages(a.np, false);  // X1's mid operand reuses its tile's A stage
@@ -1810,10 +1809,6 @@ int launch_slab(kx_plan *p, long R, const float *in, const float *in_max, float 
     a.rhs_mode = rhs_mode;
     a.status = p->d_status;
     a.timeout_cycles = 4000000000LL;  // ~2 s at the SM clock
-#ifdef KX_ROLE_CLOCKS
-    if (!g_clkbuf) cudaMallocManaged(&g_clkbuf, sizeof(long long) * kClk * 4096 * 6);
-    a.clk = g_clkbuf + 5LL * kClk * 4096;
-#endif
     a.share_v = same_axes12(p) ? 1 : 0;
     const size_t base = (size_t)4 * a.np1 * a.np1 + (a.share_v ? 0 : (size_t)4 * a.np2 * a.np2) + 1024;
     const size_t buffer = 2 * slab_half_bytes(std::max(a.np1, a.np2));
