@@ -506,7 +506,7 @@ __global__ void __launch_bounds__(256, 2) combine32_bulk_kernel(const double *__
     const int nch = (na + kDR - 1) / kDR;
     const int ntiles = (int)((N + kDX - 1) / kDX);
     const int my_tiles = ntiles > (int)blockIdx.x ? (ntiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : 0;
-    const int nitems = my_tiles * nch;  // N < 2^21: items stay far below 2^31
+    const int nitems = my_tiles * nch;  // N <= 2^21: items stay far below 2^31
     if (tid == 0) {
         for (int i = 0; i < kDStages; ++i) ptx::mbar_init(&full[i], 1);
         ptx::fence_mbar_init();
