@@ -606,11 +606,29 @@ __global__ void __launch_bounds__(kThreads, 1) tc_pass_kernel(const PassArgs a) 
         for (int it = grp; it < n_my; it += kProdGroups) {  // groups take alternate tiles
             const int s = it % S, r = it % kMetaRing;
             long long tw = KX_CLK_NOW();
-            if (it >= S && !wait_bar_warp(&bars.empty[s], (uint32_t)(((it / S) - 1) & 1), a, &s_abort)) break;
-            KX_CLK_ADD(1, tw);
-            tw = KX_CLK_NOW();
             if (!wait_bar_warp(&bars.meta_full[r], (uint32_t)((it / kMetaRing) & 1), a, &s_abort)) break;
             KX_CLK_ADD(2, tw);
+            // the tile into L2 while its stage is still in use: the producers' loads start from
+            // memory only then (X3I 2.59 -> 2.22 ms per apply at 96^3 / 64 orbitals, the separate
+            // passes at 120 x 112 x 120 / 16: X2F 0.37 -> 0.31, X1, which holds a stage through
+            // both of its products, 0.79 -> 0.72 ms).  X3F's orbitals are in L2 already.
+            if (PASS == P_X1) {
+                const int row8 = 8 * a.n1;  // eight contiguous rows per group
+                for (int e = 32 * gtid; e < 16 * row8; e += 32 * kGroupThreads) {
+                    const int g = e / row8;
+                    if (smeta[r].p0[g] != nullptr) ptx::prefetch_l2(smeta[r].p0[g] + (e - g * row8));
+                }
+            } else if (PASS != P_X3F || a.rhs_mode) {
+                const int g = gtid & 15;  // one prefetch per line: at its start or where a run of groups begins
+                const float *p = smeta[r].p0[g];
+                const long long ks = (PASS == P_X2F || PASS == P_X2I) ? a.n1 : (long long)a.n1 * a.n2;
+                if (p != nullptr && (g == 0 || p != smeta[r].p0[g - 1] + 8 ||
+                                     (reinterpret_cast<uintptr_t>(p) & 127) == 0))
+                    for (int k = gtid >> 4; k < a.nc; k += kGroupThreads / 16) ptx::prefetch_l2(p + k * ks);
+            }
+            tw = KX_CLK_NOW();
+            if (it >= S && !wait_bar_warp(&bars.empty[s], (uint32_t)(((it / S) - 1) & 1), a, &s_abort)) break;
+            KX_CLK_ADD(1, tw);
             tw = KX_CLK_NOW();
             uint8_t *Ahi = stage0 + s * stage_bytes;
             produce_tile<PASS, U>(a, smeta[r], Ahi, Ahi + half_bytes, gtid);
