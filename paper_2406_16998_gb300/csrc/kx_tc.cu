@@ -612,8 +612,12 @@ __global__ void __launch_bounds__(kThreads, 1) tc_pass_kernel(const PassArgs a) 
             // memory only then (X3I 2.59 -> 2.22 ms per apply at 96^3 / 64 orbitals, the separate
             // passes at 120 x 112 x 120 / 16: X2F 0.37 -> 0.31, X1, which holds a stage through
             // both of its products, 0.79 -> 0.72 ms).  X3F's orbitals are in L2 already.
-            if (PASS == P_X1) {
+            // Not for a first tile, which has no wait to hide it behind, and not unrolled (the
+            // longer code cost calls of a few tiles 1 of 40 us).
+            if (it < S) {
+            } else if (PASS == P_X1) {
                 const int row8 = 8 * a.n1;  // eight contiguous rows per group
+#pragma unroll 1
                 for (int e = 32 * gtid; e < 16 * row8; e += 32 * kGroupThreads) {
                     const int g = e / row8;
                     if (smeta[r].p0[g] != nullptr) ptx::prefetch_l2(smeta[r].p0[g] + (e - g * row8));
@@ -624,6 +628,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_pass_kernel(const PassArgs a) 
                 const long long ks = (PASS == P_X2F || PASS == P_X2I) ? a.n1 : (long long)a.n1 * a.n2;
                 if (p != nullptr && (g == 0 || p != smeta[r].p0[g - 1] + 8 ||
                                      (reinterpret_cast<uintptr_t>(p) & 127) == 0))
+#pragma unroll 1
                     for (int k = gtid >> 4; k < a.nc; k += kGroupThreads / 16) ptx::prefetch_l2(p + k * ks);
             }
             tw = KX_CLK_NOW();
