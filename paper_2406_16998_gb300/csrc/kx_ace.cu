@@ -495,7 +495,7 @@ __host__ __device__ constexpr size_t comb_bulk_smem(int na) {
 __global__ void __launch_bounds__(256, 2) combine32_bulk_kernel(const double *__restrict__ A, int na,
                                                                 const double *__restrict__ C, int nb, long long N,
                                                                 float sgn, bool accumulate, double *__restrict__ out,
-                                                                int *status) {
+                                                                int *status, long long wait_cycles) {
     extern __shared__ __align__(16) uint8_t smem_raw[];
     double *raw = reinterpret_cast<double *>(smem_raw);                                  // [stage][kDR][kDX]
     float *As = reinterpret_cast<float *>(raw + (size_t)kDStages * kDR * kDX);           // [2][kDR][kDX]
@@ -544,14 +544,17 @@ __global__ void __launch_bounds__(256, 2) combine32_bulk_kernel(const double *__
     int ch = 0, st = 0, tile = blockIdx.x;
     uint32_t par = 0;
     for (int i = 0; i < nitems; ++i) {
-        const bool ok = ptx::mbar_wait_bounded(&full[st], par, 2000000000LL);
+        const bool ok = wait_cycles >= 0 && ptx::mbar_wait_bounded(&full[st], par, wait_cycles);
         float *at = As + (i & 1) * kDR * kDX;
         const int rows = min(kDR, na - ch * kDR);
         const double *src = raw + st * kDR * kDX + tid;
 #pragma unroll
         for (int r = 0; r < kDR; ++r) at[r * kDX + tid] = ok && r < rows ? f64_to_f32(src[r * kDX]) : 0.f;
         if (!ok) atomicExch(status, KX_ERR_TIMEOUT);
-        if (__syncthreads_or(!ok)) return;  // a wait gave up
+        if (__syncthreads_or(!ok)) {  // a wait gave up
+            if (tid == 0) ptx::bulk_ring_drain(full, kDStages, i, min(nitems, i + kDStages), kWaitCycles);
+            return;
+        }
         if (tid == 0 && i + kDStages < nitems) issue_next();  // every thread has read this stage
         if (++st == kDStages) {
             st = 0;
@@ -664,7 +667,8 @@ int launch_combination(kx_plan *p, const double *A, int na, const double *C, int
         if (bulk) {
             KX_CUDA_TRY(cudaFuncSetAttribute(combine32_bulk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)smem));
-            combine32_bulk_kernel<<<grid, 256, smem, s>>>(A, na, C, nb, N, fs, accumulate, out, p->d_status);
+            combine32_bulk_kernel<<<grid, 256, smem, s>>>(A, na, C, nb, N, fs, accumulate, out, p->d_status,
+                                                          ring_wait_cycles());
         } else {
             KX_CUDA_TRY(cudaFuncSetAttribute(combine32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
             combine32_kernel<<<grid, 256, smem, s>>>(A, na, C, nb, N, fs, accumulate, out);

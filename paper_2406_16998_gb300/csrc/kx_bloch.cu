@@ -1847,6 +1847,7 @@ struct AccBoth {
     double wq, wk;
     double2 *out_k, *out_q;
     int *status;
+    long long wait_cycles;
 };
 
 // a b - c d and a b + c d, rounded as the compiler rounds them in the kernels above
@@ -1908,7 +1909,8 @@ __global__ void __launch_bounds__(kAccPoints) bloch_accum_both_kernel(const AccB
         const float2 f = f_next;
         const float ck = REV ? (float)(a.wk * w_next) : 0.f;
         if (v < v_hi) next(v + 1);
-        const bool ok = ptx::mbar_wait_bounded(&full[i % kAccStages], (uint32_t)((i / kAccStages) & 1), 2000000000LL);
+        const bool ok = a.wait_cycles >= 0 && ptx::mbar_wait_bounded(&full[i % kAccStages],
+                                                                     (uint32_t)((i / kAccStages) & 1), a.wait_cycles);
         if (ok) {
             const float2 *xs = ring + (i % kAccStages) * MB * kAccPoints + tid;
             float sr = 0.f, si = 0.f;
@@ -1930,7 +1932,11 @@ __global__ void __launch_bounds__(kAccPoints) bloch_accum_both_kernel(const AccB
         } else {
             atomicExch(a.status, KX_ERR_TIMEOUT);
         }
-        if (__syncthreads_or(!ok)) break;  // every thread is done with this stage, or a wait gave up
+        if (__syncthreads_or(!ok)) {  // every thread is done with this stage, or a wait gave up
+            if (tid == 0)
+                ptx::bulk_ring_drain(full, kAccStages, i, min(v_hi - v_lo + 1, i + kAccStages), kWaitCycles);
+            break;
+        }
         if (tid == 0 && v + kAccStages <= v_hi) fill(v + kAccStages);
     }
     if constexpr (REV) {
@@ -2613,7 +2619,7 @@ int bloch_sweep(kx_plan *p, int n_kpt, const double *theta, const double *wk, in
             if constexpr (sizeof(T) == 4) {
                 if (both) {
                     const AccBoth acc = {B,     Pq, F, r0, r1, N, n_orb, occ_q, occ_k, wk[q], wk[k], reinterpret_cast<double2 *>(out_k),
-                                         out_q, p->d_status};
+                                         out_q, p->d_status, ring_wait_cycles()};
                     rc = n_orb <= 4    ? launch_accum_both<4>(acc, s)
                          : n_orb <= 8  ? launch_accum_both<8>(acc, s)
                          : n_orb <= 16 ? launch_accum_both<16>(acc, s)

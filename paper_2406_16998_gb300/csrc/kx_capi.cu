@@ -31,12 +31,15 @@ int cuda_error(cudaError_t e, const char *what) {
     return set_error(code, std::string(what) + ": " + cudaGetErrorString(e));
 }
 
-// Host-side fault injection for the failure-path tests: KX_FAULT=alloc makes the
-// next workspace allocation report KX_ERR_NOMEM without touching the device.
-static bool fault_alloc() {
+// Host-side fault injection for the failure-path tests, read at each call: KX_FAULT=alloc
+// makes the next workspace allocation report KX_ERR_NOMEM without touching the device,
+// KX_FAULT=wait makes the kernels with a ring of bulk copies give up their first wait.
+static bool fault(const char *what) {
     const char *f = std::getenv("KX_FAULT");
-    return f && std::strcmp(f, "alloc") == 0;
+    return f && std::strcmp(f, what) == 0;
 }
+static bool fault_alloc() { return fault("alloc"); }
+long long ring_wait_cycles() { return fault("wait") ? -1 : kWaitCycles; }
 
 int ensure_workspace(kx_plan *p, size_t bytes) {
     if (p->ws.bytes >= bytes) return KX_OK;
