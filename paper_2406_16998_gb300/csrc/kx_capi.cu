@@ -80,7 +80,6 @@ int leading_columns(int nb) {
 // With p->blk_mode set, the block pairs of p->blk_req (I <= J each, in the
 // given order) are enumerated instead, each whole; begin / end are ignored.
 int ensure_pairs(kx_plan *p, int n_orb, cudaStream_t s, long long begin, long long end) {
-    (void)s;
     const long long P_all = (long long)n_orb * (n_orb + 1) / 2;
     if (end < 0) end = P_all;
     if (p->blk_mode) {
@@ -90,7 +89,6 @@ int ensure_pairs(kx_plan *p, int n_orb, cudaStream_t s, long long begin, long lo
     } else if (p->ws_norb == n_orb && p->blk_cur.empty() && p->pr_begin == begin && p->pr_end == end) {
         return KX_OK;
     }
-    ++p->config_version;  // the list is rebuilt in place
     std::vector<int> pairs, slots;
     std::vector<Group> groups;
     std::vector<int> first;
@@ -155,48 +153,56 @@ int ensure_pairs(kx_plan *p, int n_orb, cudaStream_t s, long long begin, long lo
                 span[2 * o + 1] = (int)gi;
                 maxorb[gi] = std::max(maxorb[gi], o);
             }
-    const size_t P = pairs.size() / 2;
-    if (P > p->pairs_cap) {
-        cudaFree(p->d_pairs);
-        cudaFree(p->d_item_slot);
-        p->d_pairs = p->d_item_slot = nullptr;
-        p->pairs_cap = 0;
-        cudaError_t e = cudaMalloc(&p->d_pairs, sizeof(int) * 2 * std::max<size_t>(P, 1));
-        if (e == cudaSuccess) e = cudaMalloc(&p->d_item_slot, sizeof(int) * 2 * std::max<size_t>(P, 1));
-        if (e != cudaSuccess) return cuda_error(e, "pair list cudaMalloc");
-        p->pairs_cap = P;
+    // one block for all tables: one allocation and one copy a list
+    size_t bytes = 0;
+    auto place = [&](size_t n) {
+        const size_t at = bytes;
+        bytes += (n + 15) & ~size_t(15);
+        return at;
+    };
+    const size_t at_pairs = place(sizeof(int) * pairs.size()), at_slots = place(sizeof(int) * slots.size());
+    const size_t at_groups = place(sizeof(Group) * groups.size()), at_span = place(sizeof(int) * span.size());
+    const size_t at_mask = place(mask.size());
+    std::vector<unsigned char> host(bytes);
+    auto put = [&](size_t at, const void *src, size_t n) {
+        if (n) std::memcpy(host.data() + at, src, n);
+    };
+    put(at_pairs, pairs.data(), sizeof(int) * pairs.size());
+    put(at_slots, slots.data(), sizeof(int) * slots.size());
+    put(at_groups, groups.data(), sizeof(Group) * groups.size());
+    put(at_span, span.data(), sizeof(int) * span.size());
+    put(at_mask, mask.data(), mask.size());
+    // Kernels queued earlier may still read the old tables, and the copy of the old host
+    // block may not have run: both are on s, or ordered before it.  A stream being captured
+    // takes a blocking copy instead (refused by the runtime where the capture forbids it).
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    KX_CUDA_TRY(cudaStreamIsCapturing(s, &cap));
+    if (cap == cudaStreamCaptureStatusNone) KX_CUDA_TRY(cudaStreamSynchronize(s));
+    // from here on the old list is gone, whatever fails below
+    p->ws_norb = -1;
+    ++p->config_version;
+    if (bytes > p->tables.bytes) {
+        cudaFree(p->tables.ptr);
+        p->tables = Workspace();
+        if (fault_alloc()) return set_error(KX_ERR_NOMEM, "pair table allocation failed (injected by KX_FAULT=alloc)");
+        cudaError_t e = cudaMalloc(&p->tables.ptr, bytes);
+        if (e != cudaSuccess) {
+            p->tables.ptr = nullptr;
+            return cuda_error(e, "pair table cudaMalloc");
+        }
+        p->tables.bytes = bytes;
     }
-    if (groups.size() > p->groups_cap) {
-        cudaFree(p->d_groups);
-        p->d_groups = nullptr;
-        p->groups_cap = 0;
-        cudaError_t e = cudaMalloc(&p->d_groups, sizeof(Group) * groups.size());
-        if (e != cudaSuccess) return cuda_error(e, "group table cudaMalloc");
-        p->groups_cap = groups.size();
-    }
-    if (mask.size() > p->pair_mask_cap) {
-        cudaFree(p->d_pair_mask);
-        p->d_pair_mask = nullptr;
-        p->pair_mask_cap = 0;
-        cudaError_t e = cudaMalloc(&p->d_pair_mask, mask.size());
-        if (e != cudaSuccess) return cuda_error(e, "pair mask cudaMalloc");
-        p->pair_mask_cap = mask.size();
-    }
-    if ((size_t)n_orb > p->orb_span_cap) {
-        cudaFree(p->d_orb_span);
-        p->d_orb_span = nullptr;
-        p->orb_span_cap = 0;
-        cudaError_t e = cudaMalloc(&p->d_orb_span, sizeof(int) * 2 * n_orb);
-        if (e != cudaSuccess) return cuda_error(e, "orbital span cudaMalloc");
-        p->orb_span_cap = (size_t)n_orb;
-    }
-    KX_CUDA_TRY(cudaMemcpy(p->d_orb_span, span.data(), sizeof(int) * span.size(), cudaMemcpyHostToDevice));
-    KX_CUDA_TRY(cudaMemcpy(p->d_pair_mask, mask.data(), mask.size(), cudaMemcpyHostToDevice));
-    if (P) {
-        KX_CUDA_TRY(cudaMemcpy(p->d_pairs, pairs.data(), sizeof(int) * 2 * P, cudaMemcpyHostToDevice));
-        KX_CUDA_TRY(cudaMemcpy(p->d_item_slot, slots.data(), sizeof(int) * 2 * P, cudaMemcpyHostToDevice));
-        KX_CUDA_TRY(cudaMemcpy(p->d_groups, groups.data(), sizeof(Group) * groups.size(), cudaMemcpyHostToDevice));
-    }
+    p->h_tables.swap(host);
+    if (cap == cudaStreamCaptureStatusNone)
+        KX_CUDA_TRY(cudaMemcpyAsync(p->tables.ptr, p->h_tables.data(), bytes, cudaMemcpyHostToDevice, s));
+    else
+        KX_CUDA_TRY(cudaMemcpy(p->tables.ptr, p->h_tables.data(), bytes, cudaMemcpyHostToDevice));
+    unsigned char *d = static_cast<unsigned char *>(p->tables.ptr);
+    p->d_pairs = reinterpret_cast<int *>(d + at_pairs);
+    p->d_item_slot = reinterpret_cast<int *>(d + at_slots);
+    p->d_groups = reinterpret_cast<int *>(d + at_groups);
+    p->d_orb_span = reinterpret_cast<int *>(d + at_span);
+    p->d_pair_mask = d + at_mask;
     p->h_group_first = first;
     p->h_orb_last = last;
     p->h_group_maxorb = maxorb;
@@ -239,8 +245,8 @@ int prof_end(kx_plan *p, cudaStream_t s) {
     return KX_OK;
 }
 
-static int reserve(kx_plan *p, int n_orb) {
-    int rc = ensure_pairs(p, n_orb, nullptr);
+static int reserve(kx_plan *p, int n_orb, cudaStream_t s) {
+    int rc = ensure_pairs(p, n_orb, s);
     if (rc) return rc;
     if ((rc = mp_reserve(p, n_orb))) return rc;
     if (p->precision == KX_FP64) {
@@ -835,14 +841,15 @@ int kx_batch_create(int n_sys, kx_plan *const *plans, const int *n_orb, kx_batch
         }
     }
     for (int i = 0; i < n_sys; ++i) {
-        int rc = reserve(plans[i], n_orb[i]);
+        int rc = reserve(plans[i], n_orb[i], nullptr);
         if (rc) {
             delete b;
             return rc;
         }
     }
     cudaGetDevice(&b->device);
-    cudaError_t e = cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking);
+    cudaError_t e = cudaStreamSynchronize(nullptr);  // the pair tables are there, whatever stream the batch runs on
+    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking);
     if (e != cudaSuccess) {
         delete b;
         return cuda_error(e, "kx_batch_create: stream");
@@ -866,7 +873,7 @@ int kx_batch_run(kx_batch *batch, const double *const *psi, double *const *vx_ps
         // the plans may have been used or reconfigured since the last capture:
         // restore each one's full pair list and buffers outside the capture
         for (int i = 0; i < n; ++i)
-            if (int rc = reserve(batch->plans[i], batch->n_orb[i])) return rc;
+            if (int rc = reserve(batch->plans[i], batch->n_orb[i], reinterpret_cast<cudaStream_t>(stream))) return rc;
         KX_CUDA_TRY(cudaStreamBeginCapture(batch->cap, cudaStreamCaptureModeThreadLocal));
         int rc = KX_OK;
         for (int i = 0; i < n && rc == KX_OK; ++i)

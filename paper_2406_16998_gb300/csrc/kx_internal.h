@@ -138,12 +138,15 @@ struct kx_plan_s {
     // blk_cur is the list the current enumeration was built from (empty: range)
     bool blk_mode = false;
     std::vector<int> blk_req, blk_cur;
+    // the tables of the list, all in `tables` (uploaded from h_tables, which the copy may
+    // still be reading until the next list)
+    kx::Workspace tables;
+    std::vector<unsigned char> h_tables;
     int *d_pairs = nullptr;       // int2 per item (i, j), i <= j
     int *d_item_slot = nullptr;   // int2 per item: slots of i and j inside its group
     int *d_groups = nullptr;      // kx::Group per group
     int *d_orb_span = nullptr;    // int2 per orbital: its first and last group (-1: none)
-    size_t orb_span_cap = 0;
-    size_t pairs_cap = 0, groups_cap = 0;
+    unsigned char *d_pair_mask = nullptr;  // pair {i, j} in the current range (n_orb x n_orb bytes, symmetric)
     std::vector<int> h_group_first;  // first item of each group (+ sentinel)
     std::vector<int> h_orb_last;     // per orbital: index of the last group that touches it (-1: none)
     kx::Profiler prof;
@@ -156,9 +159,6 @@ struct kx_plan_s {
     cudaStream_t h2d_stream = nullptr;
     std::vector<cudaEvent_t> h2d_events;
     std::vector<int> h_group_maxorb;          // per group: its largest orbital index
-    // pair {i, j} in the current pair range (n_orb x n_orb bytes, symmetric)
-    unsigned char *d_pair_mask = nullptr;
-    size_t pair_mask_cap = 0;
     // multipole boundary values (kx_plan_set_multipole): order, number of
     // harmonics K = (l_max + 1)^2, and per harmonic the regular solid harmonic
     // R_k and the correction field h_k on the grid (K x N, float64 and float32)

@@ -292,12 +292,7 @@ void plan_free(kx_plan *p) {
     cudaFree(p->d_status);
     cudaFree(p->ws.ptr);
     cudaFree(p->ws_host.ptr);
-    cudaFree(p->d_pairs);
-    cudaFree(p->d_item_slot);
-    cudaFree(p->d_groups);
-    cudaFree(p->d_orb_span);
-    cudaFree(p->d_pair_mask);
-    p->d_pair_mask = nullptr;
+    cudaFree(p->tables.ptr);
     mp_free(p);
     for (cudaEvent_t e : p->copy_events) cudaEventDestroy(e);
     p->copy_events.clear();
