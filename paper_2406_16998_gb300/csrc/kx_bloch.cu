@@ -2279,8 +2279,16 @@ inline bool bp0_axis(const kx_plan *p) {
 // Two products per kernel (kx_bloch_fused.cu): planes of 64 x 64 points, two of which are
 // a tile of 128 rows (1428 -> 873 us for the six products of 256 pairs at 64^3).  A
 // plane of 32-point axes would fill half the tile's columns and leave the kernel's time
-// per value as it is, so those sizes keep the single products.
-inline bool bp_fused(const kx_plan *p) { return bp_axes(p) && tc_axis(p, 0) && p->n[0] == 64 && p->n[1] == 64; }
+// per value as it is, and other axes have no tensor-core product at all (tc_axis), so those
+// sizes keep the single products; so does a device too small for CTAs that wait for each
+// other (bloch_fused_fits), and KX_BLOCH_FUSED=0 (comparison runs).
+inline int bp_fused(const kx_plan *p, bool *fused) {
+    *fused = false;
+    if (const char *e = std::getenv("KX_BLOCH_FUSED"))
+        if (std::atoi(e) == 0) return KX_OK;
+    if (!(bp_axes(p) && tc_axis(p, 0) && p->n[0] == 64 && p->n[1] == 64)) return KX_OK;
+    return bloch_fused_fits(p, fused);
+}
 
 template <bool FORM>
 int launch_bp0(kx_plan *p, long long R, const float2 *in, float2 *out, const __half *Bs, const float2 *P,
@@ -2340,7 +2348,7 @@ struct BlochLayout {
 };
 
 template <typename T>
-BlochLayout bloch_layout(const kx_plan *p, int n_orb, int n_vec, int n_kpt, size_t partial_doubles = 0) {
+BlochLayout bloch_layout(const kx_plan *p, int n_orb, int n_vec, int n_kpt, bool fused, size_t partial_doubles = 0) {
     using T2 = typename Cx<T>::t;
     BlochLayout L;
     const size_t N = p->N;
@@ -2384,7 +2392,7 @@ BlochLayout bloch_layout(const kx_plan *p, int n_orb, int n_vec, int n_kpt, size
     L.mx1 = off;
     off += f32 ? al256(sizeof(float) * chunk) : 0;
     L.mid = off;  // tiles' maxima between fused products, 32 per item, two sets
-    off += f32 && bp_fused(p) ? al256(sizeof(int) * 64 * chunk) : 0;
+    off += f32 && fused ? al256(sizeof(int) * 64 * chunk) : 0;
     L.A = off;
     off += al256(sizeof(T2) * N * chunk);
     L.B = off;
@@ -2459,7 +2467,9 @@ int bloch_sweep(kx_plan *p, int n_kpt, const double *theta, const double *wk, in
                 double *out_all, cudaStream_t s) {
     using T2 = typename Cx<T>::t;
     const long long N = (long long)p->N;
-    BlochLayout L = bloch_layout<T>(p, n_orb, n_vec, n_kpt);
+    bool fused;
+    if (int rc = bp_fused(p, &fused)) return rc;
+    BlochLayout L = bloch_layout<T>(p, n_orb, n_vec, n_kpt, fused);
     if (int rc = ensure_workspace(p, L.total)) return rc;
     char *ws = static_cast<char *>(p->ws.ptr);
     T2 *Mf[3], *Mi[3];
@@ -2544,35 +2554,45 @@ int bloch_sweep(kx_plan *p, int n_kpt, const double *theta, const double *wk, in
             if constexpr (sizeof(T) == 4) {
                 auto Bf = [&](int a) { return reinterpret_cast<const __half *>(ws + L.Bf[a]); };
                 auto Bi = [&](int a) { return reinterpret_cast<const __half *>(ws + L.Bi[a]); };
-                if (bp_fused(p)) {
+                float *mx0 = reinterpret_cast<float *>(ws + L.mx0), *mx1 = reinterpret_cast<float *>(ws + L.mx1);
+                const float *pm = reinterpret_cast<const float *>(ws + L.Pmax);
+                const float *fm = reinterpret_cast<const float *>(ws + L.Fmax);
+                int done = 0;  // products the fused kernels did: 2 leave B and mx0, 4 leave A and mx1
+                if (fused) {
                     // two products at a time; the items' and tiles' maxima zeroed together
-                    float *mx0 = reinterpret_cast<float *>(ws + L.mx0), *mx1 = reinterpret_cast<float *>(ws + L.mx1);
                     int *mid = reinterpret_cast<int *>(ws + L.mid);
                     KX_CUDA_TRY(cudaMemsetAsync(mx0, 0, L.A - L.mx0, s));
-                    if ((rc = bloch_fused_forward(p, R, Pq, F, B, Bf(0), Bf(1), reinterpret_cast<const float *>(ws + L.Pmax),
-                                                  reinterpret_cast<const float *>(ws + L.Fmax), r0, n_orb, mx0, s)))
-                        return rc;
-                    if ((rc = bloch_fused_middle(p, R, B, A, Bf(2), Bi(2), f, mx0, mid, mx1, s))) return rc;
-                    rc = bloch_fused_inverse(p, R, A, B, Bi(1), Bi(0), mx1, mid + 32 * R, s);
+                    if ((rc = bloch_fused_forward(p, R, Pq, F, B, Bf(0), Bf(1), pm, fm, r0, n_orb, mx0, s))) return rc;
+                    done = 2;
+                    rc = bloch_fused_middle(p, R, B, A, Bf(2), Bi(2), f, mx0, mid, mx1, s);
+                    if (!rc) {
+                        done = 4;
+                        rc = bloch_fused_inverse(p, R, A, B, Bi(1), Bi(0), mx1, mid + 32 * R, s);
+                        if (!rc) done = 6;
+                    }
+                    if (rc == kFusedRefused) rc = KX_OK;  // the rest by the single products
                 } else if (bp0_axis(p))
-                    rc = launch_bp0<true>(p, R, nullptr, A, Bf(0), Pq, F, nullptr, reinterpret_cast<const float *>(ws + L.Pmax),
-                                          reinterpret_cast<const float *>(ws + L.Fmax), r0, n_orb, s);
+                    rc = launch_bp0<true>(p, R, nullptr, A, Bf(0), Pq, F, nullptr, pm, fm, r0, n_orb, s);
                 else
                     rc = tc_axis(p, 0) ? launch_tc<true, 0>(p, 0, R, nullptr, A, Bf(0), nullptr, Pq, F, n_orb, r0, s)
                                        : launch_form<T>(p, R, A, Mf[0], Pq, F, n_orb, r0, s);
                 if (rc) return rc;
-                if (bp_fused(p)) {
-                    // done above
+                if (done == 6) {
+                    // all six done
                 } else if (bp_axes(p)) {
                     // axes 2 and 3 with per-item scales: the bound from the orbital
                     // maxima, then the maxima each product records
-                    float *mx0 = reinterpret_cast<float *>(ws + L.mx0), *mx1 = reinterpret_cast<float *>(ws + L.mx1);
-                    const float *pm = reinterpret_cast<const float *>(ws + L.Pmax);
-                    const float *fm = reinterpret_cast<const float *>(ws + L.Fmax);
-                    if ((rc = launch_bp<0>(p, 1, R, A, B, Bf(1), nullptr, nullptr, pm, fm, r0, n_orb, mx0, s))) return rc;
-                    if ((rc = launch_bp<1>(p, 2, R, B, A, Bf(2), f, mx0, nullptr, nullptr, 0, n_orb, mx1, s))) return rc;
-                    if ((rc = launch_bp<0>(p, 2, R, A, B, Bi(2), nullptr, mx1, nullptr, nullptr, 0, n_orb, mx0, s)))
+                    if (done < 2 &&
+                        (rc = launch_bp<0>(p, 1, R, A, B, Bf(1), nullptr, nullptr, pm, fm, r0, n_orb, mx0, s)))
                         return rc;
+                    if (done < 4) {
+                        if ((rc = launch_bp<1>(p, 2, R, B, A, Bf(2), f, mx0, nullptr, nullptr, 0, n_orb, mx1, s))) return rc;
+                        if ((rc = launch_bp<0>(p, 2, R, A, B, Bi(2), nullptr, mx1, nullptr, nullptr, 0, n_orb, mx0, s)))
+                            return rc;
+                    } else {
+                        std::swap(A, B);
+                        std::swap(mx0, mx1);
+                    }
                     if ((rc = launch_bp<0>(p, 1, R, B, A, Bi(1), nullptr, mx0, nullptr, nullptr, 0, n_orb,
                                            bp0_axis(p) ? mx1 : nullptr, s)))
                         return rc;
@@ -2593,11 +2613,10 @@ int bloch_sweep(kx_plan *p, int n_kpt, const double *theta, const double *wk, in
                              : launch_pipe<T, 0>(p, 1, R, B, A, Mi[1], nullptr, s);
                     if (rc) return rc;
                 }
-                if (bp_fused(p))
+                if (done == 6)
                     rc = KX_OK;
                 else if (bp0_axis(p))
-                    rc = launch_bp0<false>(p, R, A, B, Bi(0), nullptr, nullptr,
-                                           reinterpret_cast<const float *>(ws + L.mx1), nullptr, nullptr, 0, n_orb, s);
+                    rc = launch_bp0<false>(p, R, A, B, Bi(0), nullptr, nullptr, mx1, nullptr, nullptr, 0, n_orb, s);
                 else
                     rc = tc_axis(p, 0)
                              ? launch_tc<false, 0>(p, 0, R, A, B, Bi(0), nullptr, nullptr, nullptr, n_orb, 0, s)
@@ -2693,7 +2712,9 @@ int bloch_all(kx_plan *p, int n_kpt, const double *theta, const double *wk, int 
     // the energy partials live in the plan workspace; an empty block range ran
     // no sweep, so the workspace may still be unsized (or sized for a smaller
     // call): size it here before any kernel writes into it
-    BlochLayout L = bloch_layout<T>(p, n_orb, n_orb, n_kpt);
+    bool fused;
+    if (int rc = bp_fused(p, &fused)) return rc;
+    BlochLayout L = bloch_layout<T>(p, n_orb, n_orb, n_kpt, fused);
     if (int rc = ensure_workspace(p, L.total)) return rc;
     double *partial = reinterpret_cast<double *>(static_cast<char *>(p->ws.ptr) + L.partial);
     const int nb = 2 * p->num_sms;
@@ -2720,10 +2741,12 @@ int bloch_energy_only(kx_plan *p, int n_kpt, const double *theta, const double *
     using T2 = typename Cx<T>::t;
     const long long N = (long long)p->N;
     const long long pairs = (long long)n_orb * n_orb;
-    const long long chunk = bloch_layout<T>(p, n_orb, n_orb, n_kpt).chunk;
+    bool fused;
+    if (int rc = bp_fused(p, &fused)) return rc;
+    const long long chunk = bloch_layout<T>(p, n_orb, n_orb, n_kpt, fused).chunk;
     const long long n_launch = (pairs + chunk - 1) / chunk * ((long long)n_kpt * (n_kpt + 1) / 2);
     const size_t slot = (size_t)kBMaxPerSm * p->num_sms;
-    BlochLayout L = bloch_layout<T>(p, n_orb, n_orb, n_kpt, (size_t)n_launch * slot);
+    BlochLayout L = bloch_layout<T>(p, n_orb, n_orb, n_kpt, fused, (size_t)n_launch * slot);
     if (int rc = ensure_workspace(p, L.total)) return rc;
     char *ws = static_cast<char *>(p->ws.ptr);
     T2 *Mf[3];
@@ -2815,7 +2838,7 @@ int bloch_energy_only(kx_plan *p, int n_kpt, const double *theta, const double *
                 int rc;
                 if constexpr (sizeof(T) == 4) {
                     auto Bf = [&](int a) { return reinterpret_cast<const __half *>(ws + L.Bf[a]); };
-                    if (bp_fused(p)) {
+                    if (fused) {
                         KX_CUDA_TRY(cudaMemsetAsync(ws + L.mx0, 0, sizeof(float) * R, s));
                         rc = bloch_fused_forward(p, R, Pq, F, B, Bf(0), Bf(1), reinterpret_cast<const float *>(ws + L.Pmax),
                                                  reinterpret_cast<const float *>(ws + L.Fmax), r0, n_orb,
@@ -2831,7 +2854,7 @@ int bloch_energy_only(kx_plan *p, int n_kpt, const double *theta, const double *
                         float *mx0 = reinterpret_cast<float *>(ws + L.mx0);
                         const float *pm = reinterpret_cast<const float *>(ws + L.Pmax);
                         const float *fm = reinterpret_cast<const float *>(ws + L.Fmax);
-                        if (!bp_fused(p) &&
+                        if (!fused &&
                             (rc = launch_bp<0>(p, 1, R, A, B, Bf(1), nullptr, nullptr, pm, fm, r0, n_orb, mx0, s)))
                             return rc;
                         if ((rc = launch_bp<2>(p, 2, R, B, nullptr, Bf(2), f, mx0, nullptr, nullptr, 0, n_orb, nullptr,

@@ -611,6 +611,19 @@ __global__ void __launch_bounds__(kFuThreads, 1) bloch_fused_kernel(const FuArgs
     }
 }
 
+constexpr int kFuItemTiles = 32;  // most tiles of an item (F_MID3: 4096 / 128, F_INV21: n3 / 2)
+
+template <int KIND, int NK>
+int fused_resident(const kx_plan *p, int *ctas) {
+    int per_sm = 0;
+    KX_CUDA_TRY(cudaFuncSetAttribute(bloch_fused_kernel<KIND, NK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     fu_smem_bytes(NK)));
+    KX_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, bloch_fused_kernel<KIND, NK>, kFuThreads,
+                                                              fu_smem_bytes(NK)));
+    *ctas = std::min(*ctas, per_sm * p->num_sms);
+    return KX_OK;
+}
+
 template <int KIND, int NK>
 int launch_fused(kx_plan *p, FuArgs a, long long R, cudaStream_t s) {
     a.N = (long long)p->N;
@@ -632,14 +645,39 @@ int launch_fused(kx_plan *p, FuArgs a, long long R, cudaStream_t s) {
         bloch_fused_kernel<KIND, NK><<<grid, kFuThreads, fu_smem_bytes(NK), s>>>(a);
     } else {
         void *args[] = {&a};
-        KX_CUDA_TRY(cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(bloch_fused_kernel<KIND, NK>), grid,
-                                                dim3(kFuThreads), args, (size_t)fu_smem_bytes(NK), s));
+        const cudaError_t e =
+            cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(bloch_fused_kernel<KIND, NK>), grid,
+                                        dim3(kFuThreads), args, (size_t)fu_smem_bytes(NK), s);
+        if (e == cudaErrorCooperativeLaunchTooLarge) {
+            // the stream has fewer SMs than the device
+            cudaGetLastError();
+            p->prof.launches[PK_BLOCH] -= 1;
+            if (int rc = prof_end(p, s)) return rc;
+            return kFusedRefused;
+        }
+        KX_CUDA_TRY(e);
     }
     KX_LAUNCH_CHECK("bloch_fused_kernel launch");
     return prof_end(p, s);
 }
 
 }  // namespace
+
+// Whether F_MID3 and F_INV21 can run: their CTAs wait for each other, so they must all be
+// resident (one per SM), and a CTA must never hold two tiles of one item, as it would wait
+// for its own next tile: tiles go to the CTAs in turn and an item has up to 32 neighbouring
+// ones, so 32 CTAs are enough.  *fits = 0 on a smaller share of a device, whose calls
+// take the single products.
+int bloch_fused_fits(const kx_plan *p, bool *fits) {
+    *fits = false;
+    int coop = 0, ctas = p->num_sms;
+    KX_CUDA_TRY(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, p->device));
+    int rc = p->n[2] == 64 ? fused_resident<F_MID3, 64>(p, &ctas) : fused_resident<F_MID3, 32>(p, &ctas);
+    if (!rc) rc = fused_resident<F_INV21, 64>(p, &ctas);
+    if (rc) return rc;
+    *fits = coop && ctas >= p->num_sms && ctas >= kFuItemTiles;
+    return KX_OK;
+}
 
 // items [r0, r0 + R): conj(P_m) F_v, both plane axes forward, into out; per-item maxima into out_max (zeroed)
 int bloch_fused_forward(kx_plan *p, long long R, const float2 *P, const float2 *F, float2 *out, const __half *B1,

@@ -238,7 +238,10 @@ int bloch_vx_all(kx_plan *p, int n_kpt, const double *theta, const double *wk, i
 // E_x alone into ex[0] (forward transforms and Parseval).
 int bloch_energy(kx_plan *p, int n_kpt, const double *theta, const double *wk, int n_orb, const double *psi,
                  const double *occ, double *ex, cudaStream_t s);
-// two products per kernel (kx_bloch_fused.cu)
+// two products per kernel (kx_bloch_fused.cu); the second and third return kFusedRefused,
+// with nothing launched, where their CTAs cannot all be resident
+constexpr int kFusedRefused = -1;
+int bloch_fused_fits(const kx_plan *p, bool *fits);
 int bloch_fused_forward(kx_plan *p, long long R, const float2 *P, const float2 *F, float2 *out, const __half *B1,
                         const __half *B2, const float *pmax, const float *fmax, long long r0, int n_orb,
                         float *out_max, cudaStream_t s);

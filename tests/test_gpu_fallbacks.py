@@ -1,10 +1,12 @@
 """GPU tests of the ways out: waits that give up, devices smaller than a kernel wants,
 state after a failed allocation."""
+import ctypes
+import os
+import subprocess
+
 import numpy as np
 import pytest
 
-import oracle
-import workloads
 from workloads import DIRICHLET as D, PERIODIC as P, UNSCREENED as U, SCREENED as S
 
 torch = pytest.importorskip("torch")
@@ -19,6 +21,18 @@ def kx():
     build.build()
     import paper_2406_16998_gb300 as k
     return k
+
+
+@pytest.fixture(scope="module")
+def hooks(kx, tmp_path_factory):
+    """plan_hooks.cu, compiled against the library."""
+    from paper_2406_16998_gb300 import build
+    here = os.path.dirname(os.path.abspath(__file__))
+    out = str(tmp_path_factory.mktemp("hooks") / "plan_hooks.so")
+    cmd = [build.nvcc(), *build.ARCH, *build.FLAGS, "-I", build.CSRC, "-shared", os.path.join(here, "plan_hooks.cu"),
+           build.LIB, "-lcudart", "-o", out, "-Xlinker", "-rpath", "-Xlinker", os.path.dirname(build.LIB)]
+    subprocess.run(cmd, check=True, capture_output=True, text=True)
+    return ctypes.CDLL(out)
 
 
 def rand(*shape, seed=1, cplx=False):
@@ -89,3 +103,63 @@ def test_pair_lists_in_turn_on_a_side_stream(kx, prec):
     assert plan.status() == kx.KX_OK
     for i, (vx, ex) in enumerate(got):
         assert torch.equal(vx, want[i % 4][0]) and torch.equal(ex, want[i % 4][1])
+
+
+# bands, third axis, boundaries and k-points of a plane of 64 x 64 points, where two
+# products run per kernel
+FUSED = [(3, 64, (P, P, D), U, 3, None), (4, 32, (P, D, P), U, 2, "5"), (3, 64, (P, P, P), S, 2, "7"),
+         (1, 32, (D, P, P), S, 2, None)]
+
+
+def fused_case(kx, n_orb, n3, bc, kind, nk):
+    plan = kx.Plan((64, 64, n3), (0.3, 0.35, 0.4), bc, kind, precision=1)
+    theta = np.random.default_rng(n3).uniform(-3, 3, (nk, 3))
+    # bands of very different sizes: the splits' scales span many octaves
+    psi = rand(nk, n_orb, plan.N, seed=n3, cplx=True) * torch.logspace(-4, 3, n_orb, device="cuda")[:, None]
+    wk = [1.0 / nk] * nk
+
+    def run():
+        vx, ex = kx.kx_vx_kpoints(plan, theta, wk, psi)
+        one = kx.kx_vx_apply_kpoint(plan, theta, wk, psi, nk - 1, psi[0].contiguous())
+        e_only = kx.kx_energy_kpoints(plan, theta, wk, psi)
+        launches = plan.profile_read()["bloch"][1]
+        assert plan.status() == kx.KX_OK
+        return [vx, one, ex, e_only], launches
+
+    plan.profile(False)
+    return plan, run
+
+
+@pytest.mark.parametrize("n_orb,n3,bc,kind,nk,chunk", FUSED)
+def test_fused_kpoint_products_bit_for_bit(kx, n_orb, n3, bc, kind, nk, chunk, monkeypatch):
+    """The kernels with two products and the single products (KX_BLOCH_FUSED=0) give the same bits."""
+    if chunk:
+        monkeypatch.setenv("KX_CHUNK_PAIRS", chunk)
+    plan, run = fused_case(kx, n_orb, n3, bc, kind, nk)
+    two, n_two = run()
+    monkeypatch.setenv("KX_BLOCH_FUSED", "0")
+    one, n_one = run()
+    assert n_one - n_two > n_two  # other kernels: twice as many launches and more
+    for a, b in zip(two, one):
+        assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("sms", [16, 31, 4096])
+@pytest.mark.parametrize("n_orb,n3,bc,kind,nk,chunk", FUSED[:3])
+def test_fused_kpoint_products_on_another_share_of_the_device(kx, hooks, sms, n_orb, n3, bc, kind, nk, chunk,
+                                                              monkeypatch):
+    """With fewer SMs than an item has tiles (a CTA would wait for its own next tile), and with
+    more CTAs than the device holds at once (the launch is refused), the calls take the
+    single products and give the same bits; E_x differs by the grouping of its partial sums."""
+    if chunk:
+        monkeypatch.setenv("KX_CHUNK_PAIRS", chunk)
+    plan, run = fused_case(kx, n_orb, n3, bc, kind, nk)
+    want, _ = run()
+    old = hooks.hook_num_sms(plan.handle, sms)
+    try:
+        got, _ = run()
+    finally:
+        hooks.hook_num_sms(plan.handle, old)
+    assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
+    for a, b in zip(got[2:], want[2:]):
+        assert abs(a.item() - b.item()) < 1e-6 * abs(b.item())
