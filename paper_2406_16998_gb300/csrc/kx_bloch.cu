@@ -1958,19 +1958,12 @@ __global__ void __launch_bounds__(kAccPoints) bloch_accum_both_kernel(const AccB
 }
 
 template <int MB>
-int launch_accum_both(const AccBoth &a, cudaStream_t s) {
+int launch_accum_both(kx_plan *p, const AccBoth &a, cudaStream_t s) {
     const int smem = kAccStages * MB * kAccPoints * (int)sizeof(float2);
-    static bool attr = false;  // once per instantiation
-    if (!attr) {
-        KX_CUDA_TRY(cudaFuncSetAttribute(bloch_accum_both_kernel<MB, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         smem));
-        KX_CUDA_TRY(cudaFuncSetAttribute(bloch_accum_both_kernel<MB, false>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-        attr = true;
-    }
+    const auto kernel = a.out_q ? bloch_accum_both_kernel<MB, true> : bloch_accum_both_kernel<MB, false>;
+    if (int rc = raise_smem(p, reinterpret_cast<const void *>(kernel), smem)) return rc;
     const unsigned blocks = (unsigned)((a.N + kAccPoints - 1) / kAccPoints);
-    if (a.out_q) bloch_accum_both_kernel<MB, true><<<blocks, kAccPoints, smem, s>>>(a);
-    else bloch_accum_both_kernel<MB, false><<<blocks, kAccPoints, smem, s>>>(a);
+    kernel<<<blocks, kAccPoints, smem, s>>>(a);
     KX_LAUNCH_CHECK("bloch_accum_both_kernel launch");
     return KX_OK;
 }
@@ -2042,15 +2035,10 @@ void choose_split(int n, int *nc, int *n_split, int *U, size_t *smem) {
 }
 
 template <typename T, int U>
-int launch_form_u(unsigned blocks, size_t smem, cudaStream_t s, typename Cx<T>::t *out, int n_cols, int n,
+int launch_form_u(kx_plan *p, unsigned blocks, size_t smem, cudaStream_t s, typename Cx<T>::t *out, int n_cols, int n,
                   const typename Cx<T>::t *M, int nc, int n_split, const typename Cx<T>::t *P,
                   const typename Cx<T>::t *F, int n_orb, long long r0, long long N) {
-    static bool attr = false;  // once per instantiation
-    if (!attr) {
-        KX_CUDA_TRY(cudaFuncSetAttribute(bloch_form_kernel<T, U>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         200 * 1024));
-        attr = true;
-    }
+    if (int rc = raise_smem(p, reinterpret_cast<const void *>(bloch_form_kernel<T, U>), 200 * 1024)) return rc;
     bloch_form_kernel<T, U><<<blocks, kBThreads, smem, s>>>(out, n_cols, n, M, nc, n_split, P, F, n_orb, r0, N);
     KX_LAUNCH_CHECK("bloch_form_kernel launch");
     return KX_OK;
@@ -2073,7 +2061,7 @@ int launch_form(kx_plan *p, long long R, typename Cx<T>::t *out, const typename 
     if (int rc = prof_begin(p, PK_BLOCH, s)) return rc;
     const unsigned b = (unsigned)blocks;
     const int nco = (int)n_cols;
-#define KX_BLOCH_FORM(UU) launch_form_u<T, UU>(b, smem, s, out, nco, n, M, nc, n_split, P, F, n_orb, r0, N)
+#define KX_BLOCH_FORM(UU) launch_form_u<T, UU>(p, b, smem, s, out, nco, n, M, nc, n_split, P, F, n_orb, r0, N)
     int rc;
     if (U == 2) rc = KX_BLOCH_FORM(2);
     else if (U == 4) rc = KX_BLOCH_FORM(4);
@@ -2113,16 +2101,11 @@ template <typename T, int EPI, int U>
 int launch_pipe_u(kx_plan *p, long long n_tiles, size_t smem, cudaStream_t s, const typename Cx<T>::t *in,
                   typename Cx<T>::t *out, int n_cols, int n, int inner, const typename Cx<T>::t *M, int nc,
                   int n_split, const T *f, const EnergyArgs &ea) {
-    static int per_sm = 0;  // resident CTAs per SM at this instantiation's shared memory (set once)
-    static size_t per_sm_smem = 0;
-    if (per_sm == 0 || per_sm_smem != smem) {
-        KX_CUDA_TRY(cudaFuncSetAttribute(bloch_mode_pipe_kernel<T, EPI, U>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBSmemPipeMax));
-        KX_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, bloch_mode_pipe_kernel<T, EPI, U>,
-                                                                  kBThreads, smem));
-        per_sm = std::max(per_sm, 1);
-        per_sm_smem = smem;
-    }
+    const void *kernel = reinterpret_cast<const void *>(bloch_mode_pipe_kernel<T, EPI, U>);
+    int per_sm = 0;
+    if (int rc = raise_smem(p, kernel, kBSmemPipeMax)) return rc;
+    if (int rc = resident_ctas(p, kernel, kBThreads, smem, &per_sm)) return rc;
+    per_sm = std::max(per_sm, 1);
     const long long per_split =
         std::max(1LL, std::min(n_tiles, (long long)std::min(per_sm, kBMaxPerSm) * p->num_sms / n_split));
     const unsigned blocks = (unsigned)(per_split * n_split);
@@ -2192,21 +2175,12 @@ int launch_tc(kx_plan *p, int axis, long long R, const float2 *in, float2 *out, 
     const long long n_tiles = (n_cols + 127) / 128;
     const int grid = (int)std::min<long long>(n_tiles, p->num_sms);
     const size_t smem = tc_smem_bytes(n);
-    static bool attr = false;  // once per instantiation
-    if (!attr) {
-        KX_CUDA_TRY(cudaFuncSetAttribute(bloch_tc_kernel<FORM, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)tc_smem_bytes(kTcMaxN)));
-        attr = true;
-    }
     // warp-specialised form unless KX_BLOCH_WS=0 (comparison runs)
     const char *ws_env = std::getenv("KX_BLOCH_WS");
     const bool ws = !(ws_env && std::atoi(ws_env) == 0);
-    static bool attr_ws = false;
-    if (ws && !attr_ws) {
-        KX_CUDA_TRY(cudaFuncSetAttribute(bloch_tc_ws_kernel<FORM, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)tc_smem_bytes(kTcMaxN)));
-        attr_ws = true;
-    }
+    const void *kernel = ws ? reinterpret_cast<const void *>(bloch_tc_ws_kernel<FORM, EPI>)
+                            : reinterpret_cast<const void *>(bloch_tc_kernel<FORM, EPI>);
+    if (int rc = raise_smem(p, kernel, tc_smem_bytes(kTcMaxN))) return rc;
     if (int rc = prof_begin(p, PK_BLOCH, s)) return rc;
     if (ws)
         bloch_tc_ws_kernel<FORM, EPI><<<grid, kTwThreads, smem, s>>>(in, out, (int)n_cols, n, inner, Bs, f, P, F,
@@ -2256,12 +2230,8 @@ int launch_bp(kx_plan *p, int axis, long long R, const float2 *in, float2 *out, 
     const long long n_tiles = (a.n_cols + 127) / 128;
     if (n_tiles == 0) return KX_OK;
     if (out_max) KX_CUDA_TRY(cudaMemsetAsync(out_max, 0, sizeof(float) * R, s));
-    static bool attr = false;  // once per instantiation
-    if (!attr) {
-        KX_CUDA_TRY(cudaFuncSetAttribute(bloch_pass_kernel<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)bp_smem_bytes(kTcMaxN)));
-        attr = true;
-    }
+    if (int rc = raise_smem(p, reinterpret_cast<const void *>(bloch_pass_kernel<EPI>), bp_smem_bytes(kTcMaxN)))
+        return rc;
     const int grid = (int)std::min<long long>(n_tiles, p->num_sms);
     if (int rc = prof_begin(p, PK_BLOCH, s)) return rc;
     bloch_pass_kernel<EPI><<<grid, kBpThreads, bp_smem_bytes(n), s>>>(a);
@@ -2282,7 +2252,7 @@ inline bool bp0_axis(const kx_plan *p) {
 // per value as it is, and other axes have no tensor-core product at all (tc_axis), so those
 // sizes keep the single products; so does a device too small for CTAs that wait for each
 // other (bloch_fused_fits), and KX_BLOCH_FUSED=0 (comparison runs).
-inline int bp_fused(const kx_plan *p, bool *fused) {
+inline int bp_fused(kx_plan *p, bool *fused) {
     *fused = false;
     if (const char *e = std::getenv("KX_BLOCH_FUSED"))
         if (std::atoi(e) == 0) return KX_OK;
@@ -2317,12 +2287,8 @@ int launch_bp0(kx_plan *p, long long R, const float2 *in, float2 *out, const __h
     a.timeout_cycles = 2000000000LL;
     const long long n_tiles = (a.n_cols + 127) / 128;
     if (n_tiles == 0) return KX_OK;
-    static bool attr = false;  // once per instantiation
-    if (!attr) {
-        KX_CUDA_TRY(cudaFuncSetAttribute(bloch_pass0_kernel<FORM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)bp_smem_bytes(kTcMaxN)));
-        attr = true;
-    }
+    if (int rc = raise_smem(p, reinterpret_cast<const void *>(bloch_pass0_kernel<FORM>), bp_smem_bytes(kTcMaxN)))
+        return rc;
     const int grid = (int)std::min<long long>(n_tiles, p->num_sms);
     if (int rc = prof_begin(p, PK_BLOCH, s)) return rc;
     bloch_pass0_kernel<FORM><<<grid, kBpThreads, bp_smem_bytes(n), s>>>(a, P, F, N);
@@ -2639,10 +2605,10 @@ int bloch_sweep(kx_plan *p, int n_kpt, const double *theta, const double *wk, in
                 if (both) {
                     const AccBoth acc = {B,     Pq, F, r0, r1, N, n_orb, occ_q, occ_k, wk[q], wk[k], reinterpret_cast<double2 *>(out_k),
                                          out_q, p->d_status, ring_wait_cycles()};
-                    rc = n_orb <= 4    ? launch_accum_both<4>(acc, s)
-                         : n_orb <= 8  ? launch_accum_both<8>(acc, s)
-                         : n_orb <= 16 ? launch_accum_both<16>(acc, s)
-                                       : launch_accum_both<24>(acc, s);
+                    rc = n_orb <= 4    ? launch_accum_both<4>(p, acc, s)
+                         : n_orb <= 8  ? launch_accum_both<8>(p, acc, s)
+                         : n_orb <= 16 ? launch_accum_both<16>(p, acc, s)
+                                       : launch_accum_both<24>(p, acc, s);
                     if (rc) return rc;
                 }
             }

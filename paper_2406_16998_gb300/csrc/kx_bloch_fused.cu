@@ -614,12 +614,11 @@ __global__ void __launch_bounds__(kFuThreads, 1) bloch_fused_kernel(const FuArgs
 constexpr int kFuItemTiles = 32;  // most tiles of an item (F_MID3: 4096 / 128, F_INV21: n3 / 2)
 
 template <int KIND, int NK>
-int fused_resident(const kx_plan *p, int *ctas) {
+int fused_resident(kx_plan *p, int *ctas) {
+    const void *kernel = reinterpret_cast<const void *>(bloch_fused_kernel<KIND, NK>);
     int per_sm = 0;
-    KX_CUDA_TRY(cudaFuncSetAttribute(bloch_fused_kernel<KIND, NK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     fu_smem_bytes(NK)));
-    KX_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, bloch_fused_kernel<KIND, NK>, kFuThreads,
-                                                              fu_smem_bytes(NK)));
+    if (int rc = raise_smem(p, kernel, fu_smem_bytes(NK))) return rc;
+    if (int rc = resident_ctas(p, kernel, kFuThreads, fu_smem_bytes(NK), &per_sm)) return rc;
     *ctas = std::min(*ctas, per_sm * p->num_sms);
     return KX_OK;
 }
@@ -633,12 +632,8 @@ int launch_fused(kx_plan *p, FuArgs a, long long R, cudaStream_t s) {
     a.n_tiles = (int)(R * a.tiles_per_item);
     a.status = p->d_status;
     a.timeout_cycles = 2000000000LL;
-    static bool attr = false;  // once per instantiation
-    if (!attr) {
-        KX_CUDA_TRY(cudaFuncSetAttribute(bloch_fused_kernel<KIND, NK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         fu_smem_bytes(NK)));
-        attr = true;
-    }
+    const void *kernel = reinterpret_cast<const void *>(bloch_fused_kernel<KIND, NK>);
+    if (int rc = raise_smem(p, kernel, fu_smem_bytes(NK))) return rc;
     if (int rc = prof_begin(p, PK_BLOCH, s)) return rc;
     const dim3 grid((unsigned)std::min(a.n_tiles, p->num_sms));  // one CTA per SM, all resident
     if constexpr (KIND == F_FWD12) {
@@ -646,8 +641,7 @@ int launch_fused(kx_plan *p, FuArgs a, long long R, cudaStream_t s) {
     } else {
         void *args[] = {&a};
         const cudaError_t e =
-            cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(bloch_fused_kernel<KIND, NK>), grid,
-                                        dim3(kFuThreads), args, (size_t)fu_smem_bytes(NK), s);
+            cudaLaunchCooperativeKernel(kernel, grid, dim3(kFuThreads), args, (size_t)fu_smem_bytes(NK), s);
         if (e == cudaErrorCooperativeLaunchTooLarge) {
             // the stream has fewer SMs than the device
             cudaGetLastError();
@@ -668,7 +662,7 @@ int launch_fused(kx_plan *p, FuArgs a, long long R, cudaStream_t s) {
 // for its own next tile: tiles go to the CTAs in turn and an item has up to 32 neighbouring
 // ones, so 32 CTAs are enough.  *fits = 0 on a smaller share of a device, whose calls
 // take the single products.
-int bloch_fused_fits(const kx_plan *p, bool *fits) {
+int bloch_fused_fits(kx_plan *p, bool *fits) {
     *fits = false;
     int coop = 0, ctas = p->num_sms;
     KX_CUDA_TRY(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, p->device));

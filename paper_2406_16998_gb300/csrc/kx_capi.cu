@@ -41,6 +41,25 @@ static bool fault(const char *what) {
 static bool fault_alloc() { return fault("alloc"); }
 long long ring_wait_cycles() { return fault("wait") ? -1 : kWaitCycles; }
 
+int raise_smem(kx_plan *p, const void *kernel, size_t bytes) {
+    size_t &limit = p->smem_limit[kernel];
+    if (limit >= bytes) return KX_OK;
+    KX_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+    limit = bytes;
+    return KX_OK;
+}
+
+int resident_ctas(kx_plan *p, const void *kernel, int threads, size_t smem, int *per_sm) {
+    const auto known = p->resident.find({kernel, smem});
+    if (known != p->resident.end()) {
+        *per_sm = known->second;
+        return KX_OK;
+    }
+    KX_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, kernel, threads, smem));
+    p->resident[{kernel, smem}] = *per_sm;
+    return KX_OK;
+}
+
 int ensure_workspace(kx_plan *p, size_t bytes) {
     if (p->ws.bytes >= bytes) return KX_OK;
     if (fault_alloc()) return set_error(KX_ERR_NOMEM, "workspace allocation failed (injected by KX_FAULT=alloc)");

@@ -5,7 +5,9 @@
 #include <cuda_fp16.h>
 #include <cstddef>
 #include <cstdint>
+#include <map>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "../../include/kronx.h"
@@ -173,9 +175,17 @@ struct kx_plan_s {
     // reallocated or refilled (workspaces, pair list, multipole fields)
     unsigned long long config_version = 0;
     kx::Workspace mp_scratch;
+    std::map<const void *, size_t> smem_limit;                 // raise_smem
+    std::map<std::pair<const void *, size_t>, int> resident;  // resident_ctas
 };
 
 namespace kx {
+
+// A kernel's shared-memory limit raised to `bytes`, once per plan: it is an attribute of the
+// function on the plan's device, in the plan's context.
+int raise_smem(kx_plan *p, const void *kernel, size_t bytes);
+// Resident CTAs per SM at that shared memory, asked once per plan.
+int resident_ctas(kx_plan *p, const void *kernel, int threads, size_t smem, int *per_sm);
 
 // Bracket one kernel launch with profiling events (no-ops unless kx_profile is on).
 int prof_begin(kx_plan *p, int kind, cudaStream_t s);
@@ -241,7 +251,7 @@ int bloch_energy(kx_plan *p, int n_kpt, const double *theta, const double *wk, i
 // two products per kernel (kx_bloch_fused.cu); the second and third return kFusedRefused,
 // with nothing launched, where their CTAs cannot all be resident
 constexpr int kFusedRefused = -1;
-int bloch_fused_fits(const kx_plan *p, bool *fits);
+int bloch_fused_fits(kx_plan *p, bool *fits);
 int bloch_fused_forward(kx_plan *p, long long R, const float2 *P, const float2 *F, float2 *out, const __half *B1,
                         const __half *B2, const float *pmax, const float *fmax, long long r0, int n_orb,
                         float *out_max, cudaStream_t s);

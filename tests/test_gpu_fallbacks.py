@@ -3,6 +3,7 @@ state after a failed allocation."""
 import ctypes
 import os
 import subprocess
+import sys
 
 import numpy as np
 import pytest
@@ -163,3 +164,50 @@ def test_fused_kpoint_products_on_another_share_of_the_device(kx, hooks, sms, n_
     assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
     for a, b in zip(got[2:], want[2:]):
         assert abs(a.item() - b.item()) < 1e-6 * abs(b.item())
+
+
+# Three kinds of k-point products (two per kernel, single ones, CUDA cores with up to 200 KB
+# of shared memory) and the widest sums, before and after a reset of the device: what was
+# set for the kernels in the first context is gone in the second.
+RESET = """
+import ctypes, sys
+import numpy as np
+import paper_2406_16998_gb300 as kx
+L = kx.lib()
+rt = ctypes.CDLL("libcudart.so.13")  # the one the library is linked to
+dp = ctypes.POINTER(ctypes.c_double)
+
+def buf(a):
+    p = ctypes.c_void_p()
+    assert rt.cudaMalloc(ctypes.byref(p), ctypes.c_size_t(a.nbytes)) == 0
+    assert rt.cudaMemcpy(p, a.ctypes.data_as(ctypes.c_void_p), ctypes.c_size_t(a.nbytes), 1) == 0
+    return p
+
+def run(n, n_orb):
+    plan = kx.Plan(n, (0.4, 0.45, 0.5), (1, 1, 1), 1, precision=1)
+    psi = np.random.default_rng(n_orb).standard_normal((2, n_orb, plan.N, 2))
+    theta, wk = np.array([[0.0, 0.0, 0.0], [1.0, 0.5, -0.7]]), np.array([0.5, 0.5])
+    d_psi, d_vx = buf(psi), buf(np.zeros_like(psi))
+    host = lambda a: a.ctypes.data_as(L.kx_vx_kpoints.argtypes[2])
+    rc = L.kx_vx_kpoints(plan.handle, 2, host(theta), host(wk), n_orb, d_psi, None, d_vx, None, None)
+    detail = ctypes.create_string_buffer(256)
+    L.kx_last_error_detail(detail, 256)
+    assert rc == 0, (n, rc, detail.value)
+    out = np.empty_like(psi)
+    assert rt.cudaMemcpy(out.ctypes.data_as(ctypes.c_void_p), d_vx, ctypes.c_size_t(out.nbytes), 2) == 0
+    plan.close()
+    assert np.isfinite(out).all() and np.abs(out).max() > 0
+    return out.tobytes()
+
+calls = [((64, 64, 32), 5), ((64, 32, 32), 2), ((48, 40, 56), 2), ((16, 16, 16), 20)]
+first = [run(*c) for c in calls]
+assert rt.cudaDeviceReset() == 0
+assert [run(*c) for c in calls] == first
+print("same")
+"""
+
+
+def test_kpoints_in_a_second_context(kx):
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", RESET], cwd=root, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0 and r.stdout.strip() == "same", r.stdout + r.stderr
