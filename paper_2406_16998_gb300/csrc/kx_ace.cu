@@ -364,6 +364,7 @@ __global__ void __launch_bounds__(256, 2) proj32_kernel(const double *__restrict
         }
 }
 
+constexpr int kMaxAce = 256;  // vectors of the compressed operator
 constexpr int kCX = 128;  // combination tile: 128 grid points x 64 output vectors
 constexpr int kCB = 64;
 constexpr int kCA = 16;   // input vectors per pipeline step
@@ -621,12 +622,10 @@ int launch_projection(kx_plan *p, const double *A, int na, const double *B, int 
         // 16-byte copies need even N (so every row starts 16-byte aligned) and aligned bases
         const bool vec2 = N % 2 == 0 && ((reinterpret_cast<uintptr_t>(A) | reinterpret_cast<uintptr_t>(B)) & 15) == 0;
         if (vec2) {
-            KX_CUDA_TRY(cudaFuncSetAttribute(proj32_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)kProjSmem));
+            if (int rc = raise_smem(p, reinterpret_cast<const void *>(proj32_kernel<true>), kProjSmem)) return rc;
             proj32_kernel<true><<<grid, 256, kProjSmem, s>>>(A, na, B, nb, w32, N, span, part);
         } else {
-            KX_CUDA_TRY(cudaFuncSetAttribute(proj32_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)kProjSmem));
+            if (int rc = raise_smem(p, reinterpret_cast<const void *>(proj32_kernel<false>), kProjSmem)) return rc;
             proj32_kernel<false><<<grid, 256, kProjSmem, s>>>(A, na, B, nb, w32, N, span, part);
         }
         KX_LAUNCH_CHECK("proj32_kernel launch");
@@ -665,12 +664,12 @@ int launch_combination(kx_plan *p, const double *A, int na, const double *C, int
         const size_t smem = bulk ? comb_bulk_smem(na) : comb_smem(na);
         const dim3 grid(gx, tiles_b);
         if (bulk) {
-            KX_CUDA_TRY(cudaFuncSetAttribute(combine32_bulk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)smem));
+            if (int rc = raise_smem(p, reinterpret_cast<const void *>(combine32_bulk_kernel), comb_bulk_smem(kMaxAce)))
+                return rc;
             combine32_bulk_kernel<<<grid, 256, smem, s>>>(A, na, C, nb, N, fs, accumulate, out, p->d_status,
                                                           ring_wait_cycles());
         } else {
-            KX_CUDA_TRY(cudaFuncSetAttribute(combine32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+            if (int rc = raise_smem(p, reinterpret_cast<const void *>(combine32_kernel), comb_smem(kMaxAce))) return rc;
             combine32_kernel<<<grid, 256, smem, s>>>(A, na, C, nb, N, fs, accumulate, out);
         }
         KX_LAUNCH_CHECK("combine32_kernel launch");
@@ -697,8 +696,8 @@ int ace_run(kx_plan *p, int n_orb, const double *psi, const double *W, double *x
     gram_reduce_kernel<<<(unsigned)((nn + 31) / 32), 32 * kRedWarps, 0, s>>>(part, n_slab, (int)nn, p->dV, M, M_out, A);
     KX_LAUNCH_CHECK("gram_reduce_kernel launch");
     const size_t chol_smem = n_orb <= kCholSmemN ? sizeof(double) * nn : 0;
-    KX_CUDA_TRY(cudaFuncSetAttribute(cholesky_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)(sizeof(double) * kCholSmemN * kCholSmemN)));
+    if ((rc = raise_smem(p, reinterpret_cast<const void *>(cholesky_kernel), sizeof(double) * kCholSmemN * kCholSmemN)))
+        return rc;
     cholesky_kernel<<<1, kCholThreads, chol_smem, s>>>(A, n_orb, bad);
     KX_LAUNCH_CHECK("cholesky_kernel launch");
     triinv_kernel<<<(n_orb + 3) / 4, 128, 0, s>>>(A, n_orb, Rinv);

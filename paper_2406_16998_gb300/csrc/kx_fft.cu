@@ -37,6 +37,7 @@ constexpr int kFftPlaneThreads = 512;  // passes A and C: two planes (2 x 104 KB
 // planes transformed in place: one buffer (52 KB at 80^2), four CTAs per SM whose barriers
 // fall apart
 constexpr int kFftInPlaceThreads = 256;
+constexpr size_t kFftPlaneSmem = 200 * 1024;  // most a plane may take (fft_supported)
 
 struct FftAxis {
     int n, nr;
@@ -616,7 +617,7 @@ bool fft_supported(const int *n, const int *bc) {
     FftAxis ax;
     for (int a = 0; a < 3; ++a)  // the twiddle tables hold 128 entries per axis
         if (bc[a] != KX_PERIODIC || n[a] > 128 || !factor_235(n[a], ax)) return false;
-    return sizeof(float2) * 2 * (size_t)n[1] * (n[0] + 1) <= 200 * 1024;
+    return sizeof(float2) * 2 * (size_t)n[1] * (n[0] + 1) <= kFftPlaneSmem;
 }
 
 int fft_setup(kx_plan *p) {
@@ -681,10 +682,11 @@ int fft_passes(kx_plan *p, long R, const int2 *pairs, const float *src32, int rh
     auto fwd = ip ? fft_plane_fwd_kernel<true> : fft_plane_fwd_kernel<false>;
     auto inv = ip ? fft_plane_inv_kernel<true> : fft_plane_inv_kernel<false>;
     const int pt = ip ? kFftInPlaceThreads : kFftPlaneThreads;
-    KX_CUDA_TRY(cudaFuncSetAttribute(fwd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ps));
-    KX_CUDA_TRY(cudaFuncSetAttribute(inv, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ps));
-    KX_CUDA_TRY(cudaFuncSetAttribute(fft_axis3_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ls));
     int rc;
+    if ((rc = raise_smem(p, reinterpret_cast<const void *>(fwd), kFftPlaneSmem))) return rc;
+    if ((rc = raise_smem(p, reinterpret_cast<const void *>(inv), kFftPlaneSmem))) return rc;
+    if ((rc = raise_smem(p, reinterpret_cast<const void *>(fft_axis3_kernel), sizeof(float2) * 2 * kMaxN * kFftLine)))
+        return rc;
     const dim3 gp((unsigned)p->n[2], (unsigned)R);
     if ((rc = prof_begin(p, PK_FFT, s))) return rc;
     fwd<<<gp, pt, ps, s>>>(G, pairs, src32, rhs, C);

@@ -339,9 +339,10 @@ __global__ void ftable64_kernel(int n1, int n2, int n3, const double *lam, int k
     }
 }
 
-template <int MODE, int U> int launch_u(const Args64 &a, unsigned blocks, int threads, size_t smem, cudaStream_t s) {
-    KX_CUDA_TRY(cudaFuncSetAttribute(mode64_kernel<U, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)(sizeof(double) * kMaxN * 65)));
+template <int MODE, int U>
+int launch_u(kx_plan *p, const Args64 &a, unsigned blocks, int threads, size_t smem, cudaStream_t s) {
+    if (int rc = raise_smem(p, reinterpret_cast<const void *>(mode64_kernel<U, MODE>), sizeof(double) * kMaxN * 65))
+        return rc;
     mode64_kernel<U, MODE><<<blocks, threads, smem, s>>>(a);
     KX_LAUNCH_CHECK("mode64_kernel launch");
     return KX_OK;
@@ -384,17 +385,17 @@ int launch_mode(kx_plan *p, int axis, int R, Args64 a, cudaStream_t s, int *bloc
     const int u = (he + a.groups - 1) / a.groups;
     if (int rc = prof_begin(p, PK_FP64_MODE, s)) return rc;
     int rc;
-    if (u <= 1) rc = launch_u<MODE, 1>(a, blocks, threads, smem, s);
-    else if (u <= 2) rc = launch_u<MODE, 2>(a, blocks, threads, smem, s);
-    else if (u <= 3) rc = launch_u<MODE, 3>(a, blocks, threads, smem, s);
-    else if (u <= 4) rc = launch_u<MODE, 4>(a, blocks, threads, smem, s);
-    else if (u <= 5) rc = launch_u<MODE, 5>(a, blocks, threads, smem, s);
-    else if (u <= 6) rc = launch_u<MODE, 6>(a, blocks, threads, smem, s);
-    else if (u <= 8) rc = launch_u<MODE, 8>(a, blocks, threads, smem, s);
-    else if (u <= 10) rc = launch_u<MODE, 10>(a, blocks, threads, smem, s);
-    else if (u <= 12) rc = launch_u<MODE, 12>(a, blocks, threads, smem, s);
-    else if (u <= 17) rc = launch_u<MODE, 17>(a, blocks, threads, smem, s);
-    else rc = launch_u<MODE, 32>(a, blocks, threads, smem, s);  // no parity
+    if (u <= 1) rc = launch_u<MODE, 1>(p, a, blocks, threads, smem, s);
+    else if (u <= 2) rc = launch_u<MODE, 2>(p, a, blocks, threads, smem, s);
+    else if (u <= 3) rc = launch_u<MODE, 3>(p, a, blocks, threads, smem, s);
+    else if (u <= 4) rc = launch_u<MODE, 4>(p, a, blocks, threads, smem, s);
+    else if (u <= 5) rc = launch_u<MODE, 5>(p, a, blocks, threads, smem, s);
+    else if (u <= 6) rc = launch_u<MODE, 6>(p, a, blocks, threads, smem, s);
+    else if (u <= 8) rc = launch_u<MODE, 8>(p, a, blocks, threads, smem, s);
+    else if (u <= 10) rc = launch_u<MODE, 10>(p, a, blocks, threads, smem, s);
+    else if (u <= 12) rc = launch_u<MODE, 12>(p, a, blocks, threads, smem, s);
+    else if (u <= 17) rc = launch_u<MODE, 17>(p, a, blocks, threads, smem, s);
+    else rc = launch_u<MODE, 32>(p, a, blocks, threads, smem, s);  // no parity
     if (rc) return rc;
     return prof_end(p, s);
 }

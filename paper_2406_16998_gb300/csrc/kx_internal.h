@@ -182,7 +182,9 @@ struct kx_plan_s {
 namespace kx {
 
 // A kernel's shared-memory limit raised to `bytes`, once per plan: it is an attribute of the
-// function on the plan's device, in the plan's context.
+// function on the plan's device, in the plan's context.  Always the same bytes for a kernel
+// (the most any launch of it takes): another plan's thread may launch it in between, and a
+// smaller limit set there would fail a launch here.
 int raise_smem(kx_plan *p, const void *kernel, size_t bytes);
 // Resident CTAs per SM at that shared memory, asked once per plan.
 int resident_ctas(kx_plan *p, const void *kernel, int threads, size_t smem, int *per_sm);

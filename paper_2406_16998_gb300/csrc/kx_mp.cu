@@ -905,8 +905,7 @@ int weighted_moments(kx_plan *p, int n, const double *psi, const double *W64, co
         const int n_split = moments_tc_split(p);
         const long long span = ((N + n_split - 1) / n_split + kMtX - 1) / kMtX * kMtX;
         const dim3 grid(n_split, ((K + 1) / 2 + kMtPairs - 1) / kMtPairs);
-        KX_CUDA_TRY(cudaFuncSetAttribute(mp_moments_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)kMtSmem));
+        if (int rc = raise_smem(p, reinterpret_cast<const void *>(mp_moments_tc_kernel), kMtSmem)) return rc;
         mp_moments_tc_kernel<<<grid, 256, kMtSmem, s>>>(psi, n, W32, K, Wmax, psimax, N, span, part, p->d_status,
                                                          4000000000LL);
         KX_LAUNCH_CHECK("mp_moments_tc_kernel launch");
@@ -1095,7 +1094,8 @@ int mp_correct_vx(kx_plan *p, int n_orb, const double *psi, const double *occ, d
     KX_LAUNCH_CHECK("mp_coef_kernel launch");
     const dim3 grid((unsigned)((N + kMcX - 1) / kMcX), (unsigned)((n + 63) / 64));
     const size_t smem = sizeof(float) * (size_t)n * (kMcX + 64);
-    KX_CUDA_TRY(cudaFuncSetAttribute(mp_combine32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    if (int rc = raise_smem(p, reinterpret_cast<const void *>(mp_combine32_kernel), sizeof(float) * 256 * (kMcX + 64)))
+        return rc;
     mp_combine32_kernel<<<grid, 256, smem, s>>>(psi, n, C, sym ? p->d_mpR32 : p->d_mpH32, Kc, occ, N, vx, part);
     KX_LAUNCH_CHECK("mp_combine32_kernel launch");
     if (ex) {
@@ -1141,7 +1141,7 @@ int mp_correct_into_acc(kx_plan *p, int n_orb, const double *psi, const double *
     mp_ct_bsplit_kernel<<<(unsigned)(((long long)Kc * 4096 + 255) / 256), 256, 0, s>>>(C, n, Kc, sc, Bs);
     KX_LAUNCH_CHECK("mp_ct_bsplit_kernel launch");
     const int grid = (int)std::min<long long>((N + kCtM - 1) / kCtM, p->num_sms);
-    KX_CUDA_TRY(cudaFuncSetAttribute(mp_combine_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCtSmem));
+    if (int rc = raise_smem(p, reinterpret_cast<const void *>(mp_combine_tc_kernel), kCtSmem)) return rc;
     mp_combine_tc_kernel<<<grid, 256, kCtSmem, s>>>(psi, n, Bs, sym ? p->d_mpR32 : p->d_mpH32, Kc, sc, occ, N, acc,
                                                      part, p->d_status, 4000000000LL);
     KX_LAUNCH_CHECK("mp_combine_tc_kernel launch");

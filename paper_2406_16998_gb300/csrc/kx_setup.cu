@@ -245,7 +245,7 @@ int plan_setup(kx_plan *p) {
 
     int nmax = std::max(p->n[0], std::max(p->n[1], p->n[2]));
     size_t smem = sizeof(double) * nmax * nmax;
-    KX_CUDA_TRY(cudaFuncSetAttribute(eig1d_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    if (int rc = raise_smem(p, reinterpret_cast<const void *>(eig1d_kernel), sizeof(double) * kMaxN * kMaxN)) return rc;
     eig1d_kernel<<<3, kEigThreads, smem>>>(p->n[0], p->n[1], p->n[2], p->h[0], p->h[1], p->h[2], p->bc[0],
                                            p->bc[1], p->bc[2], p->fd_order, p->d_lam[0], p->d_lam[1],
                                            p->d_lam[2], p->d_V[0], p->d_V[1], p->d_V[2]);

@@ -1738,15 +1738,15 @@ int pass_batch(int np) {
 }
 
 template <int PASS, int U>
-int launch_pass_u(const PassArgs &a, int grid, size_t smem, cudaStream_t s) {
-    KX_CUDA_TRY(cudaFuncSetAttribute(tc_pass_kernel<PASS, U>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+int launch_pass_u(kx_plan *p, const PassArgs &a, int grid, size_t smem, cudaStream_t s) {
+    if (int rc = raise_smem(p, reinterpret_cast<const void *>(tc_pass_kernel<PASS, U>), kSmemBudget + 1024)) return rc;
     tc_pass_kernel<PASS, U><<<grid, kThreads, smem, s>>>(a);
     KX_LAUNCH_CHECK("tc_pass_kernel launch");
     return KX_OK;
 }
 
 template <int PASS>
-int launch_pass(const kx_plan *p, PassArgs a, int axis, cudaStream_t s, int *grid_out) {
+int launch_pass(kx_plan *p, PassArgs a, int axis, cudaStream_t s, int *grid_out) {
     a.nc = p->n[axis];
     a.np = p->np[axis];
     a.Vs = p->d_Vs[axis];
@@ -1766,14 +1766,14 @@ int launch_pass(const kx_plan *p, PassArgs a, int axis, cudaStream_t s, int *gri
     const long long n_tiles = (a.total_rows + 127) / 128;
     const int grid = (int)std::max(1LL, std::min<long long>(n_tiles, (long long)p->num_sms));
     if (grid_out) *grid_out = grid;
-    if (int rc = prof_begin(const_cast<kx_plan *>(p), PK_X3F + PASS, s)) return rc;
+    if (int rc = prof_begin(p, PK_X3F + PASS, s)) return rc;
     const int u = PASS == P_X3F ? 8 : pass_batch(a.np);  // X3F has its own batches
     int rc;
-    if (PASS == P_X3F || u == 8) rc = launch_pass_u<PASS, 8>(a, grid, smem, s);
-    else if (u == 7) rc = launch_pass_u<PASS, PASS == P_X3F ? 8 : 7>(a, grid, smem, s);
-    else rc = launch_pass_u<PASS, PASS == P_X3F ? 8 : 5>(a, grid, smem, s);
+    if (PASS == P_X3F || u == 8) rc = launch_pass_u<PASS, 8>(p, a, grid, smem, s);
+    else if (u == 7) rc = launch_pass_u<PASS, PASS == P_X3F ? 8 : 7>(p, a, grid, smem, s);
+    else rc = launch_pass_u<PASS, PASS == P_X3F ? 8 : 5>(p, a, grid, smem, s);
     if (rc) return rc;
-    return prof_end(const_cast<kx_plan *>(p), s);
+    return prof_end(p, s);
 }
 
 // axes 1 and 2 of the same size, spacing and boundary have the same eigenvectors
@@ -1845,10 +1845,11 @@ int launch_slab(kx_plan *p, long R, const float *in, const float *in_max, float 
     smem = std::max<size_t>(smem, 120 * 1024);
     const int grid = (int)std::max(1LL, std::min<long long>(a.total_units, (long long)p->num_sms));
     if (grid_out) *grid_out = grid;
-    if (int rc = prof_begin(p, PK_SLAB, s)) return rc;
+    int rc;
+    if ((rc = prof_begin(p, PK_SLAB, s))) return rc;
     auto kernel = energy_only ? (a.pp > 1 ? tc_slab_kernel<true, true> : tc_slab_kernel<true, false>)
                               : (a.pp > 1 ? tc_slab_kernel<false, true> : tc_slab_kernel<false, false>);
-    KX_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    if ((rc = raise_smem(p, reinterpret_cast<const void *>(kernel), kSlabSmemMax))) return rc;
     kernel<<<grid, kSlabThreads, smem, s>>>(a);
     KX_LAUNCH_CHECK("tc_slab_kernel launch");
     return prof_end(p, s);
@@ -2160,8 +2161,7 @@ int tc_vx(kx_plan *p, int n_orb, const double *psi, const double *occ, double *v
             ac.ex = ex;
             if ((rc = prof_begin(p, PK_ACC, s))) return rc;
             if (N % 4 == 0) {  // rows of whole 16-byte pieces
-                KX_CUDA_TRY(cudaFuncSetAttribute(acc_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 (int)acc_smem<4>()));
+                if ((rc = raise_smem(p, reinterpret_cast<const void *>(acc_kernel<4>), acc_smem<4>()))) return rc;
                 acc_kernel<4><<<(unsigned)((N / 4 + kAccThreads - 1) / kAccThreads), kAccThreads, acc_smem<4>(), s>>>(ac);
             } else {
                 acc_kernel<1><<<(unsigned)((N + kAccThreads - 1) / kAccThreads), kAccThreads, acc_smem<1>(), s>>>(ac);

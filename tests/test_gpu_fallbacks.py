@@ -211,3 +211,18 @@ def test_kpoints_in_a_second_context(kx):
     root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
     r = subprocess.run([sys.executable, "-c", RESET], cwd=root, capture_output=True, text=True, timeout=300)
     assert r.returncode == 0 and r.stdout.strip() == "same", r.stdout + r.stderr
+
+
+@pytest.mark.parametrize("prec,big,small", [(2, (96, 96, 4), (8, 9, 5)), (1, (96, 96, 8), (16, 8, 8))])
+def test_two_threads_with_kernels_of_different_size(kx, hooks, prec, big, small):
+    """Two host threads, each with its own plan and stream, launch the same kernels with much and
+    with little shared memory: neither takes the other's limit away."""
+    plans = [kx.Plan(n, (0.5,) * 3, (P, P, P), S, precision=prec) for n in (big, small)]
+    b = [rand(1, p.N) for p in plans]
+    want = [kx.kx_apply_fL(p, x).clone() for p, x in zip(plans, b)]
+    got = [torch.zeros_like(x) for x in b]
+    torch.cuda.synchronize()
+    ptr = lambda t: ctypes.c_void_p(t.data_ptr())
+    assert hooks.hook_two_threads(plans[0].handle, ptr(b[0]), ptr(got[0]), plans[1].handle, ptr(b[1]), ptr(got[1]),
+                                  5000) == 0
+    assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
