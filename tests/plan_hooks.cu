@@ -1,8 +1,10 @@
 // Handles for the tests on what no public call reaches: a device of another size, calls
-// from two host threads without a pause.
+// from two host threads without a pause, eigenvectors without parity.
 #include "kx_internal.h"
 
+#include <cmath>
 #include <thread>
+#include <vector>
 
 // The number of SMs the plan's launches count on; returns the number before.
 extern "C" int hook_num_sms(kx_plan *p, int n) {
@@ -30,4 +32,22 @@ extern "C" int hook_two_threads(kx_plan *p0, const double *b0, double *x0, kx_pl
     loop(1, p1, b1, x1);
     t.join();
     return rc[0] ? rc[0] : rc[1];
+}
+
+// Mixes eigenvectors k and k + 1 of an axis by `angle` and makes the float64 tables again.
+extern "C" int hook_mix_eigenvectors(kx_plan *p, int axis, int k, double angle) {
+    const int n = p->n[axis];
+    std::vector<double> V((size_t)n * n);
+    if (cudaMemcpy(V.data(), p->d_V[axis], sizeof(double) * V.size(), cudaMemcpyDeviceToHost) != cudaSuccess) return -1;
+    const double c = std::cos(angle), s = std::sin(angle);
+    for (int x = 0; x < n; ++x) {
+        double &a = V[(size_t)x * n + k], &b = V[(size_t)x * n + k + 1];
+        const double t = c * a + s * b;
+        b = c * b - s * a;
+        a = t;
+    }
+    if (cudaMemcpy(p->d_V[axis], V.data(), sizeof(double) * V.size(), cudaMemcpyHostToDevice) != cudaSuccess) return -1;
+    cudaFree(p->d_p64_f);
+    p->d_p64_f = nullptr;
+    return kx::fp64_setup(p);
 }

@@ -226,3 +226,38 @@ def test_two_threads_with_kernels_of_different_size(kx, hooks, prec, big, small)
     assert hooks.hook_two_threads(plans[0].handle, ptr(b[0]), ptr(got[0]), plans[1].handle, ptr(b[1]), ptr(got[1]),
                                   5000) == 0
     assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
+
+
+@pytest.mark.parametrize("n,axis,n_rhs", [
+    ((12, 9, 16), 0, 3), ((9, 13, 8), 1, 2), ((8, 16, 70), 2, 2),
+    ((128, 32, 40), 0, 64), ((8, 128, 8), 1, 3), ((40, 32, 101), 2, 64),  # the widest forms, many and few pencils
+])
+@pytest.mark.parametrize("angle", [1e-7, 0.6])
+def test_float64_eigenvectors_without_parity(kx, hooks, n, axis, n_rhs, angle):
+    """Eigenvectors of a Dirichlet axis that are neither even nor odd, by a little or altogether,
+    take the dense form, which drops nothing of them."""
+    bc = [P, P, P]
+    bc[axis] = D
+    plan = kx.Plan(n, (0.4, 0.45, 0.5), bc, S, precision=0)
+    assert hooks.hook_mix_eigenvectors(plan.handle, axis, 1, ctypes.c_double(angle)) == 0
+    V = [torch.from_numpy(np.asarray(plan.eig(a)[1])).cuda() for a in range(3)]
+    f = torch.from_numpy(np.asarray(plan.ftable()).reshape(n[2], n[1], n[0])).cuda()
+
+    def solve(b):
+        t = b.view(-1, n[2], n[1], n[0])
+        t = torch.einsum("rzyx,zk,yj,xi->rkji", t, V[2], V[1], V[0]) * f
+        return torch.einsum("rkji,zk,yj,xi->rzyx", t, V[2], V[1], V[0]).reshape(b.shape)
+
+    b = rand(n_rhs, plan.N)
+    ref, x = solve(b), kx.kx_apply_fL(plan, b)
+    assert (x - ref).abs().max() < 1e-11 * ref.abs().max()
+    psi = b[:2].contiguous()
+    rho = torch.stack([psi[0] * psi[0], psi[0] * psi[1], psi[1] * psi[1]])
+    phi = solve(rho)
+    vx_ref = -torch.stack([psi[0] * phi[0] + psi[1] * phi[1], psi[0] * phi[1] + psi[1] * phi[2]])
+    dV = 0.4 * 0.45 * 0.5
+    ex_ref = -0.5 * dV * ((rho * phi).sum(1) * torch.tensor([1.0, 2.0, 1.0], device="cuda", dtype=torch.float64)).sum()
+    vx, ex = kx.kx_vx_apply(plan, psi)
+    assert (vx - vx_ref).abs().max() < 1e-11 * vx_ref.abs().max()
+    for e in (ex.item(), kx.kx_energy(plan, psi).item()):
+        assert abs(e - ex_ref.item()) < 1e-11 * abs(ex_ref.item())
