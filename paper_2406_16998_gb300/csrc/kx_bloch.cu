@@ -1957,6 +1957,17 @@ __global__ void __launch_bounds__(kAccPoints) bloch_accum_both_kernel(const AccB
     }
 }
 
+// Float32 sums of up to 24 bands (more would not fit the registers), even N (16-byte copies)
+// and enough blocks of points: a block takes a chunk's vectors one after the other, where
+// the kernels above spread them over the SMs too.  Whole calls, kernels above / one
+// pass, both directions: 32^3 (256 blocks) 24 bands 2645 / 2680 us and 16^3 (32) 550 / 681,
+// 40^3 (500) 6436 / 6390, 64^3 (2048) 7799 / 7405; forward alone, one band and 200
+// vectors: 16^3 219 / 396, 40^3 1896 / 1942, 48^3 (864) 3331 / 3275, 64^3 2922 / 2655.
+inline bool accum_both_fits(const kx_plan *p, int n_orb, bool reverse) {
+    const long long N = (long long)p->N, blocks = (N + kAccPoints - 1) / kAccPoints;
+    return n_orb <= 24 && N % 2 == 0 && blocks >= (reverse ? 3 : 5) * (long long)p->num_sms;
+}
+
 template <int MB>
 int launch_accum_both(kx_plan *p, const AccBoth &a, cudaStream_t s) {
     const int smem = kAccStages * MB * kAccPoints * (int)sizeof(float2);
@@ -2597,10 +2608,8 @@ int bloch_sweep(kx_plan *p, int n_kpt, const double *theta, const double *wk, in
                 if ((rc = launch_pipe<T, 0>(p, 0, R, A, B, Mi[0], nullptr, s))) return rc;
             }
             if ((rc = prof_begin(p, PK_BLOCH_OTHER, s))) return rc;
-            // float32 sums of up to 24 bands, even N (16-byte copies): both in one pass; more bands would
-            // not fit the registers
             double2 *out_q = reverse ? reinterpret_cast<double2 *>(out_all) + (size_t)q * n_orb * N : nullptr;
-            const bool both = sizeof(T) == 4 && n_orb <= 24 && N % 2 == 0;
+            const bool both = sizeof(T) == 4 && accum_both_fits(p, n_orb, reverse);
             if constexpr (sizeof(T) == 4) {
                 if (both) {
                     const AccBoth acc = {B,     Pq, F, r0, r1, N, n_orb, occ_q, occ_k, wk[q], wk[k], reinterpret_cast<double2 *>(out_k),

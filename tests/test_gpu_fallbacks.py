@@ -43,11 +43,12 @@ def rand(*shape, seed=1, cplx=False):
 
 
 @pytest.mark.parametrize("call", ["ace_apply", "kpoints"])
-def test_bulk_copy_ring_given_up(kx, call, monkeypatch):
+def test_bulk_copy_ring_given_up(kx, hooks, call, monkeypatch):
     """A kernel whose bulk copies run ahead of it gives up its first wait (KX_FAULT=wait): it
     waits for the copies in flight, reports the timeout and returns; the next call is right."""
     n = (24, 16, 24)
     plan = kx.Plan(n, (0.4, 0.45, 0.5), (P, P, P), S, precision=1)
+    hooks.hook_num_sms(plan.handle, 1)  # few SMs: the forms for many points per SM
     if call == "ace_apply":  # three steps of eight vectors per tile of points
         xi, phi = rand(20, plan.N), rand(70, plan.N, seed=2)
         run = lambda: (kx.kx_ace_apply(plan, xi, phi),)
@@ -261,3 +262,28 @@ def test_float64_eigenvectors_without_parity(kx, hooks, n, axis, n_rhs, angle):
     assert (vx - vx_ref).abs().max() < 1e-11 * vx_ref.abs().max()
     for e in (ex.item(), kx.kx_energy(plan, psi).item()):
         assert abs(e - ex_ref.item()) < 1e-11 * abs(ex_ref.item())
+
+
+@pytest.mark.parametrize("n,n_orb,n_vec,chunk", [
+    ((16, 8, 8), 1, 9, None), ((16, 16, 8), 4, 6, "7"), ((8, 16, 16), 5, 8, "11"), ((16, 8, 16), 9, 3, "20"),
+    ((16, 16, 16), 17, 5, "50"), ((16, 8, 16), 24, 2, None), ((12, 10, 9), 6, 7, "11"),
+])
+def test_kpoint_sums_of_few_and_of_many_points(kx, hooks, n, n_orb, n_vec, chunk, monkeypatch):
+    """The one-pass sums (many points per SM) and the kernels that spread a chunk's vectors over
+    the SMs (few) give the same bits, forward alone and both ways, over the band counts a
+    thread holds and chunks that split a vector's bands."""
+    if chunk:
+        monkeypatch.setenv("KX_CHUNK_PAIRS", chunk)
+    plan = kx.Plan(n, (0.4, 0.45, 0.5), (P, P, P), S, precision=1 if all(m % 8 == 0 for m in n) else 2)
+    psi, phi = rand(3, n_orb, plan.N, cplx=True), rand(n_vec, plan.N, seed=2, cplx=True)
+    occ = torch.linspace(0.2, 1.0, 3 * n_orb, dtype=torch.float64, device="cuda").view(3, n_orb)
+    theta, wk = np.random.default_rng(n_orb).uniform(-3, 3, (3, 3)), [0.5, 0.3, 0.2]
+    run = lambda: [kx.kx_vx_kpoints(plan, theta, wk, psi, occ)[0],
+                   kx.kx_vx_apply_kpoint(plan, theta, wk, psi, 1, phi, occ)]
+    few = run()  # the device's SMs: at most 36 blocks of points
+    sms = hooks.hook_num_sms(plan.handle, 1)
+    many = run()
+    hooks.hook_num_sms(plan.handle, sms)
+    assert plan.status() == kx.KX_OK
+    for a, b in zip(few, many):
+        assert torch.equal(a, b)
