@@ -385,7 +385,9 @@ __host__ __device__ constexpr size_t comb_smem(int na) {
 // C row piece it needs is the same for the whole warp (two broadcast float4
 // reads), the A values are consecutive across lanes.  Sums over a stay in
 // float32 (na <= 256 terms).
-// (For rows that are not 16-byte aligned; combine32_bulk_kernel otherwise.)
+// (For rows that are not 16-byte aligned, copied 8 bytes at a time, and for few points;
+// combine32_bulk_kernel otherwise.)
+template <bool VEC2>
 __global__ void __launch_bounds__(256, 2) combine32_kernel(const double *__restrict__ A, int na,
                                                            const double *__restrict__ C, int nb, long long N,
                                                            float sgn, bool accumulate, double *__restrict__ out) {
@@ -408,14 +410,19 @@ __global__ void __launch_bounds__(256, 2) combine32_kernel(const double *__restr
         double *dst = raw + (size_t)(i % kCStages) * kCA * kCX;
         const long long xt = (blockIdx.x + (i / nch) * gridDim.x) * kCX;
         const int r0 = (int)(i % nch) * kCA;
+        constexpr int V = VEC2 ? 2 : 1, per_row = kCX / V;
 #pragma unroll
-        for (int m = 0; m < kCA * kCX / 256; ++m) {
+        for (int m = 0; m < kCA * per_row / 256; ++m) {
             const int piece = tid + 256 * m;
-            const int r = piece / kCX, c = piece % kCX;
+            const int r = piece / per_row, c = piece % per_row * V;
             const long long x = xt + c;
             long long nbytes = (r0 + r < na) ? (N - x) * 8 : 0;
-            nbytes = nbytes < 0 ? 0 : min(nbytes, 8LL);
-            ptx::cp_async8(dst + r * kCX + c, nbytes > 0 ? A + (long long)(r0 + r) * N + x : A, (uint32_t)nbytes);
+            nbytes = nbytes < 0 ? 0 : min(nbytes, 8LL * V);
+            const double *src = nbytes > 0 ? A + (long long)(r0 + r) * N + x : A;
+            if (VEC2)
+                ptx::cp_async16(dst + r * kCX + c, src, (uint32_t)nbytes);
+            else
+                ptx::cp_async8(dst + r * kCX + c, src, (uint32_t)nbytes);
         }
     };
 #pragma unroll
@@ -657,8 +664,13 @@ int launch_combination(kx_plan *p, const double *A, int na, const double *C, int
     } else {
         const int tiles_b = (nb + kCB - 1) / kCB;
         const float fs = sgn < 0.0 ? -1.f : 1.f;
-        // bulk copies: 16-byte aligned rows
-        const bool bulk = N % 2 == 0 && (reinterpret_cast<uintptr_t>(A) & 15) == 0;
+        // bulk copies: 16-byte aligned rows, and CTAs for five SMs of eight; fewer take twice as
+        // long as those of the other kernel, which has twice as many.  An apply (vectors in, out),
+        // other / bulk: 16^3 (16 tiles of points) 64, 64 37 / 45 us, 256, 8 62 / 82; 24 x 24 x 32 (72)
+        // 64, 64 37 / 46; 16 x 16 x 24 (24, four CTAs each) 256, 256 126 / 111; 32^3 (128) 64, 64
+        // 46 / 48, 256, 8 125 / 109
+        const bool aligned = N % 2 == 0 && (reinterpret_cast<uintptr_t>(A) & 15) == 0;
+        const bool bulk = aligned && 8 * ((N + kDX - 1) / kDX) * tiles_b >= 5LL * p->num_sms;
         const long long ntiles = (N + (bulk ? kDX : kCX) - 1) / (bulk ? kDX : kCX);
         const int gx = (int)std::max(1LL, std::min<long long>(ntiles, std::max(1, 2 * p->num_sms / tiles_b)));
         const size_t smem = bulk ? comb_bulk_smem(na) : comb_smem(na);
@@ -669,8 +681,9 @@ int launch_combination(kx_plan *p, const double *A, int na, const double *C, int
             combine32_bulk_kernel<<<grid, 256, smem, s>>>(A, na, C, nb, N, fs, accumulate, out, p->d_status,
                                                           ring_wait_cycles());
         } else {
-            if (int rc = raise_smem(p, reinterpret_cast<const void *>(combine32_kernel), comb_smem(kMaxAce))) return rc;
-            combine32_kernel<<<grid, 256, smem, s>>>(A, na, C, nb, N, fs, accumulate, out);
+            const auto kernel = aligned ? combine32_kernel<true> : combine32_kernel<false>;
+            if (int rc = raise_smem(p, reinterpret_cast<const void *>(kernel), comb_smem(kMaxAce))) return rc;
+            kernel<<<grid, 256, smem, s>>>(A, na, C, nb, N, fs, accumulate, out);
         }
         KX_LAUNCH_CHECK("combine32_kernel launch");
     }

@@ -287,3 +287,21 @@ def test_kpoint_sums_of_few_and_of_many_points(kx, hooks, n, n_orb, n_vec, chunk
     assert plan.status() == kx.KX_OK
     for a, b in zip(few, many):
         assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("n,n_xi,n_vec", [
+    ((16, 8, 8), 1, 1), ((24, 40, 16), 7, 33), ((24, 40, 16), 64, 64), ((32, 16, 40), 65, 130), ((16, 8, 8), 200, 3),
+])
+def test_combinations_of_few_and_of_many_points(kx, hooks, n, n_xi, n_vec):
+    """The combination of grid vectors by bulk copies (many points per SM) and by 8-byte copies (few)
+    against the products in float64: the projections are rounded alike, 2e-6 as elsewhere."""
+    plan = kx.Plan(n, (0.4, 0.45, 0.5), (D, P, D), U, precision=1)
+    xi, phi = rand(n_xi, plan.N) * 0.3, rand(n_vec, plan.N, seed=2)
+    ref = -(0.4 * 0.45 * 0.5) * (phi @ xi.T) @ xi
+    for sms in (1, None):
+        old = hooks.hook_num_sms(plan.handle, sms) if sms else None
+        out = kx.kx_ace_apply(plan, xi, phi)
+        if sms:
+            hooks.hook_num_sms(plan.handle, old)
+        assert plan.status() == kx.KX_OK
+        assert (out - ref).abs().max() < 2e-6 * ref.abs().max()
