@@ -39,6 +39,15 @@ constexpr int kFftPlaneThreads = 512;  // passes A and C: two planes (2 x 104 KB
 constexpr int kFftInPlaceThreads = 256;
 constexpr size_t kFftPlaneSmem = 200 * 1024;  // most a plane may take (fft_supported)
 
+// Axes of kFourStep points have a transform in place (fft80_lines) beside the Stockham
+// stages.  Its second phase has five tasks a line and at most one a thread: every kernel
+// must have five threads for each of the lines it may take at once.
+constexpr int kFourStep = 80;
+__host__ __device__ constexpr bool four_step(int n) { return n == kFourStep; }
+static_assert(5 * kFftLine <= kFftLineThreads, "pass B: a task per thread");
+static_assert(5 * (kMaxN / 2 + 1) <= kFftPlaneThreads, "passes A and C: n1 / 2 + 1 columns, (n2 + 1) / 2 packed rows");
+static_assert(5 * (kFourStep / 2 + 1) <= kFftInPlaceThreads, "planes in place: the same, of 80 points");
+
 struct FftAxis {
     int n, nr;
     int radix[8];
@@ -274,7 +283,7 @@ __device__ __forceinline__ void fft80_lines(float2 *a, int nl, int lstride, int 
 template <int NL, int LS, int ST>
 __device__ __forceinline__ float2 *fft_lines(float2 *a, float2 *b, const FftAxis &ax, int nl, int lstride, int st,
                                              const float2 *W, bool inv) {
-    if (ax.n == 80) {
+    if (four_step(ax.n)) {
         fft80_lines<NL, LS, ST>(a, nl, lstride, st, W, inv);
         return a;
     }
@@ -604,12 +613,12 @@ FftGeom geom(const kx_plan *p) {
     return G;
 }
 
-// both plane axes by the four-step transform, whose second phase has a task per thread at most
-bool plane_in_place(const kx_plan *p) { return p->n[0] == 80 && p->n[1] == 80; }
+// both plane axes have a transform in place
+bool plane_in_place(const kx_plan *p) { return four_step(p->n[0]) && four_step(p->n[1]); }
 size_t plane_smem(const kx_plan *p) {
     return sizeof(float2) * (plane_in_place(p) ? 1 : 2) * (size_t)p->n[1] * (p->n[0] + 1);
 }
-size_t line_smem(const kx_plan *p) { return sizeof(float2) * (p->n[2] == 80 ? 1 : 2) * (size_t)p->n[2] * kFftLine; }
+size_t line_smem(const kx_plan *p) { return sizeof(float2) * (four_step(p->n[2]) ? 1 : 2) * (size_t)p->n[2] * kFftLine; }
 
 }  // namespace
 
