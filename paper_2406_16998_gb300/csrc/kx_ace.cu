@@ -664,13 +664,17 @@ int launch_combination(kx_plan *p, const double *A, int na, const double *C, int
     } else {
         const int tiles_b = (nb + kCB - 1) / kCB;
         const float fs = sgn < 0.0 ? -1.f : 1.f;
-        // bulk copies: 16-byte aligned rows, and CTAs for five SMs of eight; fewer take twice as
-        // long as those of the other kernel, which has twice as many.  An apply (vectors in, out),
-        // other / bulk: 16^3 (16 tiles of points) 64, 64 37 / 45 us, 256, 8 62 / 82; 24 x 24 x 32 (72)
-        // 64, 64 37 / 46; 16 x 16 x 24 (24, four CTAs each) 256, 256 126 / 111; 32^3 (128) 64, 64
-        // 46 / 48, 256, 8 125 / 109
+        // bulk copies: 16-byte aligned rows, and CTAs for three SMs of four; fewer take twice as
+        // long as those of the other kernel, which has twice as many.  Where C leaves room for
+        // one CTA per SM (more than 192 vectors), whole rounds of CTAs count, and one takes 1.56 times
+        // as long as the other's.  An apply (vectors in, out), other / bulk: 16^3 (16 tiles of
+        // points) 64, 64 37 / 45 us, 256, 8 62 / 82; 24 x 24 x 32 (72) 64, 64 37 / 46; 32^3 (128)
+        // 64, 64 46 / 48, 256, 8 125 / 109; 32 x 32 x 40 (160) 64, 64 72 / 64, 256, 8 163 / 171
         const bool aligned = N % 2 == 0 && (reinterpret_cast<uintptr_t>(A) & 15) == 0;
-        const bool bulk = aligned && 8 * ((N + kDX - 1) / kDX) * tiles_b >= 5LL * p->num_sms;
+        const long long c256 = (N + kDX - 1) / kDX * tiles_b, c128 = (N + kCX - 1) / kCX * tiles_b;
+        auto rounds = [&](long long ctas) { return (ctas + p->num_sms - 1) / p->num_sms; };
+        const bool alone = 2 * comb_bulk_smem(na) > 226 * 1024;
+        const bool bulk = aligned && (alone ? 25 * rounds(c128) >= 39 * rounds(c256) : 4 * c256 >= 3LL * p->num_sms);
         const long long ntiles = (N + (bulk ? kDX : kCX) - 1) / (bulk ? kDX : kCX);
         const int gx = (int)std::max(1LL, std::min<long long>(ntiles, std::max(1, 2 * p->num_sms / tiles_b)));
         const size_t smem = bulk ? comb_bulk_smem(na) : comb_smem(na);
