@@ -503,7 +503,7 @@ __host__ __device__ constexpr size_t comb_bulk_smem(int na) {
 __global__ void __launch_bounds__(256, 2) combine32_bulk_kernel(const double *__restrict__ A, int na,
                                                                 const double *__restrict__ C, int nb, long long N,
                                                                 float sgn, bool accumulate, double *__restrict__ out,
-                                                                int *status, long long wait_cycles) {
+                                                                int *status, bool give_up) {
     extern __shared__ __align__(16) uint8_t smem_raw[];
     double *raw = reinterpret_cast<double *>(smem_raw);                                  // [stage][kDR][kDX]
     float *As = reinterpret_cast<float *>(raw + (size_t)kDStages * kDR * kDX);           // [2][kDR][kDX]
@@ -552,7 +552,7 @@ __global__ void __launch_bounds__(256, 2) combine32_bulk_kernel(const double *__
     int ch = 0, st = 0, tile = blockIdx.x;
     uint32_t par = 0;
     for (int i = 0; i < nitems; ++i) {
-        const bool ok = wait_cycles >= 0 && ptx::mbar_wait_bounded(&full[st], par, wait_cycles);
+        const bool ok = !give_up && ptx::mbar_wait_bounded(&full[st], par, kWaitCycles);
         float *at = As + (i & 1) * kDR * kDX;
         const int rows = min(kDR, na - ch * kDR);
         const double *src = raw + st * kDR * kDX + tid;
@@ -683,7 +683,7 @@ int launch_combination(kx_plan *p, const double *A, int na, const double *C, int
             if (int rc = raise_smem(p, reinterpret_cast<const void *>(combine32_bulk_kernel), comb_bulk_smem(kMaxAce)))
                 return rc;
             combine32_bulk_kernel<<<grid, 256, smem, s>>>(A, na, C, nb, N, fs, accumulate, out, p->d_status,
-                                                          ring_wait_cycles());
+                                                          fault_wait());
         } else {
             const auto kernel = aligned ? combine32_kernel<true> : combine32_kernel<false>;
             if (int rc = raise_smem(p, reinterpret_cast<const void *>(kernel), comb_smem(kMaxAce))) return rc;

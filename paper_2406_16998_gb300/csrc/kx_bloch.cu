@@ -1847,7 +1847,7 @@ struct AccBoth {
     double wq, wk;
     double2 *out_k, *out_q;
     int *status;
-    long long wait_cycles;
+    bool give_up;
 };
 
 // a b - c d and a b + c d, rounded as the compiler rounds them in the kernels above
@@ -1909,8 +1909,8 @@ __global__ void __launch_bounds__(kAccPoints) bloch_accum_both_kernel(const AccB
         const float2 f = f_next;
         const float ck = REV ? (float)(a.wk * w_next) : 0.f;
         if (v < v_hi) next(v + 1);
-        const bool ok = a.wait_cycles >= 0 && ptx::mbar_wait_bounded(&full[i % kAccStages],
-                                                                     (uint32_t)((i / kAccStages) & 1), a.wait_cycles);
+        const bool ok =
+            !a.give_up && ptx::mbar_wait_bounded(&full[i % kAccStages], (uint32_t)((i / kAccStages) & 1), kWaitCycles);
         if (ok) {
             const float2 *xs = ring + (i % kAccStages) * MB * kAccPoints + tid;
             float sr = 0.f, si = 0.f;
@@ -2613,7 +2613,7 @@ int bloch_sweep(kx_plan *p, int n_kpt, const double *theta, const double *wk, in
             if constexpr (sizeof(T) == 4) {
                 if (both) {
                     const AccBoth acc = {B,     Pq, F, r0, r1, N, n_orb, occ_q, occ_k, wk[q], wk[k], reinterpret_cast<double2 *>(out_k),
-                                         out_q, p->d_status, ring_wait_cycles()};
+                                         out_q, p->d_status, fault_wait()};
                     rc = n_orb <= 4    ? launch_accum_both<4>(p, acc, s)
                          : n_orb <= 8  ? launch_accum_both<8>(p, acc, s)
                          : n_orb <= 16 ? launch_accum_both<16>(p, acc, s)

@@ -198,10 +198,9 @@ int plan_setup(kx_plan *p);          // eig, f tables, split operands (synchrono
 void plan_free(kx_plan *p);
 
 // ---- workspace (kx_capi.cu)
-// Limit of a wait on a ring of bulk copies (about a second); ring_wait_cycles() is what a
-// launch passes on: this, or -1 (give up untried) under KX_FAULT=wait.
+// Limit of a wait on a ring of bulk copies (about a second).
 constexpr long long kWaitCycles = 2000000000LL;
-long long ring_wait_cycles();
+bool fault_wait();  // KX_FAULT=wait: such a kernel gives up its first wait untried
 int ensure_workspace(kx_plan *p, size_t bytes);
 int ensure_pairs(kx_plan *p, int n_orb, cudaStream_t s, long long begin = 0, long long end = -1);
 

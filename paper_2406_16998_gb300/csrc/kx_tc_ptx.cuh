@@ -333,8 +333,8 @@ __device__ __forceinline__ void bulk_store(void *gdst, const void *ssrc, uint32_
 // A ring of bulk copies left early: item i's copy signals full[i % stages], and the items
 // [first, end) are issued but not waited for.  They land here (bounded waits) before the
 // CTA leaves: a late one would write into the shared memory of the CTA that follows and
-// complete a barrier that is gone.
-__device__ __forceinline__ void bulk_ring_drain(uint64_t *full, int stages, int first, int end, long long max_cycles) {
+// complete a barrier that is gone.  Not inlined: the kernels' loops stay as they are without it.
+inline __device__ __noinline__ void bulk_ring_drain(uint64_t *full, int stages, int first, int end, long long max_cycles) {
     for (int i = first; i < end; ++i) mbar_wait_bounded(&full[i % stages], (uint32_t)((i / stages) & 1), max_cycles);
 }
 __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
