@@ -172,12 +172,14 @@ int ensure_pairs(kx_plan *p, int n_orb, cudaStream_t s, long long begin, long lo
                 span[2 * o + 1] = (int)gi;
                 maxorb[gi] = std::max(maxorb[gi], o);
             }
-    // one block for all tables: one allocation and one copy a list (each table on 256 bytes: on 16
-    // the multipole correction, whose kernels read the mask, took 10 us more of 3,308)
+    // one block for all tables: one allocation and one copy a list.  Each table on a page of its
+    // own: every CTA reads the same entries at the same time, and closer together they cost
+    // the accumulation 15 us of 1,085 (64 x 64 x 96, 64 orbitals, on 256 bytes) and the multipole
+    // correction 10 us (72^3, 40 orbitals, on 16)
     size_t bytes = 0;
     auto place = [&](size_t n) {
         const size_t at = bytes;
-        bytes += (n + 255) & ~size_t(255);
+        bytes += (n + 4095) & ~size_t(4095);
         return at;
     };
     const size_t at_pairs = place(sizeof(int) * pairs.size()), at_slots = place(sizeof(int) * slots.size());
