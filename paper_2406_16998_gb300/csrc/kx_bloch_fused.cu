@@ -10,7 +10,8 @@
 // value far below it keeps fewer bits, and f(Lambda) spans many octaves: with the scale
 // of a row or a tile instead the results differ by 1.6e-8), so in F_MID3 and F_INV21 the
 // CTAs that share an item wait for its maximum between the two products: a cooperative
-// launch, bounded waits, and the store of the tile before in the meantime.
+// launch, bounded waits, and the store of the tile before in the meantime.  Where the CTAs
+// cannot all be resident (bloch_fused_fits) the single products run.
 //
 // What bounds it: six single products move 11 times a chunk's values (537 MB at 64^3 and
 // 256 pairs), these move 5.  Per chunk, forward 523 -> 238 us, middle 459 -> 310 us,
@@ -498,8 +499,8 @@ __global__ void __launch_bounds__(kFuThreads, 1) bloch_fused_kernel(const FuArgs
         };
         // F_MID3, F_INV21: the values between the products into the second A, with the
         // scale of their item's maximum once all its tiles (of this and other CTAs) are in.
-        // Tiles go to the CTAs in order, so a wait is for a tile of this item whose first
-        // product depends on earlier items only.
+        // Tiles go to the CTAs in order and no CTA has two of an item (bloch_fused_fits), so a
+        // wait is for another CTA's tile whose first product depends on earlier items only.
         auto between = [&](int it) {
             const int s = it & 1, t = tile_of(it);
             // a tile's word is its maximum and the mark that it is there: a lane per tile

@@ -26,8 +26,8 @@ namespace kx {
 namespace {
 
 // What bounds the passes is instruction issue and the barriers between their phases, not
-// memory (588 pairs at 80^3, passes A, B, C: 1588, 1042, 1202 us; floors 89, 178 and
-// 177 us): hence lines fixed per thread in pass B (885 us, 768 with five CTAs per SM),
+// memory (588 pairs at 80^3, passes A, B, C: 1588, 1042, 1202 us; floors 182, 363 and
+// 359 us): hence lines fixed per thread in pass B (885 us, 768 with five CTAs per SM),
 // neighbouring values loaded and stored together, packed sums, and planes in place
 // (A 1480 -> 1261 us, with the paired loads 862; C 1034 -> 824 us).
 constexpr int kFftLine = 32;  // lines per CTA in pass B (five CTAs per SM)
@@ -160,10 +160,10 @@ __device__ __forceinline__ void fft_stage(const float2 *a, float2 *b, int n, int
 // With x_p,q = x[p + 16 q] (p < 16, q < 5):
 //   X[k5 + 5 k16] = sum_p W80^(p k5) W16^(p k16) sum_q x_p,q W5^(q k5),
 // so phase 1 takes each p's five values through a 5-point DFT and the twiddle
-// W80^(p k5) (into the scratch buffer at k5 16 + p) and phase 2 takes each
+// W80^(p k5), back into the places it read (k5 16 + p), and phase 2 takes each
 // k5's sixteen values through a 16-point DFT (4 x 4 with twiddles W16^(b k4))
 // into X.  Tasks are ordered lines first, so that with the padded plane rows
-// (or the 64-line columns of pass B) consecutive threads touch distinct banks.
+// (or the 32 lines of pass B) consecutive threads touch distinct banks.
 // W5 and W16 are the constants cos, sin of 2 pi k / 5 and 2 pi k / 16; W80
 // comes from the line's twiddle table.  sg = -1 conjugates (inverse).
 __device__ __forceinline__ void dft4_reg(float2 &v0, float2 &v1, float2 &v2, float2 &v3, float sg) {

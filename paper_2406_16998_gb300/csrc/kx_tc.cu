@@ -1200,7 +1200,9 @@ __global__ void __launch_bounds__(kSlabThreads, 1) tc_slab_kernel(const SlabArgs
             if (a.stage_in) {
                 // task: 8 rows x1 at one x2.  Two tasks' loads first, without branches between them
                 // (batches of 3, 4 and 6 measured 1, 3 and 3% slower): a task past the end
-                // repeats the last one, a padding one reads real values and scales them to zero.  Row groups past np1 are never read (see the quadrants above).
+                // repeats the last one, a padding one reads the plane's first values and scales them to
+                // zero (an infinity or NaN there reaches the padding too; its item is lost with or without
+                // that).  Row groups past np1 are never read (see the quadrants above).
                 for (int t0 = ptid; t0 < ntask; t0 += 2 * n_prod) {
                     float4 x[2][2];
                     int off[2];
@@ -1730,7 +1732,9 @@ size_t pass_smem(int np, int stages, bool with_mid) {
 
 // Producer batch of a pass kernel: a thread has ceil(16 np / kGroupThreads) tasks a
 // tile; at np = 96 its 10 tasks take 2.60 ms as 5 + 5 and 2.70 as 8 + 2 (X3I per apply
-// at 96^3 / 64 orbitals), at np = 80 its 8 are one batch.
+// at 96^3 / 64 orbitals), at np = 80 its 8 are one batch.  Calls of a few tiles take the same
+// either way (one or two vectors at 72^3 42 us with the rule, 43-45 with batches of 7 or 5;
+// 80^3 to 128 x 128 x 64 within 1 us of the best).
 int pass_batch(int np) {
     const int tasks = (16 * np + kGroupThreads - 1) / kGroupThreads;
     if (tasks == 9 || tasks == 10) return 5;
@@ -1791,7 +1795,9 @@ bool slab_fits(const kx_plan *p) {
 // whatever the planes hold, the two passes it replaces go with their values.  Per call
 // (40 orbitals), slab against passes: 48^3 0.48 / 0.45 ms, (80, 48, 64) 1.03 / 0.86 at
 // 4608 and 3840 values a unit; (64, 48, 80) 0.84 / 0.86, 80^3 1.58 / 1.78, 96^3
-// 2.57 / 3.12 at 6144, 6400 and 9216.
+// 2.57 / 3.12 at 6144, 6400 and 9216.  With one to nine orbitals the slab is ahead on every
+// plane, by launches (four orbitals: 16^3 23 / 30 us, (80, 48, 64) 41 / 45, 96^3 67 / 82);
+// the line is drawn where the calls are long.
 bool slab_for_energy(const kx_plan *p) {
     return slab_planes(std::max(p->np[0], p->np[1])) * p->np[0] * p->np[1] >= 6000;
 }
