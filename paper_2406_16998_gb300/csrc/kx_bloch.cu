@@ -2263,12 +2263,12 @@ inline bool bp0_axis(const kx_plan *p) {
 // per value as it is, and other axes have no tensor-core product at all (tc_axis), so those
 // sizes keep the single products; so does a device too small for CTAs that wait for each
 // other (bloch_fused_fits), and KX_BLOCH_FUSED=0 (comparison runs).
-inline int bp_fused(kx_plan *p, bool *fused) {
+inline int bp_fused(kx_plan *p, cudaStream_t s, bool *fused) {
     *fused = false;
     if (const char *e = std::getenv("KX_BLOCH_FUSED"))
         if (std::atoi(e) == 0) return KX_OK;
     if (!(bp_axes(p) && tc_axis(p, 0) && p->n[0] == 64 && p->n[1] == 64)) return KX_OK;
-    return bloch_fused_fits(p, fused);
+    return bloch_fused_fits(p, s, fused);
 }
 
 template <bool FORM>
@@ -2445,7 +2445,7 @@ int bloch_sweep(kx_plan *p, int n_kpt, const double *theta, const double *wk, in
     using T2 = typename Cx<T>::t;
     const long long N = (long long)p->N;
     bool fused;
-    if (int rc = bp_fused(p, &fused)) return rc;
+    if (int rc = bp_fused(p, s, &fused)) return rc;
     BlochLayout L = bloch_layout<T>(p, n_orb, n_vec, n_kpt, fused);
     if (int rc = ensure_workspace(p, L.total)) return rc;
     char *ws = static_cast<char *>(p->ws.ptr);
@@ -2688,7 +2688,7 @@ int bloch_all(kx_plan *p, int n_kpt, const double *theta, const double *wk, int 
     // no sweep, so the workspace may still be unsized (or sized for a smaller
     // call): size it here before any kernel writes into it
     bool fused;
-    if (int rc = bp_fused(p, &fused)) return rc;
+    if (int rc = bp_fused(p, s, &fused)) return rc;
     BlochLayout L = bloch_layout<T>(p, n_orb, n_orb, n_kpt, fused);
     if (int rc = ensure_workspace(p, L.total)) return rc;
     double *partial = reinterpret_cast<double *>(static_cast<char *>(p->ws.ptr) + L.partial);
@@ -2717,7 +2717,7 @@ int bloch_energy_only(kx_plan *p, int n_kpt, const double *theta, const double *
     const long long N = (long long)p->N;
     const long long pairs = (long long)n_orb * n_orb;
     bool fused;
-    if (int rc = bp_fused(p, &fused)) return rc;
+    if (int rc = bp_fused(p, s, &fused)) return rc;
     const long long chunk = bloch_layout<T>(p, n_orb, n_orb, n_kpt, fused).chunk;
     const long long n_launch = (pairs + chunk - 1) / chunk * ((long long)n_kpt * (n_kpt + 1) / 2);
     const size_t slot = (size_t)kBMaxPerSm * p->num_sms;

@@ -646,6 +646,7 @@ int launch_fused(kx_plan *p, FuArgs a, long long R, cudaStream_t s) {
         if (e == cudaErrorCooperativeLaunchTooLarge) {
             // the stream has fewer SMs than the device
             cudaGetLastError();
+            p->fused_refused = true;
             p->prof.launches[PK_BLOCH] -= 1;
             if (int rc = prof_end(p, s)) return rc;
             return kFusedRefused;
@@ -662,9 +663,15 @@ int launch_fused(kx_plan *p, FuArgs a, long long R, cudaStream_t s) {
 // resident (one per SM), and a CTA must never hold two tiles of one item, as it would wait
 // for its own next tile: tiles go to the CTAs in turn and an item has up to 32 neighbouring
 // ones, so 32 CTAs are enough.  *fits = 0 on a smaller share of a device, whose calls
-// take the single products.
-int bloch_fused_fits(kx_plan *p, bool *fits) {
+// take the single products, and, as a refused launch would invalidate it, for a capture
+// with a plan one of whose launches was refused before.
+int bloch_fused_fits(kx_plan *p, cudaStream_t s, bool *fits) {
     *fits = false;
+    if (p->fused_refused) {
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        KX_CUDA_TRY(cudaStreamIsCapturing(s, &cap));
+        if (cap != cudaStreamCaptureStatusNone) return KX_OK;
+    }
     int coop = 0, ctas = p->num_sms;
     KX_CUDA_TRY(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, p->device));
     int rc = p->n[2] == 64 ? fused_resident<F_MID3, 64>(p, &ctas) : fused_resident<F_MID3, 32>(p, &ctas);

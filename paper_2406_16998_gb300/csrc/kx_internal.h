@@ -177,6 +177,7 @@ struct kx_plan_s {
     kx::Workspace mp_scratch;
     std::map<const void *, size_t> smem_limit;                 // raise_smem
     std::map<std::pair<const void *, size_t>, int> resident;  // resident_ctas
+    bool fused_refused = false;  // a cooperative launch of the plan was refused once
 };
 
 namespace kx {
@@ -252,7 +253,7 @@ int bloch_energy(kx_plan *p, int n_kpt, const double *theta, const double *wk, i
 // two products per kernel (kx_bloch_fused.cu); the second and third return kFusedRefused,
 // with nothing launched, where their CTAs cannot all be resident
 constexpr int kFusedRefused = -1;
-int bloch_fused_fits(kx_plan *p, bool *fits);
+int bloch_fused_fits(kx_plan *p, cudaStream_t s, bool *fits);
 int bloch_fused_forward(kx_plan *p, long long R, const float2 *P, const float2 *F, float2 *out, const __half *B1,
                         const __half *B2, const float *pmax, const float *fmax, long long r0, int n_orb,
                         float *out_max, cudaStream_t s);

@@ -305,3 +305,27 @@ def test_combinations_of_few_and_of_many_points(kx, hooks, n, n_xi, n_vec):
             hooks.hook_num_sms(plan.handle, old)
         assert plan.status() == kx.KX_OK
         assert (out - ref).abs().max() < 2e-6 * ref.abs().max()
+
+
+def test_fused_kpoint_products_refused_then_captured(kx, hooks):
+    """A launch that is refused inside a capture would invalidate it: a plan that has met a
+    refusal captures the single products, with the same bits."""
+    plan = kx.Plan((64, 64, 64), (0.3, 0.35, 0.4), (P, P, D), U, precision=1)
+    psi = rand(2, 4, plan.N, cplx=True)
+    theta, wk = [[0.0, 0.0, 0.0], [0.5, 0.2, 0.1]], [0.5, 0.5]
+    want = kx.kx_vx_kpoints(plan, theta, wk, psi)[0].clone()
+    vx, ex = torch.empty_like(psi), torch.empty(1, dtype=torch.float64, device="cuda")
+    old = hooks.hook_num_sms(plan.handle, 4096)
+    try:
+        kx.kx_vx_kpoints(plan, theta, wk, psi, out=vx, e_x=ex)  # refused; sizes the workspace
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            kx.kx_vx_kpoints(plan, theta, wk, psi, out=vx, e_x=ex)
+    finally:
+        hooks.hook_num_sms(plan.handle, old)
+    vx.zero_()
+    graph.replay()
+    torch.cuda.synchronize()
+    assert plan.status() == kx.KX_OK
+    assert torch.equal(vx, want)
