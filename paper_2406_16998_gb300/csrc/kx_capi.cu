@@ -33,7 +33,8 @@ int cuda_error(cudaError_t e, const char *what) {
 
 // Host-side fault injection for the failure-path tests, read at each call: KX_FAULT=alloc
 // makes the next workspace allocation report KX_ERR_NOMEM without touching the device,
-// KX_FAULT=wait makes the kernels with a ring of bulk copies give up their first wait.
+// KX_FAULT=host makes the host allocation of a pair list throw, KX_FAULT=wait makes the
+// kernels with a ring of bulk copies give up their first wait.
 static bool fault(const char *what) {
     const char *f = std::getenv("KX_FAULT");
     return f && std::strcmp(f, what) == 0;
@@ -42,10 +43,13 @@ static bool fault_alloc() { return fault("alloc"); }
 bool fault_wait() { return fault("wait"); }
 
 int raise_smem(kx_plan *p, const void *kernel, size_t bytes) {
-    size_t &limit = p->smem_limit[kernel];
-    if (limit >= bytes) return KX_OK;
+    const auto known = p->smem_limit.find(kernel);
+    if (known != p->smem_limit.end() && known->second >= bytes) return KX_OK;
     KX_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
-    limit = bytes;
+    try {
+        p->smem_limit[kernel] = bytes;
+    } catch (const std::bad_alloc &) {  // asked again next time
+    }
     return KX_OK;
 }
 
@@ -56,7 +60,10 @@ int resident_ctas(kx_plan *p, const void *kernel, int threads, size_t smem, int 
         return KX_OK;
     }
     KX_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, kernel, threads, smem));
-    p->resident[{kernel, smem}] = *per_sm;
+    try {
+        p->resident[{kernel, smem}] = *per_sm;
+    } catch (const std::bad_alloc &) {  // asked again next time
+    }
     return KX_OK;
 }
 
@@ -98,7 +105,7 @@ int leading_columns(int nb) {
 
 // With p->blk_mode set, the block pairs of p->blk_req (I <= J each, in the
 // given order) are enumerated instead, each whole; begin / end are ignored.
-int ensure_pairs(kx_plan *p, int n_orb, cudaStream_t s, long long begin, long long end) {
+static int build_pairs(kx_plan *p, int n_orb, cudaStream_t s, long long begin, long long end) {
     const long long P_all = (long long)n_orb * (n_orb + 1) / 2;
     if (end < 0) end = P_all;
     if (p->blk_mode) {
@@ -185,6 +192,7 @@ int ensure_pairs(kx_plan *p, int n_orb, cudaStream_t s, long long begin, long lo
     const size_t at_pairs = place(sizeof(int) * pairs.size()), at_slots = place(sizeof(int) * slots.size());
     const size_t at_groups = place(sizeof(Group) * groups.size()), at_span = place(sizeof(int) * span.size());
     const size_t at_mask = place(mask.size());
+    if (fault("host")) throw std::bad_alloc();
     std::vector<unsigned char> host(bytes);
     auto put = [&](size_t at, const void *src, size_t n) {
         if (n) std::memcpy(host.data() + at, src, n);
@@ -236,6 +244,14 @@ int ensure_pairs(kx_plan *p, int n_orb, cudaStream_t s, long long begin, long lo
     else
         p->blk_cur.clear();
     return KX_OK;
+}
+
+int ensure_pairs(kx_plan *p, int n_orb, cudaStream_t s, long long begin, long long end) {
+    try {
+        return build_pairs(p, n_orb, s, begin, end);
+    } catch (const std::bad_alloc &) {
+        return set_error(KX_ERR_NOMEM, "host allocation of the pair list failed");
+    }
 }
 
 static int prof_event(kx_plan *p, cudaEvent_t *out) {

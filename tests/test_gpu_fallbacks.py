@@ -88,6 +88,24 @@ def test_pair_list_after_a_failed_allocation(kx, prec, monkeypatch):
 
 
 @pytest.mark.parametrize("prec", [0, 1])
+def test_pair_list_without_host_memory(kx, prec, monkeypatch):
+    """A host allocation that throws while a pair list is made becomes an error code at the C
+    boundary; the list before it, and the plain one after a call with explicit blocks, hold."""
+    plan = kx.Plan((16, 24, 16), (0.4, 0.45, 0.5), (D, P, D), U, precision=prec)
+    psi = rand(12, plan.N)
+    want, ex = (t.clone() for t in kx.kx_vx_apply(plan, psi))
+    monkeypatch.setenv("KX_FAULT", "host")
+    for call in (lambda: kx.kx_vx_apply(plan, psi[:7].contiguous()),
+                 lambda: kx.kx_vx_apply_block_pairs(plan, psi, [(0, 1), (2, 2)])):
+        with pytest.raises(kx.KxError) as ei:
+            call()
+        assert ei.value.code == kx.KX_ERR_NOMEM
+    monkeypatch.delenv("KX_FAULT")
+    got, ex2 = kx.kx_vx_apply(plan, psi)
+    assert torch.equal(got, want) and torch.equal(ex2, ex)
+
+
+@pytest.mark.parametrize("prec", [0, 1])
 def test_pair_lists_in_turn_on_a_side_stream(kx, prec):
     """Calls with two orbital counts back to back on a stream that does not synchronise with
     the default one: each runs with its own pair list."""
